@@ -40,30 +40,64 @@ template <typename C> __device__ __forceinline__ C from64(double2 a);
 template <> __device__ __forceinline__ float2 from64<float2>(double2 a) { return make_float2((float)a.x, (float)a.y); }
 template <> __device__ __forceinline__ double2 from64<double2>(double2 a) { return a; }
 
-// Sum NV values over the CTA in a fixed order (warp shuffle tree, then warps in
-// index order).  Warp stages run in the accumulator type; the cross-warp stage
-// in double.  Result valid in thread 0.  `red` must hold 32*NV doubles.
+// Sum V values (a power of two <= 32) over the warp; lane l returns the total
+// of value l % V.  At each shuffle a lane gives away half of the sums it holds:
+// V - 1 + log2(32 / V) adds instead of 5 V.  On this GPU a warp's FP64 add
+// occupies its FP64 pipe for 64 cycles, so reductions count their instructions.
+template <int V, typename A>
+__device__ __forceinline__ A warp_sum_many(A (&v)[V]) {
+  const int lane = threadIdx.x & 31;
+#pragma unroll
+  for (int w = V / 2; w >= 1; w >>= 1) {
+    const bool up = (lane & w) != 0;
+#pragma unroll
+    for (int j = 0; j < w; ++j) {
+      const A send = up ? v[j] : v[j + w];
+      const A keep = up ? v[j + w] : v[j];
+      v[j] = keep + __shfl_xor_sync(0xffffffffu, send, w);
+    }
+  }
+  A t = v[0];
+#pragma unroll
+  for (int w = V; w < 32; w <<= 1) t += __shfl_xor_sync(0xffffffffu, t, w);
+  return t;
+}
+
+// a / b on a whole warp (every lane passes the same operands): the two real
+// divisions run in different lanes of one instruction stream
+__device__ __forceinline__ double2 cdiv_warp(double2 a, double2 b) {
+  const bool im = (threadIdx.x & 1) != 0;
+  const double den = b.x * b.x + b.y * b.y;
+  const double num = im ? a.y * b.x - a.x * b.y : a.x * b.x + a.y * b.y;
+  const double q = num / den;
+  return make_double2(__shfl_sync(0xffffffffu, q, 0), __shfl_sync(0xffffffffu, q, 1));
+}
+
+// Sum NV values over the CTA in a fixed order (warp tree, then the warps' sums
+// over the first warp's lanes).  Warp stages run in the accumulator type; the
+// cross-warp stage in double.  Result valid in thread 0 (every lane of warp 0).
+// `red` must hold 32 * (NV rounded up to a power of two) doubles.
 template <int NV, typename A>
 __device__ __forceinline__ void block_sum(A (&v)[NV], double* red, double (&out)[NV]) {
+  constexpr int V = NV <= 1 ? 1 : NV <= 2 ? 2 : 4;
+  static_assert(NV <= 4, "block_sum");
+  A w[V];
 #pragma unroll
-  for (int i = 0; i < NV; ++i) {
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) v[i] += __shfl_down_sync(0xffffffffu, v[i], o);
-  }
+  for (int i = 0; i < V; ++i) w[i] = i < NV ? v[i < NV ? i : 0] : (A)0;
+  const A t = warp_sum_many<V>(w);
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  if (lane == 0) {
-#pragma unroll
-    for (int i = 0; i < NV; ++i) red[warp * NV + i] = (double)v[i];
-  }
+  A* part = reinterpret_cast<A*>(red);
+  if (lane < V) part[warp * V + lane] = t;
   __syncthreads();
-  if (threadIdx.x == 0) {
-    const int nw = (blockDim.x + 31) >> 5;
+  if (warp == 0) {
+    const int n = ((blockDim.x + 31) >> 5) * V;
+    double s = 0.0;
+    for (int e = lane; e < n; e += 32) s += (double)part[e];
 #pragma unroll
-    for (int i = 0; i < NV; ++i) {
-      double s = 0.0;
-      for (int w = 0; w < nw; ++w) s += red[w * NV + i];
-      out[i] = s;
-    }
+    for (int o = V; o < 32; o <<= 1)
+      if (o < n) s += __shfl_xor_sync(0xffffffffu, s, o);
+#pragma unroll
+    for (int i = 0; i < NV; ++i) out[i] = __shfl_sync(0xffffffffu, s, i);
   }
   __syncthreads();
 }

@@ -364,14 +364,29 @@ __device__ __forceinline__ void op_tile(const JuncDev* __restrict__ jt, const Ba
     double out[2];
     block_sum<2>(v, red, out);
     if (tid == 0) b.mu_part[(size_t)s * b.PA + tile] = make_double2(out[0], out[1]);
+    if (tid < 32) mu_arrive(b, J, s);
   } else if constexpr (MODE == OP_RESID) {
     CT v[4] = {acc0, acc1, acc2, acc3};
     double out[4];
     block_sum<4>(v, red, out);
-    if (tid == 0) {
-      b.t0_part[(size_t)s * b.PA + tile] = out[3];
-      b.nrm0_part[(size_t)s * b.PA + tile] = out[0];
-      b.rho0_part[(size_t)s * b.PA + tile] = make_double2(out[1], out[2]);
+    // the slot's last CTA adds the partials: ||r||^2, r^T r, T partial
+    if (tid < 32) {
+      double* part = b.res_part + 4 * (size_t)s * b.PA;
+      int done = 0;
+      if (tid == 0) {
+        for (int i = 0; i < 4; ++i) part[4 * tile + i] = out[i];
+        __threadfence();
+        done = atomicAdd(b.res_cnt + s, 1);
+      }
+      if (__shfl_sync(0xffffffffu, done, 0) == J.nA - 1) {
+        __threadfence();
+        double w[4] = {0.0, 0.0, 0.0, 0.0};
+        for (int t = tid; t < J.nA; t += 32)
+          for (int i = 0; i < 4; ++i) w[i] += __ldcg(part + 4 * t + i);
+        const double t = warp_sum_many<4>(w);
+        if (tid < 4) b.res_tot[4 * s + tid] = t;
+        if (tid == 0) b.res_cnt[s] = 0;
+      }
     }
   }
 }
@@ -623,6 +638,7 @@ op_kernel_tma(const JuncDev* __restrict__ jt, const BatchDev* __restrict__ bp, c
     double out[2];
     block_sum<2>(vv, red, out);
     if (tid == 0) b.mu_part[(size_t)s * b.PA + tile] = make_double2(out[0], out[1]);
+    if (tid < 32) mu_arrive(b, J, s);
   }
 }
 

@@ -53,6 +53,38 @@ __device__ __forceinline__ void kahan_add_f(float& sum, float& carry, float term
   sum = t;
 }
 
+// End of an operator or projection CTA of slot s, by its first warp once lane 0
+// has written the CTA's partial of mu = p^T A p: the CTA that arrives last adds
+// the J.nA operator partials and the J.n_groups projection partials (lanes in
+// stride, then a shuffle tree: a fixed order for a given tiling) and forms
+// alpha = rho / mu, once per system instead of in every update CTA.
+__device__ __forceinline__ void mu_arrive(const BatchDev& b, const JuncDev& J, const int s) {
+  const int lane = threadIdx.x & 31;
+  const int n = J.nA + J.n_groups;
+  int done = 0;
+  if (lane == 0) {
+    __threadfence();
+    done = atomicAdd(b.mu_cnt + s, 1);
+  }
+  done = __shfl_sync(0xffffffffu, done, 0);
+  if (done != n - 1) return;
+  __threadfence();
+  double v[2] = {0.0, 0.0};
+  for (int t = lane; t < n; t += 32) {
+    const double2 w = __ldcg(b.mu_part + (size_t)s * b.PA + t);
+    v[0] += w.x;
+    v[1] += w.y;
+  }
+  const double t = warp_sum_many<2>(v);
+  const double2 mu = make_double2(__shfl_sync(0xffffffffu, t, 0), __shfl_sync(0xffffffffu, t, 1));
+  const double2 a = cdiv_warp(b.rho_cur[s], mu);
+  if (lane == 0) {
+    b.mu_cnt[s] = 0;
+    b.alpha[s] = a;
+    if (b.n_shift > 0) b.salpha[(size_t)(b.iters[s] & 1) * b.nslots + s] = a;
+  }
+}
+
 struct Pair {
   float2 a, b;  // values at x0 and x0 + 1
 };
@@ -315,6 +347,7 @@ op_pair_kernel(const JuncDev* __restrict__ jt, const BatchDev* __restrict__ bp, 
     double out[2];
     block_sum<2>(vv, red, out);
     if (tid == 0) b.mu_part[(size_t)s * b.PA + tile] = make_double2(out[0], out[1]);
+    if (tid < 32) mu_arrive(b, J, s);
   }
 }
 
@@ -537,6 +570,7 @@ op_plane_kernel(const JuncDev* __restrict__ jt, const BatchDev* __restrict__ bp,
     double out[2];
     block_sum<2>(vv, red, out);
     if (tid == 0) b.mu_part[(size_t)s * b.PA + tile] = make_double2(out[0], out[1]);
+    if (tid < 32) mu_arrive(b, J, s);
   }
 }
 

@@ -12,6 +12,7 @@
 // (queue position, busy slots).  Everything else stays on the GPU.
 #include <algorithm>
 #include <chrono>
+#include <climits>
 #include <cmath>
 #include <cstdio>
 #include <cstdlib>
@@ -75,7 +76,7 @@ struct Workspace {
   DevBuf Xslot, r, p0, p1, q, d;
   DevBuf state, sys, junc, E, col, voff, xo, xfo, iters, total_iters, cyc_iters, n_upd, restart, stall, warm, rho_cur, beta_cur;
   DevBuf bnorm2, sigma, rlast2, rrec2, tol2;
-  DevBuf rho0, nrm0, t0, tlast, gcnt, gphase, tgoal, rgoal, rho, nrm, mu, c_r, c_p, c_x, sched, counters, lst, lst_n,
+  DevBuf res_part, res_cnt, res_tot, tlast, gcnt, gphase, tgoal, rgoal, rho, nrm, mu, mu_cnt, alpha, upd_cnt, c_r, c_p, c_x, sched, counters, lst, lst_n,
       inlist, fslot, c_e;
   int generation = 0;
 };
@@ -108,7 +109,7 @@ struct ShiftSpec {
 struct PoolSpec {
   int K = 0, R = 0;
   long long N = 0;  // the largest junction: slot vectors are this long
-  int n_proj = 0, n_groups = 0, max_np = 1, nB = 0, nS = 0, PA = 0, PB = 0;
+  int n_proj = 0, n_groups = 0, max_np = 1, nB = 0, PA = 0, PB = 0;
   Tiling inner[4];                        // launch configuration per operator kind (OpKind)
   bool has[4] = {false, false, false, false};
   Tiling resid;                           // launch configuration of the true-residual kernel
@@ -139,7 +140,9 @@ struct rsn_ctx {
   cudaStream_t user_stream = nullptr;
   cudaStream_t st = nullptr;
   cudaStream_t st2 = nullptr;  // second stream: the true-residual path beside the COCG step
-  cudaEvent_t ev_in = nullptr, ev_out = nullptr, t0 = nullptr, t1 = nullptr, ev_fork = nullptr, ev_join = nullptr;
+  cudaStream_t st3 = nullptr;  // third stream: the projections of r beside the COCG operator
+  cudaEvent_t ev_in = nullptr, ev_out = nullptr, t0 = nullptr, t1 = nullptr, ev_fork = nullptr, ev_join = nullptr, ev_step = nullptr,
+              ev_proj = nullptr;
   std::string err;
 
   bool has_grid = false, has_v = false, has_cap = false;
@@ -154,8 +157,7 @@ struct rsn_ctx {
   bool dirty = true;
 
   // device operator data
-  DevBuf dg64, dg32, gld, L_idx, L_gam, inv_ptr, inv_p0, inv_q64, inv_q32, sup_pts;
-  int n_sup = 0;
+  DevBuf dg64, dg32, gld, L_idx, L_gam, inv_ptr, inv_p0, inv_q64, inv_q32, blk_row, row_meta, row_loc, row_q64, row_q32;
   DevBuf grp_ptr, grp_p0, grp_np, grp_voff, grp_idx, grp_val64, grp_val32, ekb;
   int n_groups = 0, nL = 0, max_np = 1;
   JuncDev jh{};
@@ -415,12 +417,7 @@ static rsn_status commit_setup(rsn_ctx* c) {
   const int G = c->n_groups;
   for (int g = 0; g < G; ++g)
     for (int k = gptr[g]; k < gptr[g + 1]; ++k) cnt[gidx[k] + 1]++;
-  std::vector<int> sup;  // grid points inside at least one projector support
-  for (long long i = 0; i < N; ++i) {
-    if (cnt[i + 1] > 0) sup.push_back((int)i);
-    cnt[i + 1] += cnt[i];
-  }
-  c->n_sup = (int)sup.size();
+  for (long long i = 0; i < N; ++i) cnt[i + 1] += cnt[i];
   const size_t nent = (size_t)cnt[N];
   std::vector<int> ip0(std::max<size_t>(1, nent)), fill(cnt.begin(), cnt.end() - 1);
   std::vector<double> iq64(std::max<size_t>(1, nent) * 4 * nq, 0.0);
@@ -434,6 +431,51 @@ static rsn_status commit_setup(rsn_ctx* c) {
     }
   }
   std::vector<float> iq32(iq64.begin(), iq64.end()), gvalf(gval.begin(), gval.end());
+  // the same entries by blocks of kBlkPts points, for the update kernel: rows of
+  // up to 32 points of one atom inside one block, atoms in order.  A point that
+  // an atom's index list repeats goes to a further row, so that a row holds each
+  // of its points once.
+  const int nblk = (int)((N + kBlkPts - 1) / kBlkPts);
+  std::vector<int> brow(nblk + 1, 0);
+  std::vector<int2> rmeta;
+  std::vector<unsigned char> rloc;
+  std::vector<double> rq64;
+  {
+    struct Ent { int blk, g, rep, loc, k; };
+    std::vector<Ent> ents;
+    ents.reserve(nent);
+    std::vector<int> seen(N, -1), rep(N, 0);
+    for (int g = 0; g < G; ++g)
+      for (int k = 0; k < gptr[g + 1] - gptr[g]; ++k) {
+        const int i = gidx[gptr[g] + k];
+        rep[i] = seen[i] == g ? rep[i] + 1 : 0;
+        seen[i] = g;
+        ents.push_back({i / kBlkPts, g, rep[i], i % kBlkPts, k});
+      }
+    std::sort(ents.begin(), ents.end(), [](const Ent& a, const Ent& b) {
+      return std::tie(a.blk, a.g, a.rep, a.loc) < std::tie(b.blk, b.g, b.rep, b.loc);
+    });
+    for (size_t e = 0; e < ents.size();) {
+      const Ent& f = ents[e];
+      size_t e1 = e;
+      while (e1 < ents.size() && e1 - e < 32 && ents[e1].blk == f.blk && ents[e1].g == f.g && ents[e1].rep == f.rep) ++e1;
+      const size_t row = rmeta.size();
+      rmeta.push_back(make_int2(gp0[f.g], (int)(e1 - e)));
+      rloc.resize((row + 1) * 32, 0);
+      rq64.resize((row + 1) * 32 * 4 * nq, 0.0);
+      const int len = gptr[f.g + 1] - gptr[f.g];
+      for (size_t x = e; x < e1; ++x) {
+        const int lane = (int)(x - e);
+        rloc[row * 32 + lane] = (unsigned char)ents[x].loc;
+        for (int j = 0; j < gnp[f.g]; ++j)
+          rq64[((row * nq + j / 4) * 32 + lane) * 4 + j % 4] = gval[gvoff[f.g] + (size_t)j * len + ents[x].k];
+      }
+      brow[f.blk + 1] += 1;
+      e = e1;
+    }
+    for (int k = 0; k < nblk; ++k) brow[k + 1] += brow[k];
+  }
+  std::vector<float> rq32(rq64.begin(), rq64.end());
   auto up = [&](DevBuf& b, const void* src, size_t bytes) -> cudaError_t {
     cudaError_t e = b.ensure(std::max<size_t>(bytes, 16));
     if (e != cudaSuccess) return e;
@@ -442,7 +484,11 @@ static rsn_status commit_setup(rsn_ctx* c) {
   };
   RSN_CUDA(c, up(c->inv_ptr, cnt.data(), (N + 1) * sizeof(int)));
   RSN_CUDA(c, up(c->inv_p0, ip0.data(), nent * sizeof(int)));
-  RSN_CUDA(c, up(c->sup_pts, sup.data(), sup.size() * sizeof(int)));
+  RSN_CUDA(c, up(c->blk_row, brow.data(), brow.size() * sizeof(int)));
+  RSN_CUDA(c, up(c->row_meta, rmeta.data(), rmeta.size() * sizeof(int2)));
+  RSN_CUDA(c, up(c->row_loc, rloc.data(), rloc.size()));
+  RSN_CUDA(c, up(c->row_q64, rq64.data(), rq64.size() * sizeof(double)));
+  RSN_CUDA(c, up(c->row_q32, rq32.data(), rq32.size() * sizeof(float)));
   RSN_CUDA(c, up(c->inv_q64, iq64.data(), nent * 4 * nq * sizeof(double)));
   RSN_CUDA(c, up(c->inv_q32, iq32.data(), nent * 4 * nq * sizeof(float)));
   RSN_CUDA(c, up(c->grp_ptr, gptr.data(), gptr.size() * sizeof(int)));
@@ -479,9 +525,11 @@ static rsn_status commit_setup(rsn_ctx* c) {
   J.inv_p0 = c->inv_p0.as<int>();
   J.inv_q64 = c->inv_q64.as<double2>();
   J.inv_q32 = c->inv_q32.as<float4>();
-  J.sup_pts = c->sup_pts.as<int>();
-  J.n_sup = c->n_sup;
-  J.nS = (c->n_sup + kVecPts - 1) / kVecPts;
+  J.blk_row = c->blk_row.as<int>();
+  J.row_meta = c->row_meta.as<int2>();
+  J.row_loc = c->row_loc.as<unsigned char>();
+  J.row_q64 = c->row_q64.as<double2>();
+  J.row_q32 = c->row_q32.as<float4>();
   J.grp_ptr = c->grp_ptr.as<int>();
   J.grp_p0 = c->grp_p0.as<int>();
   J.grp_np = c->grp_np.as<int>();
@@ -499,7 +547,7 @@ static rsn_status commit_setup(rsn_ctx* c) {
 
 // Device JuncDev copies for one launch configuration: copy 0 carries the tiling
 // of the COCG / apply operator kernel, copy 1 that of the FP64 true-residual
-// kernel; both record the residual kernel's CTA count (nR) for its partials.
+// kernel.
 struct LaunchCfg {
   Tiling inner, resid;
   const JuncDev* jt_inner;  // device pointer: tiling of the COCG / apply kernel
@@ -517,7 +565,6 @@ static rsn_status make_cfg(rsn_ctx* c, const Tiling& inner, const Tiling& resid,
     js[k].ytiles = t.ytiles;
     js[k].ztiles = t.ztiles;
     js[k].nA = t.n;
-    js[k].nR = cfg.resid.n;
     js[k].kind = k == 1 ? kOpReg : t.plane ? kOpPlane : t.pair ? kOpPair : t.tma ? kOpTma : kOpReg;
   }
   RSN_CUDA(c, cudaMemcpyAsync(c->jd.p, js, 2 * sizeof(JuncDev), cudaMemcpyHostToDevice, c->st));
@@ -580,6 +627,9 @@ rsn_status rsn_create(rsn_ctx** out, int device, void* cuda_stream) {
   c->user_stream = reinterpret_cast<cudaStream_t>(cuda_stream);
   if (cudaStreamCreateWithFlags(&c->st, cudaStreamNonBlocking) != cudaSuccess ||
       cudaStreamCreateWithFlags(&c->st2, cudaStreamNonBlocking) != cudaSuccess ||
+      cudaStreamCreateWithFlags(&c->st3, cudaStreamNonBlocking) != cudaSuccess ||
+      cudaEventCreateWithFlags(&c->ev_step, cudaEventDisableTiming) != cudaSuccess ||
+      cudaEventCreateWithFlags(&c->ev_proj, cudaEventDisableTiming) != cudaSuccess ||
       cudaEventCreateWithFlags(&c->ev_fork, cudaEventDisableTiming) != cudaSuccess ||
       cudaEventCreateWithFlags(&c->ev_join, cudaEventDisableTiming) != cudaSuccess ||
       cudaEventCreateWithFlags(&c->ev_in, cudaEventDisableTiming) != cudaSuccess ||
@@ -601,6 +651,7 @@ rsn_status rsn_destroy(rsn_ctx* c) {
   cudaSetDevice(c->device);
   if (c->st) cudaStreamSynchronize(c->st);
   if (c->st2) cudaStreamSynchronize(c->st2);
+  if (c->st3) cudaStreamSynchronize(c->st3);
   clear_graphs(c);
   for (cudaEvent_t e : c->tev) cudaEventDestroy(e);
   if (c->sched_host) cudaFreeHost(c->sched_host);
@@ -611,6 +662,9 @@ rsn_status rsn_destroy(rsn_ctx* c) {
   if (c->t1) cudaEventDestroy(c->t1);
   if (c->ev_fork) cudaEventDestroy(c->ev_fork);
   if (c->ev_join) cudaEventDestroy(c->ev_join);
+  if (c->ev_step) cudaEventDestroy(c->ev_step);
+  if (c->ev_proj) cudaEventDestroy(c->ev_proj);
+  if (c->st3) cudaStreamDestroy(c->st3);
   if (c->st2) cudaStreamDestroy(c->st2);
   if (c->st) cudaStreamDestroy(c->st);
   delete c;
@@ -779,7 +833,7 @@ static rsn_status ensure_ws(rsn_ctx* c, bool fp32, int S, const PoolSpec* pool =
     const Tiling ti = choose_tiling(c, !fp32, OP_COCG, S), tr = choose_tiling(c, true, OP_RESID, S);
     // mu partials: the operator tiles', then one per atom (projection kernel)
     PA = std::max(ti.n + c->n_groups, tr.n);
-    PB = c->jh.nB;
+    PB = upd_ctas(N, upd_warps(N, S));
   }
   if (w.slots == S && w.fp32 == fp32 && w.N == N && w.PA == PA && w.PB == PB && w.n_proj == n_proj)
     return RSN_OK;
@@ -814,15 +868,18 @@ static rsn_status ensure_ws(rsn_ctx* c, bool fp32, int S, const PoolSpec* pool =
   RSN_CUDA(c, w.rlast2.ensure(sd));
   RSN_CUDA(c, w.rrec2.ensure(sd));
   RSN_CUDA(c, w.tol2.ensure(sd));
-  RSN_CUDA(c, w.rho0.ensure((size_t)S * PA * sizeof(double2)));
-  RSN_CUDA(c, w.nrm0.ensure((size_t)S * PA * sizeof(double)));
-  RSN_CUDA(c, w.t0.ensure((size_t)S * PA * sizeof(double)));
+  RSN_CUDA(c, w.res_part.ensure(4 * (size_t)S * PA * sizeof(double)));
+  RSN_CUDA(c, w.res_cnt.ensure(si));
+  RSN_CUDA(c, w.res_tot.ensure(4 * sd));
   RSN_CUDA(c, w.tlast.ensure(sd));
   RSN_CUDA(c, w.gcnt.ensure(si));
   RSN_CUDA(c, w.gphase.ensure(si));
   RSN_CUDA(c, w.tgoal.ensure(sd));
   RSN_CUDA(c, w.rgoal.ensure(sd));
   RSN_CUDA(c, w.mu.ensure((size_t)S * PA * sizeof(double2)));
+  RSN_CUDA(c, w.mu_cnt.ensure(si));
+  RSN_CUDA(c, w.alpha.ensure(S * sizeof(double2)));
+  RSN_CUDA(c, w.upd_cnt.ensure(si));
   RSN_CUDA(c, w.rho.ensure((size_t)S * PB * sizeof(double2)));
   RSN_CUDA(c, w.nrm.ensure((size_t)S * PB * sizeof(double)));
   const size_t npj = std::max(1, n_proj);
@@ -940,9 +997,9 @@ static BatchDev slot_batch(rsn_ctx* c, int S, const rsn_solver_opts* o) {
   b.p1 = w.p1.p;
   b.q = w.q.p;
   b.d = w.d.p;
-  b.rho0_part = w.rho0.as<double2>();
-  b.nrm0_part = w.nrm0.as<double>();
-  b.t0_part = w.t0.as<double>();
+  b.res_part = w.res_part.as<double>();
+  b.res_cnt = w.res_cnt.as<int>();
+  b.res_tot = w.res_tot.as<double>();
   b.tlast = w.tlast.as<double>();
   b.gcnt = w.gcnt.as<int>();
   b.gphase = w.gphase.as<int>();
@@ -951,6 +1008,9 @@ static BatchDev slot_batch(rsn_ctx* c, int S, const rsn_solver_opts* o) {
   b.rho_part = w.rho.as<double2>();
   b.nrm_part = w.nrm.as<double>();
   b.mu_part = w.mu.as<double2>();
+  b.mu_cnt = w.mu_cnt.as<int>();
+  b.alpha = w.alpha.as<double2>();
+  b.upd_cnt = w.upd_cnt.as<int>();
   b.c_r = w.c_r.p;
   b.c_p = w.c_p.p;
   b.c_x = w.c_x.as<double2>();
@@ -1009,6 +1069,9 @@ static rsn_status run_stream(rsn_ctx* c, const rsn_solver_opts* o, const StreamI
   if (want_t) RSN_CUDA(c, cudaMemsetAsync(q.out_t.p, 0, nsys * sizeof(double), st));
   // slot pool starts empty
   RSN_CUDA(c, cudaMemsetAsync(w.state.p, 0, S * sizeof(int), st));
+  RSN_CUDA(c, cudaMemsetAsync(w.mu_cnt.p, 0, S * sizeof(int), st));
+  RSN_CUDA(c, cudaMemsetAsync(w.upd_cnt.p, 0, S * sizeof(int), st));
+  RSN_CUDA(c, cudaMemsetAsync(w.res_cnt.p, 0, S * sizeof(int), st));
   RSN_CUDA(c, cudaMemsetAsync(w.sched.p, 0, (3 + 2 * kMaxGraphIters) * sizeof(int), st));
   RSN_CUDA(c, cudaMemsetAsync(w.counters.p, 0, 4 * sizeof(unsigned long long), st));
 
@@ -1076,7 +1139,7 @@ static rsn_status run_stream(rsn_ctx* c, const rsn_solver_opts* o, const StreamI
   LaunchCfg cfg;
   const JuncDev* ji;
   const JuncDev* jr;
-  int nB, n_groups, max_np, nS, R;
+  int nB, n_groups, max_np, R;
   bool proj;
   if (pool) {
     ji = pool->ji;
@@ -1086,7 +1149,6 @@ static rsn_status run_stream(rsn_ctx* c, const rsn_solver_opts* o, const StreamI
     proj = pool->n_proj > 0;
     n_groups = pool->n_groups;
     max_np = pool->max_np;
-    nS = pool->nS;
     R = pool->R;
   } else {
     if ((rs = make_cfg(c, fp32, S, cfg)) != RSN_OK) return rs;
@@ -1096,11 +1158,9 @@ static rsn_status run_stream(rsn_ctx* c, const rsn_solver_opts* o, const StreamI
     proj = c->n_proj > 0;
     n_groups = c->n_groups;
     max_np = c->max_np;
-    nS = c->jh.nS;
     R = c->R;
   }
   const bool multi = pool && pool->K > 1;
-  const int ce_stride = b.ce_stride;
   const int KL = std::min(S, kListRows);
   const bool goal = o->tol_T > 0 && !sh;
   const dim3 gr(cfg.resid.n, KL);
@@ -1158,10 +1218,19 @@ static rsn_status run_stream(rsn_ctx* c, const rsn_solver_opts* o, const StreamI
         if ((e = residual_path()) != cudaSuccess) return e;
         if ((e = cudaEventRecord(c->ev_join, st2)) != cudaSuccess) return e;
       }
-      // COCG step of the ACTIVE slots (main stream)
-      if (proj && (e = launch_project(0, fp32, S, n_groups, max_np, st, ji, bdev, nullptr, w.c_r.p, multi)) !=
-                      cudaSuccess)
-        return e;
+      // COCG step of the ACTIVE slots (main stream).  The operator and the
+      // projections of r need nothing of one another: they run side by side
+      // (one after the other when the launches are timed)
+      if (proj) {
+        cudaStream_t sp = timing ? st : c->st3;
+        if (!timing) {
+          if ((e = cudaEventRecord(c->ev_step, st)) != cudaSuccess) return e;
+          if ((e = cudaStreamWaitEvent(sp, c->ev_step, 0)) != cudaSuccess) return e;
+        }
+        if ((e = launch_project(0, fp32, S, n_groups, max_np, sp, ji, bdev, nullptr, w.c_r.p, multi)) != cudaSuccess)
+          return e;
+        if (!timing && (e = cudaEventRecord(c->ev_proj, sp)) != cudaSuccess) return e;
+      }
       if (timing && (e = cudaEventRecordWithFlags(c->tev[4 * it], st, evf)) != cudaSuccess) return e;
       if (pool) {
         for (int kd = 0; kd < 4; ++kd)
@@ -1174,9 +1243,9 @@ static rsn_status run_stream(rsn_ctx* c, const rsn_solver_opts* o, const StreamI
         return e;
       }
       if (timing && (e = cudaEventRecordWithFlags(c->tev[4 * it + 1], st, evf)) != cudaSuccess) return e;
-      if ((e = launch_cocg_update(fp32, S, nB, ce_stride, st, ji, bdev)) != cudaSuccess) return e;
+      if (proj && !timing && (e = cudaStreamWaitEvent(st, c->ev_proj, 0)) != cudaSuccess) return e;
+      if ((e = launch_cocg_update(fp32, S, pool ? pool->N : c->N, proj, b.ce_stride, it, st, ji, bdev)) != cudaSuccess) return e;
       if (timing && (e = cudaEventRecordWithFlags(c->tev[4 * it + 2], st, evf)) != cudaSuccess) return e;
-      if ((e = launch_book(S, it, st, ji, bdev)) != cudaSuccess) return e;
       if (sh && (e = launch_shift_update(S, sh->nT, ns, st, ji, bdev)) != cudaSuccess) return e;
       if (!sh) {
         // join: the scheduler sees both paths of this iteration
@@ -1186,7 +1255,7 @@ static rsn_status run_stream(rsn_ctx* c, const rsn_solver_opts* o, const StreamI
     }
     return cudaSuccess;
   };
-  const int per_iter = (proj ? 11 : 9) + (sh ? 3 : 0) + (goal ? 1 : 0);
+  const int per_iter = (proj ? 10 : 8) + (sh ? 3 : 0) + (goal ? 1 : 0);
   const double vbytes = (double)(pool ? pool->N : c->N) * (fp32 ? sizeof(float2) : sizeof(double2));
   cudaGraphExec_t gexec = nullptr;
   if (o->use_graph) {
@@ -1880,7 +1949,6 @@ static rsn_status block_impl(rsn_ctx* c, int n_e, const double* E, int n_cols, c
           js[k].ytiles = t.ytiles;
           js[k].ztiles = t.ztiles;
           js[k].nA = t.n;
-          js[k].nR = t.n;
           js[k].kind = t.plane ? kOpPlane : t.pair ? kOpPair : t.tma ? kOpTma : kOpReg;
         }
         RSN_CUDA(c, cudaMemcpyAsync(q.jd.p, js, 2 * sizeof(JuncDev), cudaMemcpyHostToDevice, c->st));
@@ -2349,9 +2417,8 @@ static bool make_pool(rsn_ctx* const* ctxs, int K, bool fp32, int nslots, PoolSp
     pool.n_groups = std::max(pool.n_groups, c->n_groups);
     pool.max_np = std::max(pool.max_np, c->max_np);
     pool.nB = std::max(pool.nB, c->jh.nB);
-    pool.nS = std::max(pool.nS, c->jh.nS);
     pool.PA = std::max(pool.PA, std::max(ti.n + c->n_groups, tr.n));
-    pool.PB = std::max(pool.PB, c->jh.nB);
+    
     for (int h = 0; h < 2; ++h) {
       const Tiling& t = h == 0 ? ti : tr;
       JuncDev& J = js[h * K + k];
@@ -2361,10 +2428,10 @@ static bool make_pool(rsn_ctx* const* ctxs, int K, bool fp32, int nslots, PoolSp
       J.ytiles = t.ytiles;
       J.ztiles = t.ztiles;
       J.nA = t.n;
-      J.nR = tr.n;
       J.kind = h == 0 ? kind : kOpReg;
     }
   }
+  pool.PB = upd_ctas(pool.N, upd_warps(pool.N, nslots));
   // the big point-pair variant serves every point-pair junction of the pool
   if (pool.has[kOpPair] && pool.inner[kOpPair].threads > kPairThreads) pool.inner[kOpPair].big = true;
   return true;
@@ -2666,6 +2733,10 @@ static rsn_status bench_kernel_impl(rsn_ctx* c, int precision, int kind, int S, 
   RSN_CUDA(c, cudaMemsetAsync(w.beta_cur.p, 0x3f, S * sizeof(double2), st));
   RSN_CUDA(c, cudaMemsetAsync(w.nrm.p, 0x3f, (size_t)S * w.PB * sizeof(double), st));
   RSN_CUDA(c, cudaMemsetAsync(w.mu.p, 0x3f, (size_t)S * w.PA * sizeof(double2), st));
+  RSN_CUDA(c, cudaMemsetAsync(w.alpha.p, 0x3f, S * sizeof(double2), st));
+  for (DevBuf* v : {&w.mu_cnt, &w.upd_cnt, &w.res_cnt, &w.total_iters, &w.cyc_iters, &w.gphase})
+    RSN_CUDA(c, cudaMemsetAsync(v->p, 0, S * sizeof(int), st));
+  RSN_CUDA(c, cudaMemsetAsync(w.tol2.p, 0, S * sizeof(double), st));
   const size_t npj = std::max(1, c->n_proj);
   RSN_CUDA(c, cudaMemsetAsync(w.c_r.p, 0, (size_t)S * npj * sizeof(double2), st));
   RSN_CUDA(c, cudaMemsetAsync(w.c_p.p, 0, 2 * (size_t)S * npj * sizeof(double2), st));
@@ -2684,13 +2755,14 @@ static rsn_status bench_kernel_impl(rsn_ctx* c, int precision, int kind, int S, 
   rsn_solver_opts o;
   rsn_default_opts(precision, &o);
   BatchDev b = slot_batch(c, S, &o);
+  b.max_iter = b.cycle_cap = INT_MAX;  // the update kernel's bookkeeping keeps every slot ACTIVE
   RSN_CUDA(c, cudaMemcpyAsync(c->bd.p, &b, sizeof(b), cudaMemcpyHostToDevice, st));
   const BatchDev* bdev = c->bd.as<BatchDev>();
   LaunchCfg cfg;
   if ((rs = make_cfg(c, fp32, S, cfg)) != RSN_OK) return rs;
   auto launch = [&]() -> cudaError_t {
     if (kind == 0) return launch_inner(c, cfg.inner, OP_COCG, fp32, S, st, cfg.jt_inner, bdev, nullptr, nullptr, nullptr);
-    if (kind == 1) return launch_cocg_update(fp32, S, c->jh.nB, b.ce_stride, st, cfg.jt_inner, bdev);
+    if (kind == 1) return launch_cocg_update(fp32, S, N, c->n_proj > 0, b.ce_stride, 0, st, cfg.jt_inner, bdev);
     return launch_op(OP_RESID, fp32, c->R, cfg.resid.ppt, dim3(cfg.resid.n, S), cfg.resid.threads, cfg.resid.smem,
                      st, cfg.jt_resid, bdev, nullptr, nullptr, nullptr);
   };

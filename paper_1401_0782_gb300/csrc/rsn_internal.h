@@ -36,6 +36,17 @@ constexpr int kReadyWindow = 4096;
 constexpr int kVecThreads = 256;
 constexpr int kVecPerThread = 16;  // points per thread in the streaming kernels
 constexpr int kVecPts = kVecThreads * kVecPerThread;
+// COCG update kernel: one warp per block of kBlkPts consecutive points, at most
+// kUpdThreads / 32 blocks per CTA.  Launches too small to give every SM a few
+// CTAs take two blocks per CTA.
+constexpr int kBlkPts = 128;
+constexpr int kUpdThreads = 128;
+__host__ __device__ constexpr int upd_ctas(long long N, int nw) {
+  return (int)((N + (long long)kBlkPts * nw - 1) / ((long long)kBlkPts * nw));
+}
+constexpr int upd_warps(long long N, int nslots) {
+  return (long long)upd_ctas(N, kUpdThreads / 32) * nslots < 2 * 152 ? 2 : kUpdThreads / 32;
+}
 
 struct JuncDev {
   int nx, ny, nz, plane;
@@ -43,7 +54,6 @@ struct JuncDev {
   // stencil tiling of the operator kernel for this junction
   int TY, Lz, ytiles, ztiles, nA;  // nA = ytiles*ztiles CTAs per slot (this launch's tiling)
   int kind;                        // operator kernel of this junction's slots: kOpReg, kOpTma, kOpPair, kOpPlane
-  int nR;                          // CTAs per slot of the true-residual kernel (rho_0, ||r_0||^2 partials)
   int nB;                          // streaming-kernel CTAs per slot
   double w64[kMaxR + 1];           // w[m] = c_m / (2 h^2), m = 1..R (w[0] unused)
   float w32[kMaxR + 1];
@@ -63,8 +73,14 @@ struct JuncDev {
   const int* inv_p0;
   const double2* inv_q64;
   const float4* inv_q32;
-  const int* sup_pts;  // the grid points with at least one entry, ascending
-  int n_sup, nS;       // their number; CTAs per slot of the projector-term kernel
+  // the same by blocks of kBlkPts points: block k has rows blk_row[k] .. blk_row[k+1]-1,
+  // each up to 32 support points of one atom: (first projector, points) and per
+  // lane the point within the block and its value quads ([row][quad][lane])
+  const int* blk_row;
+  const int2* row_meta;
+  const unsigned char* row_loc;
+  const double2* row_q64;
+  const float4* row_q32;
   const int* grp_ptr;
   const int* grp_p0;
   const int* grp_np;
@@ -90,7 +106,7 @@ enum SlotState {
 // captured CUDA graphs stay valid when a call changes the buffers it points to.
 struct BatchDev {
   int nslots;
-  int PA, PB;  // partial-sum strides per slot (>= nA / nR and nB of every junction)
+  int PA, PB;  // partial-sum strides per slot (>= nA / nR and the update kernel's CTAs of every junction)
   // per slot
   int* state;
   int* sys;
@@ -123,10 +139,10 @@ struct BatchDev {
   void* q;
   void* d;
   // reduction partials
-  double2* rho0_part;   // [S][PA] true-residual kernel: r^T r
-  double* nrm0_part;    // [S][PA] true-residual kernel: ||r||^2
-  double* t0_part;      // [S][PA] true-residual kernel: sum Gamma_L |x|^2 of the iterate (forward systems)
-  double* tlast;        // [S] that sum at the previous true residual (-1: none yet)
+  double* res_part;     // [S][PA][4] true-residual kernel: ||r||^2, r^T r (re, im), sum Gamma_L |x|^2 (forward systems)
+  int* res_cnt;         // [S] residual CTAs that have written theirs
+  double* res_tot;      // [S][4] the sums, by the last of them
+  double* tlast;        // [S] sum Gamma_L |x|^2 at the previous true residual (-1: none yet)
   int* gcnt;            // [S] T checks since the residual met tol (goal phase)
   int* gphase;          // [S] 1: goal phase (the residual met tol, the T partial is converging)
   double* tgoal;        // [S] T partial of x at a goal-phase check
@@ -134,6 +150,9 @@ struct BatchDev {
   double2* rho_part;    // [S][PB] COCG update kernel: r^T r
   double* nrm_part;     // [S][PB]
   double2* mu_part;     // [S][PA] operator kernel: p^T A p
+  int* mu_cnt;          // [S] operator and projection CTAs of the iteration that have written their partial
+  double2* alpha;       // [S] alpha_k = rho_k / mu_k, formed by the last of them
+  int* upd_cnt;         // [S] update CTAs of the iteration that have written their partials
   int pstride;          // per-slot stride of the projection arrays (the largest n_proj of the junctions)
   void* c_r;            // [S][n_proj] projections of r (inner precision)
   void* c_p;            // [2][S][n_proj] projections of p
@@ -286,15 +305,13 @@ cudaError_t launch_op_plane(int mode, int R, dim3 grid, int threads, size_t smem
                             const BatchDev* b, const void* x_in, void* y_out, const void* c_in);
 
 cudaError_t launch_zero(bool fp32, int nslots, int nB, cudaStream_t st, const JuncDev* jt, const BatchDev* b);
-// the COCG update with the projector term of q on the support points; ce_stride:
-// per-slot entries of e_kb c_p (BatchDev::ce_stride), staged in shared memory
-cudaError_t launch_cocg_update(bool fp32, int nslots, int nB, int ce_stride, cudaStream_t st, const JuncDev* jt,
-                               const BatchDev* b);
+// the COCG update with the projector term of q (proj: some junction has
+// projectors) and the iteration's bookkeeping; N_max: the largest junction
+cudaError_t launch_cocg_update(bool fp32, int nslots, long long N_max, bool proj, int ce_stride, int slot_it, cudaStream_t st,
+                               const JuncDev* jt, const BatchDev* b);
 cudaError_t launch_project(int mode, bool fp32, int nslots, int n_groups, int max_np, cudaStream_t st,
                            const JuncDev* jt, const BatchDev* b, const void* x_in, void* c_out,
                            bool one_slot_per_cta = false);
-cudaError_t launch_book(int nslots, int slot_it, cudaStream_t st, const JuncDev* jt, const BatchDev* b);
-constexpr int kBookWarps = 8;  // slots per CTA of the bookkeeping kernel (one warp each)
 cudaError_t launch_sched(int nslots, int slot_it, cudaStream_t st, const JuncDev* jt, const BatchDev* b);
 cudaError_t launch_x_update(bool fp32, int nslots, int nB, cudaStream_t st, const JuncDev* jt,
                             const BatchDev* b);

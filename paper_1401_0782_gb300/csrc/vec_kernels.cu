@@ -78,140 +78,330 @@ __global__ void __launch_bounds__(kVecThreads) zero_kernel(const JuncDev* __rest
 }
 
 // ---------------------------------------------------------------------------
-// COCG update (after the operator kernel of the same iteration):
-//   alpha = rho_k / mu_k,  r -= alpha q,  d += alpha p_new,
-//   partial sums of rho_{k+1} = r^T r and ||r||^2.
-// q arrives without the projector term (the operator kernel leaves it out);
-// on the points inside a projector support the term -sum_p v_p(i) e_kb[p] c_p
-// is added here, from e_kb c_p of the new direction (projection kernel, staged
-// in shared memory with its zero-padded tail), so q is never written back.
-// Each CTA covers kVecPts consecutive points of one system.  A non-finite
-// alpha leaves r and d untouched and flags the slot through a NaN norm.
+// COCG update (after the operator and projection kernels of the same iteration):
+//   r -= alpha q,  d += alpha p_new,
+//   partial sums of rho_{k+1} = r^T r and ||r||^2,
+// then, in the CTA that finishes its slot's last chunk, the bookkeeping of the
+// iteration (book_slot).  alpha = rho_k / mu_k was formed by whichever operator
+// or projection CTA of the slot finished last (mu_arrive).
+// q arrives without the projector term (the operator kernel leaves it out); it
+// is formed here, from e_kb c_p of the new direction (projection kernel), for
+// the blocks of points that hold support points, so q is never written back.
+// Each warp covers one block of one system.  A non-finite alpha leaves r and d
+// untouched and flags the slot through a NaN norm.
+// FP32 is bound by HBM (48 B a point), FP64 by the FP64 pipe (2 operations a
+// cycle and SM; 11 a point and 8 a projector value quad).
 // ---------------------------------------------------------------------------
-template <typename T>
-__global__ void __launch_bounds__(kVecThreads) cocg_update_kernel(const JuncDev* __restrict__ jt,
-                                                                  const BatchDev* __restrict__ bp) {
+// Bookkeeping after a COCG iteration, by the first warp of the slot's last
+// update CTA: rho_{k+1} and ||r||^2 from the partials (fixed-order warp tree),
+// beta_{k+1} = rho_{k+1} / rho_k, iteration counts, the recurrence target of
+// the current cycle, breakdown detection (NaN partial).
+__device__ __forceinline__ void book_slot(const BatchDev& b, const int s, const int nU, const int slot_it) {
+  const int lane = threadIdx.x & 31;
+  double v[4] = {0.0, 0.0, 0.0, 0.0};
+  for (int t = lane; t < nU; t += 32) {
+    v[0] += __ldcg(b.nrm_part + (size_t)s * b.PB + t);
+    const double2 w = __ldcg(b.rho_part + (size_t)s * b.PB + t);
+    v[1] += w.x;
+    v[2] += w.y;
+  }
+  const double sum = warp_sum_many<4>(v);
+  const double nrm = __shfl_sync(0xffffffffu, sum, 0);
+  const double2 rho = make_double2(__shfl_sync(0xffffffffu, sum, 1), __shfl_sync(0xffffffffu, sum, 2));
+  const double2 beta = cdiv_warp(rho, b.rho_cur[s]);
+  if (lane != 0) return;
+  const int k = b.iters[s] + 1;
+  b.iters[s] = k;
+  const int tot = b.total_iters[s] + 1;
+  b.total_iters[s] = tot;
+  const int cyc = b.cyc_iters[s] + 1;
+  b.cyc_iters[s] = cyc;
+  atomicAdd(b.counters, 1ull);
+  atomicAdd(b.sched + 3 + kMaxGraphIters + slot_it, 1);
+  if (b.n_shift > 0) b.rn2[s] = nrm;
+  b.beta_cur[s] = beta;
+  b.rho_cur[s] = rho;
+  if (!isfinite(nrm)) {
+    b.restart[s] = 1;
+    b.rrec2[s] = 0.0;
+    b.state[s] = SL_CHECK;
+  } else if (nrm <= b.tol2[s] || tot >= b.max_iter || cyc >= b.cycle_cap) {
+    b.rrec2[s] = nrm;
+    b.state[s] = b.gphase[s] ? SL_CHECKT : SL_CHECK;
+  }
+}
+
+// The projector term of one block of kBlkPts points, by one warp:
+// acc[l] = -sum over the block's projector rows of value * ce, acc and ce in
+// shared memory.  A row holds up to 32 support points of one atom inside the
+// block, each point once, so the lanes of a row never meet; the rows of a block
+// come in atom order, which fixes the order of the sums.  The loads of up to
+// four rows are in flight together (NQ: value quads per row entry).
+template <typename T, int NQ>
+__device__ __forceinline__ void block_nonlocal_nq(const JuncDev& J, const typename cx<T>::t* ce, const int row0,
+                                                  const int row1, typename cx<T>::t* acc) {
   using C = typename cx<T>::t;
+  constexpr int D = NQ == 1 ? 4 : NQ == 2 ? 2 : 1;
+  const int lane = threadIdx.x & 31;
+  for (int row = row0; row < row1; row += D) {
+    int2 m[D];  // first projector, points of the row
+    int l[D];
+    T a[D][4 * NQ];
+#pragma unroll
+    for (int j = 0; j < D; ++j) {
+      const int rr = min(row + j, row1 - 1);
+      m[j] = __ldg(J.row_meta + rr);
+      if (row + j >= row1) m[j].y = 0;
+      l[j] = __ldg(J.row_loc + rr * 32 + lane);
+#pragma unroll
+      for (int qd = 0; qd < NQ; ++qd) {
+        const size_t at = ((size_t)rr * NQ + qd) * 32 + lane;
+        if constexpr (sizeof(T) == 8) {
+          const double2 a01 = __ldg(J.row_q64 + 2 * at), a23 = __ldg(J.row_q64 + 2 * at + 1);
+          a[j][4 * qd] = a01.x, a[j][4 * qd + 1] = a01.y, a[j][4 * qd + 2] = a23.x, a[j][4 * qd + 3] = a23.y;
+        } else {
+          const float4 v = __ldg(J.row_q32 + at);
+          a[j][4 * qd] = v.x, a[j][4 * qd + 1] = v.y, a[j][4 * qd + 2] = v.z, a[j][4 * qd + 3] = v.w;
+        }
+      }
+    }
+#pragma unroll
+    for (int j = 0; j < D; ++j) {
+      if (lane < m[j].y) {
+        C y = acc[l[j]];
+#pragma unroll
+        for (int i = 0; i < 4 * NQ; ++i) y = rfma(-a[j][i], ce[m[j].x + i], y);
+        acc[l[j]] = y;
+      }
+      __syncwarp();
+    }
+  }
+}
+
+template <typename T>
+__device__ __forceinline__ void block_nonlocal(const JuncDev& J, const typename cx<T>::t* ce, const int row0,
+                                               const int row1, typename cx<T>::t* acc) {
+  for (int l = threadIdx.x & 31; l < kBlkPts; l += 32) acc[l] = czero<typename cx<T>::t>();
+  __syncwarp();
+  switch (J.inv_nq) {
+    case 1: block_nonlocal_nq<T, 1>(J, ce, row0, row1, acc); break;
+    case 2: block_nonlocal_nq<T, 2>(J, ce, row0, row1, acc); break;
+    case 3: block_nonlocal_nq<T, 3>(J, ce, row0, row1, acc); break;
+    default: block_nonlocal_nq<T, 4>(J, ce, row0, row1, acc); break;
+  }
+}
+
+// vectors of a thread's U points, in 16-byte pairs where `pairs` (at[u], at[u + 1]
+// neighbours, U even), else one at a time; points at or past `end` read as zero
+// and are not stored
+template <typename C, int U>
+__device__ __forceinline__ void load_pts(const C* src, const int (&at)[U], int end, bool pairs, C (&v)[U]) {
+  if constexpr (sizeof(C) == 8) {
+    if (pairs) {
+#pragma unroll
+      for (int u = 0; u < U; u += 2) {
+        float4 w = make_float4(0.f, 0.f, 0.f, 0.f);
+        if (at[u] < end) w = *reinterpret_cast<const float4*>(src + at[u]);
+        v[u] = mk2(w.x, w.y);
+        v[u + 1] = mk2(w.z, w.w);
+      }
+      return;
+    }
+  }
+#pragma unroll
+  for (int u = 0; u < U; ++u) v[u] = at[u] < end ? src[at[u]] : czero<C>();
+}
+template <typename C, int U>
+__device__ __forceinline__ void store_pts(C* dst, const int (&at)[U], int end, bool pairs, const C (&v)[U]) {
+  if constexpr (sizeof(C) == 8) {
+    if (pairs) {
+#pragma unroll
+      for (int u = 0; u < U; u += 2)
+        if (at[u] < end) *reinterpret_cast<float4*>(dst + at[u]) = make_float4(v[u].x, v[u].y, v[u + 1].x, v[u + 1].y);
+      return;
+    }
+  }
+#pragma unroll
+  for (int u = 0; u < U; ++u)
+    if (at[u] < end) dst[at[u]] = v[u];
+}
+
+template <typename T>
+__global__ void __launch_bounds__(kUpdThreads, sizeof(T) == 4 ? 8 : 6)
+cocg_update_kernel(const JuncDev* __restrict__ jt, const BatchDev* __restrict__ bp, int slot_it) {
+  using C = typename cx<T>::t;
+  constexpr int U = sizeof(T) == 4 ? 4 : 2;  // points in flight per thread
+  constexpr int NL = kBlkPts / (32 * U);
   const BatchDev& b = *bp;
   const int s = blockIdx.y;
   if (b.state[s] != SL_ACTIVE) return;
   const JuncDev& J = jt[b.junc[s]];
-  if ((int)blockIdx.x >= J.nB) return;
-  __shared__ double red[32 * 3];
-  __shared__ double2 s_mu[kVecThreads];
-  __shared__ double2 s_alpha;
-  extern __shared__ __align__(16) unsigned char upd_smem[];
-  C* s_ce = reinterpret_cast<C*>(upd_smem);  // e_kb c_p of the new direction, ce_stride entries
-  const int k = b.iters[s];
-  const int np = J.n_proj;
-  if (np > 0) {
-    const C* cen = reinterpret_cast<const C*>(b.c_e) + (size_t)s * b.ce_stride;
-    for (int p = threadIdx.x; p < b.ce_stride; p += kVecThreads) s_ce[p] = cen[p];
-  }
-  // mu = p^T A p from the operator kernel's partials (any number of tiles)
-  // followed by one partial per atom from the projection kernel: thread t adds
-  // partials t, t + 256, ... and thread 0 adds those sums in thread order, so
-  // the order is fixed for a given tiling
-  const int nA = J.nA + (J.n_proj > 0 ? J.n_groups : 0);
-  {
-    double2 m = make_double2(0.0, 0.0);
-    for (int t = threadIdx.x; t < nA; t += kVecThreads) {
-      const double2 v = b.mu_part[(size_t)s * b.PA + t];
-      m.x += v.x;
-      m.y += v.y;
-    }
-    s_mu[threadIdx.x] = m;
-  }
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    double2 mu = make_double2(0.0, 0.0);
-    for (int t = 0; t < kVecThreads && t < nA; ++t) { mu.x += s_mu[t].x; mu.y += s_mu[t].y; }
-    s_alpha = cdiv(b.rho_cur[s], mu);
-  }
-  __syncthreads();
-  const double2 a64 = s_alpha;
-  if (b.n_shift > 0 && blockIdx.x == 0 && threadIdx.x == 0) b.salpha[(size_t)(k & 1) * b.nslots + s] = a64;
-  const size_t slot_out = (size_t)s * b.PB + blockIdx.x;
-  if (!isfinite(a64.x) || !isfinite(a64.y)) {
-    if (threadIdx.x == 0) {
-      b.nrm_part[(size_t)s * b.PB + blockIdx.x] = __longlong_as_double(0x7ff8000000000000ll);
-      b.rho_part[slot_out] = make_double2(0.0, 0.0);
-    }
-    return;
-  }
-  const C alpha = from64<C>(a64);
+  const int N = (int)J.N;  // < 2^31
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nw = blockDim.x >> 5;
+  const int nU = upd_ctas(N, nw);
+  if ((int)blockIdx.x >= nU) return;
+  const int blk = blockIdx.x * nw + warp;
+  const int i0 = min(blk * kBlkPts, N), i1 = min(i0 + kBlkPts, N);
   const long long vo = b.voff[s];
-  const C* pn = reinterpret_cast<const C*>((k & 1) ? b.p0 : b.p1);
-  const C* qv = reinterpret_cast<const C*>(b.q);
-  C* rv = reinterpret_cast<C*>(b.r);
-  C* dv = reinterpret_cast<C*>(b.d);
-  const long long i0 = (long long)blockIdx.x * kVecPts;
-  const long long i1 = min(i0 + (long long)kVecPts, J.N);
-  T nrm = 0, rre = 0, rim = 0;
-  const int nq = J.inv_nq;
-  for (long long i = i0 + threadIdx.x; i < i1; i += kVecThreads) {
-    const long long g = vo + i;
-    const C p = pn[g];
-    C q = qv[g];
-    if (np > 0) {
-      const int e0 = J.inv_ptr[i], e1 = J.inv_ptr[i + 1];
-      for (int e = e0; e < e1; ++e) {
-        const C* cp = s_ce + J.inv_p0[e];
-        for (int qd = 0; qd < nq; ++qd) q = proj_quad<C, T>(J, e * nq + qd, cp + 4 * qd, q);
+  const int k = b.iters[s];
+  const double2 a64 = b.alpha[s];
+  const bool fin = isfinite(a64.x) && isfinite(a64.y);
+  extern __shared__ __align__(16) unsigned char upd_smem[];
+  C* s_ce = reinterpret_cast<C*>(upd_smem);         // e_kb c_p of the new direction, ce_stride entries
+  C* s_nl = s_ce + b.ce_stride + warp * kBlkPts;    // projector term of the warp's block
+  __shared__ double red[4 * (kUpdThreads / 32)];
+  __shared__ int s_last;
+  T sx = 0, sy = 0, sxy = 0;  // sums of r.x^2, r.y^2, r.x r.y
+  if (fin) {  // uniform across the CTA
+    const C* pn = reinterpret_cast<const C*>((k & 1) ? b.p0 : b.p1) + vo;
+    const C* qv = reinterpret_cast<const C*>(b.q) + vo;
+    C* rv = reinterpret_cast<C*>(b.r) + vo;
+    C* dv = reinterpret_cast<C*>(b.d) + vo;
+    const T ax = (T)a64.x, ay = (T)a64.y;
+    // FP32: 16-byte pairs where the slot starts on a pair and holds whole
+    // pairs; else (and in FP64, 16 bytes a point) one point at a time
+    const bool pairs = sizeof(T) == 4 && ((vo | N) & 1) == 0;
+    C q[U], r[U], p[U], d[U];
+    int at[U];
+    auto fetch = [&](int l) {
+#pragma unroll
+      for (int u = 0; u < U; ++u)
+        at[u] = i0 + l * 32 * U + (pairs ? 2 * lane + (u >> 1) * 64 + (u & 1) : u * 32 + lane);
+      load_pts(qv, at, i1, pairs, q);
+      load_pts(rv, at, i1, pairs, r);
+      load_pts(pn, at, i1, pairs, p);
+      load_pts(dv, at, i1, pairs, d);
+    };
+    int row0 = 0, row1 = 0;
+    if (J.n_proj > 0) {
+      const int nblk = (N + kBlkPts - 1) / kBlkPts;
+      const int ra = J.blk_row[blockIdx.x * nw], rb = J.blk_row[min((int)(blockIdx.x + 1) * nw, nblk)];
+      if (rb > ra) {  // uniform across the CTA
+        const C* cen = reinterpret_cast<const C*>(b.c_e) + (size_t)s * b.ce_stride;
+        for (int e = tid; e < b.ce_stride; e += blockDim.x) s_ce[e] = cen[e];
+        if (blk < nblk) {
+          row0 = J.blk_row[blk];
+          row1 = J.blk_row[blk + 1];
+        }
+        __syncthreads();
+        if (row1 > row0) block_nonlocal<T>(J, s_ce, row0, row1, s_nl);
       }
     }
-    C r = rv[g];
-    r.x -= alpha.x * q.x - alpha.y * q.y;
-    r.y -= alpha.x * q.y + alpha.y * q.x;
-    C d = dv[g];
-    d = cfma(alpha, p, d);
-    rv[g] = r;
-    dv[g] = d;
-    nrm = fma(r.x, r.x, fma(r.y, r.y, nrm));
-    rre = fma(r.x, r.x, fma(-r.y, r.y, rre));
-    rim = fma((T)2 * r.x, r.y, rim);
+#pragma unroll
+    for (int l = 0; l < NL; ++l) {
+      fetch(l);
+      if (row1 > row0) {
+#pragma unroll
+        for (int u = 0; u < U; ++u) q[u] = cadd(q[u], s_nl[at[u] - i0]);
+      }
+#pragma unroll
+      for (int u = 0; u < U; ++u) {
+        // r -= alpha q, d += alpha p (points past the end are zero and not stored)
+        r[u].x = fma(-ax, q[u].x, fma(ay, q[u].y, r[u].x));
+        r[u].y = fma(-ax, q[u].y, fma(-ay, q[u].x, r[u].y));
+        d[u].x = fma(ax, p[u].x, fma(-ay, p[u].y, d[u].x));
+        d[u].y = fma(ax, p[u].y, fma(ay, p[u].x, d[u].y));
+        const bool in = at[u] < i1;  // (a short block's accumulators past its end are not its own)
+        const T rx = in ? r[u].x : (T)0, ry = in ? r[u].y : (T)0;
+        sx = fma(rx, rx, sx);
+        sy = fma(ry, ry, sy);
+        sxy = fma(rx, ry, sxy);
+      }
+      store_pts(rv, at, i1, pairs, r);
+      store_pts(dv, at, i1, pairs, d);
+    }
   }
-  T v[3] = {nrm, rre, rim};
-  double out[3];
-  block_sum<3>(v, red, out);
-  if (threadIdx.x == 0) {
-    b.nrm_part[(size_t)s * b.PB + blockIdx.x] = out[0];
-    b.rho_part[slot_out] = make_double2(out[1], out[2]);
+  // ||r||^2 = sx + sy, r^T r = (sx - sy, 2 sxy) over the CTA, fixed order
+  T v[3] = {sx, sy, sxy};
+  double o[3];
+  block_sum<3>(v, red, o);
+  if (warp != 0) return;
+  if (lane == 0) {
+    const size_t at = (size_t)s * b.PB + blockIdx.x;
+    b.nrm_part[at] = fin ? o[0] + o[1] : __longlong_as_double(0x7ff8000000000000ll);
+    b.rho_part[at] = fin ? make_double2(o[0] - o[1], 2.0 * o[2]) : make_double2(0.0, 0.0);
+    __threadfence();
+    const int done = atomicAdd(b.upd_cnt + s, 1);
+    s_last = done == nU - 1 ? 1 : 0;
+    if (done == nU - 1) {
+      b.upd_cnt[s] = 0;
+      __threadfence();
+    }
   }
+  __syncwarp();
+  if (s_last) book_slot(b, s, nU, slot_it);
 }
 
 // ---------------------------------------------------------------------------
-// Projections c_p = v_p . v for every projector, one CTA per (atom, slot):
+// Projections c_p = v_p . v for every projector, one CTA per (atom, SPB slots):
 // the atom's support is gathered once and dotted with each of its projectors.
 //   PJ_R: v = r (inner precision), ACTIVE slots         -> c_r
 //   PJ_X: v = x64 + d (FP64), NEW / CHECK slots         -> c_x
 //   PJ_IN: v = x_in (apply entry point)                 -> c_out
+// Bound by the latency of the gather (about ten support points a thread) and by
+// the reduction of its SPB * NP complex sums: a warp reduces all of them
+// together, halving the number of sums a lane holds at each shuffle (V - 1
+// shuffles and adds for V = 32 sums instead of 5 V), and the warps' results
+// meet once in shared memory.
 // ---------------------------------------------------------------------------
 enum { PJ_R = 0, PJ_X = 1, PJ_IN = 2 };
+constexpr int kProjThreads = 256;
+
+// sum over w < NW of part[w * LD + t]: FP64, or for FP32 parts an error-free
+// FP32 sum (hi + lo) rounded to FP64 at the end, which leaves the FP64 pipe with
+// three operations
+template <int NW, int LD>
+__device__ __forceinline__ double sum_warps(const double* part, int t) {
+  double o = part[t];
+#pragma unroll
+  for (int w = 1; w < NW; ++w) o += part[w * LD + t];
+  return o;
+}
+template <int NW, int LD>
+__device__ __forceinline__ double sum_warps(const float* part, int t) {
+  float hi = part[t], lo = 0.f;
+#pragma unroll
+  for (int w = 1; w < NW; ++w) {
+    const float a = part[w * LD + t];
+    const float s = __fadd_rn(hi, a), bb = __fsub_rn(s, hi);
+    lo = __fadd_rn(lo, __fadd_rn(__fsub_rn(hi, __fsub_rn(s, bb)), __fsub_rn(a, bb)));
+    hi = s;
+  }
+  return (double)hi + (double)lo;
+}
 
 template <typename T, int MODE, int NP, int SPB>
-__global__ void __launch_bounds__(128) project_kernel(const JuncDev* __restrict__ jt, const BatchDev* __restrict__ bp,
-                                                      const void* __restrict__ x_in, void* __restrict__ c_out) {
+__global__ void __launch_bounds__(kProjThreads) project_kernel(const JuncDev* __restrict__ jt,
+                                                               const BatchDev* __restrict__ bp,
+                                                               const void* __restrict__ x_in,
+                                                               void* __restrict__ c_out) {
   // NP: projectors per atom at compile time (>= the junction's largest group);
   // SPB: slots per CTA, so each projector value is loaded once for SPB slots
   using CT = typename std::conditional<MODE == PJ_X, double, T>::type;
   using C = typename cx<CT>::t;
   using CO = typename cx<T>::t;
+  constexpr int NV = 2 * NP * SPB;            // real sums per thread: [slot][projector][re, im]
+  constexpr int V = NV >= 32 ? 32 : NV > 16 ? 32 : NV > 8 ? 16 : 8;  // reduced together
+  constexpr int NR = (NV + V - 1) / V;        // rounds of V
+  constexpr int NW = kProjThreads / 32;
+  static_assert(NR * V <= 64, "sums per thread");
   const BatchDev& b = *bp;
   const int g = blockIdx.x;
-  __shared__ double red[32 * 2];
+  __shared__ CT part[NW][NR * V];
+  __shared__ double s_mu[2 * NP * SPB];
   __shared__ int s_slot[SPB];
   __shared__ int s_any;
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   // PJ_X takes SPB entries of the NEW / CHECK list per CTA row (rows stride by
   // gridDim.y); PJ_R and PJ_IN take slots blockIdx.y * SPB + u
   int n_ent = b.nslots;
   if constexpr (MODE == PJ_X) n_ent = *b.lst_n;
   for (int base = blockIdx.y * SPB; base < n_ent; base += gridDim.y * SPB) {
-    __syncthreads();  // s_slot, s_any and red of the previous entries are consumed
-    if (threadIdx.x == 0) s_any = 0;
+    __syncthreads();  // shared memory of the previous entries is consumed
+    if (tid == 0) s_any = 0;
     __syncthreads();
-    if (threadIdx.x < SPB) {
-      const int e = base + threadIdx.x;
+    if (tid < SPB) {
+      const int e = base + tid;
       int s = e;
       if constexpr (MODE == PJ_X) s = e < n_ent ? b.lst[e] : -1;
       bool use = s >= 0 && s < b.nslots;
@@ -224,7 +414,7 @@ __global__ void __launch_bounds__(128) project_kernel(const JuncDev* __restrict_
         }
       }
       if (use && g >= jt[b.junc[s]].n_groups) use = false;
-      s_slot[threadIdx.x] = use ? s : -1;
+      s_slot[tid] = use ? s : -1;
       if (use) atomicOr(&s_any, 1);
     }
     __syncthreads();
@@ -252,129 +442,107 @@ __global__ void __launch_bounds__(128) project_kernel(const JuncDev* __restrict_
     const int p0 = J.grp_p0[g], np = J.grp_np[g];
     const int k0 = J.grp_ptr[g], k1 = J.grp_ptr[g + 1], len = k1 - k0;
     const long long vb = J.grp_voff[g];
-    C acc[SPB][NP];
+    CT acc[NR * V];
 #pragma unroll
-    for (int u = 0; u < SPB; ++u)
-#pragma unroll
-      for (int p = 0; p < NP; ++p) acc[u][p] = czero<C>();
-    for (int kk = k0 + threadIdx.x; kk < k1; kk += blockDim.x) {
-      const int gi = J.grp_idx[kk];
-      const long long vk = vb + (kk - k0);
+    for (int j = 0; j < NR * V; ++j) acc[j] = 0;
+#pragma unroll 2
+    for (int kk = tid; kk < len; kk += kProjThreads) {
+      const int gi = J.grp_idx[k0 + kk];
       CT a[NP];
 #pragma unroll
       for (int p = 0; p < NP; ++p) {
         if (p < np) {
-          if constexpr (sizeof(CT) == 8) a[p] = (CT)J.grp_val64[vk + (long long)p * len];
-          else a[p] = (CT)J.grp_val32[vk + (long long)p * len];
+          if constexpr (sizeof(CT) == 8) a[p] = (CT)J.grp_val64[vb + kk + (long long)p * len];
+          else a[p] = (CT)J.grp_val32[vb + kk + (long long)p * len];
         } else {
           a[p] = 0;
         }
       }
+      C v[SPB];
 #pragma unroll
       for (int u = 0; u < SPB; ++u) {
+        v[u] = czero<C>();
         if (slot[u] < 0) continue;
-        C v;
         if constexpr (MODE == PJ_R) {
-          v = reinterpret_cast<const CO*>(b.r)[vo[u] + gi];
+          v[u] = reinterpret_cast<const CO*>(b.r)[vo[u] + gi];
         } else if constexpr (MODE == PJ_X) {
           const double2 xx = b.x64[xo[u] + gi];
           const double2 dd = to64(reinterpret_cast<const CO*>(b.d)[vo[u] + gi]);
-          v = mk2(fma(sig[u], dd.x, xx.x), fma(sig[u], dd.y, xx.y));
+          v[u] = mk2(fma(sig[u], dd.x, xx.x), fma(sig[u], dd.y, xx.y));
         } else {
-          v = reinterpret_cast<const CO*>(x_in)[vo[u] + gi];
+          v[u] = reinterpret_cast<const CO*>(x_in)[vo[u] + gi];
         }
-#pragma unroll
-        for (int p = 0; p < NP; ++p) acc[u][p] = rfma(a[p], v, acc[u][p]);
       }
+#pragma unroll
+      for (int u = 0; u < SPB; ++u)
+#pragma unroll
+        for (int p = 0; p < NP; ++p) {
+          acc[2 * (u * NP + p)] = fma(a[p], v[u].x, acc[2 * (u * NP + p)]);
+          acc[2 * (u * NP + p) + 1] = fma(a[p], v[u].y, acc[2 * (u * NP + p) + 1]);
+        }
     }
 #pragma unroll
-    for (int u = 0; u < SPB; ++u) {
-      if (slot[u] < 0) continue;  // uniform across the CTA
-      const int sl = slot[u];
-      C* out = reinterpret_cast<C*>(c_out) + (size_t)sl * b.pstride + p0;
-      // PJ_R, thread 0: the projections of the new direction
-      // c_p = c_r + beta c_p_old (c_p = c_r in the first iteration), e_kb c_p
-      // for the update kernel, and this atom's share of mu = p^T A p,
-      // -sum_p e_kb[p] c_p^2, as one more partial after the operator tiles'
-      double2 mu_g = make_double2(0.0, 0.0);
+    for (int rd = 0; rd < NR; ++rd) {
+      CT w[V];
 #pragma unroll
-      for (int p = 0; p < NP; ++p) {
-        if (p < np) {  // uniform across the CTA
-          CT v[2] = {acc[u][p].x, acc[u][p].y};
-          double o[2];
-          block_sum<2>(v, red, o);
-          if (threadIdx.x == 0) {
-            const C cr = mk2((CT)o[0], (CT)o[1]);
-            out[p] = cr;
-            if constexpr (MODE == PJ_R) {
-              const int k = b.iters[sl];
-              const C* cpo = reinterpret_cast<const C*>(b.c_p) + ((size_t)(k & 1) * b.nslots + sl) * b.pstride;
-              C* cpn = reinterpret_cast<C*>(b.c_p) + ((size_t)((k + 1) & 1) * b.nslots + sl) * b.pstride;
-              C* cen = reinterpret_cast<C*>(b.c_e) + (size_t)sl * b.ce_stride;
-              C c = cr;
-              if (k > 0) c = cfma(from64<C>(b.beta_cur[sl]), cpo[p0 + p], c);
-              cpn[p0 + p] = c;
-              const CT e = (CT)J.ekb[p0 + p];
-              cen[p0 + p] = mk2(e * c.x, e * c.y);
-              const double cx = c.x, cy = c.y, e64 = J.ekb[p0 + p];
-              mu_g.x -= e64 * (cx * cx - cy * cy);
-              mu_g.y -= e64 * (2.0 * cx * cy);
-            }
+      for (int j = 0; j < V; ++j) w[j] = acc[rd * V + j];
+      const CT t = warp_sum_many<V>(w);
+      if (lane < V) part[warp][rd * V + lane] = t;
+    }
+    __syncthreads();
+    // thread t: real sum t of [slot][projector][re, im] over the warps, in warp order
+    constexpr int NT = 2 * NP * SPB;
+    const bool mine = tid < NT;
+    const int u = mine ? tid / (2 * NP) : 0, p = mine ? (tid >> 1) % NP : 0, sl = s_slot[u];
+    double mu = 0.0;
+    if (tid < (NT + 31) / 32 * 32) {
+      const double o = mine ? sum_warps<NW, NR * V>(&part[0][0], tid) : 0.0;
+      const double x = __shfl_sync(0xffffffffu, o, lane & ~1), y = __shfl_sync(0xffffffffu, o, lane | 1);
+      if (mine && sl >= 0 && p < np) {
+        const C cr = mk2((CT)x, (CT)y);
+        const bool re = (tid & 1) == 0;
+        if (re) reinterpret_cast<C*>(c_out)[(size_t)sl * b.pstride + p0 + p] = cr;
+        // PJ_R: the projections of the new direction c_p = c_r + beta c_p_old
+        // (c_p = c_r in the first iteration), e_kb c_p for the update kernel, and
+        // the projector's share of mu = p^T A p, -e_kb[p] c_p^2
+        if constexpr (MODE == PJ_R) {
+          const int k = b.iters[sl];
+          const C* cpo = reinterpret_cast<const C*>(b.c_p) + ((size_t)(k & 1) * b.nslots + sl) * b.pstride;
+          C* cpn = reinterpret_cast<C*>(b.c_p) + ((size_t)((k + 1) & 1) * b.nslots + sl) * b.pstride;
+          C* cen = reinterpret_cast<C*>(b.c_e) + (size_t)sl * b.ce_stride;
+          C c = cr;
+          if (k > 0) c = cfma(from64<C>(b.beta_cur[sl]), cpo[p0 + p], c);
+          const double e64 = J.ekb[p0 + p];
+          if (re) {
+            const CT e = (CT)e64;
+            cpn[p0 + p] = c;
+            cen[p0 + p] = mk2(e * c.x, e * c.y);
           }
+          // lanes of the real part -e (cx cx - cy cy), of the imaginary part -e (2 cx) cy
+          const double cx = c.x, cy = c.y;
+          mu = -e64 * (re ? fma(cx, cx, -cy * cy) : 2.0 * cx * cy);
         }
       }
-      if (MODE == PJ_R && threadIdx.x == 0) b.mu_part[(size_t)sl * b.PA + J.nA + g] = mu_g;
+    }
+    if constexpr (MODE == PJ_R) {
+      // the atom's share of mu, one more partial after the operator tiles'
+      if (mine) s_mu[tid] = mu;
+      __syncthreads();
+      if (warp == 0) {
+        double m = 0.0;
+        if (lane < 2 * SPB) {
+#pragma unroll
+          for (int q = 0; q < NP; ++q) m += s_mu[(lane >> 1) * 2 * NP + 2 * q + (lane & 1)];
+          const int sm = s_slot[lane >> 1];
+          if (sm >= 0) reinterpret_cast<double*>(b.mu_part + (size_t)sm * b.PA + J.nA + g)[lane & 1] = m;
+        }
+        __threadfence();
+        __syncwarp();
+        for (int v = 0; v < SPB; ++v)
+          if (s_slot[v] >= 0) mu_arrive(b, J, s_slot[v]);
+      }
     }
   }  // list entries
-}
-
-// ---------------------------------------------------------------------------
-// Bookkeeping after each COCG iteration, one warp per slot: rho_{k+1} and
-// ||r||^2 from the update kernel's partials (fixed-order warp tree),
-// beta_{k+1} = rho_{k+1} / rho_k, iteration counts, the recurrence target of
-// the current cycle, breakdown detection (NaN partial from the update kernel).
-// ---------------------------------------------------------------------------
-__global__ void __launch_bounds__(32 * kBookWarps) book_kernel(const JuncDev* __restrict__ jt,
-                                                              const BatchDev* __restrict__ bp, int slot_it) {
-  const BatchDev& b = *bp;
-  const int lane = threadIdx.x & 31;
-  const int s = blockIdx.x * kBookWarps + (threadIdx.x >> 5);
-  if (s >= b.nslots || b.state[s] != SL_ACTIVE) return;
-  const JuncDev& J = jt[b.junc[s]];
-  double nrm = 0.0, rx = 0.0, ry = 0.0;
-  for (int t = lane; t < J.nB; t += 32) {
-    nrm += b.nrm_part[(size_t)s * b.PB + t];
-    const double2 v = b.rho_part[(size_t)s * b.PB + t];
-    rx += v.x;
-    ry += v.y;
-  }
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) {
-    nrm += __shfl_down_sync(0xffffffffu, nrm, o);
-    rx += __shfl_down_sync(0xffffffffu, rx, o);
-    ry += __shfl_down_sync(0xffffffffu, ry, o);
-  }
-  if (lane != 0) return;
-  const int k = b.iters[s] + 1;
-  b.iters[s] = k;
-  const int tot = b.total_iters[s] + 1;
-  b.total_iters[s] = tot;
-  const int cyc = b.cyc_iters[s] + 1;
-  b.cyc_iters[s] = cyc;
-  atomicAdd(b.counters, 1ull);
-  atomicAdd(b.sched + 3 + kMaxGraphIters + slot_it, 1);
-  const double2 rho = make_double2(rx, ry);
-  if (b.n_shift > 0) b.rn2[s] = nrm;
-  b.beta_cur[s] = cdiv(rho, b.rho_cur[s]);
-  b.rho_cur[s] = rho;
-  if (!isfinite(nrm)) {
-    b.restart[s] = 1;
-    b.rrec2[s] = 0.0;
-    b.state[s] = SL_CHECK;
-  } else if (nrm <= b.tol2[s] || tot >= b.max_iter || cyc >= b.cycle_cap) {
-    b.rrec2[s] = nrm;
-    b.state[s] = b.gphase[s] ? SL_CHECKT : SL_CHECK;
-  }
 }
 
 // ---------------------------------------------------------------------------
@@ -389,7 +557,6 @@ __global__ void __launch_bounds__(kSchedThreads) sched_kernel(const JuncDev* __r
   const BatchDev& b = *bp;
   const int S = b.nslots;
   __shared__ int warp_cnt[32];
-  __shared__ double red[32 * 2];
   int upd = 0, busy = 0;
   for (int s = threadIdx.x; s < S; s += blockDim.x) {
     int st = b.state[s];
@@ -425,18 +592,8 @@ __global__ void __launch_bounds__(kSchedThreads) sched_kernel(const JuncDev* __r
         st = SL_ACTIVE;
       }
     } else if ((st == SL_NEW || st == SL_CHECK) && listed) {
-      const JuncDev& J = jt[b.junc[s]];
-      double nrm = 0.0, tcur = 0.0;
-      double2 rho = make_double2(0.0, 0.0);
-      const double* np = b.nrm0_part + (size_t)s * b.PA;
-      const double* tp = b.t0_part + (size_t)s * b.PA;
-      const double2* rp = b.rho0_part + (size_t)s * b.PA;
-      for (int t = 0; t < J.nR; ++t) {
-        nrm += np[t];
-        tcur += tp[t];
-        rho.x += rp[t].x;
-        rho.y += rp[t].y;
-      }
+      const double nrm = b.res_tot[4 * s], tcur = b.res_tot[4 * s + 3];
+      const double2 rho = make_double2(b.res_tot[4 * s + 1], b.res_tot[4 * s + 2]);
       if (st == SL_NEW) {
         // cold start: r = b, so ||b||^2 = nrm; warm start: ||b||^2 is given
         const double bn = b.warm[s] ? b.sys_bn2[b.sys[s]] : nrm;
@@ -622,14 +779,20 @@ __global__ void __launch_bounds__(kSchedThreads) sched_kernel(const JuncDev* __r
     if (found) break;
   }
   for (int s = threadIdx.x; s < S; s += blockDim.x) busy += (b.state[s] != SL_FREE) ? 1 : 0;
-  double v[2] = {(double)busy, (double)upd};
-  double out[2];
-  block_sum<2>(v, red, out);
+  busy = __reduce_add_sync(0xffffffffu, busy);
+  upd = __reduce_add_sync(0xffffffffu, upd);
+  if (threadIdx.x == 0) s_nf = s_done = 0;  // reused: the CTA's totals
+  __syncthreads();
+  if (lane == 0) {
+    if (busy) atomicAdd(&s_nf, busy);
+    if (upd) atomicAdd(&s_done, upd);
+  }
+  __syncthreads();
   if (threadIdx.x == 0) {
     b.sched[0] = s_first;
-    b.sched[1] = (int)out[0];
-    b.sched[3 + slot_it] = (int)out[0];
-    b.counters[1] += (unsigned long long)out[1];
+    b.sched[1] = s_nf;
+    b.sched[3 + slot_it] = s_nf;
+    b.counters[1] += (unsigned long long)s_done;
   }
 }
 
@@ -644,7 +807,6 @@ __global__ void __launch_bounds__(kVecThreads) x_update_kernel(const JuncDev* __
                                                                const BatchDev* __restrict__ bp) {
   using C = typename cx<T>::t;
   const BatchDev& b = *bp;
-  __shared__ double s_part[kVecThreads];
   __shared__ double s_sig;
   const int n = *b.lst_n;
   for (int li = blockIdx.y; li < n; li += gridDim.y) {
@@ -653,22 +815,15 @@ __global__ void __launch_bounds__(kVecThreads) x_update_kernel(const JuncDev* __
     if (st != SL_NEW && st != SL_CHECK && st != SL_CHECKT) continue;
     const JuncDev& J = jt[b.junc[s]];
     if ((int)blockIdx.x >= J.nB) continue;
-    __syncthreads();  // s_part / s_sig of the previous entry are consumed
-    if (st == SL_NEW) {
-      // ||b||^2 from the residual kernel's partials, in the fixed order of the
-      // update kernel's mu sum
-      double n2t = 0.0;
-      for (int t = threadIdx.x; t < J.nR; t += kVecThreads) n2t += b.nrm0_part[(size_t)s * b.PA + t];
-      s_part[threadIdx.x] = n2t;
-      __syncthreads();
-      if (threadIdx.x == 0) {
-        double n2 = 0.0;
-        for (int t = 0; t < kVecThreads && t < J.nR; ++t) n2 += s_part[t];
-        s_sig = n2 > 0.0 ? sqrt(n2) : 1.0;
-        if (blockIdx.x == 0) b.sigma[s] = s_sig;
+    __syncthreads();  // s_sig of the previous entry are consumed
+    if (threadIdx.x == 0) {
+      double sg = b.sigma[s];
+      if (st == SL_NEW) {  // ||b||^2 from the residual kernel
+        const double n2 = b.res_tot[4 * s];
+        sg = n2 > 0.0 ? sqrt(n2) : 1.0;
+        if (blockIdx.x == 0) b.sigma[s] = sg;
       }
-    } else if (threadIdx.x == 0) {
-      s_sig = b.sigma[s];
+      s_sig = sg;
     }
     __syncthreads();
     const double sig = s_sig;
@@ -1053,18 +1208,19 @@ cudaError_t launch_zero(bool fp32, int nslots, int nB, cudaStream_t st, const Ju
   return cudaGetLastError();
 }
 
-cudaError_t launch_cocg_update(bool fp32, int nslots, int nB, int ce_stride, cudaStream_t st, const JuncDev* jt,
-                               const BatchDev* b) {
-  dim3 grid(nB, nslots);
-  const size_t smem = (size_t)ce_stride * (fp32 ? sizeof(float2) : sizeof(double2));
-  if (smem > 48 * 1024) {
+cudaError_t launch_cocg_update(bool fp32, int nslots, long long N_max, bool proj, int ce_stride, int slot_it,
+                               cudaStream_t st, const JuncDev* jt, const BatchDev* b) {
+  const int nw = upd_warps(N_max, nslots);
+  const dim3 grid(upd_ctas(N_max, nw), nslots);
+  const size_t smem = proj ? ((size_t)ce_stride + nw * kBlkPts) * (fp32 ? sizeof(float2) : sizeof(double2)) : 0;
+  if (smem > 32 * 1024) {
     cudaError_t e = set_max_dynamic_smem(
         fp32 ? reinterpret_cast<const void*>(cocg_update_kernel<float>) : reinterpret_cast<const void*>(cocg_update_kernel<double>),
         smem);
     if (e != cudaSuccess) return e;
   }
-  if (fp32) cocg_update_kernel<float><<<grid, kVecThreads, smem, st>>>(jt, b);
-  else cocg_update_kernel<double><<<grid, kVecThreads, smem, st>>>(jt, b);
+  if (fp32) cocg_update_kernel<float><<<grid, 32 * nw, smem, st>>>(jt, b, slot_it);
+  else cocg_update_kernel<double><<<grid, 32 * nw, smem, st>>>(jt, b, slot_it);
   return cudaGetLastError();
 }
 
@@ -1072,14 +1228,14 @@ template <int NP, int SPB>
 static void launch_project_np(int mode, bool fp32, dim3 grid, cudaStream_t st, const JuncDev* jt, const BatchDev* b,
                               const void* x_in, void* c_out) {
   if (mode == PJ_R) {
-    if (fp32) project_kernel<float, PJ_R, NP, SPB><<<grid, 128, 0, st>>>(jt, b, x_in, c_out);
-    else project_kernel<double, PJ_R, NP, SPB><<<grid, 128, 0, st>>>(jt, b, x_in, c_out);
+    if (fp32) project_kernel<float, PJ_R, NP, SPB><<<grid, kProjThreads, 0, st>>>(jt, b, x_in, c_out);
+    else project_kernel<double, PJ_R, NP, SPB><<<grid, kProjThreads, 0, st>>>(jt, b, x_in, c_out);
   } else if (mode == PJ_X) {
-    if (fp32) project_kernel<float, PJ_X, NP, SPB><<<grid, 128, 0, st>>>(jt, b, x_in, c_out);
-    else project_kernel<double, PJ_X, NP, SPB><<<grid, 128, 0, st>>>(jt, b, x_in, c_out);
+    if (fp32) project_kernel<float, PJ_X, NP, SPB><<<grid, kProjThreads, 0, st>>>(jt, b, x_in, c_out);
+    else project_kernel<double, PJ_X, NP, SPB><<<grid, kProjThreads, 0, st>>>(jt, b, x_in, c_out);
   } else {
-    if (fp32) project_kernel<float, PJ_IN, NP, SPB><<<grid, 128, 0, st>>>(jt, b, x_in, c_out);
-    else project_kernel<double, PJ_IN, NP, SPB><<<grid, 128, 0, st>>>(jt, b, x_in, c_out);
+    if (fp32) project_kernel<float, PJ_IN, NP, SPB><<<grid, kProjThreads, 0, st>>>(jt, b, x_in, c_out);
+    else project_kernel<double, PJ_IN, NP, SPB><<<grid, kProjThreads, 0, st>>>(jt, b, x_in, c_out);
   }
 }
 
@@ -1088,25 +1244,19 @@ cudaError_t launch_project(int mode, bool fp32, int nslots, int n_groups, int ma
                            bool one_slot_per_cta) {
   // slots per CTA: the projector values of an atom are loaded once for all of
   // them; a pool over several junctions takes one slot per CTA (atom g differs
-  // between junctions)
-  if (one_slot_per_cta && max_np <= 4) {
-    launch_project_np<4, 1>(mode, fp32, dim3(n_groups, nslots), st, jt, b, x_in, c_out);
-  } else if (one_slot_per_cta && max_np <= 9) {
-    launch_project_np<9, 1>(mode, fp32, dim3(n_groups, nslots), st, jt, b, x_in, c_out);
-  } else if (max_np <= 4) {
-    launch_project_np<4, 4>(mode, fp32, dim3(n_groups, (nslots + 3) / 4), st, jt, b, x_in, c_out);
+  // between junctions), and so does a launch that would leave SMs idle
+  const bool one = one_slot_per_cta || (long long)n_groups * ((nslots + 3) / 4) < 2 * 152;
+  if (max_np <= 4) {
+    if (one) launch_project_np<4, 1>(mode, fp32, dim3(n_groups, nslots), st, jt, b, x_in, c_out);
+    else launch_project_np<4, 4>(mode, fp32, dim3(n_groups, (nslots + 3) / 4), st, jt, b, x_in, c_out);
   } else if (max_np <= 9) {
-    launch_project_np<9, 2>(mode, fp32, dim3(n_groups, (nslots + 1) / 2), st, jt, b, x_in, c_out);
+    if (one) launch_project_np<9, 1>(mode, fp32, dim3(n_groups, nslots), st, jt, b, x_in, c_out);
+    else launch_project_np<9, 2>(mode, fp32, dim3(n_groups, (nslots + 1) / 2), st, jt, b, x_in, c_out);
   } else if (max_np <= kMaxGroupNp) {
     launch_project_np<kMaxGroupNp, 1>(mode, fp32, dim3(n_groups, nslots), st, jt, b, x_in, c_out);
   } else {
     return cudaErrorInvalidValue;
   }
-  return cudaGetLastError();
-}
-
-cudaError_t launch_book(int nslots, int slot_it, cudaStream_t st, const JuncDev* jt, const BatchDev* b) {
-  book_kernel<<<(nslots + kBookWarps - 1) / kBookWarps, 32 * kBookWarps, 0, st>>>(jt, b, slot_it);
   return cudaGetLastError();
 }
 
