@@ -357,168 +357,153 @@ __global__ void __launch_bounds__(kBlkThreads) blk_q0_kernel(const BlkDev* __res
 }
 
 // ---------------------------------------------------------------------------
-// b x b algebra, one warp per listed block, FP64.
+// b x b algebra of each listed block, FP64, one CTA of B * B threads (at least a
+// warp): thread t owns entry (t / B, t % B).  A warp's FP64 instruction takes 64
+// cycles of its FP64 pipe, so what counts is the number of instructions on the
+// longest chain: entries are spread over the four pipes, every elimination step
+// takes one reciprocal (or reciprocal square root) from an FP32 seed and two
+// Newton steps, and the pivot search compares exponent words.  One warp per block
+// took 510 us a phase-2 call and 225 us a phase-1 call at B = 16.
 // ---------------------------------------------------------------------------
 namespace {
 
-// Sum the Gram partials of output o over the chunks into M (row-major B x B,
-// leading dimension ld).
-template <int B>
-__device__ void sum_parts(const BlkDev& d, int k, int o, double2* M, int ld) {
-  const int lane = threadIdx.x;
-  for (int e = lane; e < B * B; e += 32) {
-    double2 v = make_double2(0.0, 0.0);
-    for (int ch = 0; ch < d.nchunk; ++ch) {
-      const double2 r = d.part[(((size_t)k * d.nchunk + ch) * 2 + o) * B * B + e];
-      v.x += r.x;
-      v.y += r.y;
-    }
-    M[(e / B) * ld + (e % B)] = v;
-  }
-  __syncwarp();
+// 1 / a by Newton's iteration from the FP32 reciprocal (24 -> 48 -> 53 bits);
+// a plain division outside the seed's range
+__device__ __forceinline__ double rcp_newton(double a) {
+  const float f = (float)a;
+  if (!(f > 1e-30f && f < 1e30f)) return 1.0 / a;
+  double y = (double)__frcp_rn(f);
+  y = fma(fma(-a, y, 1.0), y, y);
+  return fma(fma(-a, y, 1.0), y, y);
+}
+// 1 / sqrt(a) by Newton's iteration from the FP32 reciprocal square root
+__device__ __forceinline__ double rsqrt_newton(double a) {
+  const float f = (float)a;
+  if (!(f > 1e-30f && f < 1e30f)) return 1.0 / sqrt(a);
+  double y = (double)__frsqrt_rn(f);
+  const double h = 0.5 * a;
+  y = fma(fma(-h * y, y, 0.5), y, y);
+  return fma(fma(-h * y, y, 0.5), y, y);
 }
 
-// Solve M X = Y for the B x B block X, with M and Y held side by side in
-// aug (B rows, 2B columns, leading dimension 2B): Gaussian elimination with
-// partial pivoting, lane j owning augmented column j.  The solution goes to
-// sol (row-major B x B).  Returns false on a zero or non-finite pivot.
-template <int B>
-__device__ bool warp_solve(double2* aug, double2* fac, int* s_piv, double2* sol) {
-  constexpr int L = 2 * B;
-  const int lane = threadIdx.x;
-  bool ok = true;
+__device__ __forceinline__ double2 cfma64(double2 a, double2 b, double2 acc) {
+  acc.x = fma(a.x, b.x, fma(-a.y, b.y, acc.x));
+  acc.y = fma(a.x, b.y, fma(a.y, b.x, acc.y));
+  return acc;
+}
+__device__ __forceinline__ double2 cneg(double2 a) { return make_double2(-a.x, -a.y); }
+__device__ __forceinline__ double2 cconj(double2 a) { return make_double2(a.x, -a.y); }
+
+// Solve M X = Y in place for aug = [M | Y] (B rows, 2B columns, leading
+// dimension LD): Gauss-Jordan elimination with partial pivoting (the pivot is the
+// entry with the largest real or imaginary part).  X replaces Y.  Returns false
+// (in every thread) on a zero or non-finite pivot.
+template <int B, int LD>
+__device__ bool gauss_jordan(double2* aug) {
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int er = tid / B, ec = tid % B;
   for (int kk = 0; kk < B; ++kk) {
-    if (lane == 0) {
-      int piv = kk;
-      double best = cabs2(aug[kk * L + kk]);
-      for (int r = kk + 1; r < B; ++r) {
-        const double v = cabs2(aug[r * L + kk]);
-        if (v > best) best = v, piv = r;
-      }
-      *s_piv = (best > 0.0 && best <= DBL_MAX) ? piv : -1;
+    // every warp finds the pivot for itself (integer instructions only)
+    int key = -1;
+    if (lane >= kk && lane < B) {
+      const double2 v = aug[lane * LD + kk];
+      key = max(__double2hiint(v.x) & 0x7fffffff, __double2hiint(v.y) & 0x7fffffff);
     }
-    __syncwarp();
-    const int piv = *s_piv;
-    if (piv < 0) {
-      ok = false;
-      break;
-    }
-    if (piv != kk && lane < L) {
-      const double2 tmp = aug[kk * L + lane];
-      aug[kk * L + lane] = aug[piv * L + lane];
-      aug[piv * L + lane] = tmp;
-    }
-    __syncwarp();
-    if (lane > kk && lane < B) fac[lane] = cdiv(aug[lane * L + kk], aug[kk * L + kk]);
-    __syncwarp();
-    if (lane > kk && lane < L) {
-      const double2 top = aug[kk * L + lane];
-      for (int r = kk + 1; r < B; ++r) {
-        const double2 f = fac[r];
-        double2 v = aug[r * L + lane];
-        v.x -= f.x * top.x - f.y * top.y;
-        v.y -= f.x * top.y + f.y * top.x;
-        aug[r * L + lane] = v;
+    const int best = __reduce_max_sync(0xffffffffu, key);
+    const int piv = __ffs(__ballot_sync(0xffffffffu, key == best)) - 1;
+    if (best <= 0 || best >= 0x7ff00000) return false;  // the same in every warp
+    const double2 p = aug[piv * LD + kk];
+    __syncthreads();  // every warp has read column kk
+    if (warp == 0) {
+      // row kk <- pivot row / pivot, the old row kk moves to the pivot's place
+      const double den = rcp_newton(fma(p.x, p.x, p.y * p.y));
+      const double2 inv = make_double2(p.x * den, -p.y * den);
+      for (int c = lane; c < 2 * B; c += 32) {
+        const double2 top = aug[piv * LD + c];
+        if (piv != kk) aug[piv * LD + c] = aug[kk * LD + c];
+        aug[kk * LD + c] = cfma64(top, inv, make_double2(0.0, 0.0));
       }
     }
-    __syncwarp();
+    __syncthreads();
+    if (er < B && er != kk) {
+      const double2 f = cneg(aug[er * LD + kk]);
+#pragma unroll
+      for (int h = 0; h < 2; ++h) {
+        const int c = ec + h * B;
+        if (c > kk) aug[er * LD + c] = cfma64(f, aug[kk * LD + c], aug[er * LD + c]);
+      }
+    }
+    __syncthreads();
   }
-  if (!ok) return false;
-  if (lane >= B && lane < L) {
-    const int j = lane - B;
-    for (int r = B - 1; r >= 0; --r) {
-      double2 v = aug[r * L + lane];
-      for (int m = r + 1; m < B; ++m) {
-        const double2 a = aug[r * L + m], x = sol[m * B + j];
-        v.x -= a.x * x.x - a.y * x.y;
-        v.y -= a.x * x.y + a.y * x.x;
-      }
-      sol[r * B + j] = cdiv(v, aug[r * L + r]);
-    }
-  }
-  __syncwarp();
   return true;
 }
 
-// Cholesky factor of the Hermitian positive definite A (row-major B x B):
-// A = Lc Lc^H, Lc lower triangular with a real positive diagonal; lanes own
-// rows.  Fails when a pivot is not positive or falls below 1e-12 of its
-// diagonal entry (numerically dependent columns).
+// Cholesky factor of the Hermitian positive definite A (B x B, leading dimension
+// B, destroyed above its diagonal blocks) and the inverse of its lower factor:
+// A = Lc Lc^H; U = Lc^H (upper), Li = Lc^{-1} (lower).  Fails when a pivot is not
+// positive or falls below 1e-12 of its diagonal entry (numerically dependent
+// columns).
 template <int B>
-__device__ bool warp_cholesky(const double2* A, double2* Lc, int* s_ok) {
-  const int lane = threadIdx.x;
-  for (int e = lane; e < B * B; e += 32) Lc[e] = make_double2(0.0, 0.0);
-  if (lane == 0) *s_ok = 1;
-  __syncwarp();
+__device__ bool cholesky_inverse(double2* A, double2* U, double2* Li) {
+  const int tid = threadIdx.x, er = tid / B, ec = tid % B;
+  __shared__ double s_ref[B];
+  if (er < B) {
+    U[tid] = make_double2(0.0, 0.0);
+    Li[tid] = make_double2(er == ec ? 1.0 : 0.0, 0.0);
+    if (er == ec) s_ref[er] = A[tid].x;
+  }
+  __syncthreads();
   for (int kk = 0; kk < B; ++kk) {
-    if (lane == 0) {
-      double dd = A[kk * B + kk].x;
-      for (int m = 0; m < kk; ++m) dd -= cabs2(Lc[kk * B + m]);
-      const double ref = A[kk * B + kk].x;
-      if (!(dd > 1e-12 * ref) || !(dd <= DBL_MAX)) {
-        *s_ok = 0;
-        dd = 1.0;
+    const double dd = A[kk * B + kk].x;
+    if (!(dd > 1e-12 * s_ref[kk]) || !(dd <= DBL_MAX)) return false;  // the same in every thread
+    if (tid < B) {
+      // row kk of U (columns >= kk) and of Li (columns <= kk)
+      const double rs = rsqrt_newton(dd);
+      double2 v = tid >= kk ? A[kk * B + tid] : Li[kk * B + tid];
+      v.x *= rs;
+      v.y *= rs;
+      if (tid == kk) {
+        // the diagonal: sqrt(dd) with one correction step; Li's is 1 / sqrt(dd)
+        const double q = dd * rs;
+        U[kk * B + kk] = make_double2(fma(fma(-q, q, dd), 0.5 * rs, q), 0.0);
+        Li[kk * B + kk] = make_double2(rs, 0.0);
+      } else if (tid > kk) {
+        U[kk * B + tid] = v;
+      } else {
+        Li[kk * B + tid] = v;
       }
-      Lc[kk * B + kk] = make_double2(sqrt(dd), 0.0);
     }
-    __syncwarp();
-    if (lane > kk && lane < B) {
-      double2 v = A[lane * B + kk];
-      for (int m = 0; m < kk; ++m) {
-        const double2 a = Lc[lane * B + m], b = Lc[kk * B + m];  // a conj(b)
-        v.x -= a.x * b.x + a.y * b.y;
-        v.y -= a.y * b.x - a.x * b.y;
-      }
-      const double dk = Lc[kk * B + kk].x;
-      Lc[lane * B + kk] = make_double2(v.x / dk, v.y / dk);
+    __syncthreads();
+    if (er > kk && er < B) {
+      const double2 f = cneg(cconj(U[kk * B + er]));  // -Lc[er][kk]
+      if (ec > kk) A[tid] = cfma64(f, U[kk * B + ec], A[tid]);
+      else Li[tid] = cfma64(f, Li[kk * B + ec], Li[tid]);
     }
-    __syncwarp();
+    __syncthreads();
   }
-  return *s_ok != 0;
-}
-
-// Li = Lc^{-1} (lower triangular), lane j owning column j.
-template <int B>
-__device__ void warp_lower_inverse(const double2* Lc, double2* Li) {
-  const int j = threadIdx.x;
-  if (j < B) {
-    for (int r = 0; r < B; ++r) {
-      double2 v = make_double2(r == j ? 1.0 : 0.0, 0.0);
-      if (r > j) {
-        v = make_double2(0.0, 0.0);
-        for (int m = j; m < r; ++m) {
-          const double2 a = Lc[r * B + m], x = Li[m * B + j];
-          v.x -= a.x * x.x - a.y * x.y;
-          v.y -= a.x * x.y + a.y * x.x;
-        }
-      }
-      const double dr = Lc[r * B + r].x;
-      Li[r * B + j] = r < j ? make_double2(0.0, 0.0) : make_double2(v.x / dr, v.y / dr);
-    }
-  }
-  __syncwarp();
-}
-
-// C = A Bm for row-major B x B matrices, lane j owning column j of C.
-template <int B>
-__device__ void warp_matmul(const double2* A, const double2* Bm, double2* C) {
-  const int j = threadIdx.x;
-  if (j < B) {
-    for (int r = 0; r < B; ++r) {
-      double2 v = make_double2(0.0, 0.0);
-      for (int m = 0; m < B; ++m) {
-        const double2 a = A[r * B + m];
-        const double2 b = Bm[m * B + j];
-        v.x += a.x * b.x - a.y * b.y;
-        v.y += a.x * b.y + a.y * b.x;
-      }
-      C[r * B + j] = v;
-    }
-  }
-  __syncwarp();
+  return true;
 }
 
 }  // namespace
+
+// Sums of the Gram partials over the chunks, one warp per entry:
+// d.gsum[k][o][e], o < no.
+template <int B>
+__global__ void __launch_bounds__(256) blk_psum_kernel(const BlkDev* __restrict__ dp, int no) {
+  const BlkDev& d = *dp;
+  const int k = d.blist[blockIdx.y];
+  if (d.flag[k] != 0) return;
+  const int lane = threadIdx.x & 31, e = blockIdx.x * 8 + (threadIdx.x >> 5);
+  if (e >= no * B * B) return;
+  double v[2] = {0.0, 0.0};
+  for (int ch = lane; ch < d.nchunk; ch += 32) {
+    const double2 r = d.part[((size_t)k * d.nchunk + ch) * 2 * B * B + e];
+    v[0] += r.x;
+    v[1] += r.y;
+  }
+  const double t = warp_sum_many<2>(v);
+  if (lane < 2) reinterpret_cast<double*>(d.gsum + (size_t)k * 2 * B * B + e)[lane] = t;
+}
 
 // PHASE 0: start of an inner solve (W holds the normalised residual block):
 //          tau_0, tau_0^{-1}, xi_0 = tau_0, ||xi_0[:, j]||, Q_0^T Q_0.
@@ -526,161 +511,121 @@ __device__ void warp_matmul(const double2* A, const double2* Bm, double2* C) {
 // PHASE 2: tau, tau^{-1} of the new W; xi <- tau xi; Q^T Q of the new Q;
 //          beta; iteration count and convergence of every column.
 template <int B, int PHASE>
-__global__ void __launch_bounds__(32) blk_small_kernel(const BlkDev* __restrict__ dp) {
+__global__ void __launch_bounds__(B * B < 32 ? 32 : B * B) blk_small_kernel(const BlkDev* __restrict__ dp) {
+  constexpr int LD = 2 * B + 1;
   const BlkDev& d = *dp;
   const int k = d.blist[blockIdx.x];
-  const int lane = threadIdx.x;
+  const int tid = threadIdx.x;
   if (PHASE != 0 && d.flag[k] != 0) return;
-  __shared__ double2 aug[B * 2 * B];
+  __shared__ double2 aug[B * LD];
   __shared__ double2 M0[B * B], M1[B * B], M2[B * B], M3[B * B];
-  __shared__ double2 fac[B];
-  __shared__ int s_i;
   const size_t ko = (size_t)k * B * B;
+  const bool own = tid < B * B;
+  const int a = tid / B, j = tid % B;  // the thread's entry
+  const double2 zero = make_double2(0.0, 0.0);
+  const double2* G = d.gsum + 2 * ko;
   if (PHASE == 1) {
-    sum_parts<B>(d, k, 0, aug, 2 * B);  // P^T A P
-    for (int e = lane; e < B * B; e += 32) aug[(e / B) * 2 * B + B + (e % B)] = d.QQ[ko + e];
-    __syncwarp();
-    if (!warp_solve<B>(aug, fac, &s_i, M0)) {
-      if (lane == 0) d.flag[k] = 2;
+    if (own) {
+      aug[a * LD + j] = G[tid];  // P^T A P
+      aug[a * LD + B + j] = d.QQ[ko + tid];
+      M1[tid] = d.xi[ko + tid];
+    }
+    __syncthreads();
+    if (!gauss_jordan<B, LD>(aug)) {
+      if (tid == 0) d.flag[k] = 2;
       return;
     }
-    for (int e = lane; e < B * B; e += 32) M1[e] = d.xi[ko + e];
-    __syncwarp();
-    warp_matmul<B>(M0, M1, M2);  // alpha xi
-    for (int e = lane; e < B * B; e += 32) {
-      d.alpha[ko + e] = to32(M0[e]);
-      d.axi[ko + e] = to32(M2[e]);
+    if (own) {
+      double2 v = zero;  // alpha xi
+#pragma unroll 4
+      for (int m = 0; m < B; ++m) v = cfma64(aug[a * LD + B + m], M1[m * B + j], v);
+      d.alpha[ko + tid] = to32(aug[a * LD + B + j]);
+      d.axi[ko + tid] = to32(v);
     }
     return;
   }
   // PHASE 0 / 2: Cholesky QR of W
-  sum_parts<B>(d, k, 0, M0, B);  // W^H W
-  sum_parts<B>(d, k, 1, M1, B);  // W^T W
-  if (!warp_cholesky<B>(M0, M2, &s_i)) {  // M2 = Lc, tau = Lc^H
-    if (lane == 0) d.flag[k] = 2;
+  if (own) {
+    M0[tid] = G[tid];          // W^H W
+    M1[tid] = G[B * B + tid];  // W^T W
+  }
+  __syncthreads();
+  if (!cholesky_inverse<B>(M0, M2, M3)) {  // M2 = tau = Lc^H, M3 = Lc^{-1}, tau^{-1} = M3^H
+    if (tid == 0) d.flag[k] = 2;
     return;
   }
-  warp_lower_inverse<B>(M2, M3);  // M3 = Li = Lc^{-1}, tau^{-1} = Li^H
   // tau^{-1} for the vector kernels: at a restart (PHASE 0) in FP64 for the
   // Q_0 kernel, which writes Q_0 itself into W, so that the FP32 copy is I
-  for (int e = lane; e < B * B; e += 32) {
-    const int a = e / B, c = e % B;
-    const double2 v = M3[c * B + a];
+  if (own) {
+    const double2 v = cconj(M3[j * B + a]);
     if (PHASE == 0) {
-      d.tinv64[ko + e] = make_double2(v.x, -v.y);
-      d.tinv[ko + e] = make_float2(a == c ? 1.f : 0.f, 0.f);
+      d.tinv64[ko + tid] = v;
+      d.tinv[ko + tid] = make_float2(a == j ? 1.f : 0.f, 0.f);
     } else {
-      d.tinv[ko + e] = make_float2((float)v.x, (float)-v.y);
+      d.tinv[ko + tid] = to32(v);
     }
   }
-  // Q^T Q = tau^{-T} (W^T W) tau^{-1}, with tau^{-1} = Li^H
-  {
-    // T1 = (W^T W) tau^{-1}, tau^{-1}[m][j] = conj(Li[j][m])
-    const int j = lane;
-    if (j < B) {
-      for (int r = 0; r < B; ++r) {
-        double2 v = make_double2(0.0, 0.0);
-        for (int m = 0; m < B; ++m) {
-          const double2 a = M1[r * B + m];
-          const double2 li = M3[j * B + m];
-          const double2 b = make_double2(li.x, -li.y);
-          v.x += a.x * b.x - a.y * b.y;
-          v.y += a.x * b.y + a.y * b.x;
-        }
-        M0[r * B + j] = v;
-      }
-    }
-    __syncwarp();
-    // QQn = tau^{-T} T1, tau^{-T}[a][r] = tau^{-1}[r][a] = conj(Li[a][r])
-    if (j < B) {
-      for (int a = 0; a < B; ++a) {
-        double2 v = make_double2(0.0, 0.0);
-        for (int r = 0; r < B; ++r) {
-          const double2 li = M3[a * B + r];
-          const double2 t = make_double2(li.x, -li.y);
-          const double2 b = M0[r * B + j];
-          v.x += t.x * b.x - t.y * b.y;
-          v.y += t.x * b.y + t.y * b.x;
-        }
-        M1[a * B + j] = v;  // M1 = Q_{k+1}^T Q_{k+1} (W^T W no longer needed)
-      }
-    }
-    __syncwarp();
+  // Q^T Q = tau^{-T} (W^T W) tau^{-1}.  Triangular factors: entries are owned so
+  // that a warp's lanes run sums of nearly the same length.
+  if (own) {
+    double2 v = zero;  // T1[j][a] = sum_{m <= a} (W^T W)[j][m] tau^{-1}[m][a]
+    for (int m = 0; m <= a; ++m) v = cfma64(M1[j * B + m], cconj(M3[a * B + m]), v);
+    M0[j * B + a] = v;
+  }
+  __syncthreads();
+  if (own) {
+    double2 v = zero;  // QQ[a][j] = sum_{m <= a} tau^{-1}[m][a] T1[m][j]
+    for (int m = 0; m <= a; ++m) v = cfma64(cconj(M3[a * B + m]), M0[m * B + j], v);
+    M1[tid] = v;  // W^T W is no longer needed
   }
   if (PHASE == 0) {
-    for (int e = lane; e < B * B; e += 32) {
-      const int a = e / B, c = e % B;
-      const double2 l = M2[c * B + a];  // tau[a][c] = conj(Lc[c][a])
-      d.xi[ko + e] = make_double2(l.x, -l.y);
-      d.QQ[ko + e] = M1[e];
+    __syncthreads();
+    if (own) {
+      d.xi[ko + tid] = M2[tid];
+      d.QQ[ko + tid] = M1[tid];
     }
-    if (lane < B) {
+    if (tid < B) {
       double s = 0.0;
-      for (int a = 0; a < B; ++a) s += cabs2(M2[lane * B + a]);  // column lane of tau = row lane of Lc
-      d.xi0n[(size_t)k * B + lane] = sqrt(s);
+      for (int m = 0; m < B; ++m) s += cabs2(M2[m * B + tid]);  // column tid of tau
+      d.xi0n[(size_t)k * B + tid] = sqrt(s);
     }
-    if (lane == 0) {
+    if (tid == 0) {
       d.flag[k] = 0;
       d.its[k] = 0;
     }
     return;
   }
-  // xi_{k+1} = tau xi_k, tau[a][m] = conj(Lc[m][a]) (m >= a)
-  for (int e = lane; e < B * B; e += 32) M0[e] = d.xi[ko + e];
-  __syncwarp();
-  {
-    const int j = lane;
-    if (j < B) {
-      for (int a = 0; a < B; ++a) {
-        double2 v = make_double2(0.0, 0.0);
-        for (int m = a; m < B; ++m) {
-          const double2 l = M2[m * B + a];
-          const double2 t = make_double2(l.x, -l.y);
-          const double2 x = M0[m * B + j];
-          v.x += t.x * x.x - t.y * x.y;
-          v.y += t.x * x.y + t.y * x.x;
-        }
-        aug[a * 2 * B + B + j] = v;  // staged: tau xi
-      }
-    }
-    __syncwarp();
+  // xi_{k+1} = tau xi_k
+  if (own) aug[tid] = d.xi[ko + tid];
+  __syncthreads();  // M1 and the old xi are complete
+  double2 xn = zero, rhs = zero;
+  if (own) {
+    for (int m = a; m < B; ++m) xn = cfma64(M2[a * B + m], aug[m * B + j], xn);
+    // right-hand side of beta: tau^T QQ_{k+1}
+    for (int m = 0; m <= a; ++m) rhs = cfma64(M2[m * B + a], M1[m * B + j], rhs);
+    d.xi[ko + tid] = xn;
+    M0[tid] = make_double2(cabs2(xn), 0.0);
   }
-  for (int e = lane; e < B * B; e += 32) d.xi[ko + e] = aug[(e / B) * 2 * B + B + (e % B)];
+  __syncthreads();
   // every column's residual norm ||xi[:, j]|| against its start
   bool conv = true;
-  if (lane < B) {
+  if (tid < B) {
     double s = 0.0;
-    for (int a = 0; a < B; ++a) s += cabs2(aug[a * 2 * B + B + lane]);
-    conv = sqrt(s) <= d.tol_in * d.xi0n[(size_t)k * B + lane];
+    for (int m = 0; m < B; ++m) s += M0[m * B + tid].x;
+    conv = sqrt(s) <= d.tol_in * d.xi0n[(size_t)k * B + tid];
   }
-  conv = __all_sync(0xffffffffu, conv);
-  __syncwarp();
-  // beta = QQ_k^{-1} (tau^T QQ_{k+1}); tau^T[a][m] = tau[m][a] = conj(Lc[a][m]) (m <= a)
-  {
-    const int j = lane;
-    if (j < B) {
-      for (int a = 0; a < B; ++a) {
-        double2 v = make_double2(0.0, 0.0);
-        for (int m = 0; m <= a; ++m) {
-          const double2 l = M2[a * B + m];
-          const double2 t = make_double2(l.x, -l.y);
-          const double2 q = M1[m * B + j];
-          v.x += t.x * q.x - t.y * q.y;
-          v.y += t.x * q.y + t.y * q.x;
-        }
-        aug[a * 2 * B + B + j] = v;
-      }
-    }
-    __syncwarp();
+  // beta = QQ_k^{-1} (tau^T QQ_{k+1})
+  if (own) {
+    aug[a * LD + j] = d.QQ[ko + tid];
+    aug[a * LD + B + j] = rhs;
   }
-  for (int e = lane; e < B * B; e += 32) aug[(e / B) * 2 * B + (e % B)] = d.QQ[ko + e];
-  __syncwarp();
-  const bool ok = warp_solve<B>(aug, fac, &s_i, M0);  // M0 = beta
-  for (int e = lane; e < B * B; e += 32) {
-    d.QQ[ko + e] = M1[e];
-    if (ok) d.beta[ko + e] = to32(M0[e]);
+  conv = __syncthreads_and(conv);
+  const bool ok = gauss_jordan<B, LD>(aug);
+  if (own) {
+    d.QQ[ko + tid] = M1[tid];
+    if (ok) d.beta[ko + tid] = to32(aug[a * LD + B + j]);
   }
-  if (lane == 0) {
+  if (tid == 0) {
     const int it = d.its[k] + 1;
     d.its[k] = it;
     d.flag[k] = conv ? 1 : !ok ? 2 : it >= d.icap[k] ? 3 : 0;
@@ -830,19 +775,17 @@ cudaError_t launch_blk_q0(int B, int nb, cudaStream_t st, const BlkDev* d, long 
 }
 
 cudaError_t launch_blk_small(int B, int phase, int nb, cudaStream_t st, const BlkDev* d) {
-  if (phase == 0) {
-#define L_(BB) blk_small_kernel<BB, 0><<<nb, 32, 0, st>>>(d)
-    RSN_BLK_DISPATCH(B, L_)
-#undef L_
-  } else if (phase == 1) {
-#define L_(BB) blk_small_kernel<BB, 1><<<nb, 32, 0, st>>>(d)
-    RSN_BLK_DISPATCH(B, L_)
-#undef L_
-  } else {
-#define L_(BB) blk_small_kernel<BB, 2><<<nb, 32, 0, st>>>(d)
-    RSN_BLK_DISPATCH(B, L_)
-#undef L_
+  const int no = phase == 1 ? 1 : 2, nt = B * B < 32 ? 32 : B * B;
+  const dim3 gs((no * B * B + 7) / 8, nb);
+#define L_(BB)                                                                 \
+  {                                                                            \
+    blk_psum_kernel<BB><<<gs, 256, 0, st>>>(d, no);                            \
+    if (phase == 0) blk_small_kernel<BB, 0><<<nb, nt, 0, st>>>(d);             \
+    else if (phase == 1) blk_small_kernel<BB, 1><<<nb, nt, 0, st>>>(d);        \
+    else blk_small_kernel<BB, 2><<<nb, nt, 0, st>>>(d);                        \
   }
+  RSN_BLK_DISPATCH(B, L_)
+#undef L_
   return cudaGetLastError();
 }
 

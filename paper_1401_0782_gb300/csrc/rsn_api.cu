@@ -121,7 +121,7 @@ struct PoolSpec {
 // D and the FP64 iterate / residual of every member of a wave of blocks, the
 // b x b state of each block, and the apply lists of the active members.
 struct BlkBufs {
-  DevBuf W, P, AP, D, X, R, part, xi, QQ, xi0n, alpha, axi, tinv, tinv64, beta, flag, its, rpart, rn, tt, blist, col;
+  DevBuf W, P, AP, D, X, R, part, gsum, xi, QQ, xi0n, alpha, axi, tinv, tinv64, beta, flag, its, rpart, rn, tt, blist, col;
   DevBuf vE, vjunc, voff, cbuf, dev, bdev, jd, t_all, gr_cols, Td, stat, icap;
 };
 
@@ -1871,6 +1871,7 @@ static rsn_status block_impl(rsn_ctx* c, int n_e, const double* E, int n_cols, c
       nchunkR = (int)((N + chunkR_pts - 1) / chunkR_pts);
       const size_t bb2 = (size_t)nbw * B * B;
       RSN_CUDA(c, q.part.ensure((size_t)nbw * nchunk * 2 * B * B * sizeof(double2)));
+      RSN_CUDA(c, q.gsum.ensure(2 * bb2 * sizeof(double2)));
       RSN_CUDA(c, q.xi.ensure(bb2 * sizeof(double2)));
       RSN_CUDA(c, q.QQ.ensure(bb2 * sizeof(double2)));
       RSN_CUDA(c, q.xi0n.ensure((size_t)S * sizeof(double)));
@@ -1917,6 +1918,7 @@ static rsn_status block_impl(rsn_ctx* c, int n_e, const double* E, int n_cols, c
       hd.QQ = q.QQ.as<double2>();
       hd.xi0n = q.xi0n.as<double>();
       hd.part = q.part.as<double2>();
+      hd.gsum = q.gsum.as<double2>();
       hd.alpha = q.alpha.as<float2>();
       hd.axi = q.axi.as<float2>();
       hd.tinv = q.tinv.as<float2>();

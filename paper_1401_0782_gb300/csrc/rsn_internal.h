@@ -242,6 +242,7 @@ struct BlkDev {
   double2* QQ;            // Q_k^T Q_k
   double* xi0n;           // [nb][B] column norms of xi_0
   double2* part;          // [nb][nchunk][2][B*B] Gram partials
+  double2* gsum;          // [nb][2][B*B] their sums over the chunks
   float2* alpha;          // alpha_k = (P^T A P)^{-1} Q^T Q
   float2* axi;            // alpha_k xi_k
   float2* tinv;           // tau_k^{-1} (upper triangular)
