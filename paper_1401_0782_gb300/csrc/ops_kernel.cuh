@@ -20,8 +20,8 @@
 //             projections (-sum_p e_kb[p] c_p^2).
 //   OP_RESID: v = x64 + d          (refinement iterate), writes r = b - A v,
 //             and partial sums of ||r||^2 and r^T r; computed in FP64.
-//   OP_APPLY: v = x (input),  y = A v.
-// The projector term uses ce[p] = e_kb[p] (v_p . v), prepared per CTA from the
+//   OP_APPLY: v = x (input),  y = A_loc v (nonlocal_kernel adds the projector term).
+// The projector term of OP_RESID uses ce[p] = e_kb[p] (v_p . v), prepared per CTA from the
 // projections computed by the gather kernel; each grid point adds -sum over
 // its atom entries of the projector values times ce.
 #pragma once
@@ -94,8 +94,7 @@ constexpr int kOpThreads = 256;
 // One (tile, slot) of the operator: the CTA's tile blockIdx.x of slot s.
 template <typename T, int R, int PPT, int MODE>
 __device__ __forceinline__ void op_tile(const JuncDev* __restrict__ jt, const BatchDev& b, const int s,
-                                        const void* __restrict__ x_in, void* __restrict__ y_out,
-                                        const void* __restrict__ c_in) {
+                                        const void* __restrict__ x_in, void* __restrict__ y_out) {
   // compute type: FP64 for the true residual, else the inner precision
   using CT = typename std::conditional<MODE == OP_RESID, double, T>::type;
   using C = typename cx<CT>::t;   // compute complex
@@ -146,25 +145,16 @@ __device__ __forceinline__ void op_tile(const JuncDev* __restrict__ jt, const Ba
   }
 
   // ---- projector coefficients ce[p] = e_kb[p] * (v_p . v) -------------------
-  // (COCG: none.  The projector term of q = A p is added by the update
-  // kernel, and the projection kernel forms c_p = v_p . p of the new direction,
+  // (true residual only.  COCG: the projector term of q = A p is added by the
+  // update kernel, and the projection kernel forms c_p = v_p . p of the new direction,
   // e_kb c_p and the term's share of mu, -sum_p e_kb[p] c_p^2 (p^T v_p = c_p,
-  // unconjugated), from the projections alone.)
+  // unconjugated), from the projections alone.  Apply: nonlocal_kernel adds it.)
   const int n_proj = J.n_proj;
-  if (MODE != OP_COCG && n_proj > 0) {
-    if constexpr (MODE == OP_RESID) {
-      const double2* cxp = b.c_x + (size_t)s * b.pstride;
-      for (int p = tid; p < n_proj; p += nt) {
-        const double e = J.ekb[p];
-        ce[p] = mk2((CT)(e * cxp[p].x), (CT)(e * cxp[p].y));
-      }
-    } else {
-      const CO* cin = reinterpret_cast<const CO*>(c_in) + (size_t)s * b.pstride;
-      for (int p = tid; p < n_proj; p += nt) {
-        const CT e = (CT)J.ekb[p];
-        C c = cin[p];
-        ce[p] = mk2(e * c.x, e * c.y);
-      }
+  if (MODE == OP_RESID && n_proj > 0) {
+    const double2* cxp = b.c_x + (size_t)s * b.pstride;
+    for (int p = tid; p < n_proj; p += nt) {
+      const double e = J.ekb[p];
+      ce[p] = mk2((CT)(e * cxp[p].x), (CT)(e * cxp[p].y));
     }
     for (int p = tid; p < kCePad; p += nt) ce[n_proj + p] = czero<C>();
   }
@@ -254,7 +244,7 @@ __device__ __forceinline__ void op_tile(const JuncDev* __restrict__ jt, const Ba
       if (own[u] && z < z1) {
         const long long g = (long long)z * plane + po[u];
         if constexpr (sizeof(CT) == 4) dgf_n[u] = J.dg32[g];
-        if (MODE != OP_COCG && n_proj > 0) {
+        if (MODE == OP_RESID && n_proj > 0) {
           e0_n[u] = J.inv_ptr[g];
           e1_n[u] = J.inv_ptr[g + 1];
         }
@@ -319,7 +309,7 @@ __device__ __forceinline__ void op_tile(const JuncDev* __restrict__ jt, const Ba
       } else {
         y = fd_diff_form<C, CT, R>(qv[u], smb, so[u], pitch, wst, vc, dgf_c[u], E);
       }
-      if (MODE != OP_COCG && n_proj > 0) {
+      if (MODE == OP_RESID && n_proj > 0) {
         const int e0 = e0_c[u], e1 = e1_c[u], nq = J.inv_nq;
         for (int e = e0; e < e1; ++e) {
           const C* cp = ce + J.inv_p0[e];
@@ -394,25 +384,25 @@ __device__ __forceinline__ void op_tile(const JuncDev* __restrict__ jt, const Ba
 template <typename T, int R, int PPT, int MODE>
 __global__ void __launch_bounds__(kOpThreads, (MODE == OP_RESID ? 2 : (PPT == 1 ? 4 : (PPT == 2 ? 3 : 2))))
 op_kernel(const JuncDev* __restrict__ jt, const BatchDev* __restrict__ bp, const void* __restrict__ x_in,
-          void* __restrict__ y_out, const void* __restrict__ c_in) {
+          void* __restrict__ y_out) {
   const BatchDev& b = *bp;
   if constexpr (MODE == OP_RESID) {
     // the true residual runs only for the NEW / CHECK slots of the list: CTA
     // rows take its entries in turn
     const int n = *b.lst_n;
     for (int li = blockIdx.y; li < n; li += gridDim.y) {
-      op_tile<T, R, PPT, MODE>(jt, b, b.lst[li], x_in, y_out, c_in);
+      op_tile<T, R, PPT, MODE>(jt, b, b.lst[li], x_in, y_out);
       __syncthreads();  // the shared-memory planes are reused by the next entry
     }
   } else {
-    op_tile<T, R, PPT, MODE>(jt, b, blockIdx.y, x_in, y_out, c_in);
+    op_tile<T, R, PPT, MODE>(jt, b, blockIdx.y, x_in, y_out);
   }
 }
 
 template <int R>
 cudaError_t launch_op_r(int mode, bool fp32, int ppt, dim3 grid, int threads, size_t smem, cudaStream_t st,
-                        const JuncDev* jt, const BatchDev* b, const void* x_in, void* y_out, const void* c_in) {
-  void (*kern)(const JuncDev*, const BatchDev*, const void*, void*, const void*) = nullptr;
+                        const JuncDev* jt, const BatchDev* b, const void* x_in, void* y_out) {
+  void (*kern)(const JuncDev*, const BatchDev*, const void*, void*) = nullptr;
 #define RSN_PICK(T, P)                                                   \
   if (mode == OP_COCG) kern = op_kernel<T, R, P, OP_COCG>;               \
   else if (mode == OP_RESID) kern = op_kernel<T, R, P, OP_RESID>;        \
@@ -440,7 +430,7 @@ cudaError_t launch_op_r(int mode, bool fp32, int ppt, dim3 grid, int threads, si
     if (e != cudaSuccess) return e;
   }
   cudaFuncSetAttribute(kern, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared);
-  kern<<<grid, threads, smem, st>>>(jt, b, x_in, y_out, c_in);
+  kern<<<grid, threads, smem, st>>>(jt, b, x_in, y_out);
   return cudaGetLastError();
 }
 
@@ -458,7 +448,7 @@ constexpr int kStages = 4;
 template <typename T, int R, int MODE>
 __global__ void __launch_bounds__(1024, 1)
 op_kernel_tma(const JuncDev* __restrict__ jt, const BatchDev* __restrict__ bp, const void* __restrict__ x_in,
-              void* __restrict__ y_out, const void* __restrict__ c_in) {
+              void* __restrict__ y_out) {
   using C = typename cx<T>::t;
   constexpr int Q = 2 * R + 1;
   constexpr int NIN = (MODE == OP_COCG) ? 2 : 1;
@@ -480,10 +470,8 @@ op_kernel_tma(const JuncDev* __restrict__ jt, const BatchDev* __restrict__ bp, c
   extern __shared__ __align__(16) unsigned char smem_raw[];
   C* stage = reinterpret_cast<C*>(smem_raw);          // [kStages][NIN][plane]
   C* exch = stage + kStages * NIN * plane;           // [2][prow][pitch]
-  C* ce = exch + 2 * prow * pitch;                   // [n_proj]
-  const int n_proj = J.n_proj;
   uint64_t* bars = reinterpret_cast<uint64_t*>(
-      (reinterpret_cast<uintptr_t>(ce + n_proj + kCePad) + 15) & ~static_cast<uintptr_t>(15));
+      (reinterpret_cast<uintptr_t>(exch + 2 * prow * pitch) + 15) & ~static_cast<uintptr_t>(15));
   __shared__ double red[32 * 2];
   __shared__ int s_bad;
 
@@ -506,16 +494,6 @@ op_kernel_tma(const JuncDev* __restrict__ jt, const BatchDev* __restrict__ bp, c
     pnew = reinterpret_cast<C*>((k & 1) ? b.p0 : b.p1);
   } else {
     src0 = reinterpret_cast<const C*>(x_in) + vo;
-  }
-  // APPLY only: in COCG the projector term of q is added on the support points
-  if (MODE != OP_COCG && n_proj > 0) {
-    const C* cin = reinterpret_cast<const C*>(c_in) + (size_t)s * b.pstride;
-    for (int p = tid; p < n_proj; p += nt) {
-      const T e = (T)J.ekb[p];
-      const C c = cin[p];
-      ce[p] = mk2(e * c.x, e * c.y);
-    }
-    for (int p = tid; p < kCePad; p += nt) ce[n_proj + p] = czero<C>();
   }
   __syncthreads();
 
@@ -551,15 +529,10 @@ op_kernel_tma(const JuncDev* __restrict__ jt, const BatchDev* __restrict__ bp, c
   T acc0 = 0, acc1 = 0, car0 = 0, car1 = 0;
   // per-point operator data of the next plane to compute, loaded one plane early
   float2 dg_n = make_float2(0.f, 0.f);
-  int e0_n = 0, e1_n = 0;
   auto load_pt = [&](int z) {
     if (own && z < z1) {
       const long long g = (long long)z * plane + tid;
       if constexpr (sizeof(T) == 4) dg_n = J.dg32[g];
-      if (MODE != OP_COCG && n_proj > 0) {
-        e0_n = J.inv_ptr[g];
-        e1_n = J.inv_ptr[g + 1];
-      }
     }
   };
   load_pt(z0);
@@ -597,7 +570,6 @@ op_kernel_tma(const JuncDev* __restrict__ jt, const BatchDev* __restrict__ bp, c
     }
     if (zc < z0 || !own) continue;
     const float2 dg_c = dg_n;
-    const int e0 = e0_n, e1 = e1_n;
     load_pt(zc + 1);
 
     const C vc = qv[R];
@@ -616,13 +588,6 @@ op_kernel_tma(const JuncDev* __restrict__ jt, const BatchDev* __restrict__ bp, c
       y = cfma(mk2((T)(E + t.x), (T)t.y), vc, lap);
     } else {
       y = fd_diff_form<C, T, R>(qv, smb, so, pitch, wst, vc, dg_c, E);
-    }
-    if (MODE != OP_COCG && n_proj > 0) {
-      const int nq = J.inv_nq;
-      for (int e = e0; e < e1; ++e) {
-        const C* cp = ce + J.inv_p0[e];
-        for (int qd = 0; qd < nq; ++qd) y = proj_quad<C, T>(J, e * nq + qd, cp + 4 * qd, y);
-      }
     }
     if constexpr (MODE == OP_COCG) {
       pnew[vo + gl] = vc;
@@ -644,8 +609,8 @@ op_kernel_tma(const JuncDev* __restrict__ jt, const BatchDev* __restrict__ bp, c
 
 template <int R>
 cudaError_t launch_op_tma_r(int mode, bool fp32, dim3 grid, int threads, size_t smem, cudaStream_t st,
-                            const JuncDev* jt, const BatchDev* b, const void* x_in, void* y_out, const void* c_in) {
-  void (*kern)(const JuncDev*, const BatchDev*, const void*, void*, const void*) = nullptr;
+                            const JuncDev* jt, const BatchDev* b, const void* x_in, void* y_out) {
+  void (*kern)(const JuncDev*, const BatchDev*, const void*, void*) = nullptr;
   if (mode == OP_COCG) kern = fp32 ? op_kernel_tma<float, R, OP_COCG> : op_kernel_tma<double, R, OP_COCG>;
   else if (mode == OP_APPLY) kern = fp32 ? op_kernel_tma<float, R, OP_APPLY> : op_kernel_tma<double, R, OP_APPLY>;
   else return cudaErrorInvalidValue;
@@ -654,7 +619,7 @@ cudaError_t launch_op_tma_r(int mode, bool fp32, dim3 grid, int threads, size_t 
     if (e != cudaSuccess) return e;
   }
   cudaFuncSetAttribute(kern, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared);
-  kern<<<grid, threads, smem, st>>>(jt, b, x_in, y_out, c_in);
+  kern<<<grid, threads, smem, st>>>(jt, b, x_in, y_out);
   return cudaGetLastError();
 }
 
@@ -664,22 +629,22 @@ cudaError_t launch_op_tma_r(int mode, bool fp32, dim3 grid, int threads, size_t 
   namespace rsn {                                                                                 \
   cudaError_t launch_op_R##R(int mode, bool fp32, int ppt, dim3 grid, int threads, size_t smem,  \
                              cudaStream_t st, const JuncDev* jt, const BatchDev* b,             \
-                             const void* x_in, void* y_out, const void* c_in) {                  \
-    return launch_op_r<R>(mode, fp32, ppt, grid, threads, smem, st, jt, b, x_in, y_out, c_in);   \
+                             const void* x_in, void* y_out) {                  \
+    return launch_op_r<R>(mode, fp32, ppt, grid, threads, smem, st, jt, b, x_in, y_out);   \
   }                                                                                               \
   cudaError_t launch_op_tma_R##R(int mode, bool fp32, dim3 grid, int threads, size_t smem,        \
                                  cudaStream_t st, const JuncDev* jt, const BatchDev* b,         \
-                                 const void* x_in, void* y_out, const void* c_in) {              \
-    return launch_op_tma_r<R>(mode, fp32, grid, threads, smem, st, jt, b, x_in, y_out, c_in);    \
+                                 const void* x_in, void* y_out) {              \
+    return launch_op_tma_r<R>(mode, fp32, grid, threads, smem, st, jt, b, x_in, y_out);    \
   }                                                                                               \
   cudaError_t launch_op_plane_R##R(int mode, dim3 grid, int threads, size_t smem, cudaStream_t st, \
                                    const JuncDev* jt, const BatchDev* b, const void* x_in,      \
-                                   void* y_out, const void* c_in) {                              \
-    return launch_op_plane_r<R>(mode, grid, threads, smem, st, jt, b, x_in, y_out, c_in);        \
+                                   void* y_out) {                              \
+    return launch_op_plane_r<R>(mode, grid, threads, smem, st, jt, b, x_in, y_out);        \
   }                                                                                               \
   cudaError_t launch_op_pair_R##R(int mode, bool big, dim3 grid, int threads, size_t smem,        \
                                   cudaStream_t st, const JuncDev* jt, const BatchDev* b,        \
-                                  const void* x_in, void* y_out, const void* c_in) {             \
-    return launch_op_pair_r<R>(mode, big, grid, threads, smem, st, jt, b, x_in, y_out, c_in);    \
+                                  const void* x_in, void* y_out) {             \
+    return launch_op_pair_r<R>(mode, big, grid, threads, smem, st, jt, b, x_in, y_out);    \
   }                                                                                               \
   }

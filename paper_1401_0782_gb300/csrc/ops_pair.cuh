@@ -1,7 +1,7 @@
 // FP32 operator kernel on point pairs with plane streaming: y = A_loc(E) v
-// (COCG) or y = A(E) x (apply), A(E) = E - H_KS + i(Gamma_L + Gamma_R) (Eqs. G
-// and Hop), H_KS = -1/2 lap_FD + V_loc [+ sum_p |v_p> e_kb <v_p| in the apply
-// mode] (Sec. II.C).
+// (COCG) or y = A_loc(E) x (apply), A_loc = E - H + i(Gamma_L + Gamma_R) (Eqs. G
+// and Hop) with H = -1/2 lap_FD + V_loc (Sec. II.C); the projector term is added
+// by the COCG update kernel, or by nonlocal_kernel after an application.
 //
 // One CTA owns whole x-y planes [z0, z0+Lz) of one slot and marches along z.
 //  * The input planes (r and p_old, or x) of planes z0-R .. z0+Lz+R-1 arrive by
@@ -103,7 +103,7 @@ __device__ __forceinline__ void sts_pair(float2* s, const Pair& v) {
 template <int R, int MODE, bool BIG>
 __global__ void __maxnreg__(96)
 op_pair_kernel(const JuncDev* __restrict__ jt, const BatchDev* __restrict__ bp, const void* __restrict__ x_in,
-               void* __restrict__ y_out, const void* __restrict__ c_in) {
+               void* __restrict__ y_out) {
   constexpr int Q = 2 * R + 1;
   constexpr int MD = R < 2 ? R : 2;  // distances summed in difference form
   constexpr int KX = (R + 1) / 2;    // neighbour pairs left / right in x
@@ -124,15 +124,12 @@ op_pair_kernel(const JuncDev* __restrict__ jt, const BatchDev* __restrict__ bp, 
   const int rows = ny + 2 * R;
   const int tid = threadIdx.x, nt = blockDim.x;
   const long long vo = b.voff[s];
-  const int n_proj = J.n_proj;
 
   extern __shared__ __align__(16) unsigned char smem_raw[];
   float2* stage = reinterpret_cast<float2*>(smem_raw);  // [kPairStages][NIN][plane]
   float2* exch = stage + kPairStages * NIN * plane;    // [2][rows][pitch]
-  float2* ce = exch + 2 * rows * pitch;                 // apply mode: e_kb[p] (v_p . x)
   uint64_t* bars = reinterpret_cast<uint64_t*>(
-      (reinterpret_cast<uintptr_t>(ce + (MODE == OP_APPLY ? n_proj + kCePad : 0)) + 15) &
-      ~static_cast<uintptr_t>(15));
+      (reinterpret_cast<uintptr_t>(exch + 2 * rows * pitch) + 15) & ~static_cast<uintptr_t>(15));
   __shared__ double red[32 * 2];
   __shared__ int s_bad;
 
@@ -159,15 +156,6 @@ op_pair_kernel(const JuncDev* __restrict__ jt, const BatchDev* __restrict__ bp, 
   } else {
     src0 = reinterpret_cast<const float2*>(x_in) + vo;
     yv = reinterpret_cast<float2*>(y_out) + vo;
-  }
-  if (MODE == OP_APPLY && n_proj > 0) {
-    const float2* cin = reinterpret_cast<const float2*>(c_in) + (size_t)s * b.pstride;
-    for (int p = tid; p < n_proj; p += nt) {
-      const float e = (float)J.ekb[p];
-      const float2 c = cin[p];
-      ce[p] = make_float2(e * c.x, e * c.y);
-    }
-    for (int p = tid; p < kCePad; p += nt) ce[n_proj + p] = make_float2(0.f, 0.f);
   }
   __syncthreads();
 
@@ -303,28 +291,6 @@ op_pair_kernel(const JuncDev* __restrict__ jt, const BatchDev* __restrict__ bp, 
           float2 y0v = cfma2(make_float2(Ef + dgc.x, dgc.y), c0, lap0);
           float2 y1v = cfma2(make_float2(Ef + dgc.z, dgc.w), c1, lap1);
           const int gi = zc * plane + po;
-          if constexpr (MODE == OP_APPLY) {
-            if (n_proj > 0) {
-              const int nq = J.inv_nq;
-#pragma unroll
-              for (int jj = 0; jj < 2; ++jj) {
-                float2 yy = jj ? y1v : y0v;
-                const int e0 = J.inv_ptr[gi + jj], e1 = J.inv_ptr[gi + jj + 1];
-                for (int e = e0; e < e1; ++e) {
-                  const float2* cp = ce + J.inv_p0[e];
-                  for (int qd = 0; qd < nq; ++qd) {
-                    const float4 a = J.inv_q32[e * nq + qd];
-                    yy = fma2(make_float2(-a.x, -a.x), cp[4 * qd], yy);
-                    yy = fma2(make_float2(-a.y, -a.y), cp[4 * qd + 1], yy);
-                    yy = fma2(make_float2(-a.z, -a.z), cp[4 * qd + 2], yy);
-                    yy = fma2(make_float2(-a.w, -a.w), cp[4 * qd + 3], yy);
-                  }
-                }
-                if (jj) y1v = yy;
-                else y0v = yy;
-              }
-            }
-          }
           if constexpr (MODE == OP_COCG) {
             *reinterpret_cast<float4*>(pnew + gi) = make_float4(c0.x, c0.y, c1.x, c1.y);
             // mu partial v^T y (unconjugated) of both points, Kahan-compensated
@@ -362,7 +328,7 @@ op_pair_kernel(const JuncDev* __restrict__ jt, const BatchDev* __restrict__ bp, 
 template <int R, int MODE>
 __global__ void __launch_bounds__(kPlaneThreads, 2)
 op_plane_kernel(const JuncDev* __restrict__ jt, const BatchDev* __restrict__ bp, const void* __restrict__ x_in,
-                void* __restrict__ y_out, const void* __restrict__ c_in) {
+                void* __restrict__ y_out) {
   constexpr int Q = 2 * R + 1;
   constexpr int MD = R < 2 ? R : 2;  // distances summed in difference form
   constexpr int NIN = (MODE == OP_COCG) ? 2 : 1;
@@ -381,15 +347,12 @@ op_plane_kernel(const JuncDev* __restrict__ jt, const BatchDev* __restrict__ bp,
   const int rows = ny + 2 * R;
   const int tid = threadIdx.x, nt = blockDim.x;
   const long long vo = b.voff[s];
-  const int n_proj = J.n_proj;
 
   extern __shared__ __align__(16) unsigned char smem_raw[];
   float2* stage = reinterpret_cast<float2*>(smem_raw);  // [kPairStages][NIN][plane]
   float2* exch = stage + kPairStages * NIN * plane;    // [2][rows][pitch]
-  float2* ce = exch + 2 * rows * pitch;                 // apply mode: e_kb[p] (v_p . x)
   uint64_t* bars = reinterpret_cast<uint64_t*>(
-      (reinterpret_cast<uintptr_t>(ce + (MODE == OP_APPLY ? n_proj + kCePad : 0)) + 15) &
-      ~static_cast<uintptr_t>(15));
+      (reinterpret_cast<uintptr_t>(exch + 2 * rows * pitch) + 15) & ~static_cast<uintptr_t>(15));
   __shared__ double red[32 * 2];
   __shared__ int s_bad;
   __shared__ float s_w[R + 2];
@@ -423,15 +386,6 @@ op_plane_kernel(const JuncDev* __restrict__ jt, const BatchDev* __restrict__ bp,
   } else {
     src0 = reinterpret_cast<const float2*>(x_in) + vo;
     yv = reinterpret_cast<float2*>(y_out) + vo;
-  }
-  if (MODE == OP_APPLY && n_proj > 0) {
-    const float2* cin = reinterpret_cast<const float2*>(c_in) + (size_t)s * b.pstride;
-    for (int p = tid; p < n_proj; p += nt) {
-      const float e = (float)J.ekb[p];
-      const float2 c = cin[p];
-      ce[p] = make_float2(e * c.x, e * c.y);
-    }
-    for (int p = tid; p < kCePad; p += nt) ce[n_proj + p] = make_float2(0.f, 0.f);
   }
   __syncthreads();
 
@@ -536,24 +490,6 @@ op_plane_kernel(const JuncDev* __restrict__ jt, const BatchDev* __restrict__ bp,
           const float dr = s_w[0] + dgc.x, di = dgc.y;
           float2 y = make_float2(fmaf(dr, c.x, fmaf(-di, c.y, lx)), fmaf(dr, c.y, fmaf(di, c.x, ly)));
           const int gi = zc * plane + tid;
-          if constexpr (MODE == OP_APPLY) {
-            if (n_proj > 0) {
-              const int nq = J.inv_nq;
-              const int e0 = J.inv_ptr[gi], e1 = J.inv_ptr[gi + 1];
-              for (int e = e0; e < e1; ++e) {
-                const float2* cp = ce + J.inv_p0[e];
-                for (int qd = 0; qd < nq; ++qd) {
-                  const float4 a = J.inv_q32[e * nq + qd];
-                  const float av[4] = {a.x, a.y, a.z, a.w};
-#pragma unroll
-                  for (int jj = 0; jj < 4; ++jj) {
-                    y.x = fmaf(-av[jj], cp[4 * qd + jj].x, y.x);
-                    y.y = fmaf(-av[jj], cp[4 * qd + jj].y, y.y);
-                  }
-                }
-              }
-            }
-          }
           if constexpr (MODE == OP_COCG) {
             pnew[gi] = c;
             // mu partial v^T y (unconjugated), Kahan-compensated
@@ -576,8 +512,8 @@ op_plane_kernel(const JuncDev* __restrict__ jt, const BatchDev* __restrict__ bp,
 
 template <int R>
 cudaError_t launch_op_plane_r(int mode, dim3 grid, int threads, size_t smem, cudaStream_t st, const JuncDev* jt,
-                              const BatchDev* b, const void* x_in, void* y_out, const void* c_in) {
-  void (*kern)(const JuncDev*, const BatchDev*, const void*, void*, const void*) = nullptr;
+                              const BatchDev* b, const void* x_in, void* y_out) {
+  void (*kern)(const JuncDev*, const BatchDev*, const void*, void*) = nullptr;
   if (mode == OP_COCG) kern = op_plane_kernel<R, OP_COCG>;
   else if (mode == OP_APPLY) kern = op_plane_kernel<R, OP_APPLY>;
   else return cudaErrorInvalidValue;
@@ -587,14 +523,14 @@ cudaError_t launch_op_plane_r(int mode, dim3 grid, int threads, size_t smem, cud
     if (e != cudaSuccess) return e;
   }
   cudaFuncSetAttribute(kern, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared);
-  kern<<<grid, threads, smem, st>>>(jt, b, x_in, y_out, c_in);
+  kern<<<grid, threads, smem, st>>>(jt, b, x_in, y_out);
   return cudaGetLastError();
 }
 
 template <int R>
 cudaError_t launch_op_pair_r(int mode, bool big, dim3 grid, int threads, size_t smem, cudaStream_t st,
-                             const JuncDev* jt, const BatchDev* b, const void* x_in, void* y_out, const void* c_in) {
-  void (*kern)(const JuncDev*, const BatchDev*, const void*, void*, const void*) = nullptr;
+                             const JuncDev* jt, const BatchDev* b, const void* x_in, void* y_out) {
+  void (*kern)(const JuncDev*, const BatchDev*, const void*, void*) = nullptr;
   if (mode == OP_COCG) kern = big ? op_pair_kernel<R, OP_COCG, true> : op_pair_kernel<R, OP_COCG, false>;
   else if (mode == OP_APPLY) kern = big ? op_pair_kernel<R, OP_APPLY, true> : op_pair_kernel<R, OP_APPLY, false>;
   else return cudaErrorInvalidValue;
@@ -604,7 +540,7 @@ cudaError_t launch_op_pair_r(int mode, bool big, dim3 grid, int threads, size_t 
     if (e != cudaSuccess) return e;
   }
   cudaFuncSetAttribute(kern, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared);
-  kern<<<grid, threads, smem, st>>>(jt, b, x_in, y_out, c_in);
+  kern<<<grid, threads, smem, st>>>(jt, b, x_in, y_out);
   return cudaGetLastError();
 }
 

@@ -167,7 +167,9 @@ struct rsn_ctx {
   Workspace ws;
   CallBufs cb;
   BlkBufs bb;
-  DevBuf bd;  // device BatchDev: [0] streaming solver, [1] rsn_apply
+  DevBuf bd;  // device BatchDev of the streaming solver
+  DevBuf ap;  // one rsn_apply call's BatchDev, JuncDev and per-vector tables, and their host image
+  std::vector<unsigned char> ap_host;
   std::map<GraphKey, cudaGraphExec_t> graphs;
   int* sched_host = nullptr;  // pinned mirror of BatchDev::sched
   unsigned long long* cnt_host = nullptr;  // pinned mirror of BatchDev::counters
@@ -252,7 +254,7 @@ static Tiling choose_tiling(const rsn_ctx* c, bool compute64, int mode, int nslo
   };
   if (!compute64 && mode != OP_RESID && streamable && !reg_forced && c->tile_override[3] != -3 && nx % 2 == 0) {
     const int thr = (int)(((pl / 2) + 31) / 32 * 32);
-    const size_t sm = op_pair_smem_bytes(mode, R, nx, ny, c->n_proj);
+    const size_t sm = op_pair_smem_bytes(mode, R, nx, ny);
     if (thr <= kPairThreadsBig && sm <= 200 * 1024) {
       t.pair = true;
       t.big = thr > kPairThreads;
@@ -265,7 +267,7 @@ static Tiling choose_tiling(const rsn_ctx* c, bool compute64, int mode, int nslo
   }
   if (!compute64 && mode != OP_RESID && streamable && !reg_forced && c->tile_override[3] != -2 && pl % 2 == 0 &&
       pl <= kPlaneThreads) {
-    const size_t sm = op_pair_smem_bytes(mode, R, nx, ny, c->n_proj);
+    const size_t sm = op_pair_smem_bytes(mode, R, nx, ny);
     if (sm <= 100 * 1024) {
       t.plane = true;
       t.threads = (int)((pl + 31) / 32 * 32);
@@ -317,7 +319,7 @@ static Tiling choose_tiling(const rsn_ctx* c, bool compute64, int mode, int nslo
   // whose byte sizes keep every bulk copy 16-byte aligned
   if (!compute64 && mode != OP_RESID && streamable && pl <= 1024 && (pl * 8) % 16 == 0 && (c->N * 8) % 16 == 0 &&
       c->tile_override[3] == -1) {
-    const size_t sm = op_tma_smem_bytes(true, mode, R, nx, ny, c->n_proj);
+    const size_t sm = op_tma_smem_bytes(true, mode, R, nx, ny);
     if (sm <= 200 * 1024) {
       t.TY = ny;
       t.ytiles = 1;
@@ -333,13 +335,34 @@ static Tiling choose_tiling(const rsn_ctx* c, bool compute64, int mode, int nslo
 // Operator launch (COCG or apply) with a tiling from choose_tiling; the
 // JuncDev copy `jt` must carry the same tiling.
 static cudaError_t launch_inner(const rsn_ctx* c, const Tiling& t, int mode, bool fp32, int nslots, cudaStream_t st,
-                                const JuncDev* jt, const BatchDev* b, const void* x_in, void* y_out,
-                                const void* c_in) {
+                                const JuncDev* jt, const BatchDev* b, const void* x_in, void* y_out) {
   const dim3 grid(t.n, nslots);
-  if (t.plane) return launch_op_plane(mode, c->R, grid, t.threads, t.smem, st, jt, b, x_in, y_out, c_in);
-  if (t.pair) return launch_op_pair(mode, c->R, t.big, grid, t.threads, t.smem, st, jt, b, x_in, y_out, c_in);
-  if (t.tma) return launch_op_tma(mode, fp32, c->R, grid, t.threads, t.smem, st, jt, b, x_in, y_out, c_in);
-  return launch_op(mode, fp32, c->R, t.ppt, grid, t.threads, t.smem, st, jt, b, x_in, y_out, c_in);
+  if (t.plane) return launch_op_plane(mode, c->R, grid, t.threads, t.smem, st, jt, b, x_in, y_out);
+  if (t.pair) return launch_op_pair(mode, c->R, t.big, grid, t.threads, t.smem, st, jt, b, x_in, y_out);
+  if (t.tma) return launch_op_tma(mode, fp32, c->R, grid, t.threads, t.smem, st, jt, b, x_in, y_out);
+  return launch_op(mode, fp32, c->R, t.ppt, grid, t.threads, t.smem, st, jt, b, x_in, y_out);
+}
+
+// y = A(E) x of the n vectors that bdev describes: the projections (into c) and
+// the local operator side by side, then the projector term.
+static cudaError_t launch_apply(rsn_ctx* c, const Tiling& t, bool fp32, int n, const JuncDev* jt, const BatchDev* bdev,
+                                const void* x, void* y, void* coef) {
+  const bool proj = c->n_proj > 0;
+  cudaError_t e;
+  if (proj) {
+    if ((e = cudaEventRecord(c->ev_step, c->st)) != cudaSuccess) return e;
+    if ((e = cudaStreamWaitEvent(c->st3, c->ev_step, 0)) != cudaSuccess) return e;
+    if ((e = launch_project(2, fp32, n, c->n_groups, c->max_np, c->st3, jt, bdev, x, coef)) != cudaSuccess) return e;
+    if ((e = cudaEventRecord(c->ev_proj, c->st3)) != cudaSuccess) return e;
+  }
+  e = launch_inner(c, t, OP_APPLY, fp32, n, c->st, jt, bdev, x, y);
+  // join the projections' stream whether or not the operator was launched
+  if (proj) {
+    const cudaError_t ej = cudaStreamWaitEvent(c->st, c->ev_proj, 0);
+    if (e == cudaSuccess) e = ej;
+  }
+  if (e != cudaSuccess || !proj) return e;
+  return launch_nonlocal(fp32, n, c->N, c->n_proj, c->st, jt, bdev, coef, y);
 }
 
 // ---------------------------------------------------------------------------
@@ -554,19 +577,21 @@ struct LaunchCfg {
   const JuncDev* jt_resid;  // device pointer: tiling of the residual kernel
 };
 
+static void set_tiling_dev(JuncDev& J, const Tiling& t) {
+  J.TY = t.TY;
+  J.Lz = t.Lz;
+  J.ytiles = t.ytiles;
+  J.ztiles = t.ztiles;
+  J.nA = t.n;
+  J.kind = t.plane ? kOpPlane : t.pair ? kOpPair : t.tma ? kOpTma : kOpReg;
+}
+
 static rsn_status make_cfg(rsn_ctx* c, const Tiling& inner, const Tiling& resid, LaunchCfg& cfg) {
   cfg.inner = inner;
   cfg.resid = resid;
   JuncDev js[2] = {c->jh, c->jh};
-  for (int k = 0; k < 2; ++k) {
-    const Tiling& t = k == 0 ? cfg.inner : cfg.resid;
-    js[k].TY = t.TY;
-    js[k].Lz = t.Lz;
-    js[k].ytiles = t.ytiles;
-    js[k].ztiles = t.ztiles;
-    js[k].nA = t.n;
-    js[k].kind = k == 1 ? kOpReg : t.plane ? kOpPlane : t.pair ? kOpPair : t.tma ? kOpTma : kOpReg;
-  }
+  set_tiling_dev(js[0], inner);
+  set_tiling_dev(js[1], resid);
   RSN_CUDA(c, cudaMemcpyAsync(c->jd.p, js, 2 * sizeof(JuncDev), cudaMemcpyHostToDevice, c->st));
   cfg.jt_inner = c->jd.as<JuncDev>();
   cfg.jt_resid = c->jd.as<JuncDev>() + 1;
@@ -898,7 +923,7 @@ static rsn_status ensure_ws(rsn_ctx* c, bool fp32, int S, const PoolSpec* pool =
   std::vector<long long> hvo(S);
   for (int s = 0; s < S; ++s) hvo[s] = (long long)s * N;
   RSN_CUDA(c, cudaMemcpy(w.voff.p, hvo.data(), sl, cudaMemcpyHostToDevice));
-  RSN_CUDA(c, c->bd.ensure(2 * sizeof(BatchDev)));
+  RSN_CUDA(c, c->bd.ensure(sizeof(BatchDev)));
   w.slots = S;
   w.fp32 = fp32;
   w.N = N;
@@ -1195,7 +1220,7 @@ static rsn_status run_stream(rsn_ctx* c, const rsn_solver_opts* o, const StreamI
                       cudaSuccess)
         return e2;
       if ((e2 = launch_op(OP_RESID, fp32, R, cfg.resid.ppt, gr, cfg.resid.threads, cfg.resid.smem, st2, jr, bdev,
-                          nullptr, nullptr, nullptr)) != cudaSuccess)
+                          nullptr, nullptr)) != cudaSuccess)
         return e2;
       if ((e2 = launch_x_update(fp32, KL, nB, st2, jr, bdev)) != cudaSuccess) return e2;
       if (goal && (e2 = launch_tgoal(st2, jr, bdev)) != cudaSuccess) return e2;
@@ -1235,10 +1260,10 @@ static rsn_status run_stream(rsn_ctx* c, const rsn_solver_opts* o, const StreamI
       if (pool) {
         for (int kd = 0; kd < 4; ++kd)
           if (pool->has[kd] &&
-              (e = launch_inner(c, pool->inner[kd], OP_COCG, fp32, S, st, ji, bdev, nullptr, nullptr, nullptr)) !=
+              (e = launch_inner(c, pool->inner[kd], OP_COCG, fp32, S, st, ji, bdev, nullptr, nullptr)) !=
                   cudaSuccess)
             return e;
-      } else if ((e = launch_inner(c, cfg.inner, OP_COCG, fp32, S, st, ji, bdev, nullptr, nullptr, nullptr)) !=
+      } else if ((e = launch_inner(c, cfg.inner, OP_COCG, fp32, S, st, ji, bdev, nullptr, nullptr)) !=
                  cudaSuccess) {
         return e;
       }
@@ -1415,41 +1440,43 @@ static void reset_stats(rsn_ctx* c) {
   for (int k = 0; k < 2; ++k) c->ks_launches[k] = 0, c->ks_ms[k] = 0, c->ks_bytes[k] = 0;
 }
 
-// y_k = A(E_k) x_k through the allocating per-call buffers of the context.
+// y_k = A(E_k) x_k through the allocating per-call buffers of the context.  The
+// call's descriptor, tiling and per-vector tables go to the device in one copy
+// (five pageable copies were most of a small application's time).
 static rsn_status apply_impl(rsn_ctx* c, int precision, int n_rhs, const double* E, const void* x_dev, void* y_dev) {
   const bool fp32 = precision == RSN_MIXED;
   CallBufs& q = c->cb;
-  // small per-call arrays: E, junction ids, offsets, projections
-  RSN_CUDA(c, q.sys_E.ensure(n_rhs * sizeof(double)));
-  RSN_CUDA(c, q.sys_junc.ensure(n_rhs * sizeof(int)));
-  RSN_CUDA(c, q.sys_xo.ensure(n_rhs * sizeof(long long)));
+  const size_t o_J = (sizeof(BatchDev) + 15) & ~(size_t)15, o_E = o_J + ((sizeof(JuncDev) + 15) & ~(size_t)15);
+  const size_t o_voff = o_E + (size_t)n_rhs * sizeof(double), o_junc = o_voff + (size_t)n_rhs * sizeof(long long);
+  const size_t bytes = o_junc + (size_t)n_rhs * sizeof(int);
+  RSN_CUDA(c, c->ap.ensure(bytes));
   RSN_CUDA(c, q.out_t.ensure((size_t)n_rhs * std::max(1, c->n_proj) * sizeof(double2)));
-  RSN_CUDA(c, c->bd.ensure(2 * sizeof(BatchDev)));
-  std::vector<int> hj(n_rhs, 0);
-  std::vector<long long> hvo(n_rhs);
-  for (int s = 0; s < n_rhs; ++s) hvo[s] = (long long)s * c->N;
-  RSN_CUDA(c, cudaMemcpyAsync(q.sys_E.p, E, n_rhs * sizeof(double), cudaMemcpyHostToDevice, c->st));
-  RSN_CUDA(c, cudaMemcpyAsync(q.sys_junc.p, hj.data(), n_rhs * sizeof(int), cudaMemcpyHostToDevice, c->st));
-  RSN_CUDA(c, cudaMemcpyAsync(q.sys_xo.p, hvo.data(), n_rhs * sizeof(long long), cudaMemcpyHostToDevice, c->st));
-  BatchDev b;
-  memset(&b, 0, sizeof(b));
-  b.nslots = n_rhs;
-  b.junc = q.sys_junc.as<int>();
-  b.E = q.sys_E.as<double>();
-  b.voff = q.sys_xo.as<long long>();
-  b.pstride = c->n_proj;
-  RSN_CUDA(c, cudaMemcpyAsync(c->bd.as<BatchDev>() + 1, &b, sizeof(b), cudaMemcpyHostToDevice, c->st));
-  const BatchDev* bdev = c->bd.as<BatchDev>() + 1;
   // bulk-copy kernels need 16-byte aligned vectors; otherwise a register tiling
   const bool aligned = (reinterpret_cast<uintptr_t>(x_dev) % 16) == 0 && (reinterpret_cast<uintptr_t>(y_dev) % 16) == 0;
   const Tiling t = choose_tiling(c, !fp32, OP_APPLY, n_rhs, aligned);
-  LaunchCfg cfg;
-  rsn_status rs = make_cfg(c, t, choose_tiling(c, true, OP_RESID, n_rhs), cfg);
-  if (rs != RSN_OK) return rs;
-  void* cbuf = q.out_t.p;
-  if (c->n_proj > 0)
-    RSN_CUDA(c, launch_project(2, fp32, n_rhs, c->n_groups, c->max_np, c->st, cfg.jt_inner, bdev, x_dev, cbuf));
-  RSN_CUDA(c, launch_inner(c, t, OP_APPLY, fp32, n_rhs, c->st, cfg.jt_inner, bdev, x_dev, y_dev, cbuf));
+  c->ap_host.resize(bytes);
+  unsigned char *h = c->ap_host.data(), *dev = c->ap.as<unsigned char>();
+  BatchDev b;
+  memset(&b, 0, sizeof(b));
+  b.nslots = n_rhs;
+  b.E = reinterpret_cast<double*>(dev + o_E);
+  b.voff = reinterpret_cast<long long*>(dev + o_voff);
+  b.junc = reinterpret_cast<int*>(dev + o_junc);
+  b.pstride = c->n_proj;
+  JuncDev J = c->jh;
+  set_tiling_dev(J, t);
+  memcpy(h, &b, sizeof(b));
+  memcpy(h + o_J, &J, sizeof(J));
+  memcpy(h + o_E, E, (size_t)n_rhs * sizeof(double));
+  for (int s = 0; s < n_rhs; ++s) {
+    const long long vo = (long long)s * c->N;
+    memcpy(h + o_voff + (size_t)s * sizeof(long long), &vo, sizeof(vo));
+  }
+  memset(h + o_junc, 0, (size_t)n_rhs * sizeof(int));
+  // pageable source: staged before the call returns
+  RSN_CUDA(c, cudaMemcpyAsync(dev, h, bytes, cudaMemcpyHostToDevice, c->st));
+  RSN_CUDA(c, launch_apply(c, t, fp32, n_rhs, reinterpret_cast<const JuncDev*>(dev + o_J),
+                           reinterpret_cast<const BatchDev*>(dev), x_dev, y_dev, q.out_t.p));
   return RSN_OK;
 }
 
@@ -1768,15 +1795,13 @@ static rsn_status blk_set_lists(rsn_ctx* c, const BlkRun& br, const std::vector<
   return RSN_OK;
 }
 
-// y = A(E) x over the listed members (projections first, then the operator)
+// y = A(E) x over the listed members
 static rsn_status blk_apply(rsn_ctx* c, const Tiling& t, const JuncDev* jt, bool fp32, int nm, const void* x,
                             void* y) {
   BlkBufs& q = c->bb;
   const BatchDev* bd = q.bdev.as<BatchDev>();
-  if (c->n_proj > 0)
-    RSN_CUDA(c, launch_project(2, fp32, nm, c->n_groups, c->max_np, c->st, jt, bd, x, q.cbuf.p));
-  RSN_CUDA(c, launch_inner(c, t, OP_APPLY, fp32, nm, c->st, jt, bd, x, y, q.cbuf.p));
-  c->st_launches += c->n_proj > 0 ? 2 : 1;
+  RSN_CUDA(c, launch_apply(c, t, fp32, nm, jt, bd, x, y, q.cbuf.p));
+  c->st_launches += c->n_proj > 0 ? 3 : 1;
   return RSN_OK;
 }
 
@@ -1944,15 +1969,7 @@ static rsn_status block_impl(rsn_ctx* c, int n_e, const double* E, int n_cols, c
       {
         JuncDev js[2] = {c->jh, c->jh};
         const Tiling* tt2[2] = {&t32, &t64};
-        for (int k = 0; k < 2; ++k) {
-          const Tiling& t = *tt2[k];
-          js[k].TY = t.TY;
-          js[k].Lz = t.Lz;
-          js[k].ytiles = t.ytiles;
-          js[k].ztiles = t.ztiles;
-          js[k].nA = t.n;
-          js[k].kind = t.plane ? kOpPlane : t.pair ? kOpPair : t.tma ? kOpTma : kOpReg;
-        }
+        for (int k = 0; k < 2; ++k) set_tiling_dev(js[k], *tt2[k]);
         RSN_CUDA(c, cudaMemcpyAsync(q.jd.p, js, 2 * sizeof(JuncDev), cudaMemcpyHostToDevice, c->st));
       }
       const JuncDev* j32 = q.jd.as<JuncDev>();
@@ -2425,12 +2442,7 @@ static bool make_pool(rsn_ctx* const* ctxs, int K, bool fp32, int nslots, PoolSp
       const Tiling& t = h == 0 ? ti : tr;
       JuncDev& J = js[h * K + k];
       J = c->jh;
-      J.TY = t.TY;
-      J.Lz = t.Lz;
-      J.ytiles = t.ytiles;
-      J.ztiles = t.ztiles;
-      J.nA = t.n;
-      J.kind = h == 0 ? kind : kOpReg;
+      set_tiling_dev(J, t);
     }
   }
   pool.PB = upd_ctas(pool.N, upd_warps(pool.N, nslots));
@@ -2763,10 +2775,10 @@ static rsn_status bench_kernel_impl(rsn_ctx* c, int precision, int kind, int S, 
   LaunchCfg cfg;
   if ((rs = make_cfg(c, fp32, S, cfg)) != RSN_OK) return rs;
   auto launch = [&]() -> cudaError_t {
-    if (kind == 0) return launch_inner(c, cfg.inner, OP_COCG, fp32, S, st, cfg.jt_inner, bdev, nullptr, nullptr, nullptr);
+    if (kind == 0) return launch_inner(c, cfg.inner, OP_COCG, fp32, S, st, cfg.jt_inner, bdev, nullptr, nullptr);
     if (kind == 1) return launch_cocg_update(fp32, S, N, c->n_proj > 0, b.ce_stride, 0, st, cfg.jt_inner, bdev);
     return launch_op(OP_RESID, fp32, c->R, cfg.resid.ppt, dim3(cfg.resid.n, S), cfg.resid.threads, cfg.resid.smem,
-                     st, cfg.jt_resid, bdev, nullptr, nullptr, nullptr);
+                     st, cfg.jt_resid, bdev, nullptr, nullptr);
   };
   RSN_CUDA(c, launch_list(st, bdev));  // every slot, for the true-residual kernel
   for (int i = 0; i < 2; ++i) RSN_CUDA(c, launch());
@@ -2983,9 +2995,7 @@ static rsn_status apply_noalloc_impl(rsn_ctx* c, int precision, int n_rhs, const
   LaunchCfg cfg;
   rsn_status rs = make_cfg(c, t, choose_tiling(c, true, OP_RESID, n_rhs), cfg);
   if (rs != RSN_OK) return rs;
-  if (c->n_proj > 0)
-    RSN_CUDA(c, launch_project(2, fp32, n_rhs, c->n_groups, c->max_np, c->st, cfg.jt_inner, bdev, x_dev, cbuf));
-  RSN_CUDA(c, launch_inner(c, t, OP_APPLY, fp32, n_rhs, c->st, cfg.jt_inner, bdev, x_dev, y_dev, cbuf));
+  RSN_CUDA(c, launch_apply(c, t, fp32, n_rhs, cfg.jt_inner, bdev, x_dev, y_dev, cbuf));
   return RSN_OK;
 }
 

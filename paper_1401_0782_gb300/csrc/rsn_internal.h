@@ -283,12 +283,12 @@ enum OpKind { kOpReg = 0, kOpTma = 1, kOpPair = 2, kOpPlane = 3 };
 // ---- launchers (defined in the .cu files) --------------------------------
 cudaError_t launch_op(int mode, bool fp32, int R, int ppt, dim3 grid, int threads, size_t smem,
                       cudaStream_t st, const JuncDev* jt, const BatchDev* b, const void* x_in,
-                      void* y_out, const void* c_in);
+                      void* y_out);
 size_t op_smem_bytes(bool fp32, int mode, int R, int TY, int nx, int n_proj);
 // plane-streaming (TMA) operator kernel for whole-plane tiles (OP_COCG / OP_APPLY)
 cudaError_t launch_op_tma(int mode, bool fp32, int R, dim3 grid, int threads, size_t smem, cudaStream_t st,
-                          const JuncDev* jt, const BatchDev* b, const void* x_in, void* y_out, const void* c_in);
-size_t op_tma_smem_bytes(bool fp32, int mode, int R, int nx, int ny, int n_proj);
+                          const JuncDev* jt, const BatchDev* b, const void* x_in, void* y_out);
+size_t op_tma_smem_bytes(bool fp32, int mode, int R, int nx, int ny);
 // FP32 point-pair operator kernel with plane streaming (OP_COCG / OP_APPLY):
 // whole planes, nx even, 16-byte aligned vectors; big: the one-CTA-per-SM
 // variant for planes of more than 2 * kPairThreads points
@@ -298,12 +298,12 @@ constexpr int kPairStages = 4;        // input planes in flight per CTA
 constexpr int kPlaneThreads = 576;    // one-point-per-thread plane kernel: threads per CTA (two per SM)
 constexpr int kPairXO = 8;            // zero columns left of x = 0 in the exchange tile (>= R, even)
 cudaError_t launch_op_pair(int mode, int R, bool big, dim3 grid, int threads, size_t smem, cudaStream_t st,
-                           const JuncDev* jt, const BatchDev* b, const void* x_in, void* y_out, const void* c_in);
-size_t op_pair_smem_bytes(int mode, int R, int nx, int ny, int n_proj);
+                           const JuncDev* jt, const BatchDev* b, const void* x_in, void* y_out);
+size_t op_pair_smem_bytes(int mode, int R, int nx, int ny);
 // FP32 one-point-per-thread kernel with plane streaming: whole planes of an
 // even number of at most kPlaneThreads points; same shared-memory layout
 cudaError_t launch_op_plane(int mode, int R, dim3 grid, int threads, size_t smem, cudaStream_t st, const JuncDev* jt,
-                            const BatchDev* b, const void* x_in, void* y_out, const void* c_in);
+                            const BatchDev* b, const void* x_in, void* y_out);
 
 cudaError_t launch_zero(bool fp32, int nslots, int nB, cudaStream_t st, const JuncDev* jt, const BatchDev* b);
 // the COCG update with the projector term of q (proj: some junction has
@@ -313,6 +313,9 @@ cudaError_t launch_cocg_update(bool fp32, int nslots, long long N_max, bool proj
 cudaError_t launch_project(int mode, bool fp32, int nslots, int n_groups, int max_np, cudaStream_t st,
                            const JuncDev* jt, const BatchDev* b, const void* x_in, void* c_out,
                            bool one_slot_per_cta = false);
+// y += the projector term -sum_p v_p e_kb[p] c[p] of n_rhs vectors, c [n_rhs][n_proj]
+cudaError_t launch_nonlocal(bool fp32, int n_rhs, long long N, int n_proj, cudaStream_t st, const JuncDev* jt,
+                            const BatchDev* b, const void* c, void* y);
 cudaError_t launch_sched(int nslots, int slot_it, cudaStream_t st, const JuncDev* jt, const BatchDev* b);
 cudaError_t launch_x_update(bool fp32, int nslots, int nB, cudaStream_t st, const JuncDev* jt,
                             const BatchDev* b);
