@@ -87,8 +87,9 @@ template <typename T> struct RawIn<T, OP_RESID> { double2 a; typename cx<T>::t b
 template <typename T> struct RawIn<T, OP_APPLY> { typename cx<T>::t a; };
 
 // At most kOpThreads threads per CTA; the minimum resident CTAs per SM bound
-// the registers per thread (64 / 85 / 128 for 1 / 2 / 3+ points per thread,
-// 128 for the FP64 true residual).
+// the registers per thread (FP32: 64 / 85 / 128 for 1 / 2 / 3+ points per thread;
+// FP64 and the true residual: 128, since the FP64 pipe needs few warps to stay
+// busy and spilled queues cost more than occupancy).
 constexpr int kOpThreads = 256;
 
 // One (tile, slot) of the operator: the CTA's tile blockIdx.x of slot s.
@@ -232,7 +233,7 @@ __device__ __forceinline__ void op_tile(const JuncDev* __restrict__ jt, const Ba
 
   CT acc0 = 0, acc1 = 0, acc2 = 0;  // COCG: mu(re,im) ; RESID: nrm, rho(re,im)
   double acc3 = 0.0;                // RESID: sum Gamma_L |v|^2 of the iterate (T partial)
-  CT car0 = 0, car1 = 0;            // Kahan carries of the COCG sums
+  CT car0 = 0, car1 = 0;            // FP32: Kahan carries of the COCG sums; FP64: the sums of v.y y.y and v.y y.x
   // per-point operator data of the next plane to compute, loaded one plane early
   float2 dgf_n[PPT];
   int e0_n[PPT], e1_n[PPT];
@@ -319,8 +320,18 @@ __device__ __forceinline__ void op_tile(const JuncDev* __restrict__ jt, const Ba
       if constexpr (MODE == OP_COCG) {
         pnew[vo + gl] = vc;
         reinterpret_cast<CO*>(b.q)[vo + gl] = y;
-        kahan_add(acc0, car0, fma(vc.x, y.x, -vc.y * y.y));
-        kahan_add(acc1, car1, fma(vc.x, y.y, vc.y * y.x));
+        if constexpr (sizeof(CT) == 8) {
+          // four running sums, one fused (unrounded) product each: 4 operations
+          // of the FP64 pipe that bounds this kernel instead of the 12 of
+          // compensated sums; the chain is a thread's Lz planes long
+          acc0 = fma(vc.x, y.x, acc0);
+          car0 = fma(vc.y, y.y, car0);
+          acc1 = fma(vc.x, y.y, acc1);
+          car1 = fma(vc.y, y.x, car1);
+        } else {
+          kahan_add(acc0, car0, fma(vc.x, y.x, -vc.y * y.y));
+          kahan_add(acc1, car1, fma(vc.x, y.y, vc.y * y.x));
+        }
       } else if constexpr (MODE == OP_RESID) {
         double2 bb = make_double2(0.0, 0.0);
         const int col = b.col[s];
@@ -350,7 +361,7 @@ __device__ __forceinline__ void op_tile(const JuncDev* __restrict__ jt, const Ba
   }
 
   if constexpr (MODE == OP_COCG) {
-    CT v[2] = {acc0 - car0, acc1 - car1};
+    CT v[2] = {acc0 - car0, sizeof(CT) == 8 ? acc1 + car1 : acc1 - car1};
     double out[2];
     block_sum<2>(v, red, out);
     if (tid == 0) b.mu_part[(size_t)s * b.PA + tile] = make_double2(out[0], out[1]);
@@ -382,7 +393,7 @@ __device__ __forceinline__ void op_tile(const JuncDev* __restrict__ jt, const Ba
 }
 
 template <typename T, int R, int PPT, int MODE>
-__global__ void __launch_bounds__(kOpThreads, (MODE == OP_RESID ? 2 : (PPT == 1 ? 4 : (PPT == 2 ? 3 : 2))))
+__global__ void __launch_bounds__(kOpThreads, (MODE == OP_RESID || sizeof(T) == 8 ? 2 : (PPT == 1 ? 4 : (PPT == 2 ? 3 : 2))))
 op_kernel(const JuncDev* __restrict__ jt, const BatchDev* __restrict__ bp, const void* __restrict__ x_in,
           void* __restrict__ y_out) {
   const BatchDev& b = *bp;

@@ -192,7 +192,7 @@ struct BatchDev {
   long long xs_sstride;      // xs offset of slot / system k: k * xs_sstride + e * xs_estride
   long long xs_estride;
   int xs_by_sys;             // 1: xs is indexed by system (caller's output), 0: by slot
-  double2* ps;               // shifted directions p_e: [slot][n_shift][nT]
+  double2* ps;               // scaled shifted directions pi_e p_e: [slot][n_shift][nT]
   double2* spi;              // pi_{e,k} ring: [3][slot][n_shift], iteration k in ring k % 3
   int* sconv_it;             // [slot][n_shift] iteration at which shift e converged (INT_MAX: not yet)
   double2* salpha;           // [2][slot] alpha_k of the seed recurrence, ring k % 2

@@ -988,7 +988,11 @@ __global__ void __launch_bounds__(256) grad_sys_kernel(int nsys, long long N, co
 //   pi_{k+1} = (1 + alpha_k sigma) pi_k + (alpha_k beta_{k-1} / alpha_{k-1}) (pi_k - pi_{k-1}),
 //   alpha_e = alpha_k pi_k / pi_{k+1},  beta_e = beta_k (pi_k / pi_{k+1})^2,
 //   x_e += alpha_e p_e,  p_e = r_{k+1} / pi_{k+1} + beta_e p_e
-// (alpha_{-1} = 1, beta_{-1} = 0, pi_{-1} = pi_0 = 1, p_{e,0} = b).  The seed
+// (alpha_{-1} = 1, beta_{-1} = 0, pi_{-1} = pi_0 = 1, p_{e,0} = b).  What is kept
+// is the scaled direction g_e = pi_{e,k} p_e, which needs no product with r:
+//   x_e += (alpha_k / pi_{k+1}) g_e,  g_e = r_{k+1} + (beta_k pi_k / pi_{k+1}) g_e
+// (8 instead of 12 operations of the FP64 pipe per shift and tracked point; the
+// loads of four shifts are in flight together).  The seed
 // runs the FP64 slot solver unchanged; the shifted iterates live only on the
 // tracked points (the Gamma_L support for T, every point for full columns).
 // A shift is frozen once ||r_{k+1}|| / |pi_{e,k+1}| <= tol ||b||.
@@ -1041,52 +1045,51 @@ __global__ void __launch_bounds__(kVecThreads) shift_update_kernel(const JuncDev
   const int ns = b.n_shift, nT = b.nT;
   const size_t S = (size_t)b.nslots;
   const int k = b.iters[s] - 1;  // the iteration just completed
-  extern __shared__ double2 sh[];  // [ns] alpha_e, [ns] beta_e, [ns] 1 / pi_{k+1}
+  extern __shared__ double2 sh[];  // [ns] alpha_k / pi_{k+1}, [ns] beta_k pi_k / pi_{k+1}
   __shared__ int s_left;
   double2* sa = sh;
   double2* sb = sh + ns;
-  double2* sip = sh + 2 * ns;
   if (threadIdx.x == 0) s_left = 0;
   __syncthreads();
-  const double2 al = b.salpha[(size_t)(k & 1) * S + s];
-  const double2 al_m = b.salpha[(size_t)((k + 1) & 1) * S + s];
   const double2 be = b.beta_cur[s];
-  const double2 be_m = b.sbeta[(size_t)((k + 1) & 1) * S + s];
-  const double rn2 = b.rn2[s], bn2 = b.bnorm2[s];
-  const double2 cc = cmul(al, cdiv(be_m, al_m));  // alpha_k beta_{k-1} / alpha_{k-1}
-  const double2* pi_k = b.spi + ((size_t)(k % 3) * S + s) * ns;
-  const double2* pi_m = b.spi + ((size_t)((k + 2) % 3) * S + s) * ns;
-  double2* pi_n = b.spi + ((size_t)((k + 1) % 3) * S + s) * ns;
   int* cit = b.sconv_it + (size_t)s * ns;
-  for (int e = threadIdx.x; e < ns; e += blockDim.x) {
-    if (cit[e] < k) {  // frozen at an earlier iteration
-      sa[e] = make_double2(0.0, 0.0);
-      sb[e] = make_double2(0.0, 0.0);
-      sip[e] = make_double2(0.0, 0.0);
-      continue;
-    }
-    const double sg = b.shift_sig[e];
-    const double2 p0 = pi_k[e], pm = pi_m[e];
-    // pi_{k+1} = (1 + alpha sigma) pi_k + c (pi_k - pi_{k-1})
-    const double2 f = make_double2(1.0 + al.x * sg, al.y * sg);
-    const double2 pn = cadd(cmul(f, p0), cmul(cc, csub(p0, pm)));
-    const double2 ratio = cdiv(p0, pn);
-    sa[e] = cmul(al, ratio);
-    sb[e] = cmul(be, cmul(ratio, ratio));
-    sip[e] = cdiv(make_double2(1.0, 0.0), pn);
-    const double apn2 = pn.x * pn.x + pn.y * pn.y;
-    const double est2 = rn2 / (apn2 * bn2);
-    const bool conv = est2 <= b.tol * b.tol;
-    if (!isfinite(est2)) sip[e] = make_double2(0.0, 0.0);
-    if (blockIdx.x == 0) {
-      pi_n[e] = pn;
-      const int sy = b.sys[s];
-      b.out_srel[(size_t)e * b.nsys + sy] = sqrt(est2);
-      if (conv) {
-        cit[e] = k;
-        b.out_sit[(size_t)e * b.nsys + sy] = k + 1;
-      } else {
-        atomicAdd(&s_left, 1);
+  if (threadIdx.x < 32 || ns > 32) {
+    const double2 al = b.salpha[(size_t)(k & 1) * S + s];
+    const double2 al_m = b.salpha[(size_t)((k + 1) & 1) * S + s];
+    const double2 be_m = b.sbeta[(size_t)((k + 1) & 1) * S + s];
+    const double rn2 = b.rn2[s], bn2 = b.bnorm2[s];
+    const double2 cc = cmul(al, cdiv(be_m, al_m));  // alpha_k beta_{k-1} / alpha_{k-1}
+    const double2* pi_k = b.spi + ((size_t)(k % 3) * S + s) * ns;
+    const double2* pi_m = b.spi + ((size_t)((k + 2) % 3) * S + s) * ns;
+    double2* pi_n = b.spi + ((size_t)((k + 1) % 3) * S + s) * ns;
+    for (int e = threadIdx.x; e < ns; e += blockDim.x) {
+      if (cit[e] < k) {  // frozen at an earlier iteration
+        sa[e] = sb[e] = make_double2(0.0, 0.0);
+        continue;
+      }
+      const double sg = b.shift_sig[e];
+      const double2 p0 = pi_k[e], pm = pi_m[e];
+      // pi_{k+1} = (1 + alpha sigma) pi_k + c (pi_k - pi_{k-1})
+      const double2 f = make_double2(1.0 + al.x * sg, al.y * sg);
+      const double2 pn = cadd(cmul(f, p0), cmul(cc, csub(p0, pm)));
+      const double apn2 = pn.x * pn.x + pn.y * pn.y;
+      const double inv2 = 1.0 / apn2;
+      const double2 inv = make_double2(pn.x * inv2, -pn.y * inv2);  // 1 / pi_{k+1}
+      sa[e] = cmul(al, inv);
+      sb[e] = cmul(be, cmul(p0, inv));
+      const double est2 = rn2 / (apn2 * bn2);
+      const bool conv = est2 <= b.tol * b.tol;
+      if (!isfinite(est2)) sa[e] = sb[e] = make_double2(0.0, 0.0);
+      if (blockIdx.x == 0) {
+        pi_n[e] = pn;
+        const int sy = b.sys[s];
+        b.out_srel[(size_t)e * b.nsys + sy] = sqrt(est2);
+        if (conv) {
+          cit[e] = k;
+          b.out_sit[(size_t)e * b.nsys + sy] = k + 1;
+        } else {
+          atomicAdd(&s_left, 1);
+        }
       }
     }
   }
@@ -1100,14 +1103,29 @@ __global__ void __launch_bounds__(kVecThreads) shift_update_kernel(const JuncDev
   const double2* rv = reinterpret_cast<const double2*>(b.r) + b.voff[s];
   for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < nT; i += gridDim.x * blockDim.x) {
     const double2 r = rv[b.T_idx[i]];
-    for (int e = 0; e < ns; ++e) {
-      const double2 ip = sip[e];
-      if (ip.x == 0.0 && ip.y == 0.0) continue;  // frozen (uniform across the CTA)
-      double2* xp = xb + (long long)e * b.xs_estride + i;
-      double2* pp = pb + (size_t)e * nT + i;
-      const double2 p = *pp;
-      *xp = cfma(sa[e], p, *xp);
-      *pp = cfma(sb[e], p, cmul(r, ip));
+    for (int e0 = 0; e0 < ns; e0 += 4) {
+      double2 g[4], x[4];
+      bool on[4];
+#pragma unroll
+      for (int u = 0; u < 4; ++u) {
+        const int e = e0 + u;
+        on[u] = false;
+        if (e < ns) {  // frozen shifts are skipped (uniform across the CTA)
+          const double2 a = sa[e], c = sb[e];
+          on[u] = a.x != 0.0 || a.y != 0.0 || c.x != 0.0 || c.y != 0.0;
+        }
+        if (on[u]) {
+          g[u] = pb[(size_t)e * nT + i];
+          x[u] = xb[(long long)e * b.xs_estride + i];
+        }
+      }
+#pragma unroll
+      for (int u = 0; u < 4; ++u) {
+        const int e = e0 + u;
+        if (!on[u]) continue;
+        xb[(long long)e * b.xs_estride + i] = cfma(sa[e], g[u], x[u]);
+        pb[(size_t)e * nT + i] = cfma(sb[e], g[u], r);
+      }
     }
   }
 }
@@ -1359,7 +1377,7 @@ cudaError_t launch_shift_init(int nT, cudaStream_t st, const JuncDev* jt, const 
 cudaError_t launch_shift_update(int nslots, int nT, int n_shift, cudaStream_t st, const JuncDev* jt,
                                 const BatchDev* b) {
   const int bx = std::max(1, (nT + kVecThreads - 1) / kVecThreads);
-  shift_update_kernel<<<dim3(bx, nslots), kVecThreads, 3 * n_shift * sizeof(double2), st>>>(jt, b);
+  shift_update_kernel<<<dim3(bx, nslots), kVecThreads, 2 * n_shift * sizeof(double2), st>>>(jt, b);
   return cudaGetLastError();
 }
 
