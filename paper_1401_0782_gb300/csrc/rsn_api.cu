@@ -242,9 +242,16 @@ static Tiling choose_tiling(const rsn_ctx* c, bool compute64, int mode, int nslo
   // FP32 point-pair kernel: whole planes, nx even (16-byte pairs), at most
   // 2 * kPairThreadsBig points per plane, no explicit register tile requested
   const bool reg_forced = c->tile_override[0] > 0 || c->tile_override[2] > 0 || c->tile_override[3] == -1;
+  // z chunks per tile column: chunks of 2R + 2 planes and more, so that the 2R
+  // halo planes of a chunk do not outweigh it, unless that leaves SMs without a
+  // CTA: then down to two planes a chunk, since the march (chunk + 2R planes) is
+  // what such a launch waits for (8 systems of 16x16x64 in FP32: 26 -> 17 us)
+  auto z_cap = [&](int columns) {
+    return std::max(1, std::max(nz / (2 * R + 2), std::min(nz / 2, 152 / std::max(1, columns))));
+  };
   auto z_chunks = [&](int per_sm) {
     int zt = (4 * per_sm * 152 + nslots - 1) / nslots;
-    zt = std::max(1, std::min(zt, std::max(1, nz / (2 * R + 2))));
+    zt = std::max(1, std::min(zt, z_cap(nslots)));
     if (c->tile_override[1] > 0) zt = (nz + c->tile_override[1] - 1) / c->tile_override[1];
     t.Lz = (nz + zt - 1) / zt;
     t.ztiles = (nz + t.Lz - 1) / t.Lz;
@@ -304,7 +311,7 @@ static Tiling choose_tiling(const rsn_ctx* c, bool compute64, int mode, int nslo
   t.threads = threads;
   int want = 8 * 152;
   int zt = (want + nslots * t.ytiles - 1) / (nslots * t.ytiles);
-  zt = std::max(1, std::min(zt, std::max(1, nz / (2 * R + 2))));
+  zt = std::max(1, std::min(zt, z_cap(nslots * t.ytiles)));
   if (c->tile_override[1] > 0) zt = (nz + c->tile_override[1] - 1) / c->tile_override[1];
   // few systems need a true residual at a time and it sits on every
   // iteration's critical path: two planes per CTA whatever the operator
@@ -1097,6 +1104,8 @@ static rsn_status run_stream(rsn_ctx* c, const rsn_solver_opts* o, const StreamI
   RSN_CUDA(c, cudaMemsetAsync(w.mu_cnt.p, 0, S * sizeof(int), st));
   RSN_CUDA(c, cudaMemsetAsync(w.upd_cnt.p, 0, S * sizeof(int), st));
   RSN_CUDA(c, cudaMemsetAsync(w.res_cnt.p, 0, S * sizeof(int), st));
+  RSN_CUDA(c, cudaMemsetAsync(w.lst_n.p, 0, sizeof(int), st));
+  RSN_CUDA(c, cudaMemsetAsync(w.inlist.p, 0, S * sizeof(int), st));
   RSN_CUDA(c, cudaMemsetAsync(w.sched.p, 0, (3 + 2 * kMaxGraphIters) * sizeof(int), st));
   RSN_CUDA(c, cudaMemsetAsync(w.counters.p, 0, 4 * sizeof(unsigned long long), st));
 
@@ -1196,12 +1205,12 @@ static rsn_status run_stream(rsn_ctx* c, const rsn_solver_opts* o, const StreamI
     RSN_CUDA(c, cudaEventCreate(&e));
     c->tev.push_back(e);
   }
-  // One iteration: the true-residual path of the NEW / CHECK / goal-check slots
-  // (list, zero, projections of x, FP64 residual, x update, goal check) runs on
-  // the second stream beside the COCG step of the ACTIVE slots (projections of
-  // r, operator, update, bookkeeping); both touch disjoint slots.  The
-  // scheduler then joins them: finished systems leave, checked systems resume,
-  // free slots take queued systems for the next iteration.
+  // One iteration: the outputs of the drained slots and the true-residual path of
+  // the NEW / CHECK / goal-check slots (zero, projections of x, FP64 residual, x
+  // update, goal check) run on the second stream beside the COCG step of the
+  // ACTIVE slots (projections of r, operator, update); all touch disjoint slots.
+  // The scheduler then joins them: finished systems leave, checked systems
+  // resume, free slots take queued systems and the next list is made.
   // Shifted systems keep one stream: their per-iteration shift step must see
   // exactly the slots that did a COCG iteration, so the scheduler runs first.
   cudaStream_t st2 = sh ? st : c->st2;
@@ -1213,7 +1222,8 @@ static rsn_status run_stream(rsn_ctx* c, const rsn_solver_opts* o, const StreamI
       return e;
     auto residual_path = [&]() -> cudaError_t {
       cudaError_t e2;
-      if ((e2 = launch_list(st2, bdev)) != cudaSuccess) return e2;
+      if (sh && (e2 = launch_list(st2, bdev)) != cudaSuccess) return e2;
+      if (!sh && (e2 = launch_emit(S, st2, jr, bdev)) != cudaSuccess) return e2;
       if ((e2 = launch_zero(fp32, KL, nB, st2, jr, bdev)) != cudaSuccess) return e2;
       if (sh && (e2 = launch_shift_init(sh->nT, st2, jr, bdev)) != cudaSuccess) return e2;
       if (proj && (e2 = launch_project(1, fp32, KL, n_groups, max_np, st2, jr, bdev, nullptr, w.c_x.p, multi)) !=
@@ -1228,8 +1238,8 @@ static rsn_status run_stream(rsn_ctx* c, const rsn_solver_opts* o, const StreamI
     };
     auto schedule = [&](int it) -> cudaError_t {
       cudaError_t e2;
-      if ((e2 = launch_sched(S, it, st, jr, bdev)) != cudaSuccess) return e2;
-      if ((e2 = launch_emit(S, st, jr, bdev)) != cudaSuccess) return e2;
+      if ((e2 = launch_sched(it, !sh, st, jr, bdev)) != cudaSuccess) return e2;
+      if (sh && (e2 = launch_emit(S, st, jr, bdev)) != cudaSuccess) return e2;
       if (sh && (e2 = launch_shift_emit(S, ns, st, jr, bdev)) != cudaSuccess) return e2;
       return cudaSuccess;
     };
@@ -1280,7 +1290,7 @@ static rsn_status run_stream(rsn_ctx* c, const rsn_solver_opts* o, const StreamI
     }
     return cudaSuccess;
   };
-  const int per_iter = (proj ? 10 : 8) + (sh ? 3 : 0) + (goal ? 1 : 0);
+  const int per_iter = (proj ? 9 : 7) + (sh ? 4 : 0) + (goal ? 1 : 0);
   const double vbytes = (double)(pool ? pool->N : c->N) * (fp32 ? sizeof(float2) : sizeof(double2));
   cudaGraphExec_t gexec = nullptr;
   if (o->use_graph) {
@@ -1364,6 +1374,9 @@ static rsn_status run_stream(rsn_ctx* c, const rsn_solver_opts* o, const StreamI
     }
   }
   if (!finished && !timeout && !aborted) RSN_FAIL(c, RSN_ECUDA, "streaming solver exceeded its iteration bound");
+  // a pass that stops early leaves the systems of its last scheduler call drained
+  // but not yet emitted
+  if (!finished && !sh) RSN_CUDA(c, launch_emit(S, st, jr, bdev));
   out.iters.resize(nsys);
   out.status.resize(nsys);
   out.relres.resize(nsys);

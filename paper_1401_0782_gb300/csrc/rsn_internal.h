@@ -48,6 +48,11 @@ constexpr int upd_warps(long long N, int nslots) {
   return (long long)upd_ctas(N, kUpdThreads / 32) * nslots < 2 * 152 ? 2 : kUpdThreads / 32;
 }
 
+// fewer warps than four CTAs of four on every SM: memory latency counts, not occupancy
+constexpr bool upd_early(long long N, int nslots) {
+  return (N + kBlkPts - 1) / kBlkPts * nslots < 16 * 152;
+}
+
 struct JuncDev {
   int nx, ny, nz, plane;
   long long N;
@@ -316,7 +321,7 @@ cudaError_t launch_project(int mode, bool fp32, int nslots, int n_groups, int ma
 // y += the projector term -sum_p v_p e_kb[p] c[p] of n_rhs vectors, c [n_rhs][n_proj]
 cudaError_t launch_nonlocal(bool fp32, int n_rhs, long long N, int n_proj, cudaStream_t st, const JuncDev* jt,
                             const BatchDev* b, const void* c, void* y);
-cudaError_t launch_sched(int nslots, int slot_it, cudaStream_t st, const JuncDev* jt, const BatchDev* b);
+cudaError_t launch_sched(int slot_it, bool make_list, cudaStream_t st, const JuncDev* jt, const BatchDev* b);
 cudaError_t launch_x_update(bool fp32, int nslots, int nB, cudaStream_t st, const JuncDev* jt,
                             const BatchDev* b);
 cudaError_t launch_emit(int nslots, cudaStream_t st, const JuncDev* jt, const BatchDev* b);

@@ -6,13 +6,13 @@
 //   project   (NEW|CHECK)      c_x = v_p . (x + d)                       [projectors]
 //   op RESID  (NEW|CHECK)      r = b - A (x + d) in FP64, ||r||^2, r^T r
 //   x_update  (NEW|CHECK)      x += d, d = 0
-//   sched     (all, 1 CTA)     converged? -> DRAIN; else reliable update -> ACTIVE;
-//                              DRAIN -> FREE; FREE slots take queued systems
 //   emit      (DRAIN)          T partial of the finished system
 //   project   (ACTIVE)         c_r = v_p . r                             [projectors]
-//   op COCG   (ACTIVE)         p = r + beta p, q = A p, p^T q
-//   update    (ACTIVE)         alpha = rho/mu, r -= alpha q, d += alpha p, r^T r, ||r||^2
-//   book      (ACTIVE, 1 CTA)  iteration counts; recurrence target reached -> CHECK
+//   op COCG   (ACTIVE)         p = r + beta p, q = A p, p^T q; alpha = rho/mu
+//   update    (ACTIVE)         r -= alpha q, d += alpha p, r^T r, ||r||^2, then the slot's
+//                              iteration counts; recurrence target reached -> CHECK
+//   sched     (all, 1 CTA)     converged? -> DRAIN; else reliable update -> ACTIVE;
+//                              DRAIN -> FREE; FREE slots take queued systems; list
 #include <algorithm>
 #include <type_traits>
 
@@ -23,12 +23,12 @@
 namespace rsn {
 
 // ---------------------------------------------------------------------------
-// List of the slots that need a true residual in this iteration (NEW and
+// List of the slots that need a true residual in the next iteration (NEW and
 // CHECK), in slot order: one CTA, ballot + warp-count prefix per 1024 slots.
+// Built at the end of the scheduler; shifted systems, whose scheduler runs before
+// the COCG step, take a kernel of its own at the start of the iteration.
 // ---------------------------------------------------------------------------
-__global__ void __launch_bounds__(kSchedThreads) list_kernel(const BatchDev* __restrict__ bp) {
-  const BatchDev& b = *bp;
-  __shared__ int warp_cnt[kSchedThreads / 32];
+__device__ __forceinline__ void build_list(const BatchDev& b, int* warp_cnt) {
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
   int total = 0;
   for (int base = 0; base < b.nslots; base += blockDim.x) {
@@ -50,6 +50,11 @@ __global__ void __launch_bounds__(kSchedThreads) list_kernel(const BatchDev* __r
     __syncthreads();
   }
   if (threadIdx.x == 0) *b.lst_n = total;
+}
+
+__global__ void __launch_bounds__(kSchedThreads) list_kernel(const BatchDev* __restrict__ bp) {
+  __shared__ int warp_cnt[kSchedThreads / 32];
+  build_list(*bp, warp_cnt);
 }
 
 // ---------------------------------------------------------------------------
@@ -230,8 +235,10 @@ __device__ __forceinline__ void store_pts(C* dst, const int (&at)[U], int end, b
     if (at[u] < end) dst[at[u]] = v[u];
 }
 
-template <typename T>
-__global__ void __launch_bounds__(kUpdThreads, sizeof(T) == 4 ? 8 : 6)
+// EARLY: the vectors are requested before the projector term is formed, which
+// takes 90 registers; for launches whose latency counts (upd_early).
+template <typename T, bool EARLY>
+__global__ void __launch_bounds__(kUpdThreads, EARLY ? 4 : sizeof(T) == 4 ? 8 : 6)
 cocg_update_kernel(const JuncDev* __restrict__ jt, const BatchDev* __restrict__ bp, int slot_it) {
   using C = typename cx<T>::t;
   constexpr int U = sizeof(T) == 4 ? 4 : 2;  // points in flight per thread
@@ -276,6 +283,7 @@ cocg_update_kernel(const JuncDev* __restrict__ jt, const BatchDev* __restrict__ 
       load_pts(pn, at, i1, pairs, p);
       load_pts(dv, at, i1, pairs, d);
     };
+    if constexpr (EARLY) fetch(0);
     int row0 = 0, row1 = 0;
     if (J.n_proj > 0) {
       const int nblk = (N + kBlkPts - 1) / kBlkPts;
@@ -293,7 +301,7 @@ cocg_update_kernel(const JuncDev* __restrict__ jt, const BatchDev* __restrict__ 
     }
 #pragma unroll
     for (int l = 0; l < NL; ++l) {
-      fetch(l);
+      if (!EARLY || l > 0) fetch(l);
       if (row1 > row0) {
 #pragma unroll
         for (int u = 0; u < U; ++u) q[u] = cadd(q[u], s_nl[at[u] - i0]);
@@ -609,11 +617,26 @@ __global__ void __launch_bounds__(kUpdThreads) nonlocal_kernel(const JuncDev* __
 // assigns queued systems to free slots in slot order.
 // ---------------------------------------------------------------------------
 __global__ void __launch_bounds__(kSchedThreads) sched_kernel(const JuncDev* __restrict__ jt,
-                                                             const BatchDev* __restrict__ bp, int slot_it) {
+                                                             const BatchDev* __restrict__ bp, int slot_it,
+                                                             int make_list) {
   const BatchDev& b = *bp;
   const int S = b.nslots;
   __shared__ int warp_cnt[32];
   int upd = 0, busy = 0;
+  if (make_list) {
+    // most iterations change no slot: nothing drained, listed, due for a list or
+    // waiting for a slot; the list stays empty and the busy count what it was
+    const bool queued = b.sched[0] < b.nsys;
+    bool work = false;
+    for (int s = threadIdx.x; s < S; s += blockDim.x) {
+      const int st = b.state[s];
+      work = work || !(st == SL_ACTIVE || (st == SL_FREE && !queued));
+    }
+    if (!__syncthreads_or(work)) {
+      if (threadIdx.x == 0) b.sched[3 + slot_it] = b.sched[1];
+      return;
+    }
+  }
   for (int s = threadIdx.x; s < S; s += blockDim.x) {
     int st = b.state[s];
     // NEW / CHECK / CHECKT slots are handled only if this iteration's list took
@@ -835,6 +858,7 @@ __global__ void __launch_bounds__(kSchedThreads) sched_kernel(const JuncDev* __r
     if (found) break;
   }
   for (int s = threadIdx.x; s < S; s += blockDim.x) busy += (b.state[s] != SL_FREE) ? 1 : 0;
+  if (make_list) build_list(b, warp_cnt);
   busy = __reduce_add_sync(0xffffffffu, busy);
   upd = __reduce_add_sync(0xffffffffu, upd);
   if (threadIdx.x == 0) s_nf = s_done = 0;  // reused: the CTA's totals
@@ -1286,14 +1310,15 @@ cudaError_t launch_cocg_update(bool fp32, int nslots, long long N_max, bool proj
   const int nw = upd_warps(N_max, nslots);
   const dim3 grid(upd_ctas(N_max, nw), nslots);
   const size_t smem = proj ? ((size_t)ce_stride + nw * kBlkPts) * (fp32 ? sizeof(float2) : sizeof(double2)) : 0;
+  const bool early = upd_early(N_max, nslots);
+  void (*kern)(const JuncDev*, const BatchDev*, int) =
+      fp32 ? (early ? cocg_update_kernel<float, true> : cocg_update_kernel<float, false>)
+           : (early ? cocg_update_kernel<double, true> : cocg_update_kernel<double, false>);
   if (smem > 32 * 1024) {
-    cudaError_t e = set_max_dynamic_smem(
-        fp32 ? reinterpret_cast<const void*>(cocg_update_kernel<float>) : reinterpret_cast<const void*>(cocg_update_kernel<double>),
-        smem);
+    cudaError_t e = set_max_dynamic_smem(reinterpret_cast<const void*>(kern), smem);
     if (e != cudaSuccess) return e;
   }
-  if (fp32) cocg_update_kernel<float><<<grid, 32 * nw, smem, st>>>(jt, b, slot_it);
-  else cocg_update_kernel<double><<<grid, 32 * nw, smem, st>>>(jt, b, slot_it);
+  kern<<<grid, 32 * nw, smem, st>>>(jt, b, slot_it);
   return cudaGetLastError();
 }
 
@@ -1355,9 +1380,8 @@ cudaError_t launch_nonlocal(bool fp32, int n_rhs, long long N, int n_proj, cudaS
   return cudaGetLastError();
 }
 
-cudaError_t launch_sched(int nslots, int slot_it, cudaStream_t st, const JuncDev* jt, const BatchDev* b) {
-  (void)nslots;
-  sched_kernel<<<1, kSchedThreads, 0, st>>>(jt, b, slot_it);
+cudaError_t launch_sched(int slot_it, bool make_list, cudaStream_t st, const JuncDev* jt, const BatchDev* b) {
+  sched_kernel<<<1, kSchedThreads, 0, st>>>(jt, b, slot_it, make_list ? 1 : 0);
   return cudaGetLastError();
 }
 
