@@ -44,19 +44,28 @@ template <> __device__ __forceinline__ double2 from64<double2>(double2 a) { retu
 // of value l % V.  At each shuffle a lane gives away half of the sums it holds:
 // V - 1 + log2(32 / V) adds instead of 5 V.  On this GPU a warp's FP64 add
 // occupies its FP64 pipe for 64 cycles, so reductions count their instructions.
-template <int V, typename A>
-__device__ __forceinline__ A warp_sum_many(A (&v)[V]) {
-  const int lane = threadIdx.x & 31;
+// The lanes meet in the same order for V = 8, 16 and 32.
+template <int V, int W, int DONE, typename A>
+__device__ __forceinline__ void warp_sum_step(A (&v)[V]) {
+  if constexpr (W < V) {
+    const bool up = (threadIdx.x & W) != 0;
 #pragma unroll
-  for (int w = V / 2; w >= 1; w >>= 1) {
-    const bool up = (lane & w) != 0;
-#pragma unroll
-    for (int j = 0; j < w; ++j) {
-      const A send = up ? v[j] : v[j + w];
-      const A keep = up ? v[j + w] : v[j];
-      v[j] = keep + __shfl_xor_sync(0xffffffffu, send, w);
+    for (int j = 0; j < V; ++j) {
+      if ((j & (DONE | W)) == 0) {
+        const A send = up ? v[j] : v[j | W];
+        const A keep = up ? v[j | W] : v[j];
+        v[j] = keep + __shfl_xor_sync(0xffffffffu, send, W);
+      }
     }
   }
+}
+template <int V, typename A>
+__device__ __forceinline__ A warp_sum_many(A (&v)[V]) {
+  warp_sum_step<V, 4, 0>(v);
+  warp_sum_step<V, 2, 4>(v);
+  warp_sum_step<V, 1, 6>(v);
+  warp_sum_step<V, 8, 7>(v);
+  warp_sum_step<V, 16, 15>(v);
   A t = v[0];
 #pragma unroll
   for (int w = V; w < 32; w <<= 1) t += __shfl_xor_sync(0xffffffffu, t, w);

@@ -52,33 +52,14 @@ __device__ __forceinline__ C fd_diff_form(const C* qz, const C* smb, int so, int
   return cfma(mk2((CT)((float)E + dgv.x), (CT)dgv.y), vc, lap);
 }
 
-// Kahan-compensated accumulation (sum, carry) for long FP32 dot products.
-template <typename S>
-__device__ __forceinline__ void kahan_add(S& sum, S& carry, S term) {
-  const S y = term - carry;
-  const S t = sum + y;
-  carry = (t - sum) - y;
-  sum = t;
-}
-
-// y -= sum_j a_j cp[j] over one quad of an atom entry's projector values
-// (FP64 values for an FP64 compute type, else FP32), in projector order.
-template <typename C, typename CT>
-__device__ __forceinline__ C proj_quad(const JuncDev& J, int qi, const C* cp, C y) {
-  if constexpr (sizeof(CT) == 8) {
-    const double2 a01 = J.inv_q64[2 * (size_t)qi], a23 = J.inv_q64[2 * (size_t)qi + 1];
-    y = rfma((CT)-a01.x, cp[0], y);
-    y = rfma((CT)-a01.y, cp[1], y);
-    y = rfma((CT)-a23.x, cp[2], y);
-    y = rfma((CT)-a23.y, cp[3], y);
-  } else {
-    const float4 a = J.inv_q32[qi];
-    y = rfma((CT)-a.x, cp[0], y);
-    y = rfma((CT)-a.y, cp[1], y);
-    y = rfma((CT)-a.z, cp[2], y);
-    y = rfma((CT)-a.w, cp[3], y);
-  }
-  return y;
+// y -= sum_j a_j cp[j] over one quad of an atom entry's projector values, in
+// projector order (the true residual's projector term).
+__device__ __forceinline__ double2 proj_quad(const JuncDev& J, int qi, const double2* cp, double2 y) {
+  const double2 a01 = J.inv_q64[2 * (size_t)qi], a23 = J.inv_q64[2 * (size_t)qi + 1];
+  y = rfma(-a01.x, cp[0], y);
+  y = rfma(-a01.y, cp[1], y);
+  y = rfma(-a23.x, cp[2], y);
+  return rfma(-a23.y, cp[3], y);
 }
 
 template <typename T, int MODE> struct RawIn;
@@ -92,7 +73,8 @@ template <typename T> struct RawIn<T, OP_APPLY> { typename cx<T>::t a; };
 // busy and spilled queues cost more than occupancy).
 constexpr int kOpThreads = 256;
 
-// One (tile, slot) of the operator: the CTA's tile blockIdx.x of slot s.
+// One (tile, slot) of the operator: the CTA's tile of slot s (blockIdx.y; the true
+// residual, whose CTA rows walk a list of slots: blockIdx.x).
 template <typename T, int R, int PPT, int MODE>
 __device__ __forceinline__ void op_tile(const JuncDev* __restrict__ jt, const BatchDev& b, const int s,
                                         const void* __restrict__ x_in, void* __restrict__ y_out) {
@@ -111,12 +93,14 @@ __device__ __forceinline__ void op_tile(const JuncDev* __restrict__ jt, const Ba
     if (stt != SL_NEW && stt != SL_CHECK) return;
   }
   const JuncDev& J = jt[b.junc[s]];
-  const int tile = blockIdx.x;
+  const int tile = MODE == OP_RESID ? blockIdx.x : blockIdx.y;
   if (tile >= J.nA || (MODE != OP_RESID && J.kind != kOpReg)) return;
 
   const int nx = J.nx, ny = J.ny, nz = J.nz, plane = J.plane, TY = J.TY;
   const int yt = tile % J.ytiles, zt = tile / J.ytiles;
-  const int z0 = zt * J.Lz, z1 = min(z0 + J.Lz, nz);
+  const int Lz = MODE == OP_COCG ? cocg_lz(J, b) : J.Lz;
+  const int z0 = zt * Lz, z1 = min(z0 + Lz, nz);
+  if (z0 >= nz) return;
   const int y0 = yt * TY, y1 = min(y0 + TY, ny), ty = y1 - y0;
   const int pitch = nx + 2 * R, rows = TY + 2 * R;
   const int tid = threadIdx.x, nt = blockDim.x;
@@ -129,7 +113,9 @@ __device__ __forceinline__ void op_tile(const JuncDev* __restrict__ jt, const Ba
   C* sm0 = reinterpret_cast<C*>(smem_raw);
   C* sm1 = sm0 + rows * pitch;
   C* ce = sm1 + rows * pitch;
-  __shared__ double red[32 * 4];
+  __shared__ double red[MODE == OP_RESID ? 32 * 4 : 1];
+  // mu partials (COCG): [block of planes][warp][re, im]
+  __shared__ CT s_mu[MODE == OP_COCG ? kMaxLz / kMuPlanes * (kOpThreads / 32) * 2 : 1];
 
   for (int i = tid; i < 2 * rows * pitch; i += nt) sm0[i] = czero<C>();
 
@@ -231,9 +217,8 @@ __device__ __forceinline__ void op_tile(const JuncDev* __restrict__ jt, const Ba
     else wst[m] = (CT)J.w32[m];
   }
 
-  CT acc0 = 0, acc1 = 0, acc2 = 0;  // COCG: mu(re,im) ; RESID: nrm, rho(re,im)
+  CT acc0 = 0, acc1 = 0, acc2 = 0;  // COCG: mu(re,im) of kMuPlanes planes; RESID: nrm, rho(re,im)
   double acc3 = 0.0;                // RESID: sum Gamma_L |v|^2 of the iterate (T partial)
-  CT car0 = 0, car1 = 0;            // FP32: Kahan carries of the COCG sums; FP64: the sums of v.y y.y and v.y y.x
   // per-point operator data of the next plane to compute, loaded one plane early
   float2 dgf_n[PPT];
   int e0_n[PPT], e1_n[PPT];
@@ -310,28 +295,23 @@ __device__ __forceinline__ void op_tile(const JuncDev* __restrict__ jt, const Ba
       } else {
         y = fd_diff_form<C, CT, R>(qv[u], smb, so[u], pitch, wst, vc, dgf_c[u], E);
       }
-      if (MODE == OP_RESID && n_proj > 0) {
-        const int e0 = e0_c[u], e1 = e1_c[u], nq = J.inv_nq;
-        for (int e = e0; e < e1; ++e) {
-          const C* cp = ce + J.inv_p0[e];
-          for (int qd = 0; qd < nq; ++qd) y = proj_quad<C, CT>(J, e * nq + qd, cp + 4 * qd, y);
+      if constexpr (MODE == OP_RESID) {
+        if (n_proj > 0) {
+          const int e0 = e0_c[u], e1 = e1_c[u], nq = J.inv_nq;
+          for (int e = e0; e < e1; ++e) {
+            const C* cp = ce + J.inv_p0[e];
+            for (int qd = 0; qd < nq; ++qd) y = proj_quad(J, e * nq + qd, cp + 4 * qd, y);
+          }
         }
       }
       if constexpr (MODE == OP_COCG) {
         pnew[vo + gl] = vc;
         reinterpret_cast<CO*>(b.q)[vo + gl] = y;
-        if constexpr (sizeof(CT) == 8) {
-          // four running sums, one fused (unrounded) product each: 4 operations
-          // of the FP64 pipe that bounds this kernel instead of the 12 of
-          // compensated sums; the chain is a thread's Lz planes long
-          acc0 = fma(vc.x, y.x, acc0);
-          car0 = fma(vc.y, y.y, car0);
-          acc1 = fma(vc.x, y.y, acc1);
-          car1 = fma(vc.y, y.x, car1);
-        } else {
-          kahan_add(acc0, car0, fma(vc.x, y.x, -vc.y * y.y));
-          kahan_add(acc1, car1, fma(vc.x, y.y, vc.y * y.x));
-        }
+        // fused (unrounded) products; the sums are over kMuPlanes planes of the thread's
+        // points, so FP64 needs none of the compensation that took 8 of its 12
+        // operations here
+        acc0 = fma(vc.x, y.x, fma(-vc.y, y.y, acc0));
+        acc1 = fma(vc.x, y.y, fma(vc.y, y.x, acc1));
       } else if constexpr (MODE == OP_RESID) {
         double2 bb = make_double2(0.0, 0.0);
         const int col = b.col[s];
@@ -358,14 +338,16 @@ __device__ __forceinline__ void op_tile(const JuncDev* __restrict__ jt, const Ba
         reinterpret_cast<CO*>(y_out)[vo + gl] = from64<CO>(to64(y));
       }
     }
+    if constexpr (MODE == OP_COCG) {
+      if ((zc - z0) % kMuPlanes == kMuPlanes - 1 || zc == z1 - 1) {
+        mu_flush(s_mu, (zc - z0) / kMuPlanes, acc0, acc1);
+        acc0 = acc1 = 0;
+      }
+    }
   }
 
   if constexpr (MODE == OP_COCG) {
-    CT v[2] = {acc0 - car0, sizeof(CT) == 8 ? acc1 + car1 : acc1 - car1};
-    double out[2];
-    block_sum<2>(v, red, out);
-    if (tid == 0) b.mu_part[(size_t)s * b.PA + tile] = make_double2(out[0], out[1]);
-    if (tid < 32) mu_arrive(b, J, s);
+    mu_finish(b, J, s, s_mu, yt, z0, z1);
   } else if constexpr (MODE == OP_RESID) {
     CT v[4] = {acc0, acc1, acc2, acc3};
     double out[4];
@@ -406,7 +388,7 @@ op_kernel(const JuncDev* __restrict__ jt, const BatchDev* __restrict__ bp, const
       __syncthreads();  // the shared-memory planes are reused by the next entry
     }
   } else {
-    op_tile<T, R, PPT, MODE>(jt, b, blockIdx.y, x_in, y_out);
+    op_tile<T, R, PPT, MODE>(jt, b, blockIdx.x, x_in, y_out);
   }
 }
 
@@ -436,7 +418,7 @@ cudaError_t launch_op_r(int mode, bool fp32, int ppt, dim3 grid, int threads, si
     }
   }
 #undef RSN_PICK
-  if (smem > 48 * 1024) {
+  if (smem > 16 * 1024) {  // beside the static arrays
     cudaError_t e = set_max_dynamic_smem(reinterpret_cast<const void*>(kern), smem);
     if (e != cudaSuccess) return e;
   }
@@ -464,15 +446,17 @@ op_kernel_tma(const JuncDev* __restrict__ jt, const BatchDev* __restrict__ bp, c
   constexpr int Q = 2 * R + 1;
   constexpr int NIN = (MODE == OP_COCG) ? 2 : 1;
   const BatchDev& b = *bp;
-  const int s = blockIdx.y;
+  const int s = blockIdx.x;
   if constexpr (MODE == OP_COCG) {
     if (b.state[s] != SL_ACTIVE) return;
   }
   const JuncDev& J = jt[b.junc[s]];
-  const int tile = blockIdx.x;
+  const int tile = blockIdx.y;
   if (tile >= J.nA || J.kind != kOpTma) return;
   const int nx = J.nx, ny = J.ny, nz = J.nz, plane = J.plane;
-  const int z0 = tile * J.Lz, z1 = min(z0 + J.Lz, nz);
+  const int Lz = MODE == OP_COCG ? cocg_lz(J, b) : J.Lz;
+  const int z0 = tile * Lz, z1 = min(z0 + Lz, nz);
+  if (z0 >= nz) return;
   const int pitch = nx + 2 * R, prow = ny + 2 * R;
   const int tid = threadIdx.x, nt = blockDim.x;
   const long long vo = b.voff[s];
@@ -483,7 +467,8 @@ op_kernel_tma(const JuncDev* __restrict__ jt, const BatchDev* __restrict__ bp, c
   C* exch = stage + kStages * NIN * plane;           // [2][prow][pitch]
   uint64_t* bars = reinterpret_cast<uint64_t*>(
       (reinterpret_cast<uintptr_t>(exch + 2 * prow * pitch) + 15) & ~static_cast<uintptr_t>(15));
-  __shared__ double red[32 * 2];
+  // mu partials (COCG): [block of planes][warp][re, im]
+  __shared__ T s_mu[MODE == OP_COCG ? kMaxLz / kMuPlanes * 32 * 2 : 1];
   __shared__ int s_bad;
 
   for (int i = tid; i < 2 * prow * pitch; i += nt) exch[i] = czero<C>();
@@ -537,7 +522,7 @@ op_kernel_tma(const JuncDev* __restrict__ jt, const BatchDev* __restrict__ bp, c
   C qv[Q];
 #pragma unroll
   for (int m = 0; m < Q; ++m) qv[m] = czero<C>();
-  T acc0 = 0, acc1 = 0, car0 = 0, car1 = 0;
+  T acc0 = 0, acc1 = 0;  // mu(re, im) of kMuPlanes planes
   // per-point operator data of the next plane to compute, loaded one plane early
   float2 dg_n = make_float2(0.f, 0.f);
   auto load_pt = [&](int z) {
@@ -579,7 +564,8 @@ op_kernel_tma(const JuncDev* __restrict__ jt, const BatchDev* __restrict__ bp, c
       fence_proxy_async();
       issue(zl + kStages);
     }
-    if (zc < z0 || !own) continue;
+    if (zc < z0) continue;
+    if (own) {
     const float2 dg_c = dg_n;
     load_pt(zc + 1);
 
@@ -603,19 +589,20 @@ op_kernel_tma(const JuncDev* __restrict__ jt, const BatchDev* __restrict__ bp, c
     if constexpr (MODE == OP_COCG) {
       pnew[vo + gl] = vc;
       reinterpret_cast<C*>(b.q)[vo + gl] = y;
-      kahan_add(acc0, car0, fma(vc.x, y.x, -vc.y * y.y));
-      kahan_add(acc1, car1, fma(vc.x, y.y, vc.y * y.x));
+      acc0 = fma(vc.x, y.x, fma(-vc.y, y.y, acc0));
+      acc1 = fma(vc.x, y.y, fma(vc.y, y.x, acc1));
     } else {
       reinterpret_cast<C*>(y_out)[vo + gl] = y;
     }
+    }
+    if constexpr (MODE == OP_COCG) {
+      if ((zc - z0) % kMuPlanes == kMuPlanes - 1 || zc == z1 - 1) {
+        mu_flush(s_mu, (zc - z0) / kMuPlanes, acc0, acc1);
+        acc0 = acc1 = 0;
+      }
+    }
   }
-  if constexpr (MODE == OP_COCG) {
-    T vv[2] = {acc0 - car0, acc1 - car1};
-    double out[2];
-    block_sum<2>(vv, red, out);
-    if (tid == 0) b.mu_part[(size_t)s * b.PA + tile] = make_double2(out[0], out[1]);
-    if (tid < 32) mu_arrive(b, J, s);
-  }
+  if constexpr (MODE == OP_COCG) mu_finish(b, J, s, s_mu, 0, z0, z1);
 }
 
 template <int R>
@@ -625,7 +612,7 @@ cudaError_t launch_op_tma_r(int mode, bool fp32, dim3 grid, int threads, size_t 
   if (mode == OP_COCG) kern = fp32 ? op_kernel_tma<float, R, OP_COCG> : op_kernel_tma<double, R, OP_COCG>;
   else if (mode == OP_APPLY) kern = fp32 ? op_kernel_tma<float, R, OP_APPLY> : op_kernel_tma<double, R, OP_APPLY>;
   else return cudaErrorInvalidValue;
-  if (smem > 48 * 1024) {
+  if (smem > 16 * 1024) {  // beside the static arrays
     cudaError_t e = set_max_dynamic_smem(reinterpret_cast<const void*>(kern), smem);
     if (e != cudaSuccess) return e;
   }
@@ -653,9 +640,9 @@ cudaError_t launch_op_tma_r(int mode, bool fp32, dim3 grid, int threads, size_t 
                                    void* y_out) {                              \
     return launch_op_plane_r<R>(mode, grid, threads, smem, st, jt, b, x_in, y_out);        \
   }                                                                                               \
-  cudaError_t launch_op_pair_R##R(int mode, bool big, dim3 grid, int threads, size_t smem,        \
+  cudaError_t launch_op_pair_R##R(int mode, bool big, int pitch, dim3 grid, int threads, size_t smem, \
                                   cudaStream_t st, const JuncDev* jt, const BatchDev* b,        \
                                   const void* x_in, void* y_out) {             \
-    return launch_op_pair_r<R>(mode, big, grid, threads, smem, st, jt, b, x_in, y_out);    \
+    return launch_op_pair_r<R>(mode, big, pitch, grid, threads, smem, st, jt, b, x_in, y_out); \
   }                                                                                               \
   }

@@ -45,29 +45,35 @@ __device__ __forceinline__ float2 cfma2(float2 a, float2 b, float2 acc) {
   return fma2(make_float2(-a.y, a.y), make_float2(b.y, b.x), acc);
 }
 
-// Kahan-compensated accumulation (sum, carry) for long FP32 dot products.
-__device__ __forceinline__ void kahan_add_f(float& sum, float& carry, float term) {
-  const float y = term - carry;
-  const float t = sum + y;
-  carry = (t - sum) - y;
-  sum = t;
+// Planes per z chunk of a COCG operator launch, by the number of active slots
+// (host: choose_tiling), and the operator CTAs of a slot with it.
+__device__ __forceinline__ int cocg_lz(const JuncDev& J, const BatchDev& b) {
+  const int n = *b.nact;
+  return J.lz_act[n <= 1 ? 0 : min(kActBuckets - 1, 32 - __clz(n - 1))];
+}
+__device__ __forceinline__ int cocg_tiles(const JuncDev& J, const BatchDev& b) {
+  const int lz = cocg_lz(J, b);
+  return J.ytiles * ((J.nz + lz - 1) / lz);
+}
+__device__ __forceinline__ int cocg_parts(const JuncDev& J) {
+  return J.ytiles * ((J.nz + kMuPlanes - 1) / kMuPlanes);
 }
 
-// End of an operator or projection CTA of slot s, by its first warp once lane 0
-// has written the CTA's partial of mu = p^T A p: the CTA that arrives last adds
-// the J.nA operator partials and the J.n_groups projection partials (lanes in
-// stride, then a shuffle tree: a fixed order for a given tiling) and forms
+// End of an operator or projection CTA of slot s, by its first warp once the
+// CTA's partials of mu = p^T A p are written (and seen by lane 0): the CTA that
+// arrives last adds the operator's and the J.n_groups projections' partials
+// (lanes in stride, then a shuffle tree: a fixed order) and forms
 // alpha = rho / mu, once per system instead of in every update CTA.
 __device__ __forceinline__ void mu_arrive(const BatchDev& b, const JuncDev& J, const int s) {
   const int lane = threadIdx.x & 31;
-  const int n = J.nA + J.n_groups;
+  const int ctas = cocg_tiles(J, b) + J.n_groups, n = cocg_parts(J) + J.n_groups;
   int done = 0;
   if (lane == 0) {
     __threadfence();
     done = atomicAdd(b.mu_cnt + s, 1);
   }
   done = __shfl_sync(0xffffffffu, done, 0);
-  if (done != n - 1) return;
+  if (done != ctas - 1) return;
   __threadfence();
   double v[2] = {0.0, 0.0};
   for (int t = lane; t < n; t += 32) {
@@ -85,6 +91,49 @@ __device__ __forceinline__ void mu_arrive(const BatchDev& b, const JuncDev& J, c
   }
 }
 
+// sum over w < nw of part[w * ld] (see the callers): FP64, or for FP32 parts an
+// error-free FP32 sum (hi + lo) rounded to FP64 at the end, which leaves the FP64
+// pipe with three operations
+__device__ __forceinline__ double sum_strided(const double* part, int nw, int ld) {
+  double o = part[0];
+  for (int w = 1; w < nw; ++w) o += part[w * ld];
+  return o;
+}
+__device__ __forceinline__ double sum_strided(const float* part, int nw, int ld) {
+  float hi = part[0], lo = 0.f;
+  for (int w = 1; w < nw; ++w) {
+    const float a = part[w * ld];
+    const float s = __fadd_rn(hi, a), bb = __fsub_rn(s, hi);
+    lo = __fadd_rn(lo, __fadd_rn(__fsub_rn(hi, __fsub_rn(s, bb)), __fsub_rn(a, bb)));
+    hi = s;
+  }
+  return (double)hi + (double)lo;
+}
+
+// mu partials of an operator CTA: each warp leaves its sum of every kMuPlanes
+// planes in s_mu[block][warp][re, im]; at the end the first warp's lanes (block,
+// component) add the warps' sums and write mu_part, and the CTA arrives.
+template <typename A>
+__device__ __forceinline__ void mu_flush(A* s_mu, int block, A re, A im) {
+  A v[2] = {re, im};
+  const A t = warp_sum_many<2>(v);
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
+  if (lane < 2) s_mu[(block * nw + warp) * 2 + lane] = t;
+}
+template <typename A>
+__device__ __forceinline__ void mu_finish(const BatchDev& b, const JuncDev& J, int s, const A* s_mu, int yt, int z0,
+                                          int z1) {
+  const int nw = blockDim.x >> 5, nb = (z1 - z0 + kMuPlanes - 1) / kMuPlanes;
+  __syncthreads();
+  if (threadIdx.x >= 32) return;
+  double* out = reinterpret_cast<double*>(b.mu_part + (size_t)s * b.PA +
+                                          (size_t)yt * ((J.nz + kMuPlanes - 1) / kMuPlanes) + z0 / kMuPlanes);
+  for (int e = threadIdx.x; e < 2 * nb; e += 32) out[e] = sum_strided(s_mu + (e >> 1) * nw * 2 + (e & 1), nw, 2);
+  __threadfence();
+  __syncwarp();
+  mu_arrive(b, J, s);
+}
+
 struct Pair {
   float2 a, b;  // values at x0 and x0 + 1
 };
@@ -100,7 +149,7 @@ __device__ __forceinline__ void sts_pair(float2* s, const Pair& v) {
 }
 
 
-template <int R, int MODE, bool BIG>
+template <int R, int MODE, int PITCH>
 __global__ void __maxnreg__(96)
 op_pair_kernel(const JuncDev* __restrict__ jt, const BatchDev* __restrict__ bp, const void* __restrict__ x_in,
                void* __restrict__ y_out) {
@@ -109,18 +158,20 @@ op_pair_kernel(const JuncDev* __restrict__ jt, const BatchDev* __restrict__ bp, 
   constexpr int KX = (R + 1) / 2;    // neighbour pairs left / right in x
   constexpr int NIN = (MODE == OP_COCG) ? 2 : 1;
   const BatchDev& b = *bp;
-  const int s = blockIdx.y;
+  const int s = blockIdx.x;
   if constexpr (MODE == OP_COCG) {
     if (b.state[s] != SL_ACTIVE) return;
   }
   const JuncDev& J = jt[b.junc[s]];
-  const int tile = blockIdx.x;
+  const int tile = blockIdx.y;
   if (tile >= J.nA || J.kind != kOpPair) return;
 
   const int nx = J.nx, ny = J.ny, nz = J.nz, plane = J.plane;
   const int hx = nx >> 1;  // pairs per row
-  const int z0 = tile * J.Lz, z1 = min(z0 + J.Lz, nz);
-  const int pitch = nx + 2 * kPairXO;
+  const int Lz = MODE == OP_COCG ? cocg_lz(J, b) : J.Lz;
+  const int z0 = tile * Lz, z1 = min(z0 + Lz, nz);
+  if (z0 >= nz) return;
+  const int pitch = PITCH > 0 ? PITCH : nx + 2 * kPairXO;
   const int rows = ny + 2 * R;
   const int tid = threadIdx.x, nt = blockDim.x;
   const long long vo = b.voff[s];
@@ -130,7 +181,8 @@ op_pair_kernel(const JuncDev* __restrict__ jt, const BatchDev* __restrict__ bp, 
   float2* exch = stage + kPairStages * NIN * plane;    // [2][rows][pitch]
   uint64_t* bars = reinterpret_cast<uint64_t*>(
       (reinterpret_cast<uintptr_t>(exch + 2 * rows * pitch) + 15) & ~static_cast<uintptr_t>(15));
-  __shared__ double red[32 * 2];
+  // mu partials (COCG): [block of planes][warp][re, im]
+  __shared__ float s_mu[MODE == OP_COCG ? kMaxLz / kMuPlanes * (kPairThreadsBig / 32) * 2 : 1];
   __shared__ int s_bad;
 
   for (int i = tid; i < 2 * rows * pitch; i += nt) exch[i] = make_float2(0.f, 0.f);
@@ -198,13 +250,11 @@ op_pair_kernel(const JuncDev* __restrict__ jt, const BatchDev* __restrict__ bp, 
   }
   __syncthreads();
   const float4* dg4 = reinterpret_cast<const float4*>(J.dg32);
-  float4 dgn = make_float4(0.f, 0.f, 0.f, 0.f);  // (-V_loc, Gamma) of both points of the next plane
-  if (own && z0 < z1) dgn = __ldg(dg4 + ((z0 * plane + po) >> 1));
 
   Pair zq[Q];
 #pragma unroll
   for (int m = 0; m < Q; ++m) zq[m] = zero_pair();
-  float2 macc = make_float2(0.f, 0.f), mcar = macc;  // Kahan sum of mu = v^T A_loc v
+  float2 macc = make_float2(0.f, 0.f);               // sum of mu = v^T A_loc v over kMuPlanes planes
   int sidx = 0;                                      // stage of the plane entering the ring
   uint32_t sph = 0;                                  // its mbarrier phase parity
 
@@ -215,6 +265,8 @@ op_pair_kernel(const JuncDev* __restrict__ jt, const BatchDev* __restrict__ bp, 
       if (zc < z1) {
         // plane zl = zc + R arrives in stage sidx and enters ring slot u
         const int zl = zc + R;
+        float4 dgc = make_float4(0.f, 0.f, 0.f, 0.f);  // (-V_loc, Gamma) of both points of plane zc
+        if (own && zc >= z0) dgc = __ldg(dg4 + ((zc * plane + po) >> 1));
         Pair v = zero_pair();
         if (!mbar_wait(bars + sidx, sph)) {
           s_bad = 1;
@@ -254,8 +306,6 @@ op_pair_kernel(const JuncDev* __restrict__ jt, const BatchDev* __restrict__ bp, 
           sph ^= 1u;
         }
         if (zc >= z0 && own) {
-          const float4 dgc = dgn;
-          if (zc + 1 < z1) dgn = __ldg(dg4 + (((zc + 1) * plane + po) >> 1));
           // x neighbours at offsets -2KX .. 2KX+1 from x0
           float2 X[4 * KX + 2];
 #pragma unroll
@@ -293,28 +343,23 @@ op_pair_kernel(const JuncDev* __restrict__ jt, const BatchDev* __restrict__ bp, 
           const int gi = zc * plane + po;
           if constexpr (MODE == OP_COCG) {
             *reinterpret_cast<float4*>(pnew + gi) = make_float4(c0.x, c0.y, c1.x, c1.y);
-            // mu partial v^T y (unconjugated) of both points, Kahan-compensated
-            float2 t = fma2(make_float2(c0.x, c0.x), y0v, make_float2(0.f, 0.f));
-            t = fma2(make_float2(-c0.y, c0.y), make_float2(y0v.y, y0v.x), t);
-            t = fma2(make_float2(c1.x, c1.x), y1v, t);
-            t = fma2(make_float2(-c1.y, c1.y), make_float2(y1v.y, y1v.x), t);
-            const float2 yk = sub2(t, mcar);
-            const float2 tk = add2(macc, yk);
-            mcar = sub2(sub2(tk, macc), yk);
-            macc = tk;
+            // mu partial v^T y (unconjugated) of both points
+            macc = cfma2(c0, y0v, macc);
+            macc = cfma2(c1, y1v, macc);
           }
           *reinterpret_cast<float4*>(yv + gi) = make_float4(y0v.x, y0v.y, y1v.x, y1v.y);
+        }
+        if constexpr (MODE == OP_COCG) {
+          // every kMuPlanes planes and at the chunk's end: the warp's sum so far
+          if (zc >= z0 && ((zc - z0) % kMuPlanes == kMuPlanes - 1 || zc == z1 - 1)) {
+            mu_flush(s_mu, (zc - z0) / kMuPlanes, macc.x, macc.y);
+            macc = make_float2(0.f, 0.f);
+          }
         }
       }
     }
   }
-  if constexpr (MODE == OP_COCG) {
-    float vv[2] = {macc.x - mcar.x, macc.y - mcar.y};
-    double out[2];
-    block_sum<2>(vv, red, out);
-    if (tid == 0) b.mu_part[(size_t)s * b.PA + tile] = make_double2(out[0], out[1]);
-    if (tid < 32) mu_arrive(b, J, s);
-  }
+  if constexpr (MODE == OP_COCG) mu_finish(b, J, s, s_mu, 0, z0, z1);
 }
 
 // ---------------------------------------------------------------------------
@@ -333,16 +378,18 @@ op_plane_kernel(const JuncDev* __restrict__ jt, const BatchDev* __restrict__ bp,
   constexpr int MD = R < 2 ? R : 2;  // distances summed in difference form
   constexpr int NIN = (MODE == OP_COCG) ? 2 : 1;
   const BatchDev& b = *bp;
-  const int s = blockIdx.y;
+  const int s = blockIdx.x;
   if constexpr (MODE == OP_COCG) {
     if (b.state[s] != SL_ACTIVE) return;
   }
   const JuncDev& J = jt[b.junc[s]];
-  const int tile = blockIdx.x;
+  const int tile = blockIdx.y;
   if (tile >= J.nA || J.kind != kOpPlane) return;
 
   const int nx = J.nx, ny = J.ny, nz = J.nz, plane = J.plane;
-  const int z0 = tile * J.Lz, z1 = min(z0 + J.Lz, nz);
+  const int Lz = MODE == OP_COCG ? cocg_lz(J, b) : J.Lz;
+  const int z0 = tile * Lz, z1 = min(z0 + Lz, nz);
+  if (z0 >= nz) return;
   const int pitch = nx + 2 * kPairXO;
   const int rows = ny + 2 * R;
   const int tid = threadIdx.x, nt = blockDim.x;
@@ -353,7 +400,7 @@ op_plane_kernel(const JuncDev* __restrict__ jt, const BatchDev* __restrict__ bp,
   float2* exch = stage + kPairStages * NIN * plane;    // [2][rows][pitch]
   uint64_t* bars = reinterpret_cast<uint64_t*>(
       (reinterpret_cast<uintptr_t>(exch + 2 * rows * pitch) + 15) & ~static_cast<uintptr_t>(15));
-  __shared__ double red[32 * 2];
+  __shared__ float s_mu[MODE == OP_COCG ? kMaxLz / kMuPlanes * (kPlaneThreads / 32) * 2 : 1];
   __shared__ int s_bad;
   __shared__ float s_w[R + 2];
 
@@ -418,7 +465,7 @@ op_plane_kernel(const JuncDev* __restrict__ jt, const BatchDev* __restrict__ bp,
   float2 zq[Q];
 #pragma unroll
   for (int m = 0; m < Q; ++m) zq[m] = make_float2(0.f, 0.f);
-  float ma_x = 0.f, ma_y = 0.f, mc_x = 0.f, mc_y = 0.f;  // Kahan sum of mu = v^T A_loc v
+  float ma_x = 0.f, ma_y = 0.f;  // sum of mu = v^T A_loc v over kMuPlanes planes
   int sidx = 0;
   uint32_t sph = 0;
 
@@ -492,22 +539,22 @@ op_plane_kernel(const JuncDev* __restrict__ jt, const BatchDev* __restrict__ bp,
           const int gi = zc * plane + tid;
           if constexpr (MODE == OP_COCG) {
             pnew[gi] = c;
-            // mu partial v^T y (unconjugated), Kahan-compensated
-            kahan_add_f(ma_x, mc_x, fmaf(c.x, y.x, -c.y * y.y));
-            kahan_add_f(ma_y, mc_y, fmaf(c.x, y.y, c.y * y.x));
+            // mu partial v^T y (unconjugated)
+            ma_x = fmaf(c.x, y.x, fmaf(-c.y, y.y, ma_x));
+            ma_y = fmaf(c.x, y.y, fmaf(c.y, y.x, ma_y));
           }
           yv[gi] = y;
+        }
+        if constexpr (MODE == OP_COCG) {
+          if (zc >= z0 && ((zc - z0) % kMuPlanes == kMuPlanes - 1 || zc == z1 - 1)) {
+            mu_flush(s_mu, (zc - z0) / kMuPlanes, ma_x, ma_y);
+            ma_x = ma_y = 0.f;
+          }
         }
       }
     }
   }
-  if constexpr (MODE == OP_COCG) {
-    float vv[2] = {ma_x - mc_x, ma_y - mc_y};
-    double out[2];
-    block_sum<2>(vv, red, out);
-    if (tid == 0) b.mu_part[(size_t)s * b.PA + tile] = make_double2(out[0], out[1]);
-    if (tid < 32) mu_arrive(b, J, s);
-  }
+  if constexpr (MODE == OP_COCG) mu_finish(b, J, s, s_mu, 0, z0, z1);
 }
 
 template <int R>
@@ -518,7 +565,7 @@ cudaError_t launch_op_plane_r(int mode, dim3 grid, int threads, size_t smem, cud
   else if (mode == OP_APPLY) kern = op_plane_kernel<R, OP_APPLY>;
   else return cudaErrorInvalidValue;
   if (threads > kPlaneThreads) return cudaErrorInvalidValue;
-  if (smem > 48 * 1024) {
+  if (smem > 16 * 1024) {  // beside the static arrays
     cudaError_t e = set_max_dynamic_smem(reinterpret_cast<const void*>(kern), smem);
     if (e != cudaSuccess) return e;
   }
@@ -528,14 +575,21 @@ cudaError_t launch_op_plane_r(int mode, dim3 grid, int threads, size_t smem, cud
 }
 
 template <int R>
-cudaError_t launch_op_pair_r(int mode, bool big, dim3 grid, int threads, size_t smem, cudaStream_t st,
+cudaError_t launch_op_pair_r(int mode, bool big, int pitch, dim3 grid, int threads, size_t smem, cudaStream_t st,
                              const JuncDev* jt, const BatchDev* b, const void* x_in, void* y_out) {
   void (*kern)(const JuncDev*, const BatchDev*, const void*, void*) = nullptr;
-  if (mode == OP_COCG) kern = big ? op_pair_kernel<R, OP_COCG, true> : op_pair_kernel<R, OP_COCG, false>;
-  else if (mode == OP_APPLY) kern = big ? op_pair_kernel<R, OP_APPLY, true> : op_pair_kernel<R, OP_APPLY, false>;
-  else return cudaErrorInvalidValue;
+#define RSN_PAIR(M) \
+  kern = pitch == 40 ? op_pair_kernel<R, M, 40> : pitch == 56 ? op_pair_kernel<R, M, 56> : op_pair_kernel<R, M, 0>;
+  if (mode == OP_COCG) {
+    RSN_PAIR(OP_COCG)
+  } else if (mode == OP_APPLY) {
+    RSN_PAIR(OP_APPLY)
+  } else {
+    return cudaErrorInvalidValue;
+  }
+#undef RSN_PAIR
   if (threads > (big ? kPairThreadsBig : kPairThreads)) return cudaErrorInvalidValue;
-  if (smem > 48 * 1024) {
+  if (smem > 16 * 1024) {  // beside the static arrays
     cudaError_t e = set_max_dynamic_smem(reinterpret_cast<const void*>(kern), smem);
     if (e != cudaSuccess) return e;
   }

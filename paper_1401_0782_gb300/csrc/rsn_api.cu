@@ -64,6 +64,10 @@ struct Tiling {
   bool tma = false;   // whole-plane tile streamed by bulk copies (op_kernel_tma)
   bool pair = false;  // FP32 point-pair kernel with plane streaming (op_pair_kernel)
   bool plane = false; // FP32 one-point-per-thread kernel with plane streaming (op_plane_kernel)
+  int parts = 0;      // COCG: mu partials per slot
+  // COCG: planes per chunk and CTAs per slot when at most 2^k slots are busy
+  int lz_act[kActBuckets] = {0}, n_act[kActBuckets] = {0};
+  int pitch = 0;      // its compile-time row pitch (0: none)
   bool big = false;   // its one-CTA-per-SM variant (planes of more than 2 * kPairThreads points)
 };
 
@@ -75,8 +79,8 @@ struct Workspace {
   int PA = 0, PB = 0, n_proj = 0;
   DevBuf Xslot, r, p0, p1, q, d;
   DevBuf state, sys, junc, E, col, voff, xo, xfo, iters, total_iters, cyc_iters, n_upd, restart, stall, warm, rho_cur, beta_cur;
-  DevBuf bnorm2, sigma, rlast2, rrec2, tol2;
-  DevBuf res_part, res_cnt, res_tot, tlast, gcnt, gphase, tgoal, rgoal, rho, nrm, mu, mu_cnt, alpha, upd_cnt, c_r, c_p, c_x, sched, counters, lst, lst_n,
+  DevBuf bnorm2, sigma, rlast2, rrec2, rmin2, rmin_it, tol2;
+  DevBuf res_part, res_cnt, res_tot, tlast, gcnt, gphase, tgoal, rgoal, rho, nrm, mu, mu_cnt, alpha, nact, upd_cnt, c_r, c_p, c_x, sched, counters, lst, lst_n,
       inlist, fslot, c_e;
   int generation = 0;
 };
@@ -126,10 +130,10 @@ struct BlkBufs {
 };
 
 struct GraphKey {
-  int fp32, slots, iters, generation, proj, timing, n_shift, nT;
+  int fp32, slots, iters, generation, proj, timing, n_shift, nT, busy;
   bool operator<(const GraphKey& o) const {
-    return std::tie(fp32, slots, iters, generation, proj, timing, n_shift, nT) <
-           std::tie(o.fp32, o.slots, o.iters, o.generation, o.proj, o.timing, o.n_shift, o.nT);
+    return std::tie(fp32, slots, iters, generation, proj, timing, n_shift, nT, busy) <
+           std::tie(o.fp32, o.slots, o.iters, o.generation, o.proj, o.timing, o.n_shift, o.nT, o.busy);
   }
 };
 
@@ -154,10 +158,13 @@ struct rsn_ctx {
   std::vector<int64_t> poff;
   std::vector<int32_t> pidx;
   std::vector<double> pval, pekb;
-  bool dirty = true;
+  // what the setters changed since the last upload; the projector tables and the
+  // captured graphs outlive a new potential or CAP
+  bool dirty_v = true, dirty_cap = true, dirty_proj = true;
+  bool dirty() const { return dirty_v || dirty_cap || dirty_proj; }
 
   // device operator data
-  DevBuf dg64, dg32, gld, L_idx, L_gam, inv_ptr, inv_p0, inv_q64, inv_q32, blk_row, row_meta, row_loc, row_q64, row_q32;
+  DevBuf dg64, dg32, gld, L_idx, L_gam, inv_ptr, inv_p0, inv_q64, blk_row, row_meta, row_loc, row_q64, row_q32;
   DevBuf grp_ptr, grp_p0, grp_np, grp_voff, grp_idx, grp_val64, grp_val32, ekb;
   int n_groups = 0, nL = 0, max_np = 1;
   JuncDev jh{};
@@ -242,33 +249,54 @@ static Tiling choose_tiling(const rsn_ctx* c, bool compute64, int mode, int nslo
   // FP32 point-pair kernel: whole planes, nx even (16-byte pairs), at most
   // 2 * kPairThreadsBig points per plane, no explicit register tile requested
   const bool reg_forced = c->tile_override[0] > 0 || c->tile_override[2] > 0 || c->tile_override[3] == -1;
-  // z chunks per tile column: chunks of 2R + 2 planes and more, so that the 2R
-  // halo planes of a chunk do not outweigh it, unless that leaves SMs without a
-  // CTA: then down to two planes a chunk, since the march (chunk + 2R planes) is
-  // what such a launch waits for (8 systems of 16x16x64 in FP32: 26 -> 17 us)
-  auto z_cap = [&](int columns) {
-    return std::max(1, std::max(nz / (2 * R + 2), std::min(nz / 2, 152 / std::max(1, columns))));
+  // z chunks per tile column: as many as make the launch shortest.  A CTA marches
+  // Lz + 2R planes after a start worth a plane or so, halo planes costing half a
+  // plane (FP32) or less (FP64, bound by its pipe), and waves of 152 * per_sm CTAs
+  // follow one another.  24x24x120, order 8: 144 FP32 systems 120 us at Lz 14, 84 at
+  // 60; 16 of them 23 at 10, 64 at 60; FP64, 144 systems 1,430 us at Lz 40, 1,289 at
+  // 60; 16 of them 158 at 10, 151 at 20, 252 at 60.
+  auto pick_zt = [&](long long columns, int per_sm, int zt_max) {
+    int best = 1;
+    double best_cost = 1e300;
+    for (int zt = 1; zt <= std::max(1, std::min(nz / 2, zt_max)); ++zt) {
+      const int lz = std::min(kMaxLz, ((nz + zt - 1) / zt + kMuPlanes - 1) / kMuPlanes * kMuPlanes);
+      const long long n = columns * ((nz + lz - 1) / lz), wave = 152LL * per_sm;
+      const double cost = (double)((n + wave - 1) / wave) * (compute64 ? lz + 0.35 * R + 1.0 : lz + R + 1.5);
+      if (cost < best_cost * 0.999) best_cost = cost, best = zt;
+    }
+    return best;
   };
-  auto z_chunks = [&](int per_sm) {
-    int zt = (4 * per_sm * 152 + nslots - 1) / nslots;
-    zt = std::max(1, std::min(zt, z_cap(nslots)));
-    if (c->tile_override[1] > 0) zt = (nz + c->tile_override[1] - 1) / c->tile_override[1];
-    t.Lz = (nz + zt - 1) / zt;
+  // The COCG launch picks its chunks by the number of slots still busy (lz_act[k]:
+  // at most 2^k of them), apply by its vectors.
+  auto z_chunks = [&](int per_sm, int ytiles) {
+    for (int k = 0; k < kActBuckets; ++k) {
+      const int act = mode == OP_COCG ? (int)std::min<long long>(1LL << k, nslots) : nslots;
+      const int zt = pick_zt((long long)act * ytiles, per_sm, nz);
+      int lz = (nz + zt - 1) / zt;
+      if (c->tile_override[1] > 0) lz = std::min(nz, c->tile_override[1]);
+      lz = std::min(kMaxLz, (lz + kMuPlanes - 1) / kMuPlanes * kMuPlanes);
+      t.lz_act[k] = lz;
+      t.n_act[k] = ytiles * ((nz + lz - 1) / lz);
+      t.n = std::max(t.n, t.n_act[k]);
+    }
+    t.Lz = t.lz_act[kActBuckets - 1];
     t.ztiles = (nz + t.Lz - 1) / t.Lz;
-    t.n = t.ztiles;
-    t.TY = ny;
-    t.ytiles = 1;
+    t.ytiles = ytiles;
+    if (mode != OP_COCG) t.n = ytiles * t.ztiles;
+    t.parts = ytiles * ((nz + kMuPlanes - 1) / kMuPlanes);
   };
   if (!compute64 && mode != OP_RESID && streamable && !reg_forced && c->tile_override[3] != -3 && nx % 2 == 0) {
     const int thr = (int)(((pl / 2) + 31) / 32 * 32);
     const size_t sm = op_pair_smem_bytes(mode, R, nx, ny);
     if (thr <= kPairThreadsBig && sm <= 200 * 1024) {
       t.pair = true;
+      t.pitch = pair_pitch_const(nx);
       t.big = thr > kPairThreads;
       t.threads = thr;
       t.smem = sm;
       t.ppt = 2;
-      z_chunks(t.big ? 1 : 2);
+      t.TY = ny;
+      z_chunks(t.big ? 1 : 2, 1);
       return t;
     }
   }
@@ -280,7 +308,8 @@ static Tiling choose_tiling(const rsn_ctx* c, bool compute64, int mode, int nslo
       t.threads = (int)((pl + 31) / 32 * 32);
       t.smem = sm;
       t.ppt = 1;
-      z_chunks(2);
+      t.TY = ny;
+      z_chunks(2, 1);
       return t;
     }
   }
@@ -309,18 +338,18 @@ static Tiling choose_tiling(const rsn_ctx* c, bool compute64, int mode, int nslo
   t.ytiles = (ny + TY - 1) / TY;
   t.ppt = ppt;
   t.threads = threads;
-  int want = 8 * 152;
-  int zt = (want + nslots * t.ytiles - 1) / (nslots * t.ytiles);
-  zt = std::max(1, std::min(zt, z_cap(nslots * t.ytiles)));
-  if (c->tile_override[1] > 0) zt = (nz + c->tile_override[1] - 1) / c->tile_override[1];
   // few systems need a true residual at a time and it sits on every
   // iteration's critical path: two planes per CTA whatever the operator
   // tiling, so that each CTA marches through 2R + 2 planes only (latency, not
   // bandwidth, bounds it)
-  if (mode == OP_RESID) zt = std::max(1, nz / 2);
-  t.Lz = (nz + zt - 1) / zt;
-  t.ztiles = (nz + t.Lz - 1) / t.Lz;
-  t.n = t.ytiles * t.ztiles;
+  if (mode == OP_RESID) {
+    const int zt = std::max(1, nz / 2);
+    t.Lz = (nz + zt - 1) / zt;
+    t.ztiles = (nz + t.Lz - 1) / t.Lz;
+    t.n = t.ytiles * t.ztiles;
+  } else {
+    z_chunks(compute64 ? 2 : 4, t.ytiles);
+  }
   t.smem = op_smem_bytes(!compute64, mode, R, TY, nx, c->n_proj);
   // whole-plane bulk-copy kernel (on request): FP32 COCG / apply on planes
   // whose byte sizes keep every bulk copy 16-byte aligned
@@ -331,6 +360,7 @@ static Tiling choose_tiling(const rsn_ctx* c, bool compute64, int mode, int nslo
       t.TY = ny;
       t.ytiles = 1;
       t.n = t.ztiles;
+      t.parts = (nz + kMuPlanes - 1) / kMuPlanes;
       t.tma = true;
       t.smem = sm;
       t.threads = (int)((pl + 31) / 32 * 32);
@@ -342,10 +372,11 @@ static Tiling choose_tiling(const rsn_ctx* c, bool compute64, int mode, int nslo
 // Operator launch (COCG or apply) with a tiling from choose_tiling; the
 // JuncDev copy `jt` must carry the same tiling.
 static cudaError_t launch_inner(const rsn_ctx* c, const Tiling& t, int mode, bool fp32, int nslots, cudaStream_t st,
-                                const JuncDev* jt, const BatchDev* b, const void* x_in, void* y_out) {
-  const dim3 grid(t.n, nslots);
+                                const JuncDev* jt, const BatchDev* b, const void* x_in, void* y_out, int tiles = 0) {
+  // slots fastest: the CTAs of systems that sit out come in runs and leave at once
+  const dim3 grid(nslots, tiles > 0 ? tiles : t.n);
   if (t.plane) return launch_op_plane(mode, c->R, grid, t.threads, t.smem, st, jt, b, x_in, y_out);
-  if (t.pair) return launch_op_pair(mode, c->R, t.big, grid, t.threads, t.smem, st, jt, b, x_in, y_out);
+  if (t.pair) return launch_op_pair(mode, c->R, t.big, t.pitch, grid, t.threads, t.smem, st, jt, b, x_in, y_out);
   if (t.tma) return launch_op_tma(mode, fp32, c->R, grid, t.threads, t.smem, st, jt, b, x_in, y_out);
   return launch_op(mode, fp32, c->R, t.ppt, grid, t.threads, t.smem, st, jt, b, x_in, y_out);
 }
@@ -375,43 +406,9 @@ static cudaError_t launch_apply(rsn_ctx* c, const Tiling& t, bool fp32, int n, c
 // ---------------------------------------------------------------------------
 // upload of the operator data (done lazily before the first solve/apply)
 // ---------------------------------------------------------------------------
-static rsn_status commit_setup(rsn_ctx* c) {
-  if (!c->has_grid) RSN_FAIL(c, RSN_ESTATE, "rsn_set_grid has not been called");
-  if (!c->has_v) RSN_FAIL(c, RSN_ESTATE, "rsn_set_potential has not been called");
-  if (!c->has_cap) RSN_FAIL(c, RSN_ESTATE, "rsn_set_cap has not been called");
-  if (!c->dirty) return RSN_OK;
+// Projector tables: atoms with their supports, per-point entries, rows by block.
+static rsn_status commit_projectors(rsn_ctx* c) {
   const long long N = c->N;
-  double cw[kMaxR + 1] = {0};
-  fd_weights(c->R, cw);
-  const double ih2 = 1.0 / (2.0 * c->h * c->h);
-  std::vector<double2> dg(N);
-  std::vector<float2> dgf(N);
-  for (long long i = 0; i < N; ++i) {
-    dg[i] = make_double2(-c->v[i] + 3.0 * cw[0] * ih2, c->gl[i] + c->gr[i]);
-    // FP32 kernels use the difference form of the stencil: no FD diagonal here
-    dgf[i] = make_float2((float)(-c->v[i]), (float)dg[i].y);
-  }
-  RSN_CUDA(c, c->dg64.ensure(N * sizeof(double2)));
-  RSN_CUDA(c, c->dg32.ensure(N * sizeof(float2)));
-  RSN_CUDA(c, c->gld.ensure(N * sizeof(double)));
-  RSN_CUDA(c, cudaMemcpy(c->dg64.p, dg.data(), N * sizeof(double2), cudaMemcpyHostToDevice));
-  RSN_CUDA(c, cudaMemcpy(c->dg32.p, dgf.data(), N * sizeof(float2), cudaMemcpyHostToDevice));
-  RSN_CUDA(c, cudaMemcpy(c->gld.p, c->gl.data(), N * sizeof(double), cudaMemcpyHostToDevice));
-  std::vector<int> lidx;
-  std::vector<double> lgam;
-  for (long long i = 0; i < N; ++i)
-    if (c->gl[i] > 0.0) {
-      lidx.push_back((int)i);
-      lgam.push_back(c->gl[i]);
-    }
-  c->nL = (int)lidx.size();
-  RSN_CUDA(c, c->L_idx.ensure(std::max<size_t>(1, lidx.size()) * sizeof(int)));
-  RSN_CUDA(c, c->L_gam.ensure(std::max<size_t>(1, lgam.size()) * sizeof(double)));
-  if (!lidx.empty()) {
-    RSN_CUDA(c, cudaMemcpy(c->L_idx.p, lidx.data(), lidx.size() * sizeof(int), cudaMemcpyHostToDevice));
-    RSN_CUDA(c, cudaMemcpy(c->L_gam.p, lgam.data(), lgam.size() * sizeof(double), cudaMemcpyHostToDevice));
-  }
-
   // projectors: atoms = runs of consecutive projectors with identical supports
   const int np = c->n_proj;
   std::vector<int> gptr{0}, gp0, gnp, gidx;
@@ -460,7 +457,7 @@ static rsn_status commit_setup(rsn_ctx* c) {
       for (int j = 0; j < gnp[g]; ++j) iq64[(size_t)e * 4 * nq + j] = gval[gvoff[g] + (size_t)j * len + k];
     }
   }
-  std::vector<float> iq32(iq64.begin(), iq64.end()), gvalf(gval.begin(), gval.end());
+  std::vector<float> gvalf(gval.begin(), gval.end());
   // the same entries by blocks of kBlkPts points, for the update kernel: rows of
   // up to 32 points of one atom inside one block, atoms in order.  A point that
   // an atom's index list repeats goes to a further row, so that a row holds each
@@ -471,39 +468,58 @@ static rsn_status commit_setup(rsn_ctx* c) {
   std::vector<unsigned char> rloc;
   std::vector<double> rq64;
   {
-    struct Ent { int blk, g, rep, loc, k; };
-    std::vector<Ent> ents;
-    ents.reserve(nent);
-    std::vector<int> seen(N, -1), rep(N, 0);
+    // entries by block, atoms in order inside a block: a counting sort by block;
+    // only repeated points need more
+    struct Ent { int g, rep, loc, k; };
+    std::vector<int> at(nblk + 1, 0), seen(N, -1), rep(N, 0);
+    for (int i : gidx) at[i / kBlkPts + 1]++;
+    for (int k = 0; k < nblk; ++k) at[k + 1] += at[k];
+    const std::vector<int> first(at);
+    std::vector<Ent> ents(nent);
+    bool repeats = false;
     for (int g = 0; g < G; ++g)
       for (int k = 0; k < gptr[g + 1] - gptr[g]; ++k) {
         const int i = gidx[gptr[g] + k];
         rep[i] = seen[i] == g ? rep[i] + 1 : 0;
+        repeats = repeats || rep[i] > 0;
         seen[i] = g;
-        ents.push_back({i / kBlkPts, g, rep[i], i % kBlkPts, k});
+        ents[at[i / kBlkPts]++] = {g, rep[i], i % kBlkPts, k};
       }
-    std::sort(ents.begin(), ents.end(), [](const Ent& a, const Ent& b) {
-      return std::tie(a.blk, a.g, a.rep, a.loc) < std::tie(b.blk, b.g, b.rep, b.loc);
-    });
-    for (size_t e = 0; e < ents.size();) {
-      const Ent& f = ents[e];
-      size_t e1 = e;
-      while (e1 < ents.size() && e1 - e < 32 && ents[e1].blk == f.blk && ents[e1].g == f.g && ents[e1].rep == f.rep) ++e1;
-      const size_t row = rmeta.size();
-      rmeta.push_back(make_int2(gp0[f.g], (int)(e1 - e)));
-      rloc.resize((row + 1) * 32, 0);
-      rq64.resize((row + 1) * 32 * 4 * nq, 0.0);
-      const int len = gptr[f.g + 1] - gptr[f.g];
-      for (size_t x = e; x < e1; ++x) {
-        const int lane = (int)(x - e);
-        rloc[row * 32 + lane] = (unsigned char)ents[x].loc;
-        for (int j = 0; j < gnp[f.g]; ++j)
-          rq64[((row * nq + j / 4) * 32 + lane) * 4 + j % 4] = gval[gvoff[f.g] + (size_t)j * len + ents[x].k];
+    if (repeats)
+      for (int k = 0; k < nblk; ++k)
+        std::stable_sort(ents.begin() + first[k], ents.begin() + first[k + 1], [](const Ent& a, const Ent& b) {
+          return std::tie(a.g, a.rep) < std::tie(b.g, b.rep);
+        });
+    // rows of the block: count, then fill
+    for (int pass = 0; pass < 2; ++pass) {
+      size_t row = 0;
+      for (int k = 0; k < nblk; ++k) {
+        brow[k] = (int)row;
+        for (int e = first[k]; e < first[k + 1];) {
+          const Ent& f = ents[e];
+          int e1 = e;
+          while (e1 < first[k + 1] && e1 - e < 32 && ents[e1].g == f.g && ents[e1].rep == f.rep) ++e1;
+          if (pass == 1) {
+            rmeta[row] = make_int2(gp0[f.g], e1 - e);
+            const int len = gptr[f.g + 1] - gptr[f.g];
+            for (int x = e; x < e1; ++x) {
+              const int lane = x - e;
+              rloc[row * 32 + lane] = (unsigned char)ents[x].loc;
+              for (int j = 0; j < gnp[f.g]; ++j)
+                rq64[((row * nq + j / 4) * 32 + lane) * 4 + j % 4] = gval[gvoff[f.g] + (size_t)j * len + ents[x].k];
+            }
+          }
+          ++row;
+          e = e1;
+        }
       }
-      brow[f.blk + 1] += 1;
-      e = e1;
+      brow[nblk] = (int)row;
+      if (pass == 0) {
+        rmeta.resize(row);
+        rloc.assign(row * 32, 0);
+        rq64.assign(row * 32 * 4 * nq, 0.0);
+      }
     }
-    for (int k = 0; k < nblk; ++k) brow[k + 1] += brow[k];
   }
   std::vector<float> rq32(rq64.begin(), rq64.end());
   auto up = [&](DevBuf& b, const void* src, size_t bytes) -> cudaError_t {
@@ -520,7 +536,6 @@ static rsn_status commit_setup(rsn_ctx* c) {
   RSN_CUDA(c, up(c->row_q64, rq64.data(), rq64.size() * sizeof(double)));
   RSN_CUDA(c, up(c->row_q32, rq32.data(), rq32.size() * sizeof(float)));
   RSN_CUDA(c, up(c->inv_q64, iq64.data(), nent * 4 * nq * sizeof(double)));
-  RSN_CUDA(c, up(c->inv_q32, iq32.data(), nent * 4 * nq * sizeof(float)));
   RSN_CUDA(c, up(c->grp_ptr, gptr.data(), gptr.size() * sizeof(int)));
   RSN_CUDA(c, up(c->grp_p0, gp0.data(), gp0.size() * sizeof(int)));
   RSN_CUDA(c, up(c->grp_np, gnp.data(), gnp.size() * sizeof(int)));
@@ -529,6 +544,54 @@ static rsn_status commit_setup(rsn_ctx* c) {
   RSN_CUDA(c, up(c->grp_val64, gval.data(), gval.size() * sizeof(double)));
   RSN_CUDA(c, up(c->grp_val32, gvalf.data(), gvalf.size() * sizeof(float)));
   RSN_CUDA(c, up(c->ekb, c->pekb.data(), c->pekb.size() * sizeof(double)));
+  return RSN_OK;
+}
+
+static rsn_status commit_setup(rsn_ctx* c) {
+  if (!c->has_grid) RSN_FAIL(c, RSN_ESTATE, "rsn_set_grid has not been called");
+  if (!c->has_v) RSN_FAIL(c, RSN_ESTATE, "rsn_set_potential has not been called");
+  if (!c->has_cap) RSN_FAIL(c, RSN_ESTATE, "rsn_set_cap has not been called");
+  if (!c->dirty()) return RSN_OK;
+  // an application may still be reading the data that the uploads below replace
+  RSN_CUDA(c, cudaSetDevice(c->device));
+  RSN_CUDA(c, cudaStreamSynchronize(c->st));
+  const long long N = c->N;
+  double cw[kMaxR + 1] = {0};
+  fd_weights(c->R, cw);
+  const double ih2 = 1.0 / (2.0 * c->h * c->h);
+  std::vector<double2> dg(N);
+  std::vector<float2> dgf(N);
+  for (long long i = 0; i < N; ++i) {
+    dg[i] = make_double2(-c->v[i] + 3.0 * cw[0] * ih2, c->gl[i] + c->gr[i]);
+    // FP32 kernels use the difference form of the stencil: no FD diagonal here
+    dgf[i] = make_float2((float)(-c->v[i]), (float)dg[i].y);
+  }
+  RSN_CUDA(c, c->dg64.ensure(N * sizeof(double2)));
+  RSN_CUDA(c, c->dg32.ensure(N * sizeof(float2)));
+  RSN_CUDA(c, c->gld.ensure(N * sizeof(double)));
+  RSN_CUDA(c, cudaMemcpy(c->dg64.p, dg.data(), N * sizeof(double2), cudaMemcpyHostToDevice));
+  RSN_CUDA(c, cudaMemcpy(c->dg32.p, dgf.data(), N * sizeof(float2), cudaMemcpyHostToDevice));
+  if (c->dirty_cap) {
+    RSN_CUDA(c, cudaMemcpy(c->gld.p, c->gl.data(), N * sizeof(double), cudaMemcpyHostToDevice));
+    std::vector<int> lidx;
+    std::vector<double> lgam;
+    for (long long i = 0; i < N; ++i)
+      if (c->gl[i] > 0.0) {
+        lidx.push_back((int)i);
+        lgam.push_back(c->gl[i]);
+      }
+    c->nL = (int)lidx.size();
+    RSN_CUDA(c, c->L_idx.ensure(std::max<size_t>(1, lidx.size()) * sizeof(int)));
+    RSN_CUDA(c, c->L_gam.ensure(std::max<size_t>(1, lgam.size()) * sizeof(double)));
+    if (!lidx.empty()) {
+      RSN_CUDA(c, cudaMemcpy(c->L_idx.p, lidx.data(), lidx.size() * sizeof(int), cudaMemcpyHostToDevice));
+      RSN_CUDA(c, cudaMemcpy(c->L_gam.p, lgam.data(), lgam.size() * sizeof(double), cudaMemcpyHostToDevice));
+    }
+  }
+  if (c->dirty_proj) {
+    const rsn_status rp = commit_projectors(c);
+    if (rp != RSN_OK) return rp;
+  }
 
   JuncDev& J = c->jh;
   memset(&J, 0, sizeof(J));
@@ -548,13 +611,12 @@ static rsn_status commit_setup(rsn_ctx* c) {
   J.nL = c->nL;
   J.L_idx = c->L_idx.as<int>();
   J.L_gam = c->L_gam.as<double>();
-  J.n_proj = np;
+  J.n_proj = c->n_proj;
   J.n_groups = c->n_groups;
   J.inv_ptr = c->inv_ptr.as<int>();
   J.inv_nq = (c->max_np + 3) / 4;
   J.inv_p0 = c->inv_p0.as<int>();
   J.inv_q64 = c->inv_q64.as<double2>();
-  J.inv_q32 = c->inv_q32.as<float4>();
   J.blk_row = c->blk_row.as<int>();
   J.row_meta = c->row_meta.as<int2>();
   J.row_loc = c->row_loc.as<unsigned char>();
@@ -569,9 +631,13 @@ static rsn_status commit_setup(rsn_ctx* c) {
   J.grp_val32 = c->grp_val32.as<float>();
   J.ekb = c->ekb.as<double>();
   RSN_CUDA(c, c->jd.ensure(4 * sizeof(JuncDev)));
-  c->dirty = false;
-  clear_graphs(c);
-  c->ws.generation++;
+  // captured graphs hold launch shapes and the addresses of the device-resident
+  // descriptors, which a new potential or CAP does not change
+  if (c->dirty_proj) {
+    clear_graphs(c);
+    c->ws.generation++;
+  }
+  c->dirty_v = c->dirty_cap = c->dirty_proj = false;
   return RSN_OK;
 }
 
@@ -590,6 +656,7 @@ static void set_tiling_dev(JuncDev& J, const Tiling& t) {
   J.ytiles = t.ytiles;
   J.ztiles = t.ztiles;
   J.nA = t.n;
+  for (int k = 0; k < kActBuckets; ++k) J.lz_act[k] = t.lz_act[k];
   J.kind = t.plane ? kOpPlane : t.pair ? kOpPair : t.tma ? kOpTma : kOpReg;
 }
 
@@ -724,7 +791,7 @@ rsn_status rsn_set_grid(rsn_ctx* c, int nx, int ny, int nz, double h, int R) {
   c->pidx.clear();
   c->pval.clear();
   c->pekb.clear();
-  c->dirty = true;
+  c->dirty_v = c->dirty_cap = c->dirty_proj = true;
   c->err.clear();
   return RSN_OK;
 }
@@ -737,7 +804,7 @@ rsn_status rsn_set_potential(rsn_ctx* c, const double* v) {
     if (!std::isfinite(v[i])) RSN_FAIL(c, RSN_EINVAL, "v_loc[%lld] is not finite", i);
   c->v.assign(v, v + c->N);
   c->has_v = true;
-  c->dirty = true;
+  c->dirty_v = true;
   return RSN_OK;
 }
 
@@ -751,7 +818,7 @@ rsn_status rsn_set_cap(rsn_ctx* c, const double* gl, const double* gr) {
   c->gl.assign(gl, gl + c->N);
   c->gr.assign(gr, gr + c->N);
   c->has_cap = true;
-  c->dirty = true;
+  c->dirty_cap = true;
   return RSN_OK;
 }
 
@@ -766,7 +833,7 @@ rsn_status rsn_set_projectors(rsn_ctx* c, int n_proj, const int64_t* off, const 
     c->pidx.clear();
     c->pval.clear();
     c->pekb.clear();
-    c->dirty = true;
+    c->dirty_proj = true;
     return RSN_OK;
   }
   if (!off || !idx || !val || !ekb) RSN_FAIL(c, RSN_EINVAL, "projector arrays must not be NULL");
@@ -786,7 +853,7 @@ rsn_status rsn_set_projectors(rsn_ctx* c, int n_proj, const int64_t* off, const 
   c->pidx.assign(idx, idx + nnz);
   c->pval.assign(val, val + nnz);
   c->pekb.assign(ekb, ekb + n_proj);
-  c->dirty = true;
+  c->dirty_proj = true;
   return RSN_OK;
 }
 
@@ -863,9 +930,9 @@ static rsn_status ensure_ws(rsn_ctx* c, bool fp32, int S, const PoolSpec* pool =
     PB = pool->PB;
   } else {
     const Tiling ti = choose_tiling(c, !fp32, OP_COCG, S), tr = choose_tiling(c, true, OP_RESID, S);
-    // mu partials: the operator tiles', then one per atom (projection kernel)
-    PA = std::max(ti.n + c->n_groups, tr.n);
-    PB = upd_ctas(N, upd_warps(N, S));
+    // mu partials: the operator's, then one per atom (projection kernel)
+    PA = std::max(ti.parts + c->n_groups, tr.n);
+    PB = upd_ctas(N);
   }
   if (w.slots == S && w.fp32 == fp32 && w.N == N && w.PA == PA && w.PB == PB && w.n_proj == n_proj)
     return RSN_OK;
@@ -899,6 +966,8 @@ static rsn_status ensure_ws(rsn_ctx* c, bool fp32, int S, const PoolSpec* pool =
   RSN_CUDA(c, w.sigma.ensure(sd));
   RSN_CUDA(c, w.rlast2.ensure(sd));
   RSN_CUDA(c, w.rrec2.ensure(sd));
+  RSN_CUDA(c, w.rmin2.ensure(sd));
+  RSN_CUDA(c, w.rmin_it.ensure(si));
   RSN_CUDA(c, w.tol2.ensure(sd));
   RSN_CUDA(c, w.res_part.ensure(4 * (size_t)S * PA * sizeof(double)));
   RSN_CUDA(c, w.res_cnt.ensure(si));
@@ -912,6 +981,7 @@ static rsn_status ensure_ws(rsn_ctx* c, bool fp32, int S, const PoolSpec* pool =
   RSN_CUDA(c, w.mu_cnt.ensure(si));
   RSN_CUDA(c, w.alpha.ensure(S * sizeof(double2)));
   RSN_CUDA(c, w.upd_cnt.ensure(si));
+  RSN_CUDA(c, w.nact.ensure(sizeof(int)));
   RSN_CUDA(c, w.rho.ensure((size_t)S * PB * sizeof(double2)));
   RSN_CUDA(c, w.nrm.ensure((size_t)S * PB * sizeof(double)));
   const size_t npj = std::max(1, n_proj);
@@ -1022,6 +1092,8 @@ static BatchDev slot_batch(rsn_ctx* c, int S, const rsn_solver_opts* o) {
   b.sigma = w.sigma.as<double>();
   b.rlast2 = w.rlast2.as<double>();
   b.rrec2 = w.rrec2.as<double>();
+  b.rmin2 = w.rmin2.as<double>();
+  b.rmin_it = w.rmin_it.as<int>();
   b.tol2 = w.tol2.as<double>();
   b.x64 = w.Xslot.as<double2>();
   b.r = w.r.p;
@@ -1043,6 +1115,7 @@ static BatchDev slot_batch(rsn_ctx* c, int S, const rsn_solver_opts* o) {
   b.mu_cnt = w.mu_cnt.as<int>();
   b.alpha = w.alpha.as<double2>();
   b.upd_cnt = w.upd_cnt.as<int>();
+  b.nact = w.nact.as<int>();
   b.c_r = w.c_r.p;
   b.c_p = w.c_p.p;
   b.c_x = w.c_x.as<double2>();
@@ -1214,7 +1287,7 @@ static rsn_status run_stream(rsn_ctx* c, const rsn_solver_opts* o, const StreamI
   // Shifted systems keep one stream: their per-iteration shift step must see
   // exactly the slots that did a COCG iteration, so the scheduler runs first.
   cudaStream_t st2 = sh ? st : c->st2;
-  auto body = [&](int iters, bool capturing) -> cudaError_t {
+  auto body = [&](int iters, bool capturing, int bucket) -> cudaError_t {
     // inside stream capture an event record must be an external node to be timeable
     const unsigned evf = capturing ? cudaEventRecordExternal : cudaEventRecordDefault;
     cudaError_t e;
@@ -1269,12 +1342,11 @@ static rsn_status run_stream(rsn_ctx* c, const rsn_solver_opts* o, const StreamI
       if (timing && (e = cudaEventRecordWithFlags(c->tev[4 * it], st, evf)) != cudaSuccess) return e;
       if (pool) {
         for (int kd = 0; kd < 4; ++kd)
-          if (pool->has[kd] &&
-              (e = launch_inner(c, pool->inner[kd], OP_COCG, fp32, S, st, ji, bdev, nullptr, nullptr)) !=
-                  cudaSuccess)
+          if (pool->has[kd] && (e = launch_inner(c, pool->inner[kd], OP_COCG, fp32, S, st, ji, bdev, nullptr, nullptr,
+                                                 pool->inner[kd].n_act[bucket])) != cudaSuccess)
             return e;
-      } else if ((e = launch_inner(c, cfg.inner, OP_COCG, fp32, S, st, ji, bdev, nullptr, nullptr)) !=
-                 cudaSuccess) {
+      } else if ((e = launch_inner(c, cfg.inner, OP_COCG, fp32, S, st, ji, bdev, nullptr, nullptr,
+                                   cfg.inner.n_act[bucket])) != cudaSuccess) {
         return e;
       }
       if (timing && (e = cudaEventRecordWithFlags(c->tev[4 * it + 1], st, evf)) != cudaSuccess) return e;
@@ -1292,26 +1364,37 @@ static rsn_status run_stream(rsn_ctx* c, const rsn_solver_opts* o, const StreamI
   };
   const int per_iter = (proj ? 9 : 7) + (sh ? 4 : 0) + (goal ? 1 : 0);
   const double vbytes = (double)(pool ? pool->N : c->N) * (fp32 ? sizeof(float2) : sizeof(double2));
-  cudaGraphExec_t gexec = nullptr;
-  if (o->use_graph) {
-    GraphKey key{fp32 ? 1 : 0, S, G, w.generation, proj ? 1 : 0, timing ? 1 : 0, ns, (sh ? sh->nT : 0) * 2 + (goal ? 1 : 0)};
+  // The z chunks of the COCG operator follow the number of busy slots in three
+  // steps (all, a quarter, a sixteenth of the pool): a few systems left over from a
+  // large pool would otherwise march the long chunks that suit the full one.
+  auto bucket_of = [](int n) {
+    int k = 0;
+    while ((1 << k) < n && k < kActBuckets - 1) ++k;
+    return k;
+  };
+  const int steps[3] = {S, std::max(1, S / 4), std::max(1, S / 16)};
+  auto graph_of = [&](int step, cudaGraphExec_t* out_exec) -> rsn_status {
+    GraphKey key{fp32 ? 1 : 0, S, G, w.generation, proj ? 1 : 0, timing ? 1 : 0, ns,
+                 (sh ? sh->nT : 0) * 2 + (goal ? 1 : 0), steps[step]};
     auto it = c->graphs.find(key);
     if (it != c->graphs.end()) {
-      gexec = it->second;
-    } else {
-      cudaGraph_t g = nullptr;
-      RSN_CUDA(c, cudaStreamBeginCapture(st, cudaStreamCaptureModeThreadLocal));
-      cudaError_t e = body(G, true);
-      cudaError_t e2 = cudaStreamEndCapture(st, &g);
-      if (e != cudaSuccess || e2 != cudaSuccess) {
-        if (g) cudaGraphDestroy(g);
-        RSN_FAIL(c, RSN_ECUDA, "graph capture failed: %s", cudaGetErrorString(e != cudaSuccess ? e : e2));
-      }
-      RSN_CUDA(c, cudaGraphInstantiate(&gexec, g, 0));
-      cudaGraphDestroy(g);
-      c->graphs[key] = gexec;
+      *out_exec = it->second;
+      return RSN_OK;
     }
-  }
+    cudaGraph_t g = nullptr;
+    RSN_CUDA(c, cudaStreamBeginCapture(st, cudaStreamCaptureModeThreadLocal));
+    cudaError_t e = body(G, true, bucket_of(steps[step]));
+    cudaError_t e2 = cudaStreamEndCapture(st, &g);
+    if (e != cudaSuccess || e2 != cudaSuccess) {
+      if (g) cudaGraphDestroy(g);
+      RSN_FAIL(c, RSN_ECUDA, "graph capture failed: %s", cudaGetErrorString(e != cudaSuccess ? e : e2));
+    }
+    e = cudaGraphInstantiate(out_exec, g, 0);
+    cudaGraphDestroy(g);
+    RSN_CUDA(c, e);
+    c->graphs[key] = *out_exec;
+    return RSN_OK;
+  };
 
   // every system needs at most max_iter COCG iterations plus one iteration per
   // true residual, and a dependent system starts after its dependency; this
@@ -1326,12 +1409,22 @@ static rsn_status run_stream(rsn_ctx* c, const rsn_solver_opts* o, const StreamI
   int* hs = c->sched_host;
   const auto t_run = std::chrono::steady_clock::now();
   long long reps_done = 0;
+  int step_now = -1;
   for (long long rep = 0; rep < max_replays; ++rep) {
     ++reps_done;
-    if (gexec) {
+    // busy slots after the last replay; a queue that is not empty fills every slot
+    const int busy = rep == 0 || hs[0] < nsys ? S : hs[1];
+    const int step = busy <= steps[2] ? 2 : busy <= steps[1] ? 1 : 0;
+    if (step != step_now) {
+      RSN_CUDA(c, cudaMemcpyAsync(w.nact.p, &steps[step], sizeof(int), cudaMemcpyHostToDevice, st));
+      step_now = step;
+    }
+    if (o->use_graph) {
+      cudaGraphExec_t gexec = nullptr;
+      if ((rs = graph_of(step, &gexec)) != RSN_OK) return rs;
       RSN_CUDA(c, cudaGraphLaunch(gexec, st));
     } else {
-      RSN_CUDA(c, body(G, false));
+      RSN_CUDA(c, body(G, false, bucket_of(steps[step])));
     }
     c->st_launches += (int64_t)G * per_iter;
     RSN_CUDA(c, cudaMemcpyAsync(hs, w.sched.p, (3 + 2 * kMaxGraphIters) * sizeof(int), cudaMemcpyDeviceToHost, st));
@@ -2439,7 +2532,9 @@ static bool make_pool(rsn_ctx* const* ctxs, int K, bool fp32, int nslots, PoolSp
     L.threads = std::max(L.threads, ti.threads);
     L.smem = std::max(L.smem, ti.smem);
     L.n = std::max(L.n, ti.n);
+    for (int a = 0; a < kActBuckets; ++a) L.n_act[a] = std::max(L.n_act[a], ti.n_act[a]);
     L.big = L.big || ti.big;
+    if (L.pitch != ti.pitch) L.pitch = 0;
     if (k == 0) pool.resid = tr;
     pool.resid.threads = std::max(pool.resid.threads, tr.threads);
     pool.resid.smem = std::max(pool.resid.smem, tr.smem);
@@ -2449,7 +2544,7 @@ static bool make_pool(rsn_ctx* const* ctxs, int K, bool fp32, int nslots, PoolSp
     pool.n_groups = std::max(pool.n_groups, c->n_groups);
     pool.max_np = std::max(pool.max_np, c->max_np);
     pool.nB = std::max(pool.nB, c->jh.nB);
-    pool.PA = std::max(pool.PA, std::max(ti.n + c->n_groups, tr.n));
+    pool.PA = std::max(pool.PA, std::max(ti.parts + c->n_groups, tr.n));
     
     for (int h = 0; h < 2; ++h) {
       const Tiling& t = h == 0 ? ti : tr;
@@ -2458,7 +2553,7 @@ static bool make_pool(rsn_ctx* const* ctxs, int K, bool fp32, int nslots, PoolSp
       set_tiling_dev(J, t);
     }
   }
-  pool.PB = upd_ctas(pool.N, upd_warps(pool.N, nslots));
+  pool.PB = upd_ctas(pool.N);
   // the big point-pair variant serves every point-pair junction of the pool
   if (pool.has[kOpPair] && pool.inner[kOpPair].threads > kPairThreads) pool.inner[kOpPair].big = true;
   return true;
@@ -2761,9 +2856,10 @@ static rsn_status bench_kernel_impl(rsn_ctx* c, int precision, int kind, int S, 
   RSN_CUDA(c, cudaMemsetAsync(w.nrm.p, 0x3f, (size_t)S * w.PB * sizeof(double), st));
   RSN_CUDA(c, cudaMemsetAsync(w.mu.p, 0x3f, (size_t)S * w.PA * sizeof(double2), st));
   RSN_CUDA(c, cudaMemsetAsync(w.alpha.p, 0x3f, S * sizeof(double2), st));
-  for (DevBuf* v : {&w.mu_cnt, &w.upd_cnt, &w.res_cnt, &w.total_iters, &w.cyc_iters, &w.gphase})
+  for (DevBuf* v : {&w.mu_cnt, &w.upd_cnt, &w.res_cnt, &w.total_iters, &w.cyc_iters, &w.rmin_it, &w.gphase})
     RSN_CUDA(c, cudaMemsetAsync(v->p, 0, S * sizeof(int), st));
   RSN_CUDA(c, cudaMemsetAsync(w.tol2.p, 0, S * sizeof(double), st));
+  RSN_CUDA(c, cudaMemsetAsync(w.rmin2.p, 0x7f, S * sizeof(double), st));
   const size_t npj = std::max(1, c->n_proj);
   RSN_CUDA(c, cudaMemsetAsync(w.c_r.p, 0, (size_t)S * npj * sizeof(double2), st));
   RSN_CUDA(c, cudaMemsetAsync(w.c_p.p, 0, 2 * (size_t)S * npj * sizeof(double2), st));
@@ -2774,6 +2870,7 @@ static rsn_status bench_kernel_impl(rsn_ctx* c, int precision, int kind, int S, 
   std::vector<long long> hvo(S);
   for (int s = 0; s < S; ++s) hvo[s] = (long long)s * N;
   RSN_CUDA(c, cudaMemcpyAsync(w.state.p, hstate.data(), S * sizeof(int), cudaMemcpyHostToDevice, st));
+  RSN_CUDA(c, cudaMemcpyAsync(w.nact.p, &active, sizeof(int), cudaMemcpyHostToDevice, st));
   RSN_CUDA(c, cudaMemcpyAsync(w.iters.p, hone.data(), S * sizeof(int), cudaMemcpyHostToDevice, st));
   RSN_CUDA(c, cudaMemcpyAsync(w.junc.p, hzero.data(), S * sizeof(int), cudaMemcpyHostToDevice, st));
   RSN_CUDA(c, cudaMemcpyAsync(w.col.p, hcol.data(), S * sizeof(int), cudaMemcpyHostToDevice, st));
@@ -2787,8 +2884,12 @@ static rsn_status bench_kernel_impl(rsn_ctx* c, int precision, int kind, int S, 
   const BatchDev* bdev = c->bd.as<BatchDev>();
   LaunchCfg cfg;
   if ((rs = make_cfg(c, fp32, S, cfg)) != RSN_OK) return rs;
+  int bucket = 0;
+  while ((1 << bucket) < active && bucket < kActBuckets - 1) ++bucket;
   auto launch = [&]() -> cudaError_t {
-    if (kind == 0) return launch_inner(c, cfg.inner, OP_COCG, fp32, S, st, cfg.jt_inner, bdev, nullptr, nullptr);
+    if (kind == 0)
+      return launch_inner(c, cfg.inner, OP_COCG, fp32, S, st, cfg.jt_inner, bdev, nullptr, nullptr,
+                          cfg.inner.n_act[bucket]);
     if (kind == 1) return launch_cocg_update(fp32, S, N, c->n_proj > 0, b.ce_stride, 0, st, cfg.jt_inner, bdev);
     return launch_op(OP_RESID, fp32, c->R, cfg.resid.ppt, dim3(cfg.resid.n, S), cfg.resid.threads, cfg.resid.smem,
                      st, cfg.jt_resid, bdev, nullptr, nullptr);
@@ -3019,7 +3120,7 @@ extern "C" rsn_status rsn_apply_noalloc(rsn_ctx* c, int precision, int n_rhs, co
   if (!c) return RSN_EINVAL;
   if (n_rhs < 0 || (n_rhs > 0 && (!E || !x_dev || !y_dev))) RSN_FAIL(c, RSN_EINVAL, "bad arguments");
   if (precision != RSN_FP64 && precision != RSN_MIXED) RSN_FAIL(c, RSN_EINVAL, "bad precision");
-  if (!c->has_grid || !c->has_v || !c->has_cap || c->dirty || !c->jd.p)
+  if (!c->has_grid || !c->has_v || !c->has_cap || c->dirty() || !c->jd.p)
     RSN_FAIL(c, RSN_ESTATE,
              "rsn_apply_noalloc: the operator data is not on the device yet; an allocating call "
              "(e.g. rsn_apply) after the last setter uploads it");

@@ -36,16 +36,12 @@ constexpr int kReadyWindow = 4096;
 constexpr int kVecThreads = 256;
 constexpr int kVecPerThread = 16;  // points per thread in the streaming kernels
 constexpr int kVecPts = kVecThreads * kVecPerThread;
-// COCG update kernel: one warp per block of kBlkPts consecutive points, at most
-// kUpdThreads / 32 blocks per CTA.  Launches too small to give every SM a few
-// CTAs take two blocks per CTA.
+// COCG update kernel: one warp per block of kBlkPts consecutive points,
+// kUpdThreads / 32 blocks per CTA.
 constexpr int kBlkPts = 128;
 constexpr int kUpdThreads = 128;
-__host__ __device__ constexpr int upd_ctas(long long N, int nw) {
-  return (int)((N + (long long)kBlkPts * nw - 1) / ((long long)kBlkPts * nw));
-}
-constexpr int upd_warps(long long N, int nslots) {
-  return (long long)upd_ctas(N, kUpdThreads / 32) * nslots < 2 * 152 ? 2 : kUpdThreads / 32;
+__host__ __device__ constexpr int upd_ctas(long long N) {
+  return (int)((N + kBlkPts * (kUpdThreads / 32) - 1) / (kBlkPts * (kUpdThreads / 32)));
 }
 
 // fewer warps than four CTAs of four on every SM: memory latency counts, not occupancy
@@ -53,11 +49,19 @@ constexpr bool upd_early(long long N, int nslots) {
   return (N + kBlkPts - 1) / kBlkPts * nslots < 16 * 152;
 }
 
+constexpr int kActBuckets = 14;  // up to 8192 slots
+// The COCG operator's partial sums of mu = p^T A p cover kMuPlanes planes each
+// (per y tile), whatever the z chunks, so that a system's result does not depend
+// on how many others share the launch; z chunks are multiples of it, of at most kMaxLz planes.
+constexpr int kMuPlanes = 4;
+constexpr int kMaxLz = 128;
+
 struct JuncDev {
   int nx, ny, nz, plane;
   long long N;
   // stencil tiling of the operator kernel for this junction
-  int TY, Lz, ytiles, ztiles, nA;  // nA = ytiles*ztiles CTAs per slot (this launch's tiling)
+  int TY, Lz, ytiles, ztiles, nA;  // nA = ytiles*ztiles CTAs per slot (this launch's tiling; COCG: at most)
+  int lz_act[kActBuckets];         // COCG: planes per chunk when at most 2^k slots are active
   int kind;                        // operator kernel of this junction's slots: kOpReg, kOpTma, kOpPair, kOpPlane
   int nB;                          // streaming-kernel CTAs per slot
   double w64[kMaxR + 1];           // w[m] = c_m / (2 h^2), m = 1..R (w[0] unused)
@@ -77,7 +81,6 @@ struct JuncDev {
   int inv_nq;
   const int* inv_p0;
   const double2* inv_q64;
-  const float4* inv_q32;
   // the same by blocks of kBlkPts points: block k has rows blk_row[k] .. blk_row[k+1]-1,
   // each up to 32 support points of one atom: (first projector, points) and per
   // lane the point within the block and its value quads ([row][quad][lane])
@@ -134,6 +137,8 @@ struct BatchDev {
   double* sigma;        // ||b||: the inner-precision vectors hold r / sigma and d / sigma
   double* rlast2;       // true ||r||^2 at the previous replacement (progress check)
   double* rrec2;        // recurrence ||r / sigma||^2 when the cycle ended (drift check)
+  double* rmin2;        // smallest recurrence ||r / sigma||^2 of the current cycle
+  int* rmin_it;         // its iteration within the cycle
   double* tol2;         // recurrence target ||r||^2 of the current cycle
   // vectors
   double2* x64;
@@ -154,9 +159,10 @@ struct BatchDev {
   double* rgoal;        // [S] relative true residual when the goal phase began
   double2* rho_part;    // [S][PB] COCG update kernel: r^T r
   double* nrm_part;     // [S][PB]
-  double2* mu_part;     // [S][PA] operator kernel: p^T A p
+  double2* mu_part;     // [S][PA] p^T A p: operator kernel ([ytiles][ceil(nz / kMuPlanes)]), then one per atom (projections)
   int* mu_cnt;          // [S] operator and projection CTAs of the iteration that have written their partial
   double2* alpha;       // [S] alpha_k = rho_k / mu_k, formed by the last of them
+  const int* nact;      // slots that may do a COCG iteration: picks the operator's z chunks (set with the launches)
   int* upd_cnt;         // [S] update CTAs of the iteration that have written their partials
   int pstride;          // per-slot stride of the projection arrays (the largest n_proj of the junctions)
   void* c_r;            // [S][n_proj] projections of r (inner precision)
@@ -302,7 +308,15 @@ constexpr int kPairThreadsBig = 640;  // one CTA per SM (planes of up to 1280 po
 constexpr int kPairStages = 4;        // input planes in flight per CTA
 constexpr int kPlaneThreads = 576;    // one-point-per-thread plane kernel: threads per CTA (two per SM)
 constexpr int kPairXO = 8;            // zero columns left of x = 0 in the exchange tile (>= R, even)
-cudaError_t launch_op_pair(int mode, int R, bool big, dim3 grid, int threads, size_t smem, cudaStream_t st,
+// Row pitch of the exchange tile: nx + 16 (a quarter warp that crosses a row
+// boundary still touches 32 distinct banks), as a compile-time constant for the
+// common widths, which turns the neighbour addresses into immediate offsets.
+// 40 and 56 keep the bank property for nx = 24 and 40 (and nx = 8, 16, whose rows
+// are whole quarter warps); other widths see a few two-way conflicts.
+constexpr int pair_pitch_const(int nx) { return nx + kPairXO + kMaxR <= 40 ? 40 : nx + kPairXO + kMaxR <= 56 ? 56 : 0; }
+// pitch: pair_pitch_const(nx), or 0 where there is none or junctions of several
+// share the launch (the pitch is then nx + 16 of each)
+cudaError_t launch_op_pair(int mode, int R, bool big, int pitch, dim3 grid, int threads, size_t smem, cudaStream_t st,
                            const JuncDev* jt, const BatchDev* b, const void* x_in, void* y_out);
 size_t op_pair_smem_bytes(int mode, int R, int nx, int ny);
 // FP32 one-point-per-thread kernel with plane streaming: whole planes of an

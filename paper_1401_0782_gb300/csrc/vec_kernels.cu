@@ -95,7 +95,7 @@ __global__ void __launch_bounds__(kVecThreads) zero_kernel(const JuncDev* __rest
 // Each warp covers one block of one system.  A non-finite alpha leaves r and d
 // untouched and flags the slot through a NaN norm.
 // FP32 is bound by HBM (48 B a point), FP64 by the FP64 pipe (2 operations a
-// cycle and SM; 11 a point and 8 a projector value quad).
+// cycle and SM; 12 a point and 8 a projector value quad).
 // ---------------------------------------------------------------------------
 // Bookkeeping after a COCG iteration, by the first warp of the slot's last
 // update CTA: rho_{k+1} and ||r||^2 from the partials (fixed-order warp tree),
@@ -126,9 +126,24 @@ __device__ __forceinline__ void book_slot(const BatchDev& b, const int s, const 
   if (b.n_shift > 0) b.rn2[s] = nrm;
   b.beta_cur[s] = beta;
   b.rho_cur[s] = rho;
-  if (!isfinite(nrm)) {
+  // A near-breakdown (mu or rho almost zero) costs an FP64 recurrence its
+  // conjugacy; it may then never converge (about one of 1e5 systems of the 8x8x48
+  // waveguide ran into max_iter at a relative residual of 1e-11 to 1e20).  It
+  // restarts from the true residual past 1e5 times the cycle's smallest residual,
+  // or, once within 1e-4 of ||b||, when half as many iterations as the system has
+  // done (at least 400) brought no new minimum.  (The mixed mode has its cycle
+  // cap; shifted systems must keep their one Krylov space.)
+  const double rm = b.rmin2[s];
+  const bool lower = nrm < rm;
+  if (lower) {
+    b.rmin2[s] = nrm;
+    b.rmin_it[s] = cyc;
+  }
+  const bool thrown = !b.handback && b.n_shift == 0 && !lower &&
+                      (nrm > 1e10 * rm || (rm <= 1e-8 && cyc - b.rmin_it[s] > max(400, tot / 2)));
+  if (!isfinite(nrm) || thrown) {
     b.restart[s] = 1;
-    b.rrec2[s] = 0.0;
+    b.rrec2[s] = thrown ? nrm : 0.0;
     b.state[s] = SL_CHECK;
   } else if (nrm <= b.tol2[s] || tot >= b.max_iter || cyc >= b.cycle_cap) {
     b.rrec2[s] = nrm;
@@ -249,7 +264,7 @@ cocg_update_kernel(const JuncDev* __restrict__ jt, const BatchDev* __restrict__ 
   const JuncDev& J = jt[b.junc[s]];
   const int N = (int)J.N;  // < 2^31
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nw = blockDim.x >> 5;
-  const int nU = upd_ctas(N, nw);
+  const int nU = upd_ctas(N);
   if ((int)blockIdx.x >= nU) return;
   const int blk = blockIdx.x * nw + warp;
   const int i0 = min(blk * kBlkPts, N), i1 = min(i0 + kBlkPts, N);
@@ -262,7 +277,7 @@ cocg_update_kernel(const JuncDev* __restrict__ jt, const BatchDev* __restrict__ 
   C* s_nl = s_ce + b.ce_stride + warp * kBlkPts;    // projector term of the warp's block
   __shared__ double red[4 * (kUpdThreads / 32)];
   __shared__ int s_last;
-  T sx = 0, sy = 0, sxy = 0;  // sums of r.x^2, r.y^2, r.x r.y
+  T re = 0, sy = 0, sxy = 0;  // sums of r.x^2 - r.y^2 (cancelling inside the sum), r.y^2, r.x r.y
   if (fin) {  // uniform across the CTA
     const C* pn = reinterpret_cast<const C*>((k & 1) ? b.p0 : b.p1) + vo;
     const C* qv = reinterpret_cast<const C*>(b.q) + vo;
@@ -315,7 +330,7 @@ cocg_update_kernel(const JuncDev* __restrict__ jt, const BatchDev* __restrict__ 
         d[u].y = fma(ax, p[u].y, fma(ay, p[u].x, d[u].y));
         const bool in = at[u] < i1;  // (a short block's accumulators past its end are not its own)
         const T rx = in ? r[u].x : (T)0, ry = in ? r[u].y : (T)0;
-        sx = fma(rx, rx, sx);
+        re = fma(rx, rx, fma(-ry, ry, re));
         sy = fma(ry, ry, sy);
         sxy = fma(rx, ry, sxy);
       }
@@ -323,15 +338,15 @@ cocg_update_kernel(const JuncDev* __restrict__ jt, const BatchDev* __restrict__ 
       store_pts(dv, at, i1, pairs, d);
     }
   }
-  // ||r||^2 = sx + sy, r^T r = (sx - sy, 2 sxy) over the CTA, fixed order
-  T v[3] = {sx, sy, sxy};
+  // r^T r = (re, 2 sxy), ||r||^2 = re + 2 sy over the CTA, fixed order
+  T v[3] = {re, sy, sxy};
   double o[3];
   block_sum<3>(v, red, o);
   if (warp != 0) return;
   if (lane == 0) {
     const size_t at = (size_t)s * b.PB + blockIdx.x;
-    b.nrm_part[at] = fin ? o[0] + o[1] : __longlong_as_double(0x7ff8000000000000ll);
-    b.rho_part[at] = fin ? make_double2(o[0] - o[1], 2.0 * o[2]) : make_double2(0.0, 0.0);
+    b.nrm_part[at] = fin ? fma(2.0, o[1], o[0]) : __longlong_as_double(0x7ff8000000000000ll);
+    b.rho_part[at] = fin ? make_double2(o[0], 2.0 * o[2]) : make_double2(0.0, 0.0);
     __threadfence();
     const int done = atomicAdd(b.upd_cnt + s, 1);
     s_last = done == nU - 1 ? 1 : 0;
@@ -358,29 +373,6 @@ cocg_update_kernel(const JuncDev* __restrict__ jt, const BatchDev* __restrict__ 
 // ---------------------------------------------------------------------------
 enum { PJ_R = 0, PJ_X = 1, PJ_IN = 2 };
 constexpr int kProjThreads = 256;
-
-// sum over w < NW of part[w * LD + t]: FP64, or for FP32 parts an error-free
-// FP32 sum (hi + lo) rounded to FP64 at the end, which leaves the FP64 pipe with
-// three operations
-template <int NW, int LD>
-__device__ __forceinline__ double sum_warps(const double* part, int t) {
-  double o = part[t];
-#pragma unroll
-  for (int w = 1; w < NW; ++w) o += part[w * LD + t];
-  return o;
-}
-template <int NW, int LD>
-__device__ __forceinline__ double sum_warps(const float* part, int t) {
-  float hi = part[t], lo = 0.f;
-#pragma unroll
-  for (int w = 1; w < NW; ++w) {
-    const float a = part[w * LD + t];
-    const float s = __fadd_rn(hi, a), bb = __fsub_rn(s, hi);
-    lo = __fadd_rn(lo, __fadd_rn(__fsub_rn(hi, __fsub_rn(s, bb)), __fsub_rn(a, bb)));
-    hi = s;
-  }
-  return (double)hi + (double)lo;
-}
 
 template <typename T, int MODE, int NP, int SPB>
 __global__ void __launch_bounds__(kProjThreads) project_kernel(const JuncDev* __restrict__ jt,
@@ -508,7 +500,7 @@ __global__ void __launch_bounds__(kProjThreads) project_kernel(const JuncDev* __
     const int u = mine ? tid / (2 * NP) : 0, p = mine ? (tid >> 1) % NP : 0, sl = s_slot[u];
     double mu = 0.0;
     if (tid < (NT + 31) / 32 * 32) {
-      const double o = mine ? sum_warps<NW, NR * V>(&part[0][0], tid) : 0.0;
+      const double o = mine ? sum_strided(&part[0][tid], NW, NR * V) : 0.0;
       const double x = __shfl_sync(0xffffffffu, o, lane & ~1), y = __shfl_sync(0xffffffffu, o, lane | 1);
       if (mine && sl >= 0 && p < np) {
         const C cr = mk2((CT)x, (CT)y);
@@ -541,12 +533,13 @@ __global__ void __launch_bounds__(kProjThreads) project_kernel(const JuncDev* __
       if (mine) s_mu[tid] = mu;
       __syncthreads();
       if (warp == 0) {
+        const int nP = cocg_parts(J);
         double m = 0.0;
         if (lane < 2 * SPB) {
 #pragma unroll
           for (int q = 0; q < NP; ++q) m += s_mu[(lane >> 1) * 2 * NP + 2 * q + (lane & 1)];
           const int sm = s_slot[lane >> 1];
-          if (sm >= 0) reinterpret_cast<double*>(b.mu_part + (size_t)sm * b.PA + J.nA + g)[lane & 1] = m;
+          if (sm >= 0) reinterpret_cast<double*>(b.mu_part + (size_t)sm * b.PA + nP + g)[lane & 1] = m;
         }
         __threadfence();
         __syncwarp();
@@ -773,6 +766,8 @@ __global__ void __launch_bounds__(kSchedThreads) sched_kernel(const JuncDev* __r
           ++upd;
         }
         b.cyc_iters[s] = 0;
+        b.rmin2[s] = nrm / bn2;
+        b.rmin_it[s] = 0;
         st = SL_ACTIVE;
       }
     }
@@ -1215,7 +1210,7 @@ __global__ void __launch_bounds__(256) landauer_kernel(int n_e, const double* __
                              const void*, void*);                                                 \
   cudaError_t launch_op_tma_R##R(int, bool, dim3, int, size_t, cudaStream_t, const JuncDev*, const BatchDev*,  \
                                  const void*, void*);                                             \
-  cudaError_t launch_op_pair_R##R(int, bool, dim3, int, size_t, cudaStream_t, const JuncDev*, const BatchDev*, \
+  cudaError_t launch_op_pair_R##R(int, bool, int, dim3, int, size_t, cudaStream_t, const JuncDev*, const BatchDev*, \
                                   const void*, void*);                                            \
   cudaError_t launch_op_plane_R##R(int, dim3, int, size_t, cudaStream_t, const JuncDev*, const BatchDev*,      \
                                    const void*, void*);
@@ -1253,15 +1248,15 @@ cudaError_t launch_op_tma(int mode, bool fp32, int R, dim3 grid, int threads, si
   }
 }
 
-cudaError_t launch_op_pair(int mode, int R, bool big, dim3 grid, int threads, size_t smem, cudaStream_t st,
+cudaError_t launch_op_pair(int mode, int R, bool big, int pitch, dim3 grid, int threads, size_t smem, cudaStream_t st,
                            const JuncDev* jt, const BatchDev* b, const void* x_in, void* y_out) {
   switch (R) {
-    case 1: return launch_op_pair_R1(mode, big, grid, threads, smem, st, jt, b, x_in, y_out);
-    case 2: return launch_op_pair_R2(mode, big, grid, threads, smem, st, jt, b, x_in, y_out);
-    case 3: return launch_op_pair_R3(mode, big, grid, threads, smem, st, jt, b, x_in, y_out);
-    case 4: return launch_op_pair_R4(mode, big, grid, threads, smem, st, jt, b, x_in, y_out);
-    case 5: return launch_op_pair_R5(mode, big, grid, threads, smem, st, jt, b, x_in, y_out);
-    case 6: return launch_op_pair_R6(mode, big, grid, threads, smem, st, jt, b, x_in, y_out);
+    case 1: return launch_op_pair_R1(mode, big, pitch, grid, threads, smem, st, jt, b, x_in, y_out);
+    case 2: return launch_op_pair_R2(mode, big, pitch, grid, threads, smem, st, jt, b, x_in, y_out);
+    case 3: return launch_op_pair_R3(mode, big, pitch, grid, threads, smem, st, jt, b, x_in, y_out);
+    case 4: return launch_op_pair_R4(mode, big, pitch, grid, threads, smem, st, jt, b, x_in, y_out);
+    case 5: return launch_op_pair_R5(mode, big, pitch, grid, threads, smem, st, jt, b, x_in, y_out);
+    case 6: return launch_op_pair_R6(mode, big, pitch, grid, threads, smem, st, jt, b, x_in, y_out);
     default: return cudaErrorInvalidValue;
   }
 }
@@ -1281,7 +1276,7 @@ cudaError_t launch_op_plane(int mode, int R, dim3 grid, int threads, size_t smem
 
 size_t op_pair_smem_bytes(int mode, int R, int nx, int ny) {
   const size_t nin = mode == OP_COCG ? 2 : 1;
-  const size_t pitch = (size_t)nx + 2 * kPairXO;
+  const size_t pitch = (size_t)std::max(pair_pitch_const(nx), nx + 2 * kPairXO);
   return sizeof(float2) * (kPairStages * nin * (size_t)nx * ny + 2 * (size_t)(ny + 2 * R) * pitch) + 16 +
          8 * kPairStages;
 }
@@ -1307,8 +1302,8 @@ cudaError_t launch_zero(bool fp32, int nslots, int nB, cudaStream_t st, const Ju
 
 cudaError_t launch_cocg_update(bool fp32, int nslots, long long N_max, bool proj, int ce_stride, int slot_it,
                                cudaStream_t st, const JuncDev* jt, const BatchDev* b) {
-  const int nw = upd_warps(N_max, nslots);
-  const dim3 grid(upd_ctas(N_max, nw), nslots);
+  constexpr int nw = kUpdThreads / 32;
+  const dim3 grid(upd_ctas(N_max), nslots);
   const size_t smem = proj ? ((size_t)ce_stride + nw * kBlkPts) * (fp32 ? sizeof(float2) : sizeof(double2)) : 0;
   const bool early = upd_early(N_max, nslots);
   void (*kern)(const JuncDev*, const BatchDev*, int) =
@@ -1364,7 +1359,7 @@ cudaError_t launch_nonlocal(bool fp32, int n_rhs, long long N, int n_proj, cudaS
   const size_t el = fp32 ? sizeof(float2) : sizeof(double2);
   // several vectors a warp where that still leaves every SM a few CTAs and the
   // coefficients fit beside the sums
-  const int gx = upd_ctas(N, nw), many = fp32 ? 4 : 2;
+  const int gx = upd_ctas(N), many = fp32 ? 4 : 2;
   const bool one = (long long)gx * ((n_rhs + many - 1) / many) < 4 * 152 ||
                    many * ((size_t)n_proj + kCePad) * el > 24 * 1024;
   const int spv = one ? 1 : many;
