@@ -59,22 +59,11 @@ __device__ __forceinline__ int cocg_parts(const JuncDev& J) {
   return J.ytiles * ((J.nz + kMuPlanes - 1) / kMuPlanes);
 }
 
-// End of an operator or projection CTA of slot s, by its first warp once the
-// CTA's partials of mu = p^T A p are written (and seen by lane 0): the CTA that
-// arrives last adds the operator's and the J.n_groups projections' partials
-// (lanes in stride, then a shuffle tree: a fixed order) and forms
-// alpha = rho / mu, once per system instead of in every update CTA.
-__device__ __forceinline__ void mu_arrive(const BatchDev& b, const JuncDev& J, const int s) {
-  const int lane = threadIdx.x & 31;
-  const int ctas = cocg_tiles(J, b) + J.n_groups, n = cocg_parts(J) + J.n_groups;
-  int done = 0;
-  if (lane == 0) {
-    __threadfence();
-    done = atomicAdd(b.mu_cnt + s, 1);
-  }
-  done = __shfl_sync(0xffffffffu, done, 0);
-  if (done != ctas - 1) return;
-  __threadfence();
+// alpha = rho / mu of slot s, by a warp, once all its mu partials are written: the
+// operator's and the J.n_groups projections' partials added in a fixed order
+// (lanes in stride, then a shuffle tree).
+__device__ __forceinline__ void mu_alpha(const BatchDev& b, const JuncDev& J, const int s) {
+  const int lane = threadIdx.x & 31, n = cocg_parts(J) + J.n_groups;
   double v[2] = {0.0, 0.0};
   for (int t = lane; t < n; t += 32) {
     const double2 w = __ldcg(b.mu_part + (size_t)s * b.PA + t);
@@ -89,6 +78,16 @@ __device__ __forceinline__ void mu_arrive(const BatchDev& b, const JuncDev& J, c
     b.alpha[s] = a;
     if (b.n_shift > 0) b.salpha[(size_t)(b.iters[s] & 1) * b.nslots + s] = a;
   }
+}
+
+// One lane, once the CTA's mu partials of slot s are written (and seen by it):
+// counts the CTA in; true for the last of the operator and projection CTAs, whose
+// warp then forms alpha, once per system instead of in every update CTA.
+__device__ __forceinline__ bool mu_arrive(const BatchDev& b, const JuncDev& J, const int s) {
+  __threadfence();
+  const bool last = atomicAdd(b.mu_cnt + s, 1) == cocg_tiles(J, b) + J.n_groups - 1;
+  if (last) __threadfence();
+  return last;
 }
 
 // sum over w < nw of part[w * ld] (see the callers): FP64, or for FP32 parts an
@@ -131,7 +130,8 @@ __device__ __forceinline__ void mu_finish(const BatchDev& b, const JuncDev& J, i
   for (int e = threadIdx.x; e < 2 * nb; e += 32) out[e] = sum_strided(s_mu + (e >> 1) * nw * 2 + (e & 1), nw, 2);
   __threadfence();
   __syncwarp();
-  mu_arrive(b, J, s);
+  const bool last = threadIdx.x == 0 && mu_arrive(b, J, s);
+  if (__any_sync(0xffffffffu, last)) mu_alpha(b, J, s);
 }
 
 struct Pair {

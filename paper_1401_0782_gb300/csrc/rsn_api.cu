@@ -164,7 +164,7 @@ struct rsn_ctx {
   bool dirty() const { return dirty_v || dirty_cap || dirty_proj; }
 
   // device operator data
-  DevBuf dg64, dg32, gld, L_idx, L_gam, inv_ptr, inv_p0, inv_q64, blk_row, row_meta, row_loc, row_q64, row_q32;
+  DevBuf dg64, dg32, gld, L_idx, L_gam, inv_ptr, inv_p0, inv_q64, blk_row, row_ent, row_q64, row_q32;
   DevBuf grp_ptr, grp_p0, grp_np, grp_voff, grp_idx, grp_val64, grp_val32, ekb;
   int n_groups = 0, nL = 0, max_np = 1;
   JuncDev jh{};
@@ -458,69 +458,36 @@ static rsn_status commit_projectors(rsn_ctx* c) {
     }
   }
   std::vector<float> gvalf(gval.begin(), gval.end());
-  // the same entries by blocks of kBlkPts points, for the update kernel: rows of
-  // up to 32 points of one atom inside one block, atoms in order.  A point that
-  // an atom's index list repeats goes to a further row, so that a row holds each
-  // of its points once.
+  // the same entries by blocks of kBlkPts points, for the update kernel: rows of up
+  // to 32 entries; layer k of a block holds the k-th entry of each of its points
+  // that has one, so that a row holds each point once
   const int nblk = (int)((N + kBlkPts - 1) / kBlkPts);
-  std::vector<int> brow(nblk + 1, 0);
-  std::vector<int2> rmeta;
-  std::vector<unsigned char> rloc;
+  std::vector<int> brow(nblk + 1, 0), rent;
   std::vector<double> rq64;
-  {
-    // entries by block, atoms in order inside a block: a counting sort by block;
-    // only repeated points need more
-    struct Ent { int g, rep, loc, k; };
-    std::vector<int> at(nblk + 1, 0), seen(N, -1), rep(N, 0);
-    for (int i : gidx) at[i / kBlkPts + 1]++;
-    for (int k = 0; k < nblk; ++k) at[k + 1] += at[k];
-    const std::vector<int> first(at);
-    std::vector<Ent> ents(nent);
-    bool repeats = false;
-    for (int g = 0; g < G; ++g)
-      for (int k = 0; k < gptr[g + 1] - gptr[g]; ++k) {
-        const int i = gidx[gptr[g] + k];
-        rep[i] = seen[i] == g ? rep[i] + 1 : 0;
-        repeats = repeats || rep[i] > 0;
-        seen[i] = g;
-        ents[at[i / kBlkPts]++] = {g, rep[i], i % kBlkPts, k};
-      }
-    if (repeats)
-      for (int k = 0; k < nblk; ++k)
-        std::stable_sort(ents.begin() + first[k], ents.begin() + first[k + 1], [](const Ent& a, const Ent& b) {
-          return std::tie(a.g, a.rep) < std::tie(b.g, b.rep);
-        });
-    // rows of the block: count, then fill
-    for (int pass = 0; pass < 2; ++pass) {
-      size_t row = 0;
-      for (int k = 0; k < nblk; ++k) {
-        brow[k] = (int)row;
-        for (int e = first[k]; e < first[k + 1];) {
-          const Ent& f = ents[e];
-          int e1 = e;
-          while (e1 < first[k + 1] && e1 - e < 32 && ents[e1].g == f.g && ents[e1].rep == f.rep) ++e1;
-          if (pass == 1) {
-            rmeta[row] = make_int2(gp0[f.g], e1 - e);
-            const int len = gptr[f.g + 1] - gptr[f.g];
-            for (int x = e; x < e1; ++x) {
-              const int lane = x - e;
-              rloc[row * 32 + lane] = (unsigned char)ents[x].loc;
-              for (int j = 0; j < gnp[f.g]; ++j)
-                rq64[((row * nq + j / 4) * 32 + lane) * 4 + j % 4] = gval[gvoff[f.g] + (size_t)j * len + ents[x].k];
-            }
-          }
-          ++row;
-          e = e1;
+  for (int k = 0; k < nblk; ++k) {
+    brow[k] = (int)(rent.size() / 32);
+    const long long i0 = (long long)k * kBlkPts, i1 = std::min<long long>(i0 + kBlkPts, N);
+    if (cnt[i1] == cnt[i0]) continue;
+    for (int layer = 0, more = 1; more; ++layer) {
+      more = 0;
+      int lane = 32;
+      for (long long i = i0; i < i1; ++i) {
+        const int e = cnt[i] + layer;
+        if (e >= cnt[i + 1]) continue;
+        more = 1;
+        if (lane == 32) {
+          rent.resize(rent.size() + 32, -1);
+          rq64.resize(rq64.size() + (size_t)32 * 4 * nq, 0.0);
+          lane = 0;
         }
-      }
-      brow[nblk] = (int)row;
-      if (pass == 0) {
-        rmeta.resize(row);
-        rloc.assign(row * 32, 0);
-        rq64.assign(row * 32 * 4 * nq, 0.0);
+        const size_t row = rent.size() / 32 - 1;
+        rent[row * 32 + lane] = ip0[e] * kBlkPts + (int)(i - i0);
+        for (int j = 0; j < 4 * nq; ++j) rq64[((row * nq + j / 4) * 32 + lane) * 4 + j % 4] = iq64[(size_t)e * 4 * nq + j];
+        ++lane;
       }
     }
   }
+  brow[nblk] = (int)(rent.size() / 32);
   std::vector<float> rq32(rq64.begin(), rq64.end());
   auto up = [&](DevBuf& b, const void* src, size_t bytes) -> cudaError_t {
     cudaError_t e = b.ensure(std::max<size_t>(bytes, 16));
@@ -531,8 +498,7 @@ static rsn_status commit_projectors(rsn_ctx* c) {
   RSN_CUDA(c, up(c->inv_ptr, cnt.data(), (N + 1) * sizeof(int)));
   RSN_CUDA(c, up(c->inv_p0, ip0.data(), nent * sizeof(int)));
   RSN_CUDA(c, up(c->blk_row, brow.data(), brow.size() * sizeof(int)));
-  RSN_CUDA(c, up(c->row_meta, rmeta.data(), rmeta.size() * sizeof(int2)));
-  RSN_CUDA(c, up(c->row_loc, rloc.data(), rloc.size()));
+  RSN_CUDA(c, up(c->row_ent, rent.data(), rent.size() * sizeof(int)));
   RSN_CUDA(c, up(c->row_q64, rq64.data(), rq64.size() * sizeof(double)));
   RSN_CUDA(c, up(c->row_q32, rq32.data(), rq32.size() * sizeof(float)));
   RSN_CUDA(c, up(c->inv_q64, iq64.data(), nent * 4 * nq * sizeof(double)));
@@ -618,8 +584,7 @@ static rsn_status commit_setup(rsn_ctx* c) {
   J.inv_p0 = c->inv_p0.as<int>();
   J.inv_q64 = c->inv_q64.as<double2>();
   J.blk_row = c->blk_row.as<int>();
-  J.row_meta = c->row_meta.as<int2>();
-  J.row_loc = c->row_loc.as<unsigned char>();
+  J.row_ent = c->row_ent.as<int>();
   J.row_q64 = c->row_q64.as<double2>();
   J.row_q32 = c->row_q32.as<float4>();
   J.grp_ptr = c->grp_ptr.as<int>();
@@ -1268,7 +1233,7 @@ static rsn_status run_stream(rsn_ctx* c, const rsn_solver_opts* o, const StreamI
     R = c->R;
   }
   const bool multi = pool && pool->K > 1;
-  const int KL = std::min(S, kListRows);
+  const int KL = std::min(S, kListRows), KV = list_rows(nB, S);
   const bool goal = o->tol_T > 0 && !sh;
   const dim3 gr(cfg.resid.n, KL);
   const int G = std::max(1, std::min(kMaxGraphIters, o->graph_iters));
@@ -1297,7 +1262,7 @@ static rsn_status run_stream(rsn_ctx* c, const rsn_solver_opts* o, const StreamI
       cudaError_t e2;
       if (sh && (e2 = launch_list(st2, bdev)) != cudaSuccess) return e2;
       if (!sh && (e2 = launch_emit(S, st2, jr, bdev)) != cudaSuccess) return e2;
-      if ((e2 = launch_zero(fp32, KL, nB, st2, jr, bdev)) != cudaSuccess) return e2;
+      if ((e2 = launch_zero(fp32, KV, nB, st2, jr, bdev)) != cudaSuccess) return e2;
       if (sh && (e2 = launch_shift_init(sh->nT, st2, jr, bdev)) != cudaSuccess) return e2;
       if (proj && (e2 = launch_project(1, fp32, KL, n_groups, max_np, st2, jr, bdev, nullptr, w.c_x.p, multi)) !=
                       cudaSuccess)
@@ -1305,8 +1270,8 @@ static rsn_status run_stream(rsn_ctx* c, const rsn_solver_opts* o, const StreamI
       if ((e2 = launch_op(OP_RESID, fp32, R, cfg.resid.ppt, gr, cfg.resid.threads, cfg.resid.smem, st2, jr, bdev,
                           nullptr, nullptr)) != cudaSuccess)
         return e2;
-      if ((e2 = launch_x_update(fp32, KL, nB, st2, jr, bdev)) != cudaSuccess) return e2;
-      if (goal && (e2 = launch_tgoal(st2, jr, bdev)) != cudaSuccess) return e2;
+      if ((e2 = launch_x_update(fp32, KV, nB, st2, jr, bdev)) != cudaSuccess) return e2;
+      if (goal && (e2 = launch_tgoal(KV, st2, jr, bdev)) != cudaSuccess) return e2;
       return cudaSuccess;
     };
     auto schedule = [&](int it) -> cudaError_t {

@@ -28,8 +28,14 @@ constexpr int kMaxGoalChecks = 24;   // T checks of a goal phase before it ends
 constexpr int kSchedThreads = 1024;
 // CTA rows of the kernels that work only on NEW / CHECK slots (zero, true
 // residual and its projections, x update): each row takes list entries
-// row, row + kListRows, ...; a handful of slots need them per iteration
+// row, row + rows, ...; a handful of slots need them per iteration.  Small systems,
+// of which many run and are checked together, get as many rows as fill the SMs.
 constexpr int kListRows = 32;
+constexpr int list_rows(int ctas_per_slot, int nslots) {
+  const int fill = 2 * 152 / (ctas_per_slot > 0 ? ctas_per_slot : 1);
+  const int r = fill > kListRows ? fill : kListRows;
+  return r < nslots ? r : nslots;
+}
 // systems past the first unstarted one that the scheduler examines for a
 // ready system (its dependency finished) when slots are free
 constexpr int kReadyWindow = 4096;
@@ -81,12 +87,12 @@ struct JuncDev {
   int inv_nq;
   const int* inv_p0;
   const double2* inv_q64;
-  // the same by blocks of kBlkPts points: block k has rows blk_row[k] .. blk_row[k+1]-1,
-  // each up to 32 support points of one atom: (first projector, points) and per
-  // lane the point within the block and its value quads ([row][quad][lane])
+  // the same by blocks of kBlkPts points: block k has rows blk_row[k] .. blk_row[k+1]-1
+  // of up to 32 entries of different points: per lane the atom's first projector
+  // * kBlkPts + the point within the block (-1: none) and its value quads
+  // ([row][quad][lane])
   const int* blk_row;
-  const int2* row_meta;
-  const unsigned char* row_loc;
+  const int* row_ent;
   const double2* row_q64;
   const float4* row_q32;
   const int* grp_ptr;
@@ -342,7 +348,7 @@ cudaError_t launch_emit(int nslots, cudaStream_t st, const JuncDev* jt, const Ba
 cudaError_t launch_list(cudaStream_t st, const BatchDev* b);
 cudaError_t launch_landauer(int n_e, const double* E, const double* T, int n_v, const double* V, double E_F,
                             double kT, double* I, cudaStream_t st);
-cudaError_t launch_tgoal(cudaStream_t st, const JuncDev* jt, const BatchDev* b);
+cudaError_t launch_tgoal(int rows, cudaStream_t st, const JuncDev* jt, const BatchDev* b);
 cudaError_t launch_t_final(int n_e, int n_cols, cudaStream_t st, const double* t_all,
                            const double* gr_cols, double* T_out);
 // shifted systems: initialisation of NEW slots, the per-iteration update of

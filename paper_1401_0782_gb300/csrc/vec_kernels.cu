@@ -153,11 +153,12 @@ __device__ __forceinline__ void book_slot(const BatchDev& b, const int s, const 
 
 // The projector term of one block of kBlkPts points, by one warp:
 // acc[l] = -sum over the block's projector rows of value * ce, acc and ce in
-// shared memory.  A row holds up to 32 support points of one atom inside the
-// block, each point once, so the lanes of a row never meet; the rows of a block
-// come in atom order, which fixes the order of the sums.  The loads of up to
-// four rows are in flight together (NQ: value quads per row entry).  SPV vectors
-// at once: vector v has its coefficients at ce + v * ces, its sums at acc + v * kBlkPts.
+// shared memory.  A row holds up to 32 entries (support point, atom) of different
+// points, so its lanes never meet: the rows of layer k hold the k-th atom of every
+// point that has one, which fixes the order of a point's sum and fills the lanes
+// (rows of one atom each left a third of them empty).  The loads of up to four
+// rows are in flight together (NQ: value quads per entry).  SPV vectors at once:
+// vector v has its coefficients at ce + v * ces, its sums at acc + v * kBlkPts.
 template <typename T, int NQ, int SPV>
 __device__ __forceinline__ void block_nonlocal_nq(const JuncDev& J, const typename cx<T>::t* ce, const int ces,
                                                   const int row0, const int row1, typename cx<T>::t* acc) {
@@ -165,15 +166,13 @@ __device__ __forceinline__ void block_nonlocal_nq(const JuncDev& J, const typena
   constexpr int D = NQ == 1 ? 4 : NQ == 2 ? 2 : 1;
   const int lane = threadIdx.x & 31;
   for (int row = row0; row < row1; row += D) {
-    int2 m[D];  // first projector, points of the row
-    int l[D];
+    int m[D];  // first projector * kBlkPts + point, -1: no entry
     T a[D][4 * NQ];
 #pragma unroll
     for (int j = 0; j < D; ++j) {
       const int rr = min(row + j, row1 - 1);
-      m[j] = __ldg(J.row_meta + rr);
-      if (row + j >= row1) m[j].y = 0;
-      l[j] = __ldg(J.row_loc + rr * 32 + lane);
+      m[j] = __ldg(J.row_ent + rr * 32 + lane);
+      if (row + j >= row1) m[j] = -1;
 #pragma unroll
       for (int qd = 0; qd < NQ; ++qd) {
         const size_t at = ((size_t)rr * NQ + qd) * 32 + lane;
@@ -188,13 +187,15 @@ __device__ __forceinline__ void block_nonlocal_nq(const JuncDev& J, const typena
     }
 #pragma unroll
     for (int j = 0; j < D; ++j) {
-      if (lane < m[j].y) {
+      if (m[j] >= 0) {
+        const int l = m[j] % kBlkPts;
+        const C* cp = ce + m[j] / kBlkPts;
 #pragma unroll
         for (int v = 0; v < SPV; ++v) {
-          C y = acc[v * kBlkPts + l[j]];
+          C y = acc[v * kBlkPts + l];
 #pragma unroll
-          for (int i = 0; i < 4 * NQ; ++i) y = rfma(-a[j][i], ce[v * ces + m[j].x + i], y);
-          acc[v * kBlkPts + l[j]] = y;
+          for (int i = 0; i < 4 * NQ; ++i) y = rfma(-a[j][i], cp[v * ces + i], y);
+          acc[v * kBlkPts + l] = y;
         }
       }
       __syncwarp();
@@ -426,22 +427,19 @@ __global__ void __launch_bounds__(kProjThreads) project_kernel(const JuncDev* __
     int slot[SPB];
     long long vo[SPB], xo[SPB];
     double sig[SPB];
+    // every active slot of this CTA belongs to a junction with this group; the
+    // junction of the first active slot supplies the support (batches share it)
+    int s0 = 0;
+    for (int u = SPB - 1; u >= 0; --u)
+      if (s_slot[u] >= 0) s0 = s_slot[u];
 #pragma unroll
     for (int u = 0; u < SPB; ++u) {
       slot[u] = s_slot[u];
-      const int s = slot[u] >= 0 ? slot[u] : 0;
+      const int s = slot[u] >= 0 ? slot[u] : s0;
       vo[u] = b.voff[s];
       xo[u] = (MODE == PJ_X) ? b.xo[s] : 0;
       sig[u] = (MODE == PJ_X) ? b.sigma[s] : 1.0;
     }
-    // every active slot of this CTA belongs to a junction with this group; the
-    // junction of the first active slot supplies the support (batches share it)
-    int s0 = 0;
-    for (int u = 0; u < SPB; ++u)
-      if (slot[u] >= 0) {
-        s0 = slot[u];
-        break;
-      }
     const JuncDev& J = jt[b.junc[s0]];
     const int p0 = J.grp_p0[g], np = J.grp_np[g];
     const int k0 = J.grp_ptr[g], k1 = J.grp_ptr[g + 1], len = k1 - k0;
@@ -449,24 +447,21 @@ __global__ void __launch_bounds__(kProjThreads) project_kernel(const JuncDev* __
     CT acc[NR * V];
 #pragma unroll
     for (int j = 0; j < NR * V; ++j) acc[j] = 0;
-#pragma unroll 2
+#pragma unroll(NP * SPB <= 8 ? 4 : 2)
     for (int kk = tid; kk < len; kk += kProjThreads) {
       const int gi = J.grp_idx[k0 + kk];
       CT a[NP];
 #pragma unroll
       for (int p = 0; p < NP; ++p) {
-        if (p < np) {
-          if constexpr (sizeof(CT) == 8) a[p] = (CT)J.grp_val64[vb + kk + (long long)p * len];
-          else a[p] = (CT)J.grp_val32[vb + kk + (long long)p * len];
-        } else {
-          a[p] = 0;
-        }
+        // (past the atom's projectors: its last one again, dropped at the end)
+        const long long at = vb + kk + (long long)min(p, np - 1) * len;
+        if constexpr (sizeof(CT) == 8) a[p] = (CT)J.grp_val64[at];
+        else a[p] = (CT)J.grp_val32[at];
       }
       C v[SPB];
 #pragma unroll
       for (int u = 0; u < SPB; ++u) {
-        v[u] = czero<C>();
-        if (slot[u] < 0) continue;
+        // (a slot that sits out reads another one's vector; its sums are dropped)
         if constexpr (MODE == PJ_R) {
           v[u] = reinterpret_cast<const CO*>(b.r)[vo[u] + gi];
         } else if constexpr (MODE == PJ_X) {
@@ -543,8 +538,11 @@ __global__ void __launch_bounds__(kProjThreads) project_kernel(const JuncDev* __
         }
         __threadfence();
         __syncwarp();
+        // the slots' arrivals side by side
+        const unsigned last = __ballot_sync(0xffffffffu, lane < SPB && s_slot[lane < SPB ? lane : 0] >= 0 &&
+                                                             mu_arrive(b, J, s_slot[lane < SPB ? lane : 0]));
         for (int v = 0; v < SPB; ++v)
-          if (s_slot[v] >= 0) mu_arrive(b, J, s_slot[v]);
+          if ((last >> v) & 1u) mu_alpha(b, J, s_slot[v]);
       }
     }
   }  // list entries
@@ -785,7 +783,8 @@ __global__ void __launch_bounds__(kSchedThreads) sched_kernel(const JuncDev* __r
   // (1) the free slots, compacted in slot order
   if (threadIdx.x == 0) s_nf = 0;
   __syncthreads();
-  for (int base = 0; base < S; base += blockDim.x) {
+  const int next0 = b.sched[0];
+  for (int base = 0; base < S && next0 < b.nsys; base += blockDim.x) {
     const int s = base + threadIdx.x;
     const bool fr = s < S && b.state[s] == SL_FREE;
     const unsigned m = __ballot_sync(0xffffffffu, fr);
@@ -802,7 +801,6 @@ __global__ void __launch_bounds__(kSchedThreads) sched_kernel(const JuncDev* __r
     __syncthreads();
   }
   const int nf = s_nf;
-  const int next0 = b.sched[0];
   // (2) ready systems, in queue order, to the free slots
   if (threadIdx.x == 0) s_done = 0;
   __syncthreads();
@@ -1338,10 +1336,10 @@ cudaError_t launch_project(int mode, bool fp32, int nslots, int n_groups, int ma
   // slots per CTA: the projector values of an atom are loaded once for all of
   // them; a pool over several junctions takes one slot per CTA (atom g differs
   // between junctions), and so does a launch that would leave SMs idle
-  const bool one = one_slot_per_cta || (long long)n_groups * ((nslots + 3) / 4) < 2 * 152;
+  const bool one = one_slot_per_cta || (long long)n_groups * ((nslots + 1) / 2) < 2 * 152;
   if (max_np <= 4) {
     if (one) launch_project_np<4, 1>(mode, fp32, dim3(n_groups, nslots), st, jt, b, x_in, c_out);
-    else launch_project_np<4, 4>(mode, fp32, dim3(n_groups, (nslots + 3) / 4), st, jt, b, x_in, c_out);
+    else launch_project_np<4, 2>(mode, fp32, dim3(n_groups, (nslots + 1) / 2), st, jt, b, x_in, c_out);
   } else if (max_np <= 9) {
     if (one) launch_project_np<9, 1>(mode, fp32, dim3(n_groups, nslots), st, jt, b, x_in, c_out);
     else launch_project_np<9, 2>(mode, fp32, dim3(n_groups, (nslots + 1) / 2), st, jt, b, x_in, c_out);
@@ -1405,8 +1403,8 @@ cudaError_t launch_shift_emit(int nslots, int n_shift, cudaStream_t st, const Ju
   return cudaGetLastError();
 }
 
-cudaError_t launch_tgoal(cudaStream_t st, const JuncDev* jt, const BatchDev* b) {
-  tgoal_kernel<<<kListRows, 256, 0, st>>>(jt, b);
+cudaError_t launch_tgoal(int rows, cudaStream_t st, const JuncDev* jt, const BatchDev* b) {
+  tgoal_kernel<<<rows, 256, 0, st>>>(jt, b);
   return cudaGetLastError();
 }
 
