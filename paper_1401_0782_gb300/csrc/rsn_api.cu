@@ -91,7 +91,7 @@ struct CallBufs {
       out_t;
   DevBuf X0, X1, wt, g, t_all, gr_cols, Td;
   // shifted systems
-  DevBuf sh_sig, sh_idx, sh_xs, sh_ps, sh_pi, sh_cit, sh_alpha, sh_beta, sh_rn2, sh_ts, sh_sit, sh_srel;
+  DevBuf sh_sig, sh_idx, sh_xs, sh_ps, sh_pi, sh_cit, sh_alpha, sh_beta, sh_stamp, sh_rn2, sh_ts, sh_sit, sh_srel;
   // Landauer current
   DevBuf lE, lT, lV, lI;
 };
@@ -1172,6 +1172,9 @@ static rsn_status run_stream(rsn_ctx* c, const rsn_solver_opts* o, const StreamI
     RSN_CUDA(c, q.sh_cit.ensure((size_t)S * ns * sizeof(int)));
     RSN_CUDA(c, q.sh_alpha.ensure(2 * (size_t)S * sizeof(double2)));
     RSN_CUDA(c, q.sh_beta.ensure(2 * (size_t)S * sizeof(double2)));
+    RSN_CUDA(c, q.sh_stamp.ensure(((size_t)S + 1) * sizeof(int)));
+    RSN_CUDA(c, cudaMemsetAsync(q.sh_stamp.p, 0xff, (size_t)S * sizeof(int), st));
+    RSN_CUDA(c, cudaMemsetAsync(q.sh_stamp.as<int>() + S, 0, sizeof(int), st));
     RSN_CUDA(c, q.sh_rn2.ensure((size_t)S * sizeof(double)));
     RSN_CUDA(c, q.sh_ts.ensure((size_t)nsys * ns * sizeof(double)));
     RSN_CUDA(c, q.sh_sit.ensure((size_t)nsys * ns * sizeof(int)));
@@ -1200,6 +1203,8 @@ static rsn_status run_stream(rsn_ctx* c, const rsn_solver_opts* o, const StreamI
     b.sconv_it = q.sh_cit.as<int>();
     b.salpha = q.sh_alpha.as<double2>();
     b.sbeta = q.sh_beta.as<double2>();
+    b.stamp = q.sh_stamp.as<int>();
+    b.iter_no = q.sh_stamp.as<int>() + S;
     b.rn2 = q.sh_rn2.as<double>();
     b.out_ts = q.sh_ts.as<double>();
     b.out_sit = q.sh_sit.as<int>();
@@ -1249,9 +1254,9 @@ static rsn_status run_stream(rsn_ctx* c, const rsn_solver_opts* o, const StreamI
   // ACTIVE slots (projections of r, operator, update); all touch disjoint slots.
   // The scheduler then joins them: finished systems leave, checked systems
   // resume, free slots take queued systems and the next list is made.
-  // Shifted systems keep one stream: their per-iteration shift step must see
-  // exactly the slots that did a COCG iteration, so the scheduler runs first.
-  cudaStream_t st2 = sh ? st : c->st2;
+  // Shifted systems: the shifted update follows the COCG update of the slots that
+  // did an iteration (stamps).
+  cudaStream_t st2 = c->st2;
   auto body = [&](int iters, bool capturing, int bucket) -> cudaError_t {
     // inside stream capture an event record must be an external node to be timeable
     const unsigned evf = capturing ? cudaEventRecordExternal : cudaEventRecordDefault;
@@ -1260,8 +1265,8 @@ static rsn_status run_stream(rsn_ctx* c, const rsn_solver_opts* o, const StreamI
       return e;
     auto residual_path = [&]() -> cudaError_t {
       cudaError_t e2;
-      if (sh && (e2 = launch_list(st2, bdev)) != cudaSuccess) return e2;
-      if (!sh && (e2 = launch_emit(S, st2, jr, bdev)) != cudaSuccess) return e2;
+      if ((e2 = launch_emit(S, st2, jr, bdev)) != cudaSuccess) return e2;
+      if (sh && (e2 = launch_shift_emit(S, ns, st2, jr, bdev)) != cudaSuccess) return e2;
       if ((e2 = launch_zero(fp32, KV, nB, st2, jr, bdev)) != cudaSuccess) return e2;
       if (sh && (e2 = launch_shift_init(sh->nT, st2, jr, bdev)) != cudaSuccess) return e2;
       if (proj && (e2 = launch_project(1, fp32, KL, n_groups, max_np, st2, jr, bdev, nullptr, w.c_x.p, multi)) !=
@@ -1274,23 +1279,11 @@ static rsn_status run_stream(rsn_ctx* c, const rsn_solver_opts* o, const StreamI
       if (goal && (e2 = launch_tgoal(KV, st2, jr, bdev)) != cudaSuccess) return e2;
       return cudaSuccess;
     };
-    auto schedule = [&](int it) -> cudaError_t {
-      cudaError_t e2;
-      if ((e2 = launch_sched(it, !sh, st, jr, bdev)) != cudaSuccess) return e2;
-      if (sh && (e2 = launch_emit(S, st, jr, bdev)) != cudaSuccess) return e2;
-      if (sh && (e2 = launch_shift_emit(S, ns, st, jr, bdev)) != cudaSuccess) return e2;
-      return cudaSuccess;
-    };
     for (int it = 0; it < iters; ++it) {
-      if (sh) {
-        if ((e = residual_path()) != cudaSuccess) return e;
-        if ((e = schedule(it)) != cudaSuccess) return e;
-      } else {
-        if ((e = cudaEventRecord(c->ev_fork, st)) != cudaSuccess) return e;
-        if ((e = cudaStreamWaitEvent(st2, c->ev_fork, 0)) != cudaSuccess) return e;
-        if ((e = residual_path()) != cudaSuccess) return e;
-        if ((e = cudaEventRecord(c->ev_join, st2)) != cudaSuccess) return e;
-      }
+      if ((e = cudaEventRecord(c->ev_fork, st)) != cudaSuccess) return e;
+      if ((e = cudaStreamWaitEvent(st2, c->ev_fork, 0)) != cudaSuccess) return e;
+      if ((e = residual_path()) != cudaSuccess) return e;
+      if ((e = cudaEventRecord(c->ev_join, st2)) != cudaSuccess) return e;
       // COCG step of the ACTIVE slots (main stream).  The operator and the
       // projections of r need nothing of one another: they run side by side
       // (one after the other when the launches are timed)
@@ -1319,15 +1312,13 @@ static rsn_status run_stream(rsn_ctx* c, const rsn_solver_opts* o, const StreamI
       if ((e = launch_cocg_update(fp32, S, pool ? pool->N : c->N, proj, b.ce_stride, it, st, ji, bdev)) != cudaSuccess) return e;
       if (timing && (e = cudaEventRecordWithFlags(c->tev[4 * it + 2], st, evf)) != cudaSuccess) return e;
       if (sh && (e = launch_shift_update(S, sh->nT, ns, st, ji, bdev)) != cudaSuccess) return e;
-      if (!sh) {
-        // join: the scheduler sees both paths of this iteration
-        if ((e = cudaStreamWaitEvent(st, c->ev_join, 0)) != cudaSuccess) return e;
-        if ((e = schedule(it)) != cudaSuccess) return e;
-      }
+      // join: the scheduler sees both paths of this iteration
+      if ((e = cudaStreamWaitEvent(st, c->ev_join, 0)) != cudaSuccess) return e;
+      if ((e = launch_sched(it, st, jr, bdev)) != cudaSuccess) return e;
     }
     return cudaSuccess;
   };
-  const int per_iter = (proj ? 9 : 7) + (sh ? 4 : 0) + (goal ? 1 : 0);
+  const int per_iter = (proj ? 9 : 7) + (sh ? 3 : 0) + (goal ? 1 : 0);
   const double vbytes = (double)(pool ? pool->N : c->N) * (fp32 ? sizeof(float2) : sizeof(double2));
   // The z chunks of the COCG operator follow the number of busy slots in three
   // steps (all, a quarter, a sixteenth of the pool): a few systems left over from a
@@ -1434,7 +1425,10 @@ static rsn_status run_stream(rsn_ctx* c, const rsn_solver_opts* o, const StreamI
   if (!finished && !timeout && !aborted) RSN_FAIL(c, RSN_ECUDA, "streaming solver exceeded its iteration bound");
   // a pass that stops early leaves the systems of its last scheduler call drained
   // but not yet emitted
-  if (!finished && !sh) RSN_CUDA(c, launch_emit(S, st, jr, bdev));
+  if (!finished) {
+    RSN_CUDA(c, launch_emit(S, st, jr, bdev));
+    if (sh) RSN_CUDA(c, launch_shift_emit(S, ns, st, jr, bdev));
+  }
   out.iters.resize(nsys);
   out.status.resize(nsys);
   out.relres.resize(nsys);

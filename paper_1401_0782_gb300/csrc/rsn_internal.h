@@ -214,6 +214,8 @@ struct BatchDev {
   int* sconv_it;             // [slot][n_shift] iteration at which shift e converged (INT_MAX: not yet)
   double2* salpha;           // [2][slot] alpha_k of the seed recurrence, ring k % 2
   double2* sbeta;            // [2][slot] beta_k, ring k % 2
+  int* stamp;                // [slot] solver iteration (*iter_no) of the slot's last COCG iteration
+  int* iter_no;              // solver iterations so far (scheduler)
   double* rn2;               // [slot] ||r_{k+1}||^2 of the seed (bookkeeping kernel)
   double* out_ts;            // [n_shift][system] T partial sum_{i in L} Gamma_L |x_e(i)|^2
   int* out_sit;              // [n_shift][system] seed iterations at convergence (-1: not converged)
@@ -341,7 +343,7 @@ cudaError_t launch_project(int mode, bool fp32, int nslots, int n_groups, int ma
 // y += the projector term -sum_p v_p e_kb[p] c[p] of n_rhs vectors, c [n_rhs][n_proj]
 cudaError_t launch_nonlocal(bool fp32, int n_rhs, long long N, int n_proj, cudaStream_t st, const JuncDev* jt,
                             const BatchDev* b, const void* c, void* y);
-cudaError_t launch_sched(int slot_it, bool make_list, cudaStream_t st, const JuncDev* jt, const BatchDev* b);
+cudaError_t launch_sched(int slot_it, cudaStream_t st, const JuncDev* jt, const BatchDev* b);
 cudaError_t launch_x_update(bool fp32, int nslots, int nB, cudaStream_t st, const JuncDev* jt,
                             const BatchDev* b);
 cudaError_t launch_emit(int nslots, cudaStream_t st, const JuncDev* jt, const BatchDev* b);

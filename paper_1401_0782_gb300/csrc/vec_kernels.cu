@@ -25,8 +25,7 @@ namespace rsn {
 // ---------------------------------------------------------------------------
 // List of the slots that need a true residual in the next iteration (NEW and
 // CHECK), in slot order: one CTA, ballot + warp-count prefix per 1024 slots.
-// Built at the end of the scheduler; shifted systems, whose scheduler runs before
-// the COCG step, take a kernel of its own at the start of the iteration.
+// Built at the end of the scheduler (a kernel of its own for the micro-benchmark).
 // ---------------------------------------------------------------------------
 __device__ __forceinline__ void build_list(const BatchDev& b, int* warp_cnt) {
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
@@ -123,7 +122,10 @@ __device__ __forceinline__ void book_slot(const BatchDev& b, const int s, const 
   b.cyc_iters[s] = cyc;
   atomicAdd(b.counters, 1ull);
   atomicAdd(b.sched + 3 + kMaxGraphIters + slot_it, 1);
-  if (b.n_shift > 0) b.rn2[s] = nrm;
+  if (b.n_shift > 0) {
+    b.rn2[s] = nrm;
+    b.stamp[s] = *b.iter_no;  // the shifted update of this iteration takes the slot
+  }
   b.beta_cur[s] = beta;
   b.rho_cur[s] = rho;
   // A near-breakdown (mu or rho almost zero) costs an FP64 recurrence its
@@ -608,13 +610,13 @@ __global__ void __launch_bounds__(kUpdThreads) nonlocal_kernel(const JuncDev* __
 // assigns queued systems to free slots in slot order.
 // ---------------------------------------------------------------------------
 __global__ void __launch_bounds__(kSchedThreads) sched_kernel(const JuncDev* __restrict__ jt,
-                                                             const BatchDev* __restrict__ bp, int slot_it,
-                                                             int make_list) {
+                                                             const BatchDev* __restrict__ bp, int slot_it) {
   const BatchDev& b = *bp;
   const int S = b.nslots;
   __shared__ int warp_cnt[32];
   int upd = 0, busy = 0;
-  if (make_list) {
+  if (b.n_shift > 0 && threadIdx.x == 0) *b.iter_no += 1;
+  {
     // most iterations change no slot: nothing drained, listed, due for a list or
     // waiting for a slot; the list stays empty and the busy count what it was
     const bool queued = b.sched[0] < b.nsys;
@@ -851,7 +853,7 @@ __global__ void __launch_bounds__(kSchedThreads) sched_kernel(const JuncDev* __r
     if (found) break;
   }
   for (int s = threadIdx.x; s < S; s += blockDim.x) busy += (b.state[s] != SL_FREE) ? 1 : 0;
-  if (make_list) build_list(b, warp_cnt);
+  build_list(b, warp_cnt);
   busy = __reduce_add_sync(0xffffffffu, busy);
   upd = __reduce_add_sync(0xffffffffu, upd);
   if (threadIdx.x == 0) s_nf = s_done = 0;  // reused: the CTA's totals
@@ -1049,16 +1051,16 @@ __global__ void __launch_bounds__(kVecThreads) shift_init_kernel(const JuncDev* 
   }
 }
 
-// One shifted step after iteration k of the seed (ACTIVE slots, and slots the
-// bookkeeping kernel just moved to CHECK).  Every CTA of a slot derives the
+// One shifted step after iteration k of the seed (the slots that did it: ACTIVE
+// ones, and those whose bookkeeping just moved them to CHECK).  CTA rows z take
+// the shifts z * 8 .. + 7.  Every CTA of a slot derives the
 // same scalars; CTA 0 records them (pi in a ring of three, so no CTA reads a
 // value that is being overwritten) and ends the cycle once every shift converged.
 __global__ void __launch_bounds__(kVecThreads) shift_update_kernel(const JuncDev* __restrict__ jt,
                                                                    const BatchDev* __restrict__ bp) {
   const BatchDev& b = *bp;
   const int s = blockIdx.y;
-  const int st = b.state[s];
-  if (st != SL_ACTIVE && st != SL_CHECK) return;
+  if (b.stamp[s] != *b.iter_no) return;  // no COCG iteration just now
   const int ns = b.n_shift, nT = b.nT;
   const size_t S = (size_t)b.nslots;
   const int k = b.iters[s] - 1;  // the iteration just completed
@@ -1097,7 +1099,7 @@ __global__ void __launch_bounds__(kVecThreads) shift_update_kernel(const JuncDev
       const double est2 = rn2 / (apn2 * bn2);
       const bool conv = est2 <= b.tol * b.tol;
       if (!isfinite(est2)) sa[e] = sb[e] = make_double2(0.0, 0.0);
-      if (blockIdx.x == 0) {
+      if (blockIdx.x == 0 && blockIdx.z == 0) {
         pi_n[e] = pn;
         const int sy = b.sys[s];
         b.out_srel[(size_t)e * b.nsys + sy] = sqrt(est2);
@@ -1111,7 +1113,7 @@ __global__ void __launch_bounds__(kVecThreads) shift_update_kernel(const JuncDev
     }
   }
   __syncthreads();
-  if (blockIdx.x == 0 && threadIdx.x == 0) {
+  if (blockIdx.x == 0 && blockIdx.z == 0 && threadIdx.x == 0) {
     b.sbeta[(size_t)(k & 1) * S + s] = be;
     if (s_left == 0) b.state[s] = SL_CHECK;  // every shift converged: end of the seed's cycle
   }
@@ -1120,14 +1122,14 @@ __global__ void __launch_bounds__(kVecThreads) shift_update_kernel(const JuncDev
   const double2* rv = reinterpret_cast<const double2*>(b.r) + b.voff[s];
   for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < nT; i += gridDim.x * blockDim.x) {
     const double2 r = rv[b.T_idx[i]];
-    for (int e0 = 0; e0 < ns; e0 += 4) {
+    for (int e0 = 8 * blockIdx.z; e0 < min(ns, 8 * ((int)blockIdx.z + 1)); e0 += 4) {
       double2 g[4], x[4];
       bool on[4];
 #pragma unroll
       for (int u = 0; u < 4; ++u) {
         const int e = e0 + u;
         on[u] = false;
-        if (e < ns) {  // frozen shifts are skipped (uniform across the CTA)
+        if (e < ns) {  // (e0 + 4 <= 8 (z + 1)) frozen shifts are skipped (uniform across the CTA)
           const double2 a = sa[e], c = sb[e];
           on[u] = a.x != 0.0 || a.y != 0.0 || c.x != 0.0 || c.y != 0.0;
         }
@@ -1373,8 +1375,8 @@ cudaError_t launch_nonlocal(bool fp32, int n_rhs, long long N, int n_proj, cudaS
   return cudaGetLastError();
 }
 
-cudaError_t launch_sched(int slot_it, bool make_list, cudaStream_t st, const JuncDev* jt, const BatchDev* b) {
-  sched_kernel<<<1, kSchedThreads, 0, st>>>(jt, b, slot_it, make_list ? 1 : 0);
+cudaError_t launch_sched(int slot_it, cudaStream_t st, const JuncDev* jt, const BatchDev* b) {
+  sched_kernel<<<1, kSchedThreads, 0, st>>>(jt, b, slot_it);
   return cudaGetLastError();
 }
 
@@ -1394,7 +1396,7 @@ cudaError_t launch_shift_init(int nT, cudaStream_t st, const JuncDev* jt, const 
 cudaError_t launch_shift_update(int nslots, int nT, int n_shift, cudaStream_t st, const JuncDev* jt,
                                 const BatchDev* b) {
   const int bx = std::max(1, (nT + kVecThreads - 1) / kVecThreads);
-  shift_update_kernel<<<dim3(bx, nslots), kVecThreads, 2 * n_shift * sizeof(double2), st>>>(jt, b);
+  shift_update_kernel<<<dim3(bx, nslots, (n_shift + 7) / 8), kVecThreads, 2 * n_shift * sizeof(double2), st>>>(jt, b);
   return cudaGetLastError();
 }
 
