@@ -164,7 +164,7 @@ struct rsn_ctx {
   bool dirty() const { return dirty_v || dirty_cap || dirty_proj; }
 
   // device operator data
-  DevBuf dg64, dg32, gld, L_idx, L_gam, inv_ptr, inv_p0, inv_q64, blk_row, row_ent, row_q64, row_q32;
+  DevBuf dg64, dg32, gld, L_idx, L_gam, inv_ptr, inv_p0, inv_q64, blk_row, row_ent, row_src, row_q64, row_q32;
   DevBuf grp_ptr, grp_p0, grp_np, grp_voff, grp_idx, grp_val64, grp_val32, ekb;
   int n_groups = 0, nL = 0, max_np = 1;
   JuncDev jh{};
@@ -460,35 +460,32 @@ static rsn_status commit_projectors(rsn_ctx* c) {
   std::vector<float> gvalf(gval.begin(), gval.end());
   // the same entries by blocks of kBlkPts points, for the update kernel: rows of up
   // to 32 entries; layer k of a block holds the k-th entry of each of its points
-  // that has one, so that a row holds each point once
+  // that has one, so that a row holds each point once.  The host lists the entries
+  // (rsrc); the value tables are gathered from the per-point ones on the device.
   const int nblk = (int)((N + kBlkPts - 1) / kBlkPts);
-  std::vector<int> brow(nblk + 1, 0), rent;
-  std::vector<double> rq64;
+  std::vector<int> brow(nblk + 1, 0), rent, rsrc;
+  rent.reserve(nent + nent / 2 + 32);
+  rsrc.reserve(nent + nent / 2 + 32);
   for (int k = 0; k < nblk; ++k) {
     brow[k] = (int)(rent.size() / 32);
-    const long long i0 = (long long)k * kBlkPts, i1 = std::min<long long>(i0 + kBlkPts, N);
+    const int i0 = k * kBlkPts, i1 = (int)std::min<long long>((long long)i0 + kBlkPts, N);
     if (cnt[i1] == cnt[i0]) continue;
-    for (int layer = 0, more = 1; more; ++layer) {
-      more = 0;
-      int lane = 32;
-      for (long long i = i0; i < i1; ++i) {
-        const int e = cnt[i] + layer;
-        if (e >= cnt[i + 1]) continue;
-        more = 1;
-        if (lane == 32) {
-          rent.resize(rent.size() + 32, -1);
-          rq64.resize(rq64.size() + (size_t)32 * 4 * nq, 0.0);
-          lane = 0;
-        }
-        const size_t row = rent.size() / 32 - 1;
-        rent[row * 32 + lane] = ip0[e] * kBlkPts + (int)(i - i0);
-        for (int j = 0; j < 4 * nq; ++j) rq64[((row * nq + j / 4) * 32 + lane) * 4 + j % 4] = iq64[(size_t)e * 4 * nq + j];
-        ++lane;
+    int act[kBlkPts], n = 0;  // points with an entry in the current layer
+    for (int i = i0; i < i1; ++i)
+      if (cnt[i + 1] > cnt[i]) act[n++] = i;
+    for (int layer = 0; n > 0; ++layer) {
+      int m = 0;
+      for (int u = 0; u < n; ++u) {
+        const int i = act[u], e = cnt[i] + layer;
+        rent.push_back(ip0[e] * kBlkPts + (i - i0));
+        rsrc.push_back(e);
+        if (e + 1 < cnt[i + 1]) act[m++] = i;
       }
+      while (rent.size() % 32) rent.push_back(-1), rsrc.push_back(-1);
+      n = m;
     }
   }
   brow[nblk] = (int)(rent.size() / 32);
-  std::vector<float> rq32(rq64.begin(), rq64.end());
   auto up = [&](DevBuf& b, const void* src, size_t bytes) -> cudaError_t {
     cudaError_t e = b.ensure(std::max<size_t>(bytes, 16));
     if (e != cudaSuccess) return e;
@@ -499,8 +496,9 @@ static rsn_status commit_projectors(rsn_ctx* c) {
   RSN_CUDA(c, up(c->inv_p0, ip0.data(), nent * sizeof(int)));
   RSN_CUDA(c, up(c->blk_row, brow.data(), brow.size() * sizeof(int)));
   RSN_CUDA(c, up(c->row_ent, rent.data(), rent.size() * sizeof(int)));
-  RSN_CUDA(c, up(c->row_q64, rq64.data(), rq64.size() * sizeof(double)));
-  RSN_CUDA(c, up(c->row_q32, rq32.data(), rq32.size() * sizeof(float)));
+  RSN_CUDA(c, up(c->row_src, rsrc.data(), rsrc.size() * sizeof(int)));
+  RSN_CUDA(c, c->row_q64.ensure(std::max<size_t>(16, rsrc.size() * 4 * nq * sizeof(double))));
+  RSN_CUDA(c, c->row_q32.ensure(std::max<size_t>(16, rsrc.size() * 4 * nq * sizeof(float))));
   RSN_CUDA(c, up(c->inv_q64, iq64.data(), nent * 4 * nq * sizeof(double)));
   RSN_CUDA(c, up(c->grp_ptr, gptr.data(), gptr.size() * sizeof(int)));
   RSN_CUDA(c, up(c->grp_p0, gp0.data(), gp0.size() * sizeof(int)));
@@ -510,6 +508,8 @@ static rsn_status commit_projectors(rsn_ctx* c) {
   RSN_CUDA(c, up(c->grp_val64, gval.data(), gval.size() * sizeof(double)));
   RSN_CUDA(c, up(c->grp_val32, gvalf.data(), gvalf.size() * sizeof(float)));
   RSN_CUDA(c, up(c->ekb, c->pekb.data(), c->pekb.size() * sizeof(double)));
+  RSN_CUDA(c, launch_row_values((long long)rsrc.size(), nq, c->st, c->row_src.as<int>(), c->inv_q64.as<double>(),
+                                c->row_q64.as<double>(), c->row_q32.as<float>()));
   return RSN_OK;
 }
 

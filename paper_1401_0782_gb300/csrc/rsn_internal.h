@@ -347,6 +347,10 @@ cudaError_t launch_sched(int slot_it, cudaStream_t st, const JuncDev* jt, const 
 cudaError_t launch_x_update(bool fp32, int nslots, int nB, cudaStream_t st, const JuncDev* jt,
                             const BatchDev* b);
 cudaError_t launch_emit(int nslots, cudaStream_t st, const JuncDev* jt, const BatchDev* b);
+// row tables: the value quads of n entries (src: per-point entry, -1: none) from the
+// per-point ones, FP64 and FP32
+cudaError_t launch_row_values(long long n, int nq, cudaStream_t st, const int* src, const double* inv_q64, double* q64,
+                              float* q32);
 cudaError_t launch_list(cudaStream_t st, const BatchDev* b);
 cudaError_t launch_landauer(int n_e, const double* E, const double* T, int n_v, const double* V, double E_F,
                             double kT, double* I, cudaStream_t st);

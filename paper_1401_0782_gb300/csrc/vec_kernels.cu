@@ -1202,6 +1202,20 @@ __global__ void __launch_bounds__(256) landauer_kernel(int n_e, const double* __
   if (threadIdx.x == 0) I[blockIdx.x] = out[0] / 3.14159265358979323846;
 }
 
+// Value quads of the row tables, [row][quad][lane], gathered from the per-point
+// entries (setup).
+__global__ void row_values_kernel(long long n, int nq, const int* __restrict__ src, const double* __restrict__ inv_q64,
+                                  double* __restrict__ q64, float* __restrict__ q32) {
+  const long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+  if (t >= n * 4 * nq) return;
+  const long long i = t / (4 * nq);  // entry: row * 32 + lane
+  const int j = (int)(t - i * 4 * nq), e = src[i];
+  const double v = e >= 0 ? inv_q64[(size_t)e * 4 * nq + j] : 0.0;
+  const long long at = (((i / 32) * nq + j / 4) * 32 + i % 32) * 4 + j % 4;
+  q64[at] = v;
+  q32[at] = (float)v;
+}
+
 // ---------------------------------------------------------------------------
 // launchers
 // ---------------------------------------------------------------------------
@@ -1413,6 +1427,13 @@ cudaError_t launch_tgoal(int rows, cudaStream_t st, const JuncDev* jt, const Bat
 cudaError_t launch_landauer(int n_e, const double* E, const double* T, int n_v, const double* V, double E_F,
                             double kT, double* I, cudaStream_t st) {
   landauer_kernel<<<n_v, 256, 0, st>>>(n_e, E, T, V, E_F, kT, I);
+  return cudaGetLastError();
+}
+
+cudaError_t launch_row_values(long long n, int nq, cudaStream_t st, const int* src, const double* inv_q64, double* q64,
+                              float* q32) {
+  if (n > 0)
+    row_values_kernel<<<(unsigned)((n * 4 * nq + 255) / 256), 256, 0, st>>>(n, nq, src, inv_q64, q64, q32);
   return cudaGetLastError();
 }
 
