@@ -76,6 +76,7 @@ __device__ __forceinline__ void mu_alpha(const BatchDev& b, const JuncDev& J, co
   if (lane == 0) {
     b.mu_cnt[s] = 0;
     b.alpha[s] = a;
+    b.alpha32[s] = make_float2((float)a.x, (float)a.y);
     if (b.n_shift > 0) b.salpha[(size_t)(b.iters[s] & 1) * b.nslots + s] = a;
   }
 }

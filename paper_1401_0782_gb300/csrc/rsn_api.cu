@@ -80,7 +80,7 @@ struct Workspace {
   DevBuf Xslot, r, p0, p1, q, d;
   DevBuf state, sys, junc, E, col, voff, xo, xfo, iters, total_iters, cyc_iters, n_upd, restart, stall, warm, rho_cur, beta_cur;
   DevBuf bnorm2, sigma, rlast2, rrec2, rmin2, rmin_it, tol2;
-  DevBuf res_part, res_cnt, res_tot, tlast, gcnt, gphase, tgoal, rgoal, rho, nrm, mu, mu_cnt, alpha, nact, upd_cnt, c_r, c_p, c_x, sched, counters, lst, lst_n,
+  DevBuf res_part, res_cnt, res_tot, tlast, gcnt, gphase, tgoal, rgoal, rho, nrm, mu, mu_cnt, alpha, alpha32, nact, upd_cnt, c_r, c_p, c_x, sched, counters, lst, lst_n,
       inlist, fslot, c_e;
   int generation = 0;
 };
@@ -145,8 +145,9 @@ struct rsn_ctx {
   cudaStream_t st = nullptr;
   cudaStream_t st2 = nullptr;  // second stream: the true-residual path beside the COCG step
   cudaStream_t st3 = nullptr;  // third stream: the projections of r beside the COCG operator
+  cudaStream_t st4 = nullptr;  // fourth stream: a pool's further operator kinds beside the first
   cudaEvent_t ev_in = nullptr, ev_out = nullptr, t0 = nullptr, t1 = nullptr, ev_fork = nullptr, ev_join = nullptr, ev_step = nullptr,
-              ev_proj = nullptr;
+              ev_proj = nullptr, ev_kind = nullptr;
   std::string err;
 
   bool has_grid = false, has_v = false, has_cap = false;
@@ -692,6 +693,8 @@ rsn_status rsn_create(rsn_ctx** out, int device, void* cuda_stream) {
   if (cudaStreamCreateWithFlags(&c->st, cudaStreamNonBlocking) != cudaSuccess ||
       cudaStreamCreateWithFlags(&c->st2, cudaStreamNonBlocking) != cudaSuccess ||
       cudaStreamCreateWithFlags(&c->st3, cudaStreamNonBlocking) != cudaSuccess ||
+      cudaStreamCreateWithFlags(&c->st4, cudaStreamNonBlocking) != cudaSuccess ||
+      cudaEventCreateWithFlags(&c->ev_kind, cudaEventDisableTiming) != cudaSuccess ||
       cudaEventCreateWithFlags(&c->ev_step, cudaEventDisableTiming) != cudaSuccess ||
       cudaEventCreateWithFlags(&c->ev_proj, cudaEventDisableTiming) != cudaSuccess ||
       cudaEventCreateWithFlags(&c->ev_fork, cudaEventDisableTiming) != cudaSuccess ||
@@ -716,6 +719,7 @@ rsn_status rsn_destroy(rsn_ctx* c) {
   if (c->st) cudaStreamSynchronize(c->st);
   if (c->st2) cudaStreamSynchronize(c->st2);
   if (c->st3) cudaStreamSynchronize(c->st3);
+  if (c->st4) cudaStreamSynchronize(c->st4);
   clear_graphs(c);
   for (cudaEvent_t e : c->tev) cudaEventDestroy(e);
   if (c->sched_host) cudaFreeHost(c->sched_host);
@@ -728,6 +732,8 @@ rsn_status rsn_destroy(rsn_ctx* c) {
   if (c->ev_join) cudaEventDestroy(c->ev_join);
   if (c->ev_step) cudaEventDestroy(c->ev_step);
   if (c->ev_proj) cudaEventDestroy(c->ev_proj);
+  if (c->ev_kind) cudaEventDestroy(c->ev_kind);
+  if (c->st4) cudaStreamDestroy(c->st4);
   if (c->st3) cudaStreamDestroy(c->st3);
   if (c->st2) cudaStreamDestroy(c->st2);
   if (c->st) cudaStreamDestroy(c->st);
@@ -945,6 +951,7 @@ static rsn_status ensure_ws(rsn_ctx* c, bool fp32, int S, const PoolSpec* pool =
   RSN_CUDA(c, w.mu.ensure((size_t)S * PA * sizeof(double2)));
   RSN_CUDA(c, w.mu_cnt.ensure(si));
   RSN_CUDA(c, w.alpha.ensure(S * sizeof(double2)));
+  RSN_CUDA(c, w.alpha32.ensure(S * sizeof(float2)));
   RSN_CUDA(c, w.upd_cnt.ensure(si));
   RSN_CUDA(c, w.nact.ensure(sizeof(int)));
   RSN_CUDA(c, w.rho.ensure((size_t)S * PB * sizeof(double2)));
@@ -1079,6 +1086,7 @@ static BatchDev slot_batch(rsn_ctx* c, int S, const rsn_solver_opts* o) {
   b.mu_part = w.mu.as<double2>();
   b.mu_cnt = w.mu_cnt.as<int>();
   b.alpha = w.alpha.as<double2>();
+  b.alpha32 = w.alpha32.as<float2>();
   b.upd_cnt = w.upd_cnt.as<int>();
   b.nact = w.nact.as<int>();
   b.c_r = w.c_r.p;
@@ -1287,22 +1295,34 @@ static rsn_status run_stream(rsn_ctx* c, const rsn_solver_opts* o, const StreamI
       // COCG step of the ACTIVE slots (main stream).  The operator and the
       // projections of r need nothing of one another: they run side by side
       // (one after the other when the launches are timed)
+      int kinds = 0;
+      if (pool)
+        for (int kd = 0; kd < 4; ++kd) kinds += pool->has[kd] ? 1 : 0;
+      if (!timing && (proj || kinds > 1) && (e = cudaEventRecord(c->ev_step, st)) != cudaSuccess) return e;
       if (proj) {
         cudaStream_t sp = timing ? st : c->st3;
-        if (!timing) {
-          if ((e = cudaEventRecord(c->ev_step, st)) != cudaSuccess) return e;
-          if ((e = cudaStreamWaitEvent(sp, c->ev_step, 0)) != cudaSuccess) return e;
-        }
+        if (!timing && (e = cudaStreamWaitEvent(sp, c->ev_step, 0)) != cudaSuccess) return e;
         if ((e = launch_project(0, fp32, S, n_groups, max_np, sp, ji, bdev, nullptr, w.c_r.p, multi)) != cudaSuccess)
           return e;
         if (!timing && (e = cudaEventRecord(c->ev_proj, sp)) != cudaSuccess) return e;
       }
       if (timing && (e = cudaEventRecordWithFlags(c->tev[4 * it], st, evf)) != cudaSuccess) return e;
       if (pool) {
-        for (int kd = 0; kd < 4; ++kd)
-          if (pool->has[kd] && (e = launch_inner(c, pool->inner[kd], OP_COCG, fp32, S, st, ji, bdev, nullptr, nullptr,
-                                                 pool->inner[kd].n_act[bucket])) != cudaSuccess)
+        // the junctions' operator kinds touch different slots and run side by side
+        bool first = true;
+        for (int kd = 0; kd < 4; ++kd) {
+          if (!pool->has[kd]) continue;
+          cudaStream_t so = first || timing ? st : c->st4;
+          if (so != st && (e = cudaStreamWaitEvent(so, c->ev_step, 0)) != cudaSuccess) return e;
+          if ((e = launch_inner(c, pool->inner[kd], OP_COCG, fp32, S, so, ji, bdev, nullptr, nullptr,
+                                pool->inner[kd].n_act[bucket])) != cudaSuccess)
             return e;
+          first = false;
+        }
+        if (kinds > 1 && !timing) {
+          if ((e = cudaEventRecord(c->ev_kind, c->st4)) != cudaSuccess) return e;
+          if ((e = cudaStreamWaitEvent(st, c->ev_kind, 0)) != cudaSuccess) return e;
+        }
       } else if ((e = launch_inner(c, cfg.inner, OP_COCG, fp32, S, st, ji, bdev, nullptr, nullptr,
                                    cfg.inner.n_act[bucket])) != cudaSuccess) {
         return e;
@@ -2815,6 +2835,7 @@ static rsn_status bench_kernel_impl(rsn_ctx* c, int precision, int kind, int S, 
   RSN_CUDA(c, cudaMemsetAsync(w.nrm.p, 0x3f, (size_t)S * w.PB * sizeof(double), st));
   RSN_CUDA(c, cudaMemsetAsync(w.mu.p, 0x3f, (size_t)S * w.PA * sizeof(double2), st));
   RSN_CUDA(c, cudaMemsetAsync(w.alpha.p, 0x3f, S * sizeof(double2), st));
+  RSN_CUDA(c, cudaMemsetAsync(w.alpha32.p, 0x3c, S * sizeof(float2), st));
   for (DevBuf* v : {&w.mu_cnt, &w.upd_cnt, &w.res_cnt, &w.total_iters, &w.cyc_iters, &w.rmin_it, &w.gphase})
     RSN_CUDA(c, cudaMemsetAsync(v->p, 0, S * sizeof(int), st));
   RSN_CUDA(c, cudaMemsetAsync(w.tol2.p, 0, S * sizeof(double), st));

@@ -168,6 +168,7 @@ struct BatchDev {
   double2* mu_part;     // [S][PA] p^T A p: operator kernel ([ytiles][ceil(nz / kMuPlanes)]), then one per atom (projections)
   int* mu_cnt;          // [S] operator and projection CTAs of the iteration that have written their partial
   double2* alpha;       // [S] alpha_k = rho_k / mu_k, formed by the last of them
+  float2* alpha32;      // [S] the same in FP32
   const int* nact;      // slots that may do a COCG iteration: picks the operator's z chunks (set with the launches)
   int* upd_cnt;         // [S] update CTAs of the iteration that have written their partials
   int pstride;          // per-slot stride of the projection arrays (the largest n_proj of the junctions)

@@ -273,8 +273,10 @@ cocg_update_kernel(const JuncDev* __restrict__ jt, const BatchDev* __restrict__ 
   const int i0 = min(blk * kBlkPts, N), i1 = min(i0 + kBlkPts, N);
   const long long vo = b.voff[s];
   const int k = b.iters[s];
-  const double2 a64 = b.alpha[s];
-  const bool fin = isfinite(a64.x) && isfinite(a64.y);
+  C al;  // (FP32: rounded once by mu_alpha, which keeps conversions off the FP64 pipe here)
+  if constexpr (sizeof(T) == 4) al = b.alpha32[s];
+  else al = b.alpha[s];
+  const bool fin = isfinite(al.x) && isfinite(al.y);
   extern __shared__ __align__(16) unsigned char upd_smem[];
   C* s_ce = reinterpret_cast<C*>(upd_smem);         // e_kb c_p of the new direction, ce_stride entries
   C* s_nl = s_ce + b.ce_stride + warp * kBlkPts;    // projector term of the warp's block
@@ -286,7 +288,7 @@ cocg_update_kernel(const JuncDev* __restrict__ jt, const BatchDev* __restrict__ 
     const C* qv = reinterpret_cast<const C*>(b.q) + vo;
     C* rv = reinterpret_cast<C*>(b.r) + vo;
     C* dv = reinterpret_cast<C*>(b.d) + vo;
-    const T ax = (T)a64.x, ay = (T)a64.y;
+    const T ax = al.x, ay = al.y;
     // FP32: 16-byte pairs where the slot starts on a pair and holds whole
     // pairs; else (and in FP64, 16 bytes a point) one point at a time
     const bool pairs = sizeof(T) == 4 && ((vo | N) & 1) == 0;
@@ -342,10 +344,22 @@ cocg_update_kernel(const JuncDev* __restrict__ jt, const BatchDev* __restrict__ 
     }
   }
   // r^T r = (re, 2 sxy), ||r||^2 = re + 2 sy over the CTA, fixed order
-  T v[3] = {re, sy, sxy};
   double o[3];
-  block_sum<3>(v, red, o);
-  if (warp != 0) return;
+  if constexpr (sizeof(T) == 4) {
+    float v[4] = {re, sy, sxy, 0.f};
+    const float t = warp_sum_many<4>(v);
+    float* part = reinterpret_cast<float*>(red);
+    if (lane < 4) part[warp * 4 + lane] = t;
+    __syncthreads();
+    if (warp != 0) return;
+    const double d = lane < 3 ? sum_strided(part + lane, nw, 4) : 0.0;
+#pragma unroll
+    for (int i = 0; i < 3; ++i) o[i] = __shfl_sync(0xffffffffu, d, i);
+  } else {
+    T v[3] = {re, sy, sxy};
+    block_sum<3>(v, red, o);
+    if (warp != 0) return;
+  }
   if (lane == 0) {
     const size_t at = (size_t)s * b.PB + blockIdx.x;
     b.nrm_part[at] = fin ? fma(2.0, o[1], o[0]) : __longlong_as_double(0x7ff8000000000000ll);
