@@ -115,7 +115,7 @@ __device__ __forceinline__ void op_tile(const JuncDev* __restrict__ jt, const Ba
   C* ce = sm1 + rows * pitch;
   __shared__ double red[MODE == OP_RESID ? 32 * 4 : 1];
   // mu partials (COCG): [block of planes][warp][re, im]
-  __shared__ CT s_mu[MODE == OP_COCG ? kMaxLz / kMuPlanes * (kOpThreads / 32) * 2 : 1];
+  __shared__ __align__(8) CT s_mu[MODE == OP_COCG ? kMaxLz / kMuPlanes * (kOpThreads / 32) * (sizeof(CT) == 8 ? kMuSlots64 : kMuSlots32) : 1];
 
   for (int i = tid; i < 2 * rows * pitch; i += nt) sm0[i] = czero<C>();
 
@@ -217,7 +217,8 @@ __device__ __forceinline__ void op_tile(const JuncDev* __restrict__ jt, const Ba
     else wst[m] = (CT)J.w32[m];
   }
 
-  CT acc0 = 0, acc1 = 0, acc2 = 0;  // COCG: mu(re,im) of kMuPlanes planes; RESID: nrm, rho(re,im)
+  typename std::conditional<sizeof(CT) == 8, MuSum64, MuSum32>::type mu;  // COCG: of kMuPlanes planes
+  CT acc0 = 0, acc1 = 0, acc2 = 0;  // RESID: nrm, rho(re,im)
   double acc3 = 0.0;                // RESID: sum Gamma_L |v|^2 of the iterate (T partial)
   // per-point operator data of the next plane to compute, loaded one plane early
   float2 dgf_n[PPT];
@@ -307,11 +308,15 @@ __device__ __forceinline__ void op_tile(const JuncDev* __restrict__ jt, const Ba
       if constexpr (MODE == OP_COCG) {
         pnew[vo + gl] = vc;
         reinterpret_cast<CO*>(b.q)[vo + gl] = y;
-        // fused (unrounded) products; the sums are over kMuPlanes planes of the thread's
-        // points, so FP64 needs none of the compensation that took 8 of its 12
-        // operations here
-        acc0 = fma(vc.x, y.x, fma(-vc.y, y.y, acc0));
-        acc1 = fma(vc.x, y.y, fma(vc.y, y.x, acc1));
+        // FP64: fused (unrounded) products into sums over kMuPlanes planes of the
+        // thread's points; the compensation of longer sums took 8 of 12 operations of
+        // the pipe that bounds this kernel
+        if constexpr (sizeof(CT) == 8) {
+          mu.re = fma(vc.x, y.x, fma(-vc.y, y.y, mu.re));
+          mu.im = fma(vc.x, y.y, fma(vc.y, y.x, mu.im));
+        } else {
+          mu.add(fma(vc.x, y.x, -vc.y * y.y), fma(vc.x, y.y, vc.y * y.x));
+        }
       } else if constexpr (MODE == OP_RESID) {
         double2 bb = make_double2(0.0, 0.0);
         const int col = b.col[s];
@@ -340,8 +345,7 @@ __device__ __forceinline__ void op_tile(const JuncDev* __restrict__ jt, const Ba
     }
     if constexpr (MODE == OP_COCG) {
       if ((zc - z0) % kMuPlanes == kMuPlanes - 1 || zc == z1 - 1) {
-        mu_flush(s_mu, (zc - z0) / kMuPlanes, acc0, acc1);
-        acc0 = acc1 = 0;
+        mu_flush(s_mu, (zc - z0) / kMuPlanes, mu);
       }
     }
   }
@@ -468,7 +472,7 @@ op_kernel_tma(const JuncDev* __restrict__ jt, const BatchDev* __restrict__ bp, c
   uint64_t* bars = reinterpret_cast<uint64_t*>(
       (reinterpret_cast<uintptr_t>(exch + 2 * prow * pitch) + 15) & ~static_cast<uintptr_t>(15));
   // mu partials (COCG): [block of planes][warp][re, im]
-  __shared__ T s_mu[MODE == OP_COCG ? kMaxLz / kMuPlanes * 32 * 2 : 1];
+  __shared__ __align__(8) T s_mu[MODE == OP_COCG ? kMaxLz / kMuPlanes * 32 * (sizeof(T) == 8 ? kMuSlots64 : kMuSlots32) : 1];
   __shared__ int s_bad;
 
   for (int i = tid; i < 2 * prow * pitch; i += nt) exch[i] = czero<C>();
@@ -522,7 +526,7 @@ op_kernel_tma(const JuncDev* __restrict__ jt, const BatchDev* __restrict__ bp, c
   C qv[Q];
 #pragma unroll
   for (int m = 0; m < Q; ++m) qv[m] = czero<C>();
-  T acc0 = 0, acc1 = 0;  // mu(re, im) of kMuPlanes planes
+  typename std::conditional<sizeof(T) == 8, MuSum64, MuSum32>::type mu;  // of kMuPlanes planes
   // per-point operator data of the next plane to compute, loaded one plane early
   float2 dg_n = make_float2(0.f, 0.f);
   auto load_pt = [&](int z) {
@@ -589,16 +593,19 @@ op_kernel_tma(const JuncDev* __restrict__ jt, const BatchDev* __restrict__ bp, c
     if constexpr (MODE == OP_COCG) {
       pnew[vo + gl] = vc;
       reinterpret_cast<C*>(b.q)[vo + gl] = y;
-      acc0 = fma(vc.x, y.x, fma(-vc.y, y.y, acc0));
-      acc1 = fma(vc.x, y.y, fma(vc.y, y.x, acc1));
+      if constexpr (sizeof(T) == 8) {
+        mu.re = fma(vc.x, y.x, fma(-vc.y, y.y, mu.re));
+        mu.im = fma(vc.x, y.y, fma(vc.y, y.x, mu.im));
+      } else {
+        mu.add(fma(vc.x, y.x, -vc.y * y.y), fma(vc.x, y.y, vc.y * y.x));
+      }
     } else {
       reinterpret_cast<C*>(y_out)[vo + gl] = y;
     }
     }
     if constexpr (MODE == OP_COCG) {
       if ((zc - z0) % kMuPlanes == kMuPlanes - 1 || zc == z1 - 1) {
-        mu_flush(s_mu, (zc - z0) / kMuPlanes, acc0, acc1);
-        acc0 = acc1 = 0;
+        mu_flush(s_mu, (zc - z0) / kMuPlanes, mu);
       }
     }
   }
