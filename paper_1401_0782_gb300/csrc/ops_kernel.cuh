@@ -67,6 +67,9 @@ template <typename T> struct RawIn<T, OP_COCG> { typename cx<T>::t a, b; };
 template <typename T> struct RawIn<T, OP_RESID> { double2 a; typename cx<T>::t b; };
 template <typename T> struct RawIn<T, OP_APPLY> { typename cx<T>::t a; };
 
+// FP64 is bound by the FP64 pipe: 67 operations a point at order 8, 85% of its
+// rate.  24x24x120: 16 systems 155 us (212 with 64 registers, which spilled the
+// queue, and compensated mu sums), 144 systems 1.32 ms (1.53).
 // At most kOpThreads threads per CTA; the minimum resident CTAs per SM bound
 // the registers per thread (FP32: 64 / 85 / 128 for 1 / 2 / 3+ points per thread;
 // FP64 and the true residual: 128, since the FP64 pipe needs few warps to stay

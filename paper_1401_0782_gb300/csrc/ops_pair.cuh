@@ -17,6 +17,9 @@
 //    the x and y neighbours (one barrier per plane), whose row pitch nx + 16 lets
 //    a quarter warp that crosses a row boundary still touch 32 distinct banks;
 //    the zero columns and rows around it are the Dirichlet boundary.
+// 24x24x120, order 8: 256 systems 158 us, 3.6 TB/s of the 32 B a point (235 us with
+// a run-time pitch, whose neighbour addresses spilled, and fixed z chunks); IPC 2.0
+// of 4 at 18 warps an SM, waits on shared memory, fixed latencies and the barrier.
 //
 // FP32 accuracy: the neighbour terms at distances m <= 2, whose weights carry
 // the large part of the Laplacian, are summed in difference form,
