@@ -14,9 +14,8 @@
 //    whose slot for plane z is (z - z0 + R) mod (2R+1); the march is unrolled by
 //    2R+1, so every ring index is a compile-time constant and nothing is shifted.
 //  * The current plane goes through a double-buffered shared-memory tile for
-//    the x and y neighbours (one barrier per plane), whose row pitch nx + 16 lets
-//    a quarter warp that crosses a row boundary still touch 32 distinct banks;
-//    the zero columns and rows around it are the Dirichlet boundary.
+//    the x and y neighbours (one barrier per plane), with a compile-time row pitch
+//    for the common widths (pair_pitch_const); the zero columns and rows around it are the Dirichlet boundary.
 // 24x24x120, order 8: 256 systems 158 us, 3.6 TB/s of the 32 B a point (235 us with
 // a run-time pitch, whose neighbour addresses spilled, and fixed z chunks); IPC 2.0
 // of 4 at 18 warps an SM, waits on shared memory, fixed latencies and the barrier.

@@ -4,7 +4,8 @@
 //   dg64        (N)  complex diagonal without E: (-V_loc + 3 c_0/(2h^2), Gamma_L+Gamma_R)
 //   dg32        (N)  (-V_loc, Gamma_L+Gamma_R) for the FP32 difference-form stencil
 //   gl          (N)  Gamma_L (FP64), used by T and the adjoint right-hand side
-//   inv_*            per-point list of (projector, value) for the matvec epilogue
+//   inv_*            per-point list of (projector, value) for the true residual
+//   row_*            the same by blocks of points, for the update and application
 //   grp_*            per-atom support lists for the projections c_p = v_p . x
 // Krylov vectors (r, p0, p1, q, d) are stored per slot: slot s owns elements
 // [voff[s], voff[s] + N) of each array.  The FP64 iterate of the system held by
@@ -120,7 +121,7 @@ enum SlotState {
 // captured CUDA graphs stay valid when a call changes the buffers it points to.
 struct BatchDev {
   int nslots;
-  int PA, PB;  // partial-sum strides per slot (>= nA / nR and the update kernel's CTAs of every junction)
+  int PA, PB;  // partial-sum strides per slot (mu parts and residual CTAs; update CTAs) of every junction
   // per slot
   int* state;
   int* sys;
