@@ -375,7 +375,8 @@ rsn_status rsn_bench_kernel(rsn_ctx* ctx, int precision, int kind, int nslots, i
                             double* ms_per_launch, double* bytes_per_launch);
 
 /* Autotuner: times the fused operator kernel (rsn_bench_kernel kind 0) for a
-   set of tilings of this grid -- the FP32 plane kernel, the point-pair kernel
+   set of tilings of this grid -- the automatic choice (no override: z-chunks by
+   the number of busy slots), the FP32 plane kernel, the point-pair kernel
    and the whole-plane bulk-copy kernel with several z-chunk lengths, and the
    register-prefetch kernel over rows per tile, points per thread and z-chunks
    -- and keeps on the context the one with the least launch time with all
