@@ -112,7 +112,7 @@ struct ShiftSpec {
 // junction carries its tilings, and each slot works on its system's junction.
 struct PoolSpec {
   int K = 0, R = 0;
-  long long N = 0;  // the largest junction: slot vectors are this long
+  long long N = 0;  // slot vectors are this long (pool_points: the largest junction, rounded up)
   int n_proj = 0, n_groups = 0, max_np = 1, nB = 0, PA = 0, PB = 0;
   Tiling inner[4];                        // launch configuration per operator kind (OpKind)
   bool has[4] = {false, false, false, false};
@@ -2483,6 +2483,17 @@ rsn_status rsn_transmission_vjp_reuse(rsn_ctx* c, int n_e, const double* E, int 
 
 }  // extern "C"
 
+// Points between the slots of a pool over several junctions: those of its largest
+// junction, rounded up to an even number.  In FP32 the bulk copies and 16-byte
+// accesses of the point-pair, plane and bulk-copy kernels need every slot on a
+// 16-byte boundary; each of those kernels only asks that its own junction has an
+// even number of points, and the largest junction may be another one.
+static long long pool_points(rsn_ctx* const* ctxs, int K) {
+  long long n = 0;
+  for (int k = 0; k < K; ++k) n = std::max(n, ctxs[k]->N);
+  return n + (n & 1);
+}
+
 // Slot-pool description of several junctions for one precision: per-junction
 // tilings for `nslots` slots, one launch configuration per operator kind in
 // use (largest thread count, shared memory and tile count of its junctions).
@@ -2493,11 +2504,13 @@ static bool make_pool(rsn_ctx* const* ctxs, int K, bool fp32, int nslots, PoolSp
   pool = PoolSpec();
   pool.K = K;
   pool.R = ctxs[0]->R;
+  pool.N = pool_points(ctxs, K);
+  const bool aligned = pool.N * (long long)(fp32 ? sizeof(float2) : sizeof(double2)) % 16 == 0;
   js.assign(2 * K, JuncDev{});
   int ppt_reg = 0, ppt_res = 0;
   for (int k = 0; k < K; ++k) {
     rsn_ctx* c = ctxs[k];
-    const Tiling ti = choose_tiling(c, !fp32, OP_COCG, nslots), tr = choose_tiling(c, true, OP_RESID, nslots);
+    const Tiling ti = choose_tiling(c, !fp32, OP_COCG, nslots, aligned), tr = choose_tiling(c, true, OP_RESID, nslots);
     const int kind = ti.plane ? kOpPlane : ti.pair ? kOpPair : ti.tma ? kOpTma : kOpReg;
     if (kind == kOpReg) {
       if (ppt_reg && ppt_reg != ti.ppt) return false;
@@ -2518,13 +2531,11 @@ static bool make_pool(rsn_ctx* const* ctxs, int K, bool fp32, int nslots, PoolSp
     pool.resid.threads = std::max(pool.resid.threads, tr.threads);
     pool.resid.smem = std::max(pool.resid.smem, tr.smem);
     pool.resid.n = std::max(pool.resid.n, tr.n);
-    pool.N = std::max(pool.N, c->N);
     pool.n_proj = std::max(pool.n_proj, c->n_proj);
     pool.n_groups = std::max(pool.n_groups, c->n_groups);
     pool.max_np = std::max(pool.max_np, c->max_np);
     pool.nB = std::max(pool.nB, c->jh.nB);
     pool.PA = std::max(pool.PA, std::max(ti.parts + c->n_groups, tr.n));
-    
     for (int h = 0; h < 2; ++h) {
       const Tiling& t = h == 0 ? ti : tr;
       JuncDev& J = js[h * K + k];
@@ -2587,11 +2598,8 @@ static rsn_status batch_pool_impl(int K, rsn_ctx* const* ctxs, const int* n_e, c
     auto run = [&](const rsn_solver_opts* oo, const StreamIn& sin, StreamOut& so) -> rsn_status {
       const bool f32 = oo->precision == RSN_MIXED;
       // slots first (a pool of one slot size), then the tilings for that count
-      PoolSpec probe;
       std::vector<JuncDev> js;
-      probe.N = 0;
-      for (int k = 0; k < K; ++k) probe.N = std::max(probe.N, ctxs[k]->N);
-      const int S = choose_slots(c, oo, (long long)sin.E.size(), 0, 0, probe.N);
+      const int S = choose_slots(c, oo, (long long)sin.E.size(), 0, 0, pool_points(ctxs, K));
       rsn_solver_opts o2 = *oo;
       o2.rhs_block = S;
       PoolSpec pool;

@@ -98,3 +98,29 @@ def test_one_pool_over_sixteen_uneven_junctions(B):
                 assert np.all(np.abs(Tb[k] - T_ref) <= 1e-8 * np.abs(T_ref)), (k, Tb[k], T_ref)
     for c in ctxs:
         c.close()
+
+
+@pytest.mark.parametrize("ppt", [0, -1, -2, -3])
+def test_batch_slots_stay_aligned_beside_an_odd_junction(B, ppt):
+    # The largest junction has an odd number of points (the register kernel), the
+    # others run kernels that copy whole planes in 16-byte units: even nx, odd nx
+    # with an even plane.  An odd and an even number of columns, so that the even
+    # junctions sit in odd and in even slots.  Mixed-mode bound on T: 1e-6.
+    specs = [(15, 15, 41), (12, 12, 36), (11, 12, 36), (10, 13, 33)]
+    js = [P.molecular_junction(seed=40 + k, nx=nx, ny=ny, nz=nz, n_cap=4, n_wells=3)
+          for k, (nx, ny, nz) in enumerate(specs)]
+    assert js[0].N % 2 == 1 and js[0].N == max(j.N for j in js)
+    ctxs = [B.Context(0).set_junction(j) for j in js]
+    for c in ctxs:
+        c.set_tiling(0, 12 if ppt == -1 else 0, ppt)
+    energies = [[0.19, 0.23]] * len(js)
+    cols = [j.right_columns()[: 5 + k] for k, j in enumerate(js)]
+    opts = B.default_opts(B.RSN_MIXED)
+    T = B.batch_transmission(ctxs, energies, cols, opts)
+    for k, j in enumerate(js):
+        T_ref = O.transmission(j, energies[k], cols[k])
+        assert np.all(np.abs(T[k] - T_ref) <= 1e-6), (k, T[k], T_ref)
+        T_alone = ctxs[k].transmission(energies[k], cols[k], opts)
+        assert np.all(np.abs(T[k] - T_alone) <= 1e-6), (k, T[k], T_alone)
+    for c in ctxs:
+        c.close()
