@@ -2559,10 +2559,14 @@ static rsn_status batch_pool_impl(int K, rsn_ctx* const* ctxs, const int* n_e, c
   rsn_ctx* c = ctxs[0];
   const bool fp32 = o->precision == RSN_MIXED;
   RSN_CUDA(c, cudaSetDevice(c->device));
-  // order the pool's stream after every caller stream
+  // order the pool's stream after every caller stream, and after the contexts' own
+  // streams: the upload of a junction's operator data (commit_setup) ends there with
+  // a kernel that gathers the projector rows
   for (int k = 0; k < K; ++k) {
     RSN_CUDA(c, cudaEventRecord(ctxs[k]->ev_in, ctxs[k]->user_stream));
     RSN_CUDA(c, cudaStreamWaitEvent(c->st, ctxs[k]->ev_in, 0));
+    RSN_CUDA(c, cudaEventRecord(ctxs[k]->ev_out, ctxs[k]->st));
+    RSN_CUDA(c, cudaStreamWaitEvent(c->st, ctxs[k]->ev_out, 0));
   }
   reset_stats(c);
   const auto t_start = std::chrono::steady_clock::now();
@@ -2740,12 +2744,15 @@ rsn_status rsn_batch_transmission(int n_ctx, rsn_ctx* const* ctxs, const int* n_
         }
     } else {
       const rsn_status rs = batch_pool_impl(n_ctx, ctxs, n_e, E, n_cols, cols, &base, T, st);
-      if (rs != RSN_OK)
+      if (rs != RSN_OK) {
+        // nothing of a pool that gave up may still read the other contexts' data
+        for (cudaStream_t ps : {ctxs[0]->st, ctxs[0]->st2, ctxs[0]->st3, ctxs[0]->st4}) cudaStreamSynchronize(ps);
         for (int k = 0; k < n_ctx; ++k)
           if (st[k] == RSN_OK) {
             st[k] = rs;
             if (k) ctxs[k]->err = "rsn_batch_transmission: the slot pool failed: " + ctxs[0]->err;
           }
+      }
     }
     rsn_status worst = RSN_OK;
     for (int k = 0; k < n_ctx; ++k) {

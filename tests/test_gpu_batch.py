@@ -100,6 +100,32 @@ def test_one_pool_over_sixteen_uneven_junctions(B):
         c.close()
 
 
+def test_batch_right_after_new_projectors(B):
+    # every junction but the first gets other projectors between two calls: the pool
+    # must not read the rows of the call before, nor rows still being gathered.  The
+    # second call agrees with contexts that never held the first projectors (the same
+    # launches on the same data: bit for bit in FP64).
+    first = _junctions()
+    second = [first[0]] + [P.molecular_junction(seed=60 + k, nx=j.nx, ny=j.ny, nz=j.nz, n_cap=5, n_wells=6, lmax=2)
+                           for k, j in enumerate(first[1:])]
+    cols = [j.right_columns()[:4] for j in second]
+    E = [[0.21]] * len(second)
+    o = B.default_opts(B.RSN_FP64)
+    ctxs = [B.Context(0).set_junction(j) for j in first]
+    B.batch_transmission(ctxs, E, [j.right_columns()[:4] for j in first], o)
+    for c, j in zip(ctxs[1:], second[1:]):
+        c.set_junction(j)
+    T = B.batch_transmission(ctxs, E, cols, o)
+    fresh = [B.Context(0).set_junction(j) for j in second]
+    T_fresh = B.batch_transmission(fresh, E, cols, o)
+    for k in range(len(second)):
+        assert np.array_equal(T[k], T_fresh[k]), (k, T[k], T_fresh[k])
+        T_ref = O.transmission(second[k], E[k], cols[k])
+        assert np.all(np.abs(T[k] - T_ref) <= 1e-9 * np.maximum(np.abs(T_ref), 1e-3)), (k, T[k], T_ref)
+    for c in ctxs + fresh:
+        c.close()
+
+
 @pytest.mark.parametrize("ppt", [0, -1, -2, -3])
 def test_batch_slots_stay_aligned_beside_an_odd_junction(B, ppt):
     # The largest junction has an odd number of points (the register kernel), the
