@@ -405,7 +405,10 @@ static cudaError_t launch_apply(rsn_ctx* c, const Tiling& t, bool fp32, int n, c
 }
 
 // ---------------------------------------------------------------------------
-// upload of the operator data (done lazily before the first solve/apply)
+// upload of the operator data (done lazily before the first solve/apply).  Every
+// copy goes through c->st: that stream is non-blocking, so nothing else orders a
+// copy before the kernels that read it (a blocking copy from pageable memory
+// returns once its source is staged, not when the data has arrived).
 // ---------------------------------------------------------------------------
 // Projector tables: atoms with their supports, per-point entries, rows by block.
 static rsn_status commit_projectors(rsn_ctx* c) {
@@ -490,7 +493,7 @@ static rsn_status commit_projectors(rsn_ctx* c) {
   auto up = [&](DevBuf& b, const void* src, size_t bytes) -> cudaError_t {
     cudaError_t e = b.ensure(std::max<size_t>(bytes, 16));
     if (e != cudaSuccess) return e;
-    if (bytes) return cudaMemcpy(b.p, src, bytes, cudaMemcpyHostToDevice);
+    if (bytes) return cudaMemcpyAsync(b.p, src, bytes, cudaMemcpyHostToDevice, c->st);
     return cudaSuccess;
   };
   RSN_CUDA(c, up(c->inv_ptr, cnt.data(), (N + 1) * sizeof(int)));
@@ -536,10 +539,10 @@ static rsn_status commit_setup(rsn_ctx* c) {
   RSN_CUDA(c, c->dg64.ensure(N * sizeof(double2)));
   RSN_CUDA(c, c->dg32.ensure(N * sizeof(float2)));
   RSN_CUDA(c, c->gld.ensure(N * sizeof(double)));
-  RSN_CUDA(c, cudaMemcpy(c->dg64.p, dg.data(), N * sizeof(double2), cudaMemcpyHostToDevice));
-  RSN_CUDA(c, cudaMemcpy(c->dg32.p, dgf.data(), N * sizeof(float2), cudaMemcpyHostToDevice));
+  RSN_CUDA(c, cudaMemcpyAsync(c->dg64.p, dg.data(), N * sizeof(double2), cudaMemcpyHostToDevice, c->st));
+  RSN_CUDA(c, cudaMemcpyAsync(c->dg32.p, dgf.data(), N * sizeof(float2), cudaMemcpyHostToDevice, c->st));
   if (c->dirty_cap) {
-    RSN_CUDA(c, cudaMemcpy(c->gld.p, c->gl.data(), N * sizeof(double), cudaMemcpyHostToDevice));
+    RSN_CUDA(c, cudaMemcpyAsync(c->gld.p, c->gl.data(), N * sizeof(double), cudaMemcpyHostToDevice, c->st));
     std::vector<int> lidx;
     std::vector<double> lgam;
     for (long long i = 0; i < N; ++i)
@@ -551,8 +554,8 @@ static rsn_status commit_setup(rsn_ctx* c) {
     RSN_CUDA(c, c->L_idx.ensure(std::max<size_t>(1, lidx.size()) * sizeof(int)));
     RSN_CUDA(c, c->L_gam.ensure(std::max<size_t>(1, lgam.size()) * sizeof(double)));
     if (!lidx.empty()) {
-      RSN_CUDA(c, cudaMemcpy(c->L_idx.p, lidx.data(), lidx.size() * sizeof(int), cudaMemcpyHostToDevice));
-      RSN_CUDA(c, cudaMemcpy(c->L_gam.p, lgam.data(), lgam.size() * sizeof(double), cudaMemcpyHostToDevice));
+      RSN_CUDA(c, cudaMemcpyAsync(c->L_idx.p, lidx.data(), lidx.size() * sizeof(int), cudaMemcpyHostToDevice, c->st));
+      RSN_CUDA(c, cudaMemcpyAsync(c->L_gam.p, lgam.data(), lgam.size() * sizeof(double), cudaMemcpyHostToDevice, c->st));
     }
   }
   if (c->dirty_proj) {
@@ -961,17 +964,17 @@ static rsn_status ensure_ws(rsn_ctx* c, bool fp32, int S, const PoolSpec* pool =
   RSN_CUDA(c, w.c_p.ensure(2 * (size_t)S * npj * sizeof(double2)));
   RSN_CUDA(c, w.c_x.ensure((size_t)S * npj * sizeof(double2)));
   RSN_CUDA(c, w.c_e.ensure((size_t)S * (npj + kCePad) * sizeof(double2)));
-  RSN_CUDA(c, cudaMemset(w.c_e.p, 0, (size_t)S * (npj + kCePad) * sizeof(double2)));
+  RSN_CUDA(c, cudaMemsetAsync(w.c_e.p, 0, (size_t)S * (npj + kCePad) * sizeof(double2), c->st));
   RSN_CUDA(c, w.sched.ensure((3 + 2 * kMaxGraphIters) * sizeof(int)));
   RSN_CUDA(c, w.counters.ensure(4 * sizeof(unsigned long long)));
   RSN_CUDA(c, w.lst.ensure(si));
   RSN_CUDA(c, w.lst_n.ensure(sizeof(int)));
   RSN_CUDA(c, w.inlist.ensure(si));
-  RSN_CUDA(c, cudaMemset(w.inlist.p, 0, si));
+  RSN_CUDA(c, cudaMemsetAsync(w.inlist.p, 0, si, c->st));
   RSN_CUDA(c, w.fslot.ensure(si));
   std::vector<long long> hvo(S);
   for (int s = 0; s < S; ++s) hvo[s] = (long long)s * N;
-  RSN_CUDA(c, cudaMemcpy(w.voff.p, hvo.data(), sl, cudaMemcpyHostToDevice));
+  RSN_CUDA(c, cudaMemcpyAsync(w.voff.p, hvo.data(), sl, cudaMemcpyHostToDevice, c->st));
   RSN_CUDA(c, c->bd.ensure(sizeof(BatchDev)));
   w.slots = S;
   w.fp32 = fp32;
