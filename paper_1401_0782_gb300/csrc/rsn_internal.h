@@ -47,6 +47,16 @@ constexpr int kVecPts = kVecThreads * kVecPerThread;
 // kUpdThreads / 32 blocks per CTA.
 constexpr int kBlkPts = 128;
 constexpr int kUpdThreads = 128;
+// Blocks of a system of N points (1 <= N < 2^31), and the first point and number of
+// points of block k: the last CTA's warps may ask past the last block (first = N,
+// no points).  Positions are kept relative to a block's first point, since its end
+// may lie past the largest int.
+__host__ __device__ constexpr int blk_count(int N) { return (N - 1) / kBlkPts + 1; }
+__host__ __device__ constexpr int blk_first(int k, int N) { return k < blk_count(N) ? k * kBlkPts : N; }
+__host__ __device__ constexpr int blk_len(int k, int N) {
+  const int left = N - blk_first(k, N);
+  return left < kBlkPts ? left : kBlkPts;
+}
 __host__ __device__ constexpr int upd_ctas(long long N) {
   return (int)((N + kBlkPts * (kUpdThreads / 32) - 1) / (kBlkPts * (kUpdThreads / 32)));
 }

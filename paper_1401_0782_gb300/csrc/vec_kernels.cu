@@ -176,7 +176,7 @@ __device__ __forceinline__ void block_nonlocal_nq(const JuncDev& J, const typena
 #pragma unroll
     for (int j = 0; j < D; ++j) {
       const int rr = min(row + j, row1 - 1);
-      m[j] = __ldg(J.row_ent + rr * 32 + lane);
+      m[j] = __ldg(J.row_ent + (size_t)rr * 32 + lane);
       if (row + j >= row1) m[j] = -1;
 #pragma unroll
       for (int qd = 0; qd < NQ; ++qd) {
@@ -273,8 +273,8 @@ cocg_update_kernel(const JuncDev* __restrict__ jt, const BatchDev* __restrict__ 
   const int nU = upd_ctas(N);
   if ((int)blockIdx.x >= nU) return;
   const int blk = blockIdx.x * nw + warp;
-  const int i0 = min(blk * kBlkPts, N), i1 = min(i0 + kBlkPts, N);
-  const long long vo = b.voff[s];
+  const int n = blk_len(blk, N);  // points of the warp's block
+  const long long vo = b.voff[s], bo = vo + blk_first(blk, N);
   const int k = b.iters[s];
   C al;  // (FP32: rounded once by mu_alpha, which keeps conversions off the FP64 pipe here)
   if constexpr (sizeof(T) == 4) al = b.alpha32[s];
@@ -287,10 +287,10 @@ cocg_update_kernel(const JuncDev* __restrict__ jt, const BatchDev* __restrict__ 
   __shared__ int s_last;
   T re = 0, sy = 0, sxy = 0;  // sums of r.x^2 - r.y^2 (cancelling inside the sum), r.y^2, r.x r.y
   if (fin) {  // uniform across the CTA
-    const C* pn = reinterpret_cast<const C*>((k & 1) ? b.p0 : b.p1) + vo;
-    const C* qv = reinterpret_cast<const C*>(b.q) + vo;
-    C* rv = reinterpret_cast<C*>(b.r) + vo;
-    C* dv = reinterpret_cast<C*>(b.d) + vo;
+    const C* pn = reinterpret_cast<const C*>((k & 1) ? b.p0 : b.p1) + bo;
+    const C* qv = reinterpret_cast<const C*>(b.q) + bo;
+    C* rv = reinterpret_cast<C*>(b.r) + bo;
+    C* dv = reinterpret_cast<C*>(b.d) + bo;
     const T ax = al.x, ay = al.y;
     // FP32: 16-byte pairs where the slot starts on a pair and holds whole
     // pairs; else (and in FP64, 16 bytes a point) one point at a time
@@ -300,16 +300,16 @@ cocg_update_kernel(const JuncDev* __restrict__ jt, const BatchDev* __restrict__ 
     auto fetch = [&](int l) {
 #pragma unroll
       for (int u = 0; u < U; ++u)
-        at[u] = i0 + l * 32 * U + (pairs ? 2 * lane + (u >> 1) * 64 + (u & 1) : u * 32 + lane);
-      load_pts(qv, at, i1, pairs, q);
-      load_pts(rv, at, i1, pairs, r);
-      load_pts(pn, at, i1, pairs, p);
-      load_pts(dv, at, i1, pairs, d);
+        at[u] = l * 32 * U + (pairs ? 2 * lane + (u >> 1) * 64 + (u & 1) : u * 32 + lane);
+      load_pts(qv, at, n, pairs, q);
+      load_pts(rv, at, n, pairs, r);
+      load_pts(pn, at, n, pairs, p);
+      load_pts(dv, at, n, pairs, d);
     };
     if constexpr (EARLY) fetch(0);
     int row0 = 0, row1 = 0;
     if (J.n_proj > 0) {
-      const int nblk = (N + kBlkPts - 1) / kBlkPts;
+      const int nblk = blk_count(N);
       const int ra = J.blk_row[blockIdx.x * nw], rb = J.blk_row[min((int)(blockIdx.x + 1) * nw, nblk)];
       if (rb > ra) {  // uniform across the CTA
         const C* cen = reinterpret_cast<const C*>(b.c_e) + (size_t)s * b.ce_stride;
@@ -327,7 +327,7 @@ cocg_update_kernel(const JuncDev* __restrict__ jt, const BatchDev* __restrict__ 
       if (!EARLY || l > 0) fetch(l);
       if (row1 > row0) {
 #pragma unroll
-        for (int u = 0; u < U; ++u) q[u] = cadd(q[u], s_nl[at[u] - i0]);
+        for (int u = 0; u < U; ++u) q[u] = cadd(q[u], s_nl[at[u]]);
       }
 #pragma unroll
       for (int u = 0; u < U; ++u) {
@@ -336,14 +336,14 @@ cocg_update_kernel(const JuncDev* __restrict__ jt, const BatchDev* __restrict__ 
         r[u].y = fma(-ax, q[u].y, fma(-ay, q[u].x, r[u].y));
         d[u].x = fma(ax, p[u].x, fma(-ay, p[u].y, d[u].x));
         d[u].y = fma(ax, p[u].y, fma(ay, p[u].x, d[u].y));
-        const bool in = at[u] < i1;  // (a short block's accumulators past its end are not its own)
+        const bool in = at[u] < n;  // (a short block's accumulators past its end are not its own)
         const T rx = in ? r[u].x : (T)0, ry = in ? r[u].y : (T)0;
         re = fma(rx, rx, fma(-ry, ry, re));
         sy = fma(ry, ry, sy);
         sxy = fma(rx, ry, sxy);
       }
-      store_pts(rv, at, i1, pairs, r);
-      store_pts(dv, at, i1, pairs, d);
+      store_pts(rv, at, n, pairs, r);
+      store_pts(dv, at, n, pairs, d);
     }
   }
   // r^T r = (re, 2 sxy), ||r||^2 = re + 2 sy over the CTA, fixed order
@@ -585,7 +585,7 @@ __global__ void __launch_bounds__(kUpdThreads) nonlocal_kernel(const JuncDev* __
   const JuncDev& J = jt[b.junc[v0]];
   const int N = (int)J.N;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nw = blockDim.x >> 5;
-  const int nblk = (N + kBlkPts - 1) / kBlkPts;
+  const int nblk = blk_count(N);
   const int blk0 = blockIdx.x * nw, blk = blk0 + warp;
   if (J.blk_row[min(blk0 + nw, nblk)] == J.blk_row[min(blk0, nblk)]) return;  // uniform across the CTA
   extern __shared__ __align__(16) unsigned char nl_smem[];
@@ -607,16 +607,16 @@ __global__ void __launch_bounds__(kUpdThreads) nonlocal_kernel(const JuncDev* __
   const int row0 = J.blk_row[blk], row1 = J.blk_row[blk + 1];
   if (row1 == row0) return;
   block_nonlocal<T, SPV>(J, s_ce, ces, row0, row1, s_acc);
-  const int i0 = blk * kBlkPts;
+  const int n = blk_len(blk, N);
   for (int v = 0; v < nv; ++v) {
-    C* y = reinterpret_cast<C*>(y_out) + b.voff[v0 + v] + i0;
+    C* y = reinterpret_cast<C*>(y_out) + b.voff[v0 + v] + blk_first(blk, N);
     C w[kBlkPts / 32];
 #pragma unroll
     for (int h = 0; h < kBlkPts / 32; ++h)
-      if (i0 + h * 32 + lane < N) w[h] = y[h * 32 + lane];
+      if (h * 32 + lane < n) w[h] = y[h * 32 + lane];
 #pragma unroll
     for (int h = 0; h < kBlkPts / 32; ++h)
-      if (i0 + h * 32 + lane < N) y[h * 32 + lane] = cadd(w[h], s_acc[v * kBlkPts + h * 32 + lane]);
+      if (h * 32 + lane < n) y[h * 32 + lane] = cadd(w[h], s_acc[v * kBlkPts + h * 32 + lane]);
   }
 }
 
@@ -1049,7 +1049,7 @@ __global__ void __launch_bounds__(kVecThreads) shift_init_kernel(const JuncDev* 
     const int col = b.col[s];
     double2* xb = b.xs + (long long)(b.xs_by_sys ? b.sys[s] : s) * b.xs_sstride;
     double2* pb = b.ps + (size_t)s * ns * nT;
-    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < nT; i += gridDim.x * blockDim.x) {
+    for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < nT; i += (long long)gridDim.x * blockDim.x) {
       const double one = b.T_idx[i] == col ? 1.0 : 0.0;
       for (int e = 0; e < ns; ++e) {
         xb[(long long)e * b.xs_estride + i] = make_double2(0.0, 0.0);
@@ -1140,7 +1140,7 @@ __global__ void __launch_bounds__(kVecThreads) shift_update_kernel(const JuncDev
   double2* xb = b.xs + (long long)(b.xs_by_sys ? b.sys[s] : s) * b.xs_sstride;
   double2* pb = b.ps + (size_t)s * ns * nT;
   const double2* rv = reinterpret_cast<const double2*>(b.r) + b.voff[s];
-  for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < nT; i += gridDim.x * blockDim.x) {
+  for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < nT; i += (long long)gridDim.x * blockDim.x) {
     const double2 r = rv[b.T_idx[i]];
     for (int e0 = 8 * blockIdx.z; e0 < min(ns, 8 * ((int)blockIdx.z + 1)); e0 += 4) {
       double2 g[4], x[4];
