@@ -358,13 +358,14 @@ static Tiling choose_tiling(const rsn_ctx* c, bool compute64, int mode, int nslo
       c->tile_override[3] == -1) {
     const size_t sm = op_tma_smem_bytes(true, mode, R, nx, ny);
     if (sm <= 200 * 1024) {
-      t.TY = ny;
-      t.ytiles = 1;
-      t.n = t.ztiles;
-      t.parts = (nz + kMuPlanes - 1) / kMuPlanes;
       t.tma = true;
+      t.TY = ny;
       t.smem = sm;
       t.threads = (int)((pl + 31) / 32 * 32);
+      // its own chunks: one tile column, and as many CTAs an SM as 64 registers a
+      // thread and the shared memory (16 KB of static arrays beside the planes) allow
+      t.n = 0;
+      z_chunks(std::max(1, std::min(1024 / t.threads, (int)(227 * 1024 / (sm + 16 * 1024)))), 1);
     }
   }
   return t;

@@ -207,6 +207,30 @@ def test_mixed_solves_under_every_operator_kernel(B, tiling):
     ctx.close()
 
 
+@pytest.mark.parametrize("prec,TY,ppt", [("mixed", 0, 0), ("mixed", 0, -1), ("mixed", 0, -2), ("mixed", 0, -3), ("mixed", 4, 2),
+                                         ("fp64", 0, 0), ("fp64", 4, 2)])
+def test_automatic_z_chunks_through_a_draining_pool(B, prec, TY, ppt):
+    # 64 systems that finish at different times: the automatic z chunks get shorter
+    # when a quarter and a sixteenth of the slots are left.  A result does not depend
+    # on the chunks, so every kernel gives what it gives with fixed ones, bit for bit,
+    # after as many iterations and with as many FP64 re-solves.
+    j = JUNCTIONS["junction_R4"]()
+    E = np.linspace(0.12, 0.4, 8)
+    cols = j.right_columns()[::17][:8]
+    ctx = B.Context(0).set_junction(j)
+    o = B.default_opts(B.RSN_FP64 if prec == "fp64" else B.RSN_MIXED)
+    out = []
+    for Lz in (0, 12):
+        ctx.set_tiling(TY, Lz, ppt)
+        x, iters, relres = ctx.solve_columns(E, cols, o)
+        out.append((x.clone(), np.array(iters), ctx.last_stats()["fp64_fallbacks"]))
+        assert relres.max() <= 1e-10
+    assert np.unique(out[0][1]).size > 4  # the pool drains in steps
+    assert np.array_equal(out[0][1], out[1][1]) and out[0][2] == out[1][2]
+    assert torch.equal(out[0][0], out[1][0])
+    ctx.close()
+
+
 @pytest.mark.parametrize("prec", ["fp64", "mixed"])
 def test_open_channel_junction_relative_transmission(B, prec):
     # above the leads' first transverse levels T = O(1): the relative bound is
