@@ -895,7 +895,8 @@ __global__ void __launch_bounds__(kSchedThreads) sched_kernel(const JuncDev* __r
 // inner recurrence works on O(1) numbers whatever the size of b (an adjoint
 // right-hand side Gamma_L o conj(x) can be ~1e-6 or smaller, whose squares
 // would leave the FP32 range).  For a NEW slot sigma comes from the residual
-// partials (r = b there); each thread touches only its own points.
+// kernel's sum (r = b from a cold start; a warm start, whose r is smaller, brings
+// ||b||^2 along); each thread touches only its own points.
 template <typename T>
 __global__ void __launch_bounds__(kVecThreads) x_update_kernel(const JuncDev* __restrict__ jt,
                                                                const BatchDev* __restrict__ bp) {
@@ -912,8 +913,8 @@ __global__ void __launch_bounds__(kVecThreads) x_update_kernel(const JuncDev* __
     __syncthreads();  // s_sig of the previous entry are consumed
     if (threadIdx.x == 0) {
       double sg = b.sigma[s];
-      if (st == SL_NEW) {  // ||b||^2 from the residual kernel
-        const double n2 = b.res_tot[4 * s];
+      if (st == SL_NEW) {  // ||b||^2, as the scheduler takes it
+        const double n2 = b.warm[s] ? b.sys_bn2[b.sys[s]] : b.res_tot[4 * s];
         sg = n2 > 0.0 ? sqrt(n2) : 1.0;
         if (blockIdx.x == 0) b.sigma[s] = sg;
       }

@@ -146,3 +146,24 @@ def test_block_edge_cases(B):
     T_ref = 4.0 * np.sum(j.gamma_r[cols] * _tc(j, O.solve_columns(j, 0.2, cols)))
     assert abs(T[0] - T_ref) <= 1e-6 * T_ref
     ctx.close()
+
+
+def test_handed_over_columns_keep_their_progress(B):
+    # a block stopped by max_outer at a residual of ~1e-9 hands its columns over with
+    # that iterate; the plain solver finishes the last decade in at most the
+    # iterations that it needs for all ten from a cold start
+    j = JUNCTIONS["junction_R4"]()
+    cols = P.column_subset(j, 8, seed=5)
+    ctx = B.Context(0).set_junction(j)
+    kw = dict(tol_T=0.0, max_outer=3)
+    _, _, own, rel = ctx.solve_columns_block([0.2], cols, block=8, tol_inner=1e-3, opts=B.default_opts(B.RSN_MIXED, tol=5e-9, **kw))
+    assert ctx.last_stats()["fp64_fallbacks"] == 0 and rel.max() <= 5e-9  # three outer steps, none handed over
+    x, _, its, rel = ctx.solve_columns_block([0.2], cols, block=8, tol_inner=1e-3, opts=B.default_opts(B.RSN_MIXED, **kw))
+    assert ctx.last_stats()["fp64_fallbacks"] == cols.size and rel.max() <= 1e-10
+    _, cold, _ = ctx.solve_columns([0.2], cols, B.default_opts(B.RSN_MIXED, tol_T=0.0))
+    more = its - own
+    assert more.min() >= 0 and 0 < more.max() <= cold.max(), (own, its, cold)  # (a column may have met its target already)
+    X_ref = O.solve_columns(j, 0.2, cols)
+    dx = np.linalg.norm(x[0].cpu().numpy().T - X_ref, axis=0) / np.linalg.norm(X_ref, axis=0)
+    assert dx.max() <= 1e-8
+    ctx.close()
