@@ -250,32 +250,19 @@ static Tiling choose_tiling(const rsn_ctx* c, bool compute64, int mode, int nslo
   // FP32 point-pair kernel: whole planes, nx even (16-byte pairs), at most
   // 2 * kPairThreadsBig points per plane, no explicit register tile requested
   const bool reg_forced = c->tile_override[0] > 0 || c->tile_override[2] > 0 || c->tile_override[3] == -1;
-  // z chunks per tile column: as many as make the launch shortest.  A CTA marches
-  // Lz + 2R planes after a start worth a plane or so, halo planes costing half a
-  // plane (FP32) or less (FP64, bound by its pipe), and waves of 152 * per_sm CTAs
-  // follow one another.  24x24x120, order 8: 144 FP32 systems 120 us at Lz 14, 84 at
-  // 60; 16 of them 23 at 10, 64 at 60; FP64, 144 systems 1,430 us at Lz 40, 1,289 at
-  // 60; 16 of them 158 at 10, 151 at 20, 252 at 60.
-  auto pick_zt = [&](long long columns, int per_sm, int zt_max) {
-    int best = 1;
-    double best_cost = 1e300;
-    for (int zt = 1; zt <= std::max(1, std::min(nz / 2, zt_max)); ++zt) {
-      const int lz = std::min(kMaxLz, ((nz + zt - 1) / zt + kMuPlanes - 1) / kMuPlanes * kMuPlanes);
-      const long long n = columns * ((nz + lz - 1) / lz), wave = 152LL * per_sm;
-      const double cost = (double)((n + wave - 1) / wave) * (compute64 ? lz + 0.35 * R + 1.0 : lz + R + 1.5);
-      if (cost < best_cost * 0.999) best_cost = cost, best = zt;
-    }
-    return best;
-  };
-  // The COCG launch picks its chunks by the number of slots still busy (lz_act[k]:
-  // at most 2^k of them), apply by its vectors.
+  // The COCG launch picks its z chunks by the number of slots still busy (lz_act[k]:
+  // at most 2^k of them), other launches by their vectors alone, once.
   auto z_chunks = [&](int per_sm, int ytiles) {
     for (int k = 0; k < kActBuckets; ++k) {
+      if (k > 0 && mode != OP_COCG) {
+        t.lz_act[k] = t.lz_act[0];
+        t.n_act[k] = t.n_act[0];
+        continue;
+      }
       const int act = mode == OP_COCG ? (int)std::min<long long>(1LL << k, nslots) : nslots;
-      const int zt = pick_zt((long long)act * ytiles, per_sm, nz);
-      int lz = (nz + zt - 1) / zt;
-      if (c->tile_override[1] > 0) lz = std::min(nz, c->tile_override[1]);
-      lz = std::min(kMaxLz, (lz + kMuPlanes - 1) / kMuPlanes * kMuPlanes);
+      int lz = pick_lz(nz, R, compute64, (long long)act * ytiles, per_sm);
+      if (c->tile_override[1] > 0)
+        lz = std::min(kMaxLz, (std::min(nz, c->tile_override[1]) + kMuPlanes - 1) / kMuPlanes * kMuPlanes);
       t.lz_act[k] = lz;
       t.n_act[k] = ytiles * ((nz + lz - 1) / lz);
       t.n = std::max(t.n, t.n_act[k]);

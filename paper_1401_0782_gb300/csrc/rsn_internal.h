@@ -73,6 +73,36 @@ constexpr int kActBuckets = 14;  // up to 8192 slots
 constexpr int kMuPlanes = 4;
 constexpr int kMaxLz = 128;
 
+// Planes per z chunk of an operator launch over `columns` tile columns of nz planes:
+// the length that makes the launch shortest.  A CTA marches lz + 2R planes after a
+// start worth a plane or so, halo planes costing half a plane (FP32) or less (FP64,
+// bound by its pipe), and waves of 152 * per_sm CTAs follow one another.  24x24x120,
+// order 8: 144 FP32 systems 120 us at 14 planes, 84 at 60; 16 of them 23 at 10, 64 at
+// 60; FP64, 144 systems 1,430 us at 40, 1,289 at 60; 16 of them 158 at 10, 151 at 20,
+// 252 at 60.  The lengths that even chunks can have are tried from the longest (at
+// most kMaxLz / kMuPlanes of them, however many planes there are: this runs in every
+// operator application); a shorter one has to be 0.1% better.
+inline int pick_lz(int nz, int R, bool fp64, long long columns, int per_sm) {
+  const long long wave = 152LL * per_sm;
+  const int zt_max = nz / 2 > 1 ? nz / 2 : 1;
+  int best = 0;
+  double best_cost = 1e300;
+  for (long long zt = 1; zt <= zt_max;) {
+    const long long even = (nz + zt - 1) / zt, up = (even + kMuPlanes - 1) / kMuPlanes * kMuPlanes;
+    const int lz = up < kMaxLz ? (int)up : kMaxLz;
+    const long long n = columns * (((long long)nz + lz - 1) / lz);
+    const double cost = (double)((n + wave - 1) / wave) * (fp64 ? lz + 0.35 * R + 1.0 : lz + R + 1.5);
+    if (cost < best_cost * 0.999) {
+      best_cost = cost;
+      best = lz;
+    }
+    if (lz <= kMuPlanes) break;
+    const long long next = ((long long)nz + lz - kMuPlanes - 1) / (lz - kMuPlanes);  // fewest chunks of a shorter length
+    zt = next > zt ? next : zt + 1;
+  }
+  return best;
+}
+
 struct JuncDev {
   int nx, ny, nz, plane;
   long long N;
