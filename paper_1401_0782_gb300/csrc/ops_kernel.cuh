@@ -76,7 +76,7 @@ template <typename T> struct RawIn<T, OP_APPLY> { typename cx<T>::t a; };
 // busy and spilled queues cost more than occupancy).
 constexpr int kOpThreads = 256;
 
-// One (tile, slot) of the operator: the CTA's tile of slot s (blockIdx.y; the true
+// One (tile, slot) of the operator: the CTA's tile of slot s (launch_tile; the true
 // residual, whose CTA rows walk a list of slots: blockIdx.x).
 template <typename T, int R, int PPT, int MODE>
 __device__ __forceinline__ void op_tile(const JuncDev* __restrict__ jt, const BatchDev& b, const int s,
@@ -96,7 +96,7 @@ __device__ __forceinline__ void op_tile(const JuncDev* __restrict__ jt, const Ba
     if (stt != SL_NEW && stt != SL_CHECK) return;
   }
   const JuncDev& J = jt[b.junc[s]];
-  const int tile = MODE == OP_RESID ? blockIdx.x : blockIdx.y;
+  const int tile = MODE == OP_RESID ? (int)blockIdx.x : launch_tile();
   if (tile >= J.nA || (MODE != OP_RESID && J.kind != kOpReg)) return;
 
   const int nx = J.nx, ny = J.ny, nz = J.nz, plane = J.plane, TY = J.TY;
@@ -458,7 +458,7 @@ op_kernel_tma(const JuncDev* __restrict__ jt, const BatchDev* __restrict__ bp, c
     if (b.state[s] != SL_ACTIVE) return;
   }
   const JuncDev& J = jt[b.junc[s]];
-  const int tile = blockIdx.y;
+  const int tile = launch_tile();
   if (tile >= J.nA || J.kind != kOpTma) return;
   const int nx = J.nx, ny = J.ny, nz = J.nz, plane = J.plane;
   const int Lz = MODE == OP_COCG ? cocg_lz(J, b) : J.Lz;

@@ -47,6 +47,10 @@ __device__ __forceinline__ float2 cfma2(float2 a, float2 b, float2 acc) {
   return fma2(make_float2(-a.y, a.y), make_float2(b.y, b.x), acc);
 }
 
+// The CTA's tile of its slot: tiles past the 65,535 of a grid's y dimension go on in
+// its z dimension (op_grid).
+__device__ __forceinline__ int launch_tile() { return (int)(blockIdx.z * gridDim.y + blockIdx.y); }
+
 // Planes per z chunk of a COCG operator launch, by the number of active slots
 // (host: choose_tiling), and the operator CTAs of a slot with it.
 __device__ __forceinline__ int cocg_lz(const JuncDev& J, const BatchDev& b) {
@@ -225,7 +229,7 @@ op_pair_kernel(const JuncDev* __restrict__ jt, const BatchDev* __restrict__ bp, 
     if (b.state[s] != SL_ACTIVE) return;
   }
   const JuncDev& J = jt[b.junc[s]];
-  const int tile = blockIdx.y;
+  const int tile = launch_tile();
   if (tile >= J.nA || J.kind != kOpPair) return;
 
   const int nx = J.nx, ny = J.ny, nz = J.nz, plane = J.plane;
@@ -444,7 +448,7 @@ op_plane_kernel(const JuncDev* __restrict__ jt, const BatchDev* __restrict__ bp,
     if (b.state[s] != SL_ACTIVE) return;
   }
   const JuncDev& J = jt[b.junc[s]];
-  const int tile = blockIdx.y;
+  const int tile = launch_tile();
   if (tile >= J.nA || J.kind != kOpPlane) return;
 
   const int nx = J.nx, ny = J.ny, nz = J.nz, plane = J.plane;

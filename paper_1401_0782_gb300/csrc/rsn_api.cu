@@ -363,7 +363,7 @@ static Tiling choose_tiling(const rsn_ctx* c, bool compute64, int mode, int nslo
 static cudaError_t launch_inner(const rsn_ctx* c, const Tiling& t, int mode, bool fp32, int nslots, cudaStream_t st,
                                 const JuncDev* jt, const BatchDev* b, const void* x_in, void* y_out, int tiles = 0) {
   // slots fastest: the CTAs of systems that sit out come in runs and leave at once
-  const dim3 grid(nslots, tiles > 0 ? tiles : t.n);
+  const dim3 grid = op_grid(nslots, tiles > 0 ? tiles : t.n);
   if (t.plane) return launch_op_plane(mode, c->R, grid, t.threads, t.smem, st, jt, b, x_in, y_out);
   if (t.pair) return launch_op_pair(mode, c->R, t.big, t.pitch, grid, t.threads, t.smem, st, jt, b, x_in, y_out);
   if (t.tma) return launch_op_tma(mode, fp32, c->R, grid, t.threads, t.smem, st, jt, b, x_in, y_out);

@@ -103,6 +103,13 @@ inline int pick_lz(int nz, int R, bool fp64, long long columns, int per_sm) {
   return best;
 }
 
+// Grid of an operator launch, slots fastest; a long wire has more tiles than the y
+// dimension holds.
+inline dim3 op_grid(int nslots, int tiles) {
+  const int y = tiles < 65535 ? tiles : 65535;
+  return dim3(nslots, y, (tiles + y - 1) / y);
+}
+
 struct JuncDev {
   int nx, ny, nz, plane;
   long long N;

@@ -6,6 +6,8 @@ Krylov + FP64 refinement to relative residual 1e-10, goal-oriented finish) --
 T relative 1e-6 (|dT| <= 1e-6 on the waveguide).  The operator itself is checked element-wise:
 FP64 to 1e-12 relative (rounding order only), FP32 to 2e-6 relative.
 """
+import dataclasses
+
 import numpy as np
 import pytest
 
@@ -228,6 +230,30 @@ def test_automatic_z_chunks_through_a_draining_pool(B, prec, TY, ppt):
     assert np.unique(out[0][1]).size > 4  # the pool drains in steps
     assert np.array_equal(out[0][1], out[1][1]) and out[0][2] == out[1][2]
     assert torch.equal(out[0][0], out[1][0])
+    ctx.close()
+
+
+@pytest.mark.parametrize("ppt", [0, -1, -2, -3])
+def test_more_tiles_than_a_grid_dimension(B, ppt):
+    # a wire of 262,200 planes in chunks of four: 65,550 tiles a vector.  Absorbing
+    # everywhere, so that a column converges in a few iterations.
+    j = P.waveguide(2, 2, 262200, n_cap=16)
+    j = dataclasses.replace(j, gamma_l=j.gamma_l + 0.5, gamma_r=j.gamma_r + 0.5)
+    A = O.system_matrix(j, 0.2)
+    ctx = B.Context(0).set_junction(j)
+    ctx.set_tiling(0, 4, ppt)
+    r = np.random.default_rng(1)
+    x = r.standard_normal((1, j.N)) + 1j * r.standard_normal((1, j.N))
+    for prec, dt, tol in ((B.RSN_FP64, np.complex128, 1e-13), (B.RSN_MIXED, np.complex64, 2e-6)):
+        y = ctx.apply([0.2], torch.tensor(x.astype(dt), device="cuda"), prec).cpu().numpy()
+        ref = A @ x[0]
+        assert np.abs(y[0] - ref).max() <= tol * np.abs(ref).max()
+        col = np.array([j.N // 2 + 1, j.N - 3], np.int32)
+        g, _, rel = ctx.solve_columns([0.2], col, B.default_opts(prec, tol=1e-10, tol_T=0.0))
+        for k in range(2):
+            res = -(A @ g[0, k].cpu().numpy())
+            res[col[k]] += 1.0
+            assert np.linalg.norm(res) <= 2e-10 and rel[0, k] <= 1e-10
     ctx.close()
 
 
