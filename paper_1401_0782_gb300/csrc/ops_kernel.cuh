@@ -117,8 +117,9 @@ __device__ __forceinline__ void op_tile(const JuncDev* __restrict__ jt, const Ba
   C* sm1 = sm0 + rows * pitch;
   C* ce = sm1 + rows * pitch;
   __shared__ double red[MODE == OP_RESID ? 32 * 4 : 1];
-  // mu partials (COCG): [block of planes][warp][re, im]
-  __shared__ __align__(8) CT s_mu[MODE == OP_COCG ? kMaxLz / kMuPlanes * (kOpThreads / 32) * (sizeof(CT) == 8 ? kMuSlots64 : kMuSlots32) : 1];
+  // mu partials (COCG): [block of planes][warp][re, im], behind the planes (as many
+  // as the launch's chunks need: beside the widest planes there is no room for more)
+  CT* s_mu = reinterpret_cast<CT*>(ce);
 
   for (int i = tid; i < 2 * rows * pitch; i += nt) sm0[i] = czero<C>();
 

@@ -252,7 +252,8 @@ static Tiling choose_tiling(const rsn_ctx* c, bool compute64, int mode, int nslo
   const bool reg_forced = c->tile_override[0] > 0 || c->tile_override[2] > 0 || c->tile_override[3] == -1;
   // The COCG launch picks its z chunks by the number of slots still busy (lz_act[k]:
   // at most 2^k of them), other launches by their vectors alone, once.
-  auto z_chunks = [&](int per_sm, int ytiles) {
+  // lz_max: as long as their partials fit in shared memory.
+  auto z_chunks = [&](int per_sm, int ytiles, int lz_max = kMaxLz) {
     for (int k = 0; k < kActBuckets; ++k) {
       if (k > 0 && mode != OP_COCG) {
         t.lz_act[k] = t.lz_act[0];
@@ -263,6 +264,7 @@ static Tiling choose_tiling(const rsn_ctx* c, bool compute64, int mode, int nslo
       int lz = pick_lz(nz, R, compute64, (long long)act * ytiles, per_sm);
       if (c->tile_override[1] > 0)
         lz = std::min(kMaxLz, (std::min(nz, c->tile_override[1]) + kMuPlanes - 1) / kMuPlanes * kMuPlanes);
+      lz = std::min(lz, lz_max);
       t.lz_act[k] = lz;
       t.n_act[k] = ytiles * ((nz + lz - 1) / lz);
       t.n = std::max(t.n, t.n_act[k]);
@@ -336,9 +338,11 @@ static Tiling choose_tiling(const rsn_ctx* c, bool compute64, int mode, int nslo
     t.ztiles = (nz + t.Lz - 1) / t.Lz;
     t.n = t.ytiles * t.ztiles;
   } else {
-    z_chunks(compute64 ? 2 : 4, t.ytiles);
+    const size_t tile = op_smem_bytes(!compute64, mode, R, TY, nx, c->n_proj, 0) + 64;  // (and the static variables)
+    const int fit = tile < (size_t)kMaxSmem ? (int)(((size_t)kMaxSmem - tile) / kMuBlockBytes) : 0;
+    z_chunks(compute64 ? 2 : 4, t.ytiles, mode == OP_COCG ? kMuPlanes * std::max(1, std::min(fit, kMaxLz / kMuPlanes)) : kMaxLz);
   }
-  t.smem = op_smem_bytes(!compute64, mode, R, TY, nx, c->n_proj);
+  t.smem = op_smem_bytes(!compute64, mode, R, TY, nx, c->n_proj, *std::max_element(t.lz_act, t.lz_act + kActBuckets));
   // whole-plane bulk-copy kernel (on request): FP32 COCG / apply on planes
   // whose byte sizes keep every bulk copy 16-byte aligned
   if (!compute64 && mode != OP_RESID && streamable && pl <= 1024 && (pl * 8) % 16 == 0 && (c->N * 8) % 16 == 0 &&
@@ -352,7 +356,7 @@ static Tiling choose_tiling(const rsn_ctx* c, bool compute64, int mode, int nslo
       // its own chunks: one tile column, and as many CTAs an SM as 64 registers a
       // thread and the shared memory (16 KB of static arrays beside the planes) allow
       t.n = 0;
-      z_chunks(std::max(1, std::min(1024 / t.threads, (int)(227 * 1024 / (sm + 16 * 1024)))), 1);
+      z_chunks(std::max(1, std::min(1024 / t.threads, (int)(kMaxSmem / (sm + 16 * 1024)))), 1);
     }
   }
   return t;

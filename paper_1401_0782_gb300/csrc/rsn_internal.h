@@ -72,6 +72,8 @@ constexpr int kActBuckets = 14;  // up to 8192 slots
 // on how many others share the launch; z chunks are multiples of it, of at most kMaxLz planes.
 constexpr int kMuPlanes = 4;
 constexpr int kMaxLz = 128;
+constexpr int kMuBlockBytes = 128;  // register kernel: shared memory for the partials of kMuPlanes planes
+constexpr int kMaxSmem = 227 * 1024;
 
 // Planes per z chunk of an operator launch over `columns` tile columns of nz planes:
 // the length that makes the launch shortest.  A CTA marches lz + 2R planes after a
@@ -352,7 +354,8 @@ enum OpKind { kOpReg = 0, kOpTma = 1, kOpPair = 2, kOpPlane = 3 };
 cudaError_t launch_op(int mode, bool fp32, int R, int ppt, dim3 grid, int threads, size_t smem,
                       cudaStream_t st, const JuncDev* jt, const BatchDev* b, const void* x_in,
                       void* y_out);
-size_t op_smem_bytes(bool fp32, int mode, int R, int TY, int nx, int n_proj);
+// lz (COCG): the longest z chunk
+size_t op_smem_bytes(bool fp32, int mode, int R, int TY, int nx, int n_proj, int lz);
 // plane-streaming (TMA) operator kernel for whole-plane tiles (OP_COCG / OP_APPLY)
 cudaError_t launch_op_tma(int mode, bool fp32, int R, dim3 grid, int threads, size_t smem, cudaStream_t st,
                           const JuncDev* jt, const BatchDev* b, const void* x_in, void* y_out);

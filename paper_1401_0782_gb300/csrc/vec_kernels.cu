@@ -1322,10 +1322,13 @@ size_t op_tma_smem_bytes(bool fp32, int mode, int R, int nx, int ny) {
   return el * (kStages * nin * (size_t)nx * ny + 2 * (size_t)(nx + 2 * R) * (ny + 2 * R)) + 16 + 8 * kStages;
 }
 
-size_t op_smem_bytes(bool fp32, int mode, int R, int TY, int nx, int n_proj) {
+size_t op_smem_bytes(bool fp32, int mode, int R, int TY, int nx, int n_proj, int lz) {
+  static_assert(kMuSlots64 * sizeof(double) == kMuSlots32 * sizeof(float) &&
+                kMuBlockBytes == kOpThreads / 32 * kMuSlots64 * sizeof(double), "mu partials of a block of planes");
   const size_t el = (mode == OP_RESID || !fp32) ? sizeof(double2) : sizeof(float2);
   const size_t cep = mode == OP_RESID ? (size_t)n_proj + kCePad : 0;
-  return el * (2 * (size_t)(TY + 2 * R) * (nx + 2 * R) + cep);
+  const size_t mu = mode == OP_COCG ? (size_t)((lz + kMuPlanes - 1) / kMuPlanes) * kMuBlockBytes : 0;
+  return el * (2 * (size_t)(TY + 2 * R) * (nx + 2 * R) + cep) + mu;
 }
 
 cudaError_t launch_zero(bool fp32, int nslots, int nB, cudaStream_t st, const JuncDev* jt, const BatchDev* b) {

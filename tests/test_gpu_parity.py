@@ -257,6 +257,30 @@ def test_more_tiles_than_a_grid_dimension(B, ppt):
     ctx.close()
 
 
+@pytest.mark.parametrize("nx,R", [(541, 6), (645, 5), (792, 4), (540, 6)])
+def test_planes_that_fill_the_shared_memory(B, nx, R):
+    # ribbons whose x rows with their 2R halo rows take nearly all of an SM's shared
+    # memory in FP64: the operator's partial sums get what is left.  Absorbing
+    # everywhere, so that a column converges in a few iterations.
+    j = P.waveguide(nx, 3, 200, n_cap=16, fd_half_order=R)
+    j = dataclasses.replace(j, gamma_l=j.gamma_l + 0.5, gamma_r=j.gamma_r + 0.5)
+    A = O.system_matrix(j, 0.2)
+    ctx = B.Context(0).set_junction(j)
+    r = np.random.default_rng(1)
+    x = r.standard_normal((1, j.N)) + 1j * r.standard_normal((1, j.N))
+    ref = A @ x[0]
+    y = ctx.apply([0.2], torch.tensor(x, device="cuda"), B.RSN_FP64).cpu().numpy()
+    assert np.abs(y[0] - ref).max() <= 1e-12 * np.abs(ref).max()
+    col = np.array([j.N // 2 + 1, j.N - 3], np.int32)
+    for prec in (B.RSN_FP64, B.RSN_MIXED):
+        g, _, rel = ctx.solve_columns([0.2], col, B.default_opts(prec, tol=1e-10, tol_T=0.0))
+        for k in range(2):
+            res = -(A @ g[0, k].cpu().numpy())
+            res[col[k]] += 1.0
+            assert np.linalg.norm(res) <= 2e-10 and rel[0, k] <= 1e-10
+    ctx.close()
+
+
 @pytest.mark.parametrize("prec", ["fp64", "mixed"])
 def test_open_channel_junction_relative_transmission(B, prec):
     # above the leads' first transverse levels T = O(1): the relative bound is
