@@ -257,8 +257,10 @@ __device__ __forceinline__ void store_pts(C* dst, const int (&at)[U], int end, b
 }
 
 // EARLY: the vectors are requested before the projector term is formed, which
-// takes 90 registers; for launches whose latency counts (upd_early).
-template <typename T, bool EARLY>
+// takes 90 registers; for launches whose latency counts (upd_early).  STAGED: the
+// coefficients are copied to shared memory, as long as they fit (more than about
+// 13,900 projectors in FP64 do not; they are read where they lie).
+template <typename T, bool EARLY, bool STAGED = true>
 __global__ void __launch_bounds__(kUpdThreads, EARLY ? 4 : sizeof(T) == 4 ? 8 : 6)
 cocg_update_kernel(const JuncDev* __restrict__ jt, const BatchDev* __restrict__ bp, int slot_it) {
   using C = typename cx<T>::t;
@@ -282,7 +284,7 @@ cocg_update_kernel(const JuncDev* __restrict__ jt, const BatchDev* __restrict__ 
   const bool fin = isfinite(al.x) && isfinite(al.y);
   extern __shared__ __align__(16) unsigned char upd_smem[];
   C* s_ce = reinterpret_cast<C*>(upd_smem);         // e_kb c_p of the new direction, ce_stride entries
-  C* s_nl = s_ce + b.ce_stride + warp * kBlkPts;    // projector term of the warp's block
+  C* s_nl = s_ce + (STAGED ? b.ce_stride : 0) + warp * kBlkPts;  // projector term of the warp's block
   __shared__ double red[4 * (kUpdThreads / 32)];
   __shared__ int s_last;
   T re = 0, sy = 0, sxy = 0;  // sums of r.x^2 - r.y^2 (cancelling inside the sum), r.y^2, r.x r.y
@@ -313,13 +315,14 @@ cocg_update_kernel(const JuncDev* __restrict__ jt, const BatchDev* __restrict__ 
       const int ra = J.blk_row[blockIdx.x * nw], rb = J.blk_row[min((int)(blockIdx.x + 1) * nw, nblk)];
       if (rb > ra) {  // uniform across the CTA
         const C* cen = reinterpret_cast<const C*>(b.c_e) + (size_t)s * b.ce_stride;
-        for (int e = tid; e < b.ce_stride; e += blockDim.x) s_ce[e] = cen[e];
+        if constexpr (STAGED)
+          for (int e = tid; e < b.ce_stride; e += blockDim.x) s_ce[e] = cen[e];
         if (blk < nblk) {
           row0 = J.blk_row[blk];
           row1 = J.blk_row[blk + 1];
         }
-        __syncthreads();
-        if (row1 > row0) block_nonlocal<T, 1>(J, s_ce, 0, row0, row1, s_nl);
+        if constexpr (STAGED) __syncthreads();
+        if (row1 > row0) block_nonlocal<T, 1>(J, STAGED ? s_ce : cen, 0, row0, row1, s_nl);
       }
     }
 #pragma unroll
@@ -1342,11 +1345,16 @@ cudaError_t launch_cocg_update(bool fp32, int nslots, long long N_max, bool proj
                                cudaStream_t st, const JuncDev* jt, const BatchDev* b) {
   constexpr int nw = kUpdThreads / 32;
   const dim3 grid(upd_ctas(N_max), nslots);
-  const size_t smem = proj ? ((size_t)ce_stride + nw * kBlkPts) * (fp32 ? sizeof(float2) : sizeof(double2)) : 0;
+  const size_t el = fp32 ? sizeof(float2) : sizeof(double2);
+  size_t smem = proj ? ((size_t)ce_stride + nw * kBlkPts) * el : 0;
   const bool early = upd_early(N_max, nslots);
   void (*kern)(const JuncDev*, const BatchDev*, int) =
       fp32 ? (early ? cocg_update_kernel<float, true> : cocg_update_kernel<float, false>)
            : (early ? cocg_update_kernel<double, true> : cocg_update_kernel<double, false>);
+  if (!fp32 && smem + 256 > (size_t)kMaxSmem) {  // (FP32: the true residual's limit comes first)
+    kern = cocg_update_kernel<double, false, false>;
+    smem = nw * kBlkPts * el;
+  }
   if (smem > 32 * 1024) {
     cudaError_t e = set_max_dynamic_smem(reinterpret_cast<const void*>(kern), smem);
     if (e != cudaSuccess) return e;
@@ -1393,11 +1401,12 @@ cudaError_t launch_project(int mode, bool fp32, int nslots, int n_groups, int ma
 
 cudaError_t launch_nonlocal(bool fp32, int n_rhs, long long N, int n_proj, cudaStream_t st, const JuncDev* jt,
                             const BatchDev* b, const void* c, void* y) {
-  constexpr int nw = kUpdThreads / 32;
   const size_t el = fp32 ? sizeof(float2) : sizeof(double2);
+  // four blocks a CTA, one where the coefficients leave no room for the sums of more
+  const int nw = ((size_t)n_proj + kCePad + kUpdThreads / 32 * kBlkPts) * el > (size_t)kMaxSmem ? 1 : kUpdThreads / 32;
   // several vectors a warp where that still leaves every SM a few CTAs and the
   // coefficients fit beside the sums
-  const int gx = upd_ctas(N), many = fp32 ? 4 : 2;
+  const int gx = (blk_count((int)N) + nw - 1) / nw, many = fp32 ? 4 : 2;
   const bool one = (long long)gx * ((n_rhs + many - 1) / many) < 4 * 152 ||
                    many * ((size_t)n_proj + kCePad) * el > 24 * 1024;
   const int spv = one ? 1 : many;
@@ -1409,7 +1418,7 @@ cudaError_t launch_nonlocal(bool fp32, int n_rhs, long long N, int n_proj, cudaS
     cudaError_t e = set_max_dynamic_smem(reinterpret_cast<const void*>(kern), smem);
     if (e != cudaSuccess) return e;
   }
-  kern<<<dim3(gx, (n_rhs + spv - 1) / spv), kUpdThreads, smem, st>>>(jt, b, c, y);
+  kern<<<dim3(gx, (n_rhs + spv - 1) / spv), 32 * nw, smem, st>>>(jt, b, c, y);
   return cudaGetLastError();
 }
 

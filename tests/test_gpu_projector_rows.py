@@ -119,6 +119,40 @@ def test_more_atoms_than_the_staging_holds(B):
     ctx.close()
 
 
+@pytest.mark.parametrize("n", [3000, 6000, 14200, 28700])
+def test_as_many_projectors_as_the_shared_memory_holds(B, n):
+    # coefficients beside the sums of four blocks of points: above 48 KB from 2,544
+    # projectors in FP64 (the update 1,520) and 5,616 in FP32; 14,200 fill an SM's shared
+    # memory in FP64 beside one block's sums (the update reads them where they lie),
+    # 28,700 in FP32.  Bounds as above; a point holds up to 3 n / 640 entries of about
+    # 0.01, which adds little to the roundings of an entry of the result.
+    j = P.tiny_junction(seed=3, nx=4, ny=4, nz=40, fd_half_order=1)
+    j = _with_projectors(j, n, 1, 3, False, 7)
+    j = dataclasses.replace(j, proj_ekb=0.04 * j.proj_ekb)
+    ctx = B.Context(0).set_junction(j)
+    r = np.random.default_rng(0)
+    x = r.standard_normal((5, j.N)) + 1j * r.standard_normal((5, j.N))
+    E = [0.2, 0.21, 0.22, 0.23, 0.24]
+    A = O.system_matrix(j, 0.0)
+    ref = np.stack([A @ v + e * v for e, v in zip(E, x)])
+    for prec, dt, tol in ((B.RSN_FP64, torch.complex128, 1e-13), (B.RSN_MIXED, torch.complex64, 4e-6)):
+        if n > 14200 and prec == B.RSN_FP64:
+            continue
+        y = ctx.apply(E, torch.tensor(x, device="cuda").to(dt), prec).cpu().numpy()
+        assert np.abs(y - ref).max() <= tol * np.abs(ref).max()
+    if n <= 14200:
+        cols = j.right_columns()[:3]
+        A2 = O.system_matrix(j, 0.2)
+        b = np.zeros((j.N, 3), complex)
+        b[cols, np.arange(3)] = 1.0
+        g_ref = np.linalg.solve(A2.toarray(), b).T
+        for prec in (B.RSN_FP64, B.RSN_MIXED):
+            g, _, rel = ctx.solve_columns([0.2], cols, B.default_opts(prec, tol=1e-12, tol_T=0.0))
+            assert rel.max() <= 1e-12
+            assert np.linalg.norm(g[0].cpu().numpy() - g_ref) <= 1e-9 * np.linalg.norm(g_ref)
+    ctx.close()
+
+
 def test_results_do_not_depend_on_the_number_of_systems(B):
     # FP64 columns solved alone, with a few others and in a pool whose z chunks differ
     j = P.molecular_junction(seed=9, nx=10, ny=9, nz=34, n_wells=3, n_cap=4)
