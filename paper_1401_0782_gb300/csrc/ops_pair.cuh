@@ -113,7 +113,8 @@ __device__ __forceinline__ double sum_strided(const float* part, int nw, int ld)
     lo = __fadd_rn(lo, __fadd_rn(__fsub_rn(hi, __fsub_rn(s, bb)), __fsub_rn(a, bb)));
     hi = s;
   }
-  return (double)hi + (double)lo;
+  // (an infinite part makes the error inf - inf; hi is the plain sum)
+  return isfinite(lo) ? (double)hi + (double)lo : (double)hi;
 }
 
 // A running sum that a thread keeps over kMuPlanes planes: FP64 plain, FP32

@@ -153,6 +153,30 @@ def test_as_many_projectors_as_the_shared_memory_holds(B, n):
     ctx.close()
 
 
+def test_infinities_of_an_application(B):
+    # an infinite entry at a support point: the projection is infinite, not NaN, and so
+    # is the result on the rest of the support, in both precisions
+    j = P.tiny_junction(seed=3, nx=8, ny=8, nz=24, fd_half_order=2)
+    j = _with_projectors(j, 1, 1, 700, False, 5)
+    pts = np.asarray(j.proj_idx)
+    x = np.ones((1, j.N), complex)
+    x[0, pts[3]] = np.inf
+    z, yx = np.divmod(np.arange(j.N), 64)
+    far = np.abs(z - z[pts[3]]) > 2
+    sup = np.zeros(j.N, bool)
+    sup[pts] = True
+    v = np.zeros(j.N)
+    v[pts] = np.asarray(j.proj_val)
+    sign = -np.sign(v * v[pts[3]] * j.proj_ekb[0])
+    ctx = B.Context(0).set_junction(j)
+    for prec, dt in ((B.RSN_FP64, torch.complex128), (B.RSN_MIXED, torch.complex64)):
+        y = ctx.apply([0.2], torch.tensor(x, device="cuda").to(dt), prec).cpu().numpy()[0]
+        assert np.all(np.isfinite(y[far & ~sup]))
+        assert np.array_equal(y.real[far & sup], np.where(sign > 0, np.inf, -np.inf)[far & sup]), prec
+        assert np.all(np.isfinite(y.imag[far]))
+    ctx.close()
+
+
 def test_results_do_not_depend_on_the_number_of_systems(B):
     # FP64 columns solved alone, with a few others and in a pool whose z chunks differ
     j = P.molecular_junction(seed=9, nx=10, ny=9, nz=34, n_wells=3, n_cap=4)
