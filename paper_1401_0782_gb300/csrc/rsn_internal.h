@@ -66,6 +66,25 @@ constexpr bool upd_early(long long N, int nslots) {
   return (N + kBlkPts - 1) / kBlkPts * nslots < 16 * 152;
 }
 
+// A near-breakdown (mu or rho almost zero) costs an FP64 recurrence its conjugacy; it
+// may then never converge (about one of 1e5 systems of the 8x8x48 waveguide ran into
+// max_iter at a relative residual of 1e-11 to 1e20).  After iteration `total` of a
+// system left the recurrence residual nrm = ||r||^2 / ||b||^2: true if it has to
+// restart from its true residual, that is past 1e5 times the smallest residual since
+// the last one (rmin2, found at iteration rmin_it), or, once that is within 1e-4 of
+// ||b||, when half as many iterations as the system has done (at least 400) brought no
+// new minimum.  The checks of a goal phase, which leave the recurrence alone, do not
+// touch the count.
+__host__ __device__ inline bool watch_step(double& rmin2, int& rmin_it, double nrm, int total) {
+  const double rm = rmin2;
+  if (nrm < rm) {
+    rmin2 = nrm;
+    rmin_it = total;
+    return false;
+  }
+  return nrm > 1e10 * rm || (rm <= 1e-8 && total - rmin_it > (total / 2 > 400 ? total / 2 : 400));
+}
+
 constexpr int kActBuckets = 14;  // up to 8192 slots
 // The COCG operator's partial sums of mu = p^T A p cover kMuPlanes planes each
 // (per y tile), whatever the z chunks, so that a system's result does not depend
@@ -193,8 +212,8 @@ struct BatchDev {
   double* sigma;        // ||b||: the inner-precision vectors hold r / sigma and d / sigma
   double* rlast2;       // true ||r||^2 at the previous replacement (progress check)
   double* rrec2;        // recurrence ||r / sigma||^2 when the cycle ended (drift check)
-  double* rmin2;        // smallest recurrence ||r / sigma||^2 of the current cycle
-  int* rmin_it;         // its iteration within the cycle
+  double* rmin2;        // smallest recurrence ||r / sigma||^2 since the last true residual
+  int* rmin_it;         // the system's iteration that brought it (watch_step)
   double* tol2;         // recurrence target ||r||^2 of the current cycle
   // vectors
   double2* x64;

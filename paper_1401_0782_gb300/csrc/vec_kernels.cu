@@ -131,21 +131,8 @@ __device__ __forceinline__ void book_slot(const BatchDev& b, const int s, const 
   }
   b.beta_cur[s] = beta;
   b.rho_cur[s] = rho;
-  // A near-breakdown (mu or rho almost zero) costs an FP64 recurrence its
-  // conjugacy; it may then never converge (about one of 1e5 systems of the 8x8x48
-  // waveguide ran into max_iter at a relative residual of 1e-11 to 1e20).  It
-  // restarts from the true residual past 1e5 times the cycle's smallest residual,
-  // or, once within 1e-4 of ||b||, when half as many iterations as the system has
-  // done (at least 400) brought no new minimum.  (The mixed mode has its cycle
-  // cap; shifted systems must keep their one Krylov space.)
-  const double rm = b.rmin2[s];
-  const bool lower = nrm < rm;
-  if (lower) {
-    b.rmin2[s] = nrm;
-    b.rmin_it[s] = cyc;
-  }
-  const bool thrown = !b.handback && b.n_shift == 0 && !lower &&
-                      (nrm > 1e10 * rm || (rm <= 1e-8 && cyc - b.rmin_it[s] > max(400, tot / 2)));
+  // (the mixed mode has its cycle cap; shifted systems must keep their one Krylov space)
+  const bool thrown = watch_step(b.rmin2[s], b.rmin_it[s], nrm, tot) && !b.handback && b.n_shift == 0;
   if (!isfinite(nrm) || thrown) {
     b.restart[s] = 1;
     b.rrec2[s] = thrown ? nrm : 0.0;
@@ -789,7 +776,7 @@ __global__ void __launch_bounds__(kSchedThreads) sched_kernel(const JuncDev* __r
         }
         b.cyc_iters[s] = 0;
         b.rmin2[s] = nrm / bn2;
-        b.rmin_it[s] = 0;
+        b.rmin_it[s] = tot;
         st = SL_ACTIVE;
       }
     }
