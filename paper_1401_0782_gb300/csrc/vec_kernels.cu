@@ -769,6 +769,10 @@ __global__ void __launch_bounds__(kSchedThreads) sched_kernel(const JuncDev* __r
           b.gphase[s] = 1;
           b.rgoal[s] = rel;
           b.gcnt[s] = 0;
+        } else {
+          // (a breakdown or a thrown-off recurrence in the goal phase whose true residual
+          // no longer meets tol: the system has to meet it again first)
+          b.gphase[s] = 0;
         }
         if (st == SL_CHECK) {
           b.n_upd[s] += 1;
