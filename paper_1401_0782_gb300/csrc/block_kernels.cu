@@ -14,7 +14,7 @@
 //   comb_p   P = W tau^{-1} + P beta                     (vectors, FP32)
 //   project + operator (the apply kernels)   AP = A P
 //   gram 0   partial sums of P^T AP                      (b x b, FP32 products)
-//   small 1  alpha, alpha xi                             (b x b, FP64, one warp per block)
+//   small 1  alpha, alpha xi                             (b x b, FP64, one CTA per block)
 //   comb_w   W = W tau^{-1} - AP alpha,  D += P alpha xi (vectors, FP32)
 //   gram 1   partial sums of W^H W and W^T W
 //   small 2  tau, tau^{-1}, xi, Q^T Q, beta; convergence
@@ -360,81 +360,123 @@ __global__ void __launch_bounds__(kBlkThreads) blk_q0_kernel(const BlkDev* __res
 // b x b algebra of each listed block, FP64, one CTA of B * B threads (at least a
 // warp): thread t owns entry (t / B, t % B).  A warp's FP64 instruction takes 64
 // cycles of its FP64 pipe, so what counts is the number of instructions on the
-// longest chain: entries are spread over the four pipes, every elimination step
-// takes one reciprocal (or reciprocal square root) from an FP32 seed and two
-// Newton steps, and the pivot search compares exponent words.  One warp per block
-// took 510 us a phase-2 call and 225 us a phase-1 call at B = 16.
+// longest chain: entries are spread over the four pipes, the divisions of a step over
+// the lanes of one warp, and the pivot search compares bits.  At B = 16 a phase-1 call
+// takes 32 us and a phase-2 call 73 (one warp per block: 225 and 510; Newton
+// reciprocals for the divisions and fused products: 27 and 61, at half again the error).
 // ---------------------------------------------------------------------------
 namespace {
 
-// 1 / a by Newton's iteration from the FP32 reciprocal (24 -> 48 -> 53 bits);
-// a plain division outside the seed's range
-__device__ __forceinline__ double rcp_newton(double a) {
-  const float f = (float)a;
-  if (!(f > 1e-30f && f < 1e30f)) return 1.0 / a;
-  double y = (double)__frcp_rn(f);
-  y = fma(fma(-a, y, 1.0), y, y);
-  return fma(fma(-a, y, 1.0), y, y);
+// acc + a b and acc - a b, the product rounded before it meets acc: in the nearly
+// diagonal systems of a block the products are small beside acc, and a chain of fused
+// additions rounds twice at the size of acc (median error of alpha over 193 systems of
+// three junctions at B = 16: 2.4e-16, fused and with reciprocals 3.6e-16; of the
+// Cholesky factor 8.4e-17 against 1.1e-16)
+__device__ __forceinline__ double2 cmac64(double2 a, double2 b, double2 acc) {
+  return make_double2(acc.x + fma(a.x, b.x, -(a.y * b.y)), acc.y + fma(a.x, b.y, a.y * b.x));
 }
-// 1 / sqrt(a) by Newton's iteration from the FP32 reciprocal square root
-__device__ __forceinline__ double rsqrt_newton(double a) {
-  const float f = (float)a;
-  if (!(f > 1e-30f && f < 1e30f)) return 1.0 / sqrt(a);
-  double y = (double)__frsqrt_rn(f);
-  const double h = 0.5 * a;
-  y = fma(fma(-h * y, y, 0.5), y, y);
-  return fma(fma(-h * y, y, 0.5), y, y);
+__device__ __forceinline__ double2 cmsub64(double2 a, double2 b, double2 acc) {
+  return make_double2(acc.x - fma(a.x, b.x, -(a.y * b.y)), acc.y - fma(a.x, b.y, a.y * b.x));
 }
-
+// acc + a b, fused: for sums of like terms (Q^T Q and the right-hand side of beta, whose
+// median errors are 2.27e-16 and 1.68e-16 with it, 2.34e-16 and 1.87e-16 without)
 __device__ __forceinline__ double2 cfma64(double2 a, double2 b, double2 acc) {
   acc.x = fma(a.x, b.x, fma(-a.y, b.y, acc.x));
   acc.y = fma(a.x, b.y, fma(a.y, b.x, acc.y));
   return acc;
 }
-__device__ __forceinline__ double2 cneg(double2 a) { return make_double2(-a.x, -a.y); }
 __device__ __forceinline__ double2 cconj(double2 a) { return make_double2(a.x, -a.y); }
 
+// Both factorisations below take one barrier a step: while the other warps apply step
+// kk, warp 0 brings the next step's column (or row) up to date and prepares that step,
+// whose divisions are the longest chain.  What a step hands over lies in two buffers,
+// by parity: one is written while slower warps still read the other.
+//
+// The threads that apply a step: all but warp 0 and, of eight warps, the one that
+// shares its FP64 pipe; a single warp does both.
+template <int B>
+__device__ __forceinline__ bool step_worker(int& index, int& count) {
+  constexpr int NW = B * B <= 32 ? 1 : B * B / 32, NWK = NW == 1 ? 1 : NW <= 4 ? NW - 1 : NW - NW / 4;
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  count = 32 * NWK;
+  index = (NW == 1 ? 0 : NW <= 4 ? warp - 1 : warp - warp / 4 - 1) * 32 + lane;
+  return NW == 1 || (warp & 3) != 0;
+}
+
+// Shared memory of the factorisations.
+template <int B>
+struct StepMem {
+  double2 fac[2][B];
+  double ref[B];
+  int piv[B];
+  int ok[2];
+};
+
 // Solve M X = Y in place for aug = [M | Y] (B rows, 2B columns, leading
-// dimension LD): Gauss-Jordan elimination with partial pivoting (the pivot is the
-// entry with the largest real or imaginary part).  X replaces Y.  Returns false
-// (in every thread) on a zero or non-finite pivot.
+// dimension LD): Gauss-Jordan elimination with partial pivoting.  X replaces Y.
+// Returns false (in every thread) on a zero or non-finite pivot.  Rows stay where they
+// are; step k's pivot row is piv[k].
 template <int B, int LD>
-__device__ bool gauss_jordan(double2* aug) {
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  const int er = tid / B, ec = tid % B;
-  for (int kk = 0; kk < B; ++kk) {
-    // every warp finds the pivot for itself (integer instructions only)
-    int key = -1;
-    if (lane >= kk && lane < B) {
+__device__ bool gauss_jordan(double2* aug, StepMem<B>& sm) {
+  const int tid = threadIdx.x, lane = tid & 31;
+  unsigned used = 0;  // warp 0: pivot rows so far
+  // warp 0: the pivot row of column kk (largest modulus) and the factors of the others,
+  // real and imaginary parts in different lanes
+  auto prepare = [&](int kk) {
+    long long key = -1;  // positive doubles order like their bits
+    if (lane < B && !((used >> lane) & 1u)) {
       const double2 v = aug[lane * LD + kk];
-      key = max(__double2hiint(v.x) & 0x7fffffff, __double2hiint(v.y) & 0x7fffffff);
+      key = __double_as_longlong(fma(v.x, v.x, v.y * v.y)) & 0x7fffffffffffffffll;
     }
-    const int best = __reduce_max_sync(0xffffffffu, key);
-    const int piv = __ffs(__ballot_sync(0xffffffffu, key == best)) - 1;
-    if (best <= 0 || best >= 0x7ff00000) return false;  // the same in every warp
-    const double2 p = aug[piv * LD + kk];
-    __syncthreads();  // every warp has read column kk
-    if (warp == 0) {
-      // row kk <- pivot row / pivot, the old row kk moves to the pivot's place
-      const double den = rcp_newton(fma(p.x, p.x, p.y * p.y));
-      const double2 inv = make_double2(p.x * den, -p.y * den);
-      for (int c = lane; c < 2 * B; c += 32) {
-        const double2 top = aug[piv * LD + c];
-        if (piv != kk) aug[piv * LD + c] = aug[kk * LD + c];
-        aug[kk * LD + c] = cfma64(top, inv, make_double2(0.0, 0.0));
+    const int hi = (int)(key >> 32), top = __reduce_max_sync(0xffffffffu, hi);
+    const unsigned lo = hi == top ? (unsigned)key : 0u, low = __reduce_max_sync(0xffffffffu, lo);
+    const int piv = __ffs(__ballot_sync(0xffffffffu, hi == top && lo == low)) - 1;
+    used |= 1u << piv;
+    const int r = lane % B, part = lane / B;
+    const double2 p = aug[piv * LD + kk], v = aug[r * LD + kk];
+    const double num = part ? fma(v.y, p.x, -(v.x * p.y)) : fma(v.x, p.x, v.y * p.y);
+    const double q = num / fma(p.x, p.x, p.y * p.y);
+    if (part < 2) reinterpret_cast<double*>(sm.fac[kk & 1] + r)[part] = q;
+    if (lane == 0) {
+      sm.piv[kk] = piv;
+      sm.ok[kk & 1] = top < 0x7ff00000 && (top > 0 || low > 0) ? 1 : 0;
+    }
+  };
+  if (tid < 32) prepare(0);
+  int w, nwk;
+  const bool worker = step_worker<B>(w, nwk);
+  for (int kk = 0; kk < B; ++kk) {
+    __syncthreads();
+    if (!sm.ok[kk & 1]) return false;
+    const int p = sm.piv[kk];
+    const double2* f = sm.fac[kk & 1];
+    if (tid < 32 && kk + 1 < B) {
+      const int r = lane % B, part = lane / B;
+      if (part < 2 && r != p) {
+        const double2 a = f[r], b = aug[p * LD + kk + 1];
+        const double t = part ? fma(a.x, b.y, a.y * b.x) : fma(a.x, b.x, -(a.y * b.y));
+        reinterpret_cast<double*>(aug + r * LD + kk + 1)[part] -= t;
+      }
+      __syncwarp();
+      prepare(kk + 1);
+    }
+    if (worker) {
+      const int c0 = kk + 1 < B ? kk + 2 : B, nc = 2 * B - c0;
+      for (int e = w; e < (B - 1) * nc; e += nwk) {
+        int r = e / nc;
+        const int c = c0 + e - r * nc;
+        r += r >= p ? 1 : 0;
+        aug[r * LD + c] = cmsub64(f[r], aug[p * LD + c], aug[r * LD + c]);
       }
     }
-    __syncthreads();
-    if (er < B && er != kk) {
-      const double2 f = cneg(aug[er * LD + kk]);
-#pragma unroll
-      for (int h = 0; h < 2; ++h) {
-        const int c = ec + h * B;
-        if (c > kk) aug[er * LD + c] = cfma64(f, aug[kk * LD + c], aug[er * LD + c]);
-      }
-    }
-    __syncthreads();
   }
+  __syncthreads();
+  const int er = tid / B, ec = tid % B;
+  double2 x = make_double2(0.0, 0.0);
+  if (er < B) x = cdiv(aug[sm.piv[er] * LD + B + ec], aug[sm.piv[er] * LD + er]);
+  __syncthreads();
+  if (er < B) aug[er * LD + B + ec] = x;
+  __syncthreads();
   return true;
 }
 
@@ -444,43 +486,53 @@ __device__ bool gauss_jordan(double2* aug) {
 // positive or falls below 1e-12 of its diagonal entry (numerically dependent
 // columns).
 template <int B>
-__device__ bool cholesky_inverse(double2* A, double2* U, double2* Li) {
+__device__ bool cholesky_inverse(double2* A, double2* U, double2* Li, StepMem<B>& sm) {
   const int tid = threadIdx.x, er = tid / B, ec = tid % B;
-  __shared__ double s_ref[B];
   if (er < B) {
     U[tid] = make_double2(0.0, 0.0);
     Li[tid] = make_double2(er == ec ? 1.0 : 0.0, 0.0);
-    if (er == ec) s_ref[er] = A[tid].x;
+    if (er == ec) sm.ref[er] = A[tid].x;
   }
   __syncthreads();
-  for (int kk = 0; kk < B; ++kk) {
+  // warp 0: row kk of U (columns >= kk) and of Li (columns <= kk), real and imaginary
+  // parts in different lanes
+  const int lc = (tid & 31) % B, part = (tid & 31) / B;
+  auto prepare = [&](int kk) {
     const double dd = A[kk * B + kk].x;
-    if (!(dd > 1e-12 * s_ref[kk]) || !(dd <= DBL_MAX)) return false;  // the same in every thread
-    if (tid < B) {
-      // row kk of U (columns >= kk) and of Li (columns <= kk)
-      const double rs = rsqrt_newton(dd);
-      double2 v = tid >= kk ? A[kk * B + tid] : Li[kk * B + tid];
-      v.x *= rs;
-      v.y *= rs;
-      if (tid == kk) {
-        // the diagonal: sqrt(dd) with one correction step; Li's is 1 / sqrt(dd)
-        const double q = dd * rs;
-        U[kk * B + kk] = make_double2(fma(fma(-q, q, dd), 0.5 * rs, q), 0.0);
-        Li[kk * B + kk] = make_double2(rs, 0.0);
-      } else if (tid > kk) {
-        U[kk * B + tid] = v;
-      } else {
-        Li[kk * B + tid] = v;
+    const double dk = sqrt(dd);
+    if (part < 2) {
+      const double v = lc == kk ? (part ? 0.0 : 1.0) : reinterpret_cast<const double*>((lc > kk ? A : Li) + kk * B + lc)[part];
+      reinterpret_cast<double*>((lc > kk ? U : Li) + kk * B + lc)[part] = v / dk;
+      if (tid == kk) U[kk * B + kk] = make_double2(dk, 0.0);
+    }
+    if (tid == 0) sm.ok[kk & 1] = dd > 1e-12 * sm.ref[kk] && dd <= DBL_MAX ? 1 : 0;
+  };
+  if (tid < 32) prepare(0);
+  int w, nwk;
+  const bool worker = step_worker<B>(w, nwk);
+  for (int kk = 0; kk < B; ++kk) {
+    __syncthreads();
+    if (!sm.ok[kk & 1]) return false;
+    if (tid < 32 && kk + 1 < B) {
+      const int r = kk + 1;
+      if (part < 2) {
+        const double2 a = cconj(U[kk * B + r]), b = (lc > kk ? U : Li)[kk * B + lc];
+        const double t = part ? fma(a.x, b.y, a.y * b.x) : fma(a.x, b.x, -(a.y * b.y));
+        reinterpret_cast<double*>((lc > kk ? A : Li) + r * B + lc)[part] -= t;
+      }
+      __syncwarp();
+      prepare(r);
+    }
+    if (worker) {
+      for (int e = (kk + 2) * B + w; e < B * B; e += nwk) {
+        const int r = e / B, c = e % B;
+        const double2 f = cconj(U[kk * B + r]);  // Lc[r][kk]
+        if (c > kk) A[e] = cmsub64(f, U[kk * B + c], A[e]);
+        else Li[e] = cmsub64(f, Li[kk * B + c], Li[e]);
       }
     }
-    __syncthreads();
-    if (er > kk && er < B) {
-      const double2 f = cneg(cconj(U[kk * B + er]));  // -Lc[er][kk]
-      if (ec > kk) A[tid] = cfma64(f, U[kk * B + ec], A[tid]);
-      else Li[tid] = cfma64(f, Li[kk * B + ec], Li[tid]);
-    }
-    __syncthreads();
   }
+  __syncthreads();
   return true;
 }
 
@@ -519,6 +571,7 @@ __global__ void __launch_bounds__(B * B < 32 ? 32 : B * B) blk_small_kernel(cons
   if (PHASE != 0 && d.flag[k] != 0) return;
   __shared__ double2 aug[B * LD];
   __shared__ double2 M0[B * B], M1[B * B], M2[B * B], M3[B * B];
+  __shared__ StepMem<B> sm;
   const size_t ko = (size_t)k * B * B;
   const bool own = tid < B * B;
   const int a = tid / B, j = tid % B;  // the thread's entry
@@ -531,14 +584,14 @@ __global__ void __launch_bounds__(B * B < 32 ? 32 : B * B) blk_small_kernel(cons
       M1[tid] = d.xi[ko + tid];
     }
     __syncthreads();
-    if (!gauss_jordan<B, LD>(aug)) {
+    if (!gauss_jordan<B, LD>(aug, sm)) {
       if (tid == 0) d.flag[k] = 2;
       return;
     }
     if (own) {
       double2 v = zero;  // alpha xi
 #pragma unroll 4
-      for (int m = 0; m < B; ++m) v = cfma64(aug[a * LD + B + m], M1[m * B + j], v);
+      for (int m = 0; m < B; ++m) v = cmac64(aug[a * LD + B + m], M1[m * B + j], v);
       d.alpha[ko + tid] = to32(aug[a * LD + B + j]);
       d.axi[ko + tid] = to32(v);
     }
@@ -550,7 +603,7 @@ __global__ void __launch_bounds__(B * B < 32 ? 32 : B * B) blk_small_kernel(cons
     M1[tid] = G[B * B + tid];  // W^T W
   }
   __syncthreads();
-  if (!cholesky_inverse<B>(M0, M2, M3)) {  // M2 = tau = Lc^H, M3 = Lc^{-1}, tau^{-1} = M3^H
+  if (!cholesky_inverse<B>(M0, M2, M3, sm)) {  // M2 = tau = Lc^H, M3 = Lc^{-1}, tau^{-1} = M3^H
     if (tid == 0) d.flag[k] = 2;
     return;
   }
@@ -600,7 +653,7 @@ __global__ void __launch_bounds__(B * B < 32 ? 32 : B * B) blk_small_kernel(cons
   __syncthreads();  // M1 and the old xi are complete
   double2 xn = zero, rhs = zero;
   if (own) {
-    for (int m = a; m < B; ++m) xn = cfma64(M2[a * B + m], aug[m * B + j], xn);
+    for (int m = a; m < B; ++m) xn = cmac64(M2[a * B + m], aug[m * B + j], xn);
     // right-hand side of beta: tau^T QQ_{k+1}
     for (int m = 0; m <= a; ++m) rhs = cfma64(M2[m * B + a], M1[m * B + j], rhs);
     d.xi[ko + tid] = xn;
@@ -620,7 +673,7 @@ __global__ void __launch_bounds__(B * B < 32 ? 32 : B * B) blk_small_kernel(cons
     aug[a * LD + B + j] = rhs;
   }
   conv = __syncthreads_and(conv);
-  const bool ok = gauss_jordan<B, LD>(aug);
+  const bool ok = gauss_jordan<B, LD>(aug, sm);
   if (own) {
     d.QQ[ko + tid] = M1[tid];
     if (ok) d.beta[ko + tid] = to32(aug[a * LD + B + j]);
