@@ -442,15 +442,16 @@ cudaError_t launch_op_r(int mode, bool fp32, int ppt, dim3 grid, int threads, si
 // copies (TMA) in a ring of kStages shared-memory stages, issued kStages
 // planes ahead, so the bytes in flight do not occupy registers.  One thread
 // per grid point keeps only the 2R+1-deep z queue.  Used for OP_COCG and
-// OP_APPLY when every plane and slot offset is 16-byte aligned.
+// OP_APPLY in FP32 when every plane and slot offset is 16-byte aligned.
 // ---------------------------------------------------------------------------
 constexpr int kStages = 4;
 
-template <typename T, int R, int MODE>
+template <int R, int MODE>
 __global__ void __launch_bounds__(1024, 1)
 op_kernel_tma(const JuncDev* __restrict__ jt, const BatchDev* __restrict__ bp, const void* __restrict__ x_in,
               void* __restrict__ y_out) {
-  using C = typename cx<T>::t;
+  using T = float;
+  using C = float2;
   constexpr int Q = 2 * R + 1;
   constexpr int NIN = (MODE == OP_COCG) ? 2 : 1;
   const BatchDev& b = *bp;
@@ -476,7 +477,7 @@ op_kernel_tma(const JuncDev* __restrict__ jt, const BatchDev* __restrict__ bp, c
   uint64_t* bars = reinterpret_cast<uint64_t*>(
       (reinterpret_cast<uintptr_t>(exch + 2 * prow * pitch) + 15) & ~static_cast<uintptr_t>(15));
   // mu partials (COCG): [block of planes][warp][re, im]
-  __shared__ __align__(8) T s_mu[MODE == OP_COCG ? kMaxLz / kMuPlanes * 32 * (sizeof(T) == 8 ? kMuSlots64 : kMuSlots32) : 1];
+  __shared__ __align__(8) T s_mu[MODE == OP_COCG ? kMaxLz / kMuPlanes * 32 * kMuSlots32 : 1];
   __shared__ int s_bad;
 
   for (int i = tid; i < 2 * prow * pitch; i += nt) exch[i] = czero<C>();
@@ -523,20 +524,17 @@ op_kernel_tma(const JuncDev* __restrict__ jt, const BatchDev* __restrict__ bp, c
   const int so = (yy + R) * pitch + xx + R;
   T wst[R + 1];
 #pragma unroll
-  for (int m = 1; m <= R; ++m) {
-    if constexpr (sizeof(T) == 8) wst[m] = (T)J.w64[m];
-    else wst[m] = (T)J.w32[m];
-  }
+  for (int m = 1; m <= R; ++m) wst[m] = J.w32[m];
   C qv[Q];
 #pragma unroll
   for (int m = 0; m < Q; ++m) qv[m] = czero<C>();
-  typename std::conditional<sizeof(T) == 8, MuSum64, MuSum32>::type mu;  // of kMuPlanes planes
+  MuSum32 mu;  // of kMuPlanes planes
   // per-point operator data of the next plane to compute, loaded one plane early
   float2 dg_n = make_float2(0.f, 0.f);
   auto load_pt = [&](int z) {
     if (own && z < z1) {
       const long long g = (long long)z * plane + tid;
-      if constexpr (sizeof(T) == 4) dg_n = J.dg32[g];
+      dg_n = J.dg32[g];
     }
   };
   load_pt(z0);
@@ -574,38 +572,18 @@ op_kernel_tma(const JuncDev* __restrict__ jt, const BatchDev* __restrict__ bp, c
     }
     if (zc < z0) continue;
     if (own) {
-    const float2 dg_c = dg_n;
-    load_pt(zc + 1);
-
-    const C vc = qv[R];
-    const long long gl = (long long)zc * plane + tid;
-    C y;
-    if constexpr (sizeof(T) == 8) {
-      C lap = czero<C>();
-#pragma unroll
-      for (int m = 1; m <= R; ++m) {
-        C sm = cadd(qv[R - m], qv[R + m]);
-        sm = cadd(sm, cadd(smb[so - m], smb[so + m]));
-        sm = cadd(sm, cadd(smb[so - m * pitch], smb[so + m * pitch]));
-        lap = rfma(wst[m], sm, lap);
-      }
-      const double2 t = J.dg64[gl];
-      y = cfma(mk2((T)(E + t.x), (T)t.y), vc, lap);
-    } else {
-      y = fd_diff_form<C, T, R>(qv, smb, so, pitch, wst, vc, dg_c, E);
-    }
-    if constexpr (MODE == OP_COCG) {
-      pnew[vo + gl] = vc;
-      reinterpret_cast<C*>(b.q)[vo + gl] = y;
-      if constexpr (sizeof(T) == 8) {
-        mu.re = fma(vc.x, y.x, fma(-vc.y, y.y, mu.re));
-        mu.im = fma(vc.x, y.y, fma(vc.y, y.x, mu.im));
-      } else {
+      const float2 dg_c = dg_n;
+      load_pt(zc + 1);
+      const C vc = qv[R];
+      const long long gl = (long long)zc * plane + tid;
+      const C y = fd_diff_form<C, T, R>(qv, smb, so, pitch, wst, vc, dg_c, E);
+      if constexpr (MODE == OP_COCG) {
+        pnew[vo + gl] = vc;
+        reinterpret_cast<C*>(b.q)[vo + gl] = y;
         mu.add(fma(vc.x, y.x, -vc.y * y.y), fma(vc.x, y.y, vc.y * y.x));
+      } else {
+        reinterpret_cast<C*>(y_out)[vo + gl] = y;
       }
-    } else {
-      reinterpret_cast<C*>(y_out)[vo + gl] = y;
-    }
     }
     if constexpr (MODE == OP_COCG) {
       if ((zc - z0) % kMuPlanes == kMuPlanes - 1 || zc == z1 - 1) {
@@ -620,8 +598,9 @@ template <int R>
 cudaError_t launch_op_tma_r(int mode, bool fp32, dim3 grid, int threads, size_t smem, cudaStream_t st,
                             const JuncDev* jt, const BatchDev* b, const void* x_in, void* y_out) {
   void (*kern)(const JuncDev*, const BatchDev*, const void*, void*) = nullptr;
-  if (mode == OP_COCG) kern = fp32 ? op_kernel_tma<float, R, OP_COCG> : op_kernel_tma<double, R, OP_COCG>;
-  else if (mode == OP_APPLY) kern = fp32 ? op_kernel_tma<float, R, OP_APPLY> : op_kernel_tma<double, R, OP_APPLY>;
+  if (!fp32) return cudaErrorInvalidValue;
+  if (mode == OP_COCG) kern = op_kernel_tma<R, OP_COCG>;
+  else if (mode == OP_APPLY) kern = op_kernel_tma<R, OP_APPLY>;
   else return cudaErrorInvalidValue;
   if (smem > 16 * 1024) {  // beside the static arrays
     cudaError_t e = set_max_dynamic_smem(reinterpret_cast<const void*>(kern), smem);

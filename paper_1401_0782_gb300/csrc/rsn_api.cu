@@ -347,7 +347,7 @@ static Tiling choose_tiling(const rsn_ctx* c, bool compute64, int mode, int nslo
   // whose byte sizes keep every bulk copy 16-byte aligned
   if (!compute64 && mode != OP_RESID && streamable && pl <= 1024 && (pl * 8) % 16 == 0 && (c->N * 8) % 16 == 0 &&
       c->tile_override[3] == -1) {
-    const size_t sm = op_tma_smem_bytes(true, mode, R, nx, ny);
+    const size_t sm = op_tma_smem_bytes(mode, R, nx, ny);
     if (sm <= 200 * 1024) {
       t.tma = true;
       t.TY = ny;

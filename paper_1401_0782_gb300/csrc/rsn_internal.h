@@ -378,7 +378,7 @@ size_t op_smem_bytes(bool fp32, int mode, int R, int TY, int nx, int n_proj, int
 // plane-streaming (TMA) operator kernel for whole-plane tiles (OP_COCG / OP_APPLY)
 cudaError_t launch_op_tma(int mode, bool fp32, int R, dim3 grid, int threads, size_t smem, cudaStream_t st,
                           const JuncDev* jt, const BatchDev* b, const void* x_in, void* y_out);
-size_t op_tma_smem_bytes(bool fp32, int mode, int R, int nx, int ny);
+size_t op_tma_smem_bytes(int mode, int R, int nx, int ny);
 // FP32 point-pair operator kernel with plane streaming (OP_COCG / OP_APPLY):
 // whole planes, nx even, 16-byte aligned vectors; big: the one-CTA-per-SM
 // variant for planes of more than 2 * kPairThreads points

@@ -1310,8 +1310,8 @@ size_t op_pair_smem_bytes(int mode, int R, int nx, int ny) {
          8 * kPairStages;
 }
 
-size_t op_tma_smem_bytes(bool fp32, int mode, int R, int nx, int ny) {
-  const size_t el = fp32 ? sizeof(float2) : sizeof(double2);
+size_t op_tma_smem_bytes(int mode, int R, int nx, int ny) {
+  const size_t el = sizeof(float2);
   const size_t nin = mode == OP_COCG ? 2 : 1;
   return el * (kStages * nin * (size_t)nx * ny + 2 * (size_t)(nx + 2 * R) * (ny + 2 * R)) + 16 + 8 * kStages;
 }
