@@ -63,12 +63,12 @@ struct Tiling {
   size_t smem = 0;
   bool tma = false;   // whole-plane tile streamed by bulk copies (op_kernel_tma)
   bool pair = false;  // FP32 point-pair kernel with plane streaming (op_pair_kernel)
+  int pitch = 0;      // its compile-time row pitch (0: none)
+  bool big = false;   // its one-CTA-per-SM variant (planes of more than 2 * kPairThreads points)
   bool plane = false; // FP32 one-point-per-thread kernel with plane streaming (op_plane_kernel)
   int parts = 0;      // COCG: mu partials per slot
   // COCG: planes per chunk and CTAs per slot when at most 2^k slots are busy
   int lz_act[kActBuckets] = {0}, n_act[kActBuckets] = {0};
-  int pitch = 0;      // its compile-time row pitch (0: none)
-  bool big = false;   // its one-CTA-per-SM variant (planes of more than 2 * kPairThreads points)
 };
 
 // Slot pool of the streaming solver (sized for S slots of N points).
@@ -2150,7 +2150,7 @@ static rsn_status block_impl(rsn_ctx* c, int n_e, const double* E, int n_cols, c
         RSN_CUDA(c, launch_blk_gram64(B, na2, nchunk, c->st, dd));
         RSN_CUDA(c, launch_blk_small(B, 0, na2, c->st, dd));
         RSN_CUDA(c, launch_blk_q0(B, na2, c->st, dd, N));
-        c->st_launches += 4;
+        c->st_launches += 5;
         std::vector<int> in = act;
         const int kChunk = 8;
         while (!in.empty()) {
@@ -2163,7 +2163,7 @@ static rsn_status block_impl(rsn_ctx* c, int n_e, const double* E, int n_cols, c
             RSN_CUDA(c, launch_blk_comb_w(B, ni, c->st, dd, N));
             RSN_CUDA(c, launch_blk_gram(B, 1, ni, nchunk, c->st, dd));
             RSN_CUDA(c, launch_blk_small(B, 2, ni, c->st, dd));
-            c->st_launches += 6;
+            c->st_launches += 8;
           }
           RSN_CUDA(c, cudaMemcpyAsync(flags.data(), q.flag.p, (size_t)nbw * sizeof(int), cudaMemcpyDeviceToHost, c->st));
           RSN_CUDA(c, cudaStreamSynchronize(c->st));

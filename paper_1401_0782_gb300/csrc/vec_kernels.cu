@@ -1024,7 +1024,11 @@ __global__ void __launch_bounds__(256) grad_sys_kernel(int nsys, long long N, co
 // (alpha_{-1} = 1, beta_{-1} = 0, pi_{-1} = pi_0 = 1, p_{e,0} = b).  What is kept
 // is the scaled direction g_e = pi_{e,k} p_e, which needs no product with r:
 //   x_e += (alpha_k / pi_{k+1}) g_e,  g_e = r_{k+1} + (beta_k pi_k / pi_{k+1}) g_e
-// (8 instead of 12 operations of the FP64 pipe per shift and tracked point; the
+// (products with conj(pi) / |pi|^2 instead of quotients; in a model of 288 shifted
+// systems of three junctions on the same seed scalars, the iterates' median error
+// against extended precision is 3.1e-15, 3.2e-15 with quotients and p_e, the rms 1.3e-11
+// both ways;
+// 8 instead of 12 operations of the FP64 pipe per shift and tracked point; the
 // loads of four shifts are in flight together; 16 systems x 16 shifts x 4,608
 // points: 43 -> 37 us in one CTA row, against 16 of FP64 work).  The seed
 // runs the FP64 slot solver unchanged; the shifted iterates live only on the

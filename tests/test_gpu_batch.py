@@ -126,8 +126,7 @@ def test_batch_right_after_new_projectors(B):
         c.close()
 
 
-@pytest.mark.parametrize("ppt", [0, -1, -2, -3])
-def test_batch_slots_stay_aligned_beside_an_odd_junction(B, ppt):
+def test_batch_slots_stay_aligned_beside_an_odd_junction(B):
     # The largest junction has an odd number of points (the register kernel), the
     # others run kernels that copy whole planes in 16-byte units: even nx, odd nx
     # with an even plane.  An odd and an even number of columns, so that the even
@@ -137,16 +136,17 @@ def test_batch_slots_stay_aligned_beside_an_odd_junction(B, ppt):
           for k, (nx, ny, nz) in enumerate(specs)]
     assert js[0].N % 2 == 1 and js[0].N == max(j.N for j in js)
     ctxs = [B.Context(0).set_junction(j) for j in js]
-    for c in ctxs:
-        c.set_tiling(0, 12 if ppt == -1 else 0, ppt)
     energies = [[0.19, 0.23]] * len(js)
     cols = [j.right_columns()[: 5 + k] for k, j in enumerate(js)]
     opts = B.default_opts(B.RSN_MIXED)
-    T = B.batch_transmission(ctxs, energies, cols, opts)
-    for k, j in enumerate(js):
-        T_ref = O.transmission(j, energies[k], cols[k])
-        assert np.all(np.abs(T[k] - T_ref) <= 1e-6), (k, T[k], T_ref)
-        T_alone = ctxs[k].transmission(energies[k], cols[k], opts)
-        assert np.all(np.abs(T[k] - T_alone) <= 1e-6), (k, T[k], T_alone)
+    T_ref = [O.transmission(j, e, c) for j, e, c in zip(js, energies, cols)]
+    for ppt in (0, -1, -2, -3):
+        for c in ctxs:
+            c.set_tiling(0, 0, ppt)
+        T = B.batch_transmission(ctxs, energies, cols, opts)
+        for k in range(len(js)):
+            assert np.all(np.abs(T[k] - T_ref[k]) <= 1e-6), (ppt, k, T[k], T_ref[k])
+            T_alone = ctxs[k].transmission(energies[k], cols[k], opts)
+            assert np.all(np.abs(T[k] - T_alone) <= 1e-6), (ppt, k, T[k], T_alone)
     for c in ctxs:
         c.close()
