@@ -79,8 +79,10 @@ __device__ __forceinline__ double warp_sum2_exact(double re, double im) {
   return __ll2double_rn(s) * __longlong_as_double((long long)((odd ? ti : tr) - 57) << 52);
 }
 
-// The sum of n complex values over a warp, in every lane.
-__device__ __forceinline__ double2 warp_sum_parts(const double2* part, int n) {
+// The sum of n complex values over a warp, in every lane.  Not inlined: inside the FP32
+// register operator it upset the allocation of the march's 64 registers (24 uneven
+// junctions: 619 us a launch, 506 as a call).
+static __device__ __noinline__ double2 warp_sum_parts(const double2* part, int n) {
   constexpr int KEEP = 4, GUARD = 40;  // values a lane keeps between the passes; n < 2^33
   const int lane = threadIdx.x & 31;
   const bool odd = (lane & 1) != 0;
