@@ -11,13 +11,12 @@
 
 namespace rsn {
 
-// bits of a double as a multiple of 2^(top - 1075 - GUARD), rounded; top: the largest
+// bits of a double as a multiple of 2^(top - 1075 - guard), rounded; top: the largest
 // biased exponent of the sum's values
-template <int GUARD>
-__host__ __device__ __forceinline__ long long to_fixed(long long bits, int top) {
+__host__ __device__ __forceinline__ long long to_fixed(long long bits, int top, int guard) {
   const int e = (int)(bits >> 52) & 0x7ff;
   long long m = bits & 0xfffffffffffffll;
-  m = (e ? m | 0x10000000000000ll : m) << GUARD;
+  m = (e ? m | 0x10000000000000ll : m) << guard;
   const int sh = top - (e ? e : 1);
   m = sh < 62 ? (m + ((1ll << sh) >> 1)) >> sh : 0;
   return bits < 0 ? -m : m;
@@ -71,7 +70,7 @@ __device__ __forceinline__ double warp_sum2_exact(double re, double im) {
     double v[2] = {re, im};
     return warp_sum_many<2>(v);
   }
-  const long long a = to_fixed<5>(__double_as_longlong(re), tr), b = to_fixed<5>(__double_as_longlong(im), ti);
+  const long long a = to_fixed(__double_as_longlong(re), tr, 5), b = to_fixed(__double_as_longlong(im), ti, 5);
   long long s = (odd ? b : a) + __shfl_xor_sync(0xffffffffu, odd ? a : b, 1);
 #pragma unroll
   for (int w = 2; w < 32; w <<= 1) s += __shfl_xor_sync(0xffffffffu, s, w);
@@ -79,9 +78,10 @@ __device__ __forceinline__ double warp_sum2_exact(double re, double im) {
   return __ll2double_rn(s) * __longlong_as_double((long long)((odd ? ti : tr) - 57) << 52);
 }
 
-// The sum of n complex values over a warp, in every lane.  Not inlined: inside the FP32
-// register operator it upset the allocation of the march's 64 registers (24 uneven
-// junctions: 619 us a launch, 506 as a call).
+// The sum of n >= 1 complex values over a warp, in every lane: in 64 bits, or, for many
+// values, in 128.  Not inlined: inside an operator kernel it upset the allocation of
+// the march's registers (FP32 register kernel, 24 uneven junctions: 619 us a launch,
+// 506 as a call).
 static __device__ __noinline__ double2 warp_sum_parts(const double2* part, int n) {
   constexpr int KEEP = 4, GUARD = 40;  // values a lane keeps between the passes; n < 2^33
   const int lane = threadIdx.x & 31;
@@ -114,6 +114,28 @@ static __device__ __noinline__ double2 warp_sum_parts(const double2* part, int n
     }
     const double t = warp_sum_many<2>(v);
     return make_double2(__shfl_sync(0xffffffffu, t, 0), __shfl_sync(0xffffffffu, t, 1));
+  }
+  if (n <= 512 && min(tr, ti) >= 80) {
+    // 64 bits: at least one bit below the last one of the largest value for up to 256
+    // values (110 of them, rounded to a quarter of it: 0.8 of it rms, which is less than
+    // the rounding of a total a few times as large)
+    const int guard = 9 - (32 - __clz(n - 1));
+    long long re = 0, im = 0;
+#pragma unroll
+    for (int k = 0; k < KEEP; ++k) {
+      re += to_fixed(__double_as_longlong(w[k].x), tr, guard);
+      im += to_fixed(__double_as_longlong(w[k].y), ti, guard);
+    }
+    for (int t = lane + 32 * KEEP; t < n; t += 32) {
+      const double2 v = __ldcg(part + t);
+      re += to_fixed(__double_as_longlong(v.x), tr, guard);
+      im += to_fixed(__double_as_longlong(v.y), ti, guard);
+    }
+    long long s = (odd ? im : re) + __shfl_xor_sync(0xffffffffu, odd ? re : im, 1);
+#pragma unroll
+    for (int x = 2; x < 32; x <<= 1) s += __shfl_xor_sync(0xffffffffu, s, x);
+    const double v = __ll2double_rn(s) * __longlong_as_double((long long)((odd ? ti : tr) - 52 - guard) << 52);
+    return make_double2(__shfl_sync(0xffffffffu, v, 0), __shfl_sync(0xffffffffu, v, 1));
   }
   i128 re = 0, im = 0;
 #pragma unroll

@@ -67,10 +67,25 @@ __device__ __forceinline__ int cocg_parts(const JuncDev& J) {
 }
 
 // alpha = rho / mu of slot s, by a warp, once all its mu partials are written: the
-// operator's and the J.n_groups projections' partials, rounded once.
+// operator's and the J.n_groups projections' partials added, FP64's in fixed point
+// (FP32's, which carry their own rounding errors, in a shuffle tree).
+template <bool FP64>
 __device__ __forceinline__ void mu_alpha(const BatchDev& b, const JuncDev& J, const int s) {
-  const int lane = threadIdx.x & 31;
-  const double2 mu = warp_sum_parts(b.mu_part + (size_t)s * b.PA, cocg_parts(J) + J.n_groups);
+  const int lane = threadIdx.x & 31, n = cocg_parts(J) + J.n_groups;
+  const double2* part = b.mu_part + (size_t)s * b.PA;
+  double2 mu;
+  if constexpr (FP64) {
+    mu = warp_sum_parts(part, n);
+  } else {
+    double v[2] = {0.0, 0.0};
+    for (int t = lane; t < n; t += 32) {
+      const double2 w = __ldcg(part + t);
+      v[0] += w.x;
+      v[1] += w.y;
+    }
+    const double t = warp_sum_many<2>(v);
+    mu = make_double2(__shfl_sync(0xffffffffu, t, 0), __shfl_sync(0xffffffffu, t, 1));
+  }
   const double2 a = cdiv_warp(b.rho_cur[s], mu);
   if (lane == 0) {
     b.mu_cnt[s] = 0;
@@ -196,7 +211,7 @@ __device__ __forceinline__ void mu_finish(const BatchDev& b, const JuncDev& J, i
   __threadfence();
   __syncwarp();
   const bool last = threadIdx.x == 0 && mu_arrive(b, J, s);
-  if (__any_sync(0xffffffffu, last)) mu_alpha(b, J, s);
+  if (__any_sync(0xffffffffu, last)) mu_alpha<sizeof(A) == 8>(b, J, s);
 }
 
 struct Pair {

@@ -552,7 +552,7 @@ __global__ void __launch_bounds__(kProjThreads) project_kernel(const JuncDev* __
         const unsigned last = __ballot_sync(0xffffffffu, lane < SPB && s_slot[lane < SPB ? lane : 0] >= 0 &&
                                                              mu_arrive(b, J, s_slot[lane < SPB ? lane : 0]));
         for (int v = 0; v < SPB; ++v)
-          if ((last >> v) & 1u) mu_alpha(b, J, s_slot[v]);
+          if ((last >> v) & 1u) mu_alpha<sizeof(T) == 8>(b, J, s_slot[v]);
       }
     }
   }  // list entries

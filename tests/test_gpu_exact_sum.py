@@ -98,10 +98,12 @@ def test_warp_sums(lib, kind):
             assert _off(got[k, c], exact) <= tol, (k, c, got[k, c], ref)
 
 
-@pytest.mark.parametrize("n", [1, 2, 31, 32, 33, 110, 127, 128, 129, 1000, 2000])
+@pytest.mark.parametrize("n", [1, 2, 31, 32, 33, 110, 127, 128, 129, 512, 513, 1000, 2000])
 @pytest.mark.parametrize("kind", KINDS)
 def test_sums_of_parts_are_rounded_once(lib, kind, n):
-    # values below 2^-40 of the largest one's last place are cut off there
+    # up to 512 values every one is rounded to 2^-guard of the largest one's last place,
+    # guard = 9 - ceil(log2 n); of more, what lies below 2^-40 of it is cut off
+    each = 2.0 ** -(10 - (n - 1).bit_length()) if n <= 512 else 2.0 ** -40
     v = _values(kind, (n,), np.random.default_rng(n))
     dev, out = torch.tensor(v, device="cuda"), torch.zeros(32, dtype=torch.complex128, device="cuda")
     torch.cuda.synchronize()
@@ -110,7 +112,7 @@ def test_sums_of_parts_are_rounded_once(lib, kind, n):
     assert np.all(got == got[0])
     for g, w in ((got[0].real, v.real), (got[0].imag, v.imag)):
         ref = math.fsum(w)
-        assert _off(g, _exact(w)) <= n * 2.0 ** -40 * math.ulp(np.abs(w).max()) + 0.5001 * math.ulp(abs(ref)), (g, ref)
+        assert _off(g, _exact(w)) <= n * each * math.ulp(np.abs(w).max()) + 0.5001 * math.ulp(abs(ref)), (g, ref)
 
 
 def test_many_parts(lib):
