@@ -396,8 +396,9 @@ rsn_status rsn_autotune(rsn_ctx* ctx, int precision, int nslots, int* TY, int* L
    two CTAs per SM up to 576 points); else, for planes of an even number of at
    most 576 points, the plane kernel (the same with one point per thread);
    everything else, and FP64, the register-prefetch kernel.  Lz sets the
-   planes per CTA of any of them (rounded up to a multiple of four, at most 128;
-   a COCG result does not depend on it).  TY rows of the x-y plane per CTA and ppt
+   planes per CTA of any of them (rounded up to a multiple of four, at most 128,
+   fewer where the widest planes leave little shared memory; a COCG result does
+   not depend on it).  TY rows of the x-y plane per CTA and ppt
    owned points per thread (1..4) select the register-prefetch kernel; ppt = -1
    the whole-plane bulk-copy kernel with a shifted register queue (FP32, planes
    of at most 1024 points with 16-byte aligned sizes); ppt = -2 the point-pair
